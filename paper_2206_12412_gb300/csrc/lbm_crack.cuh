@@ -59,19 +59,19 @@ struct CrackSums {
 
 // Step (1) for one end, by a group of G lanes (32: a warp; 16: a half warp,
 // so that one warp evaluates both ends at once); every lane of the group
-// gets the sums.  Reads S only.  All 32 lanes of the warp must call it.
-template <typename T, int G = 32>
-__device__ __forceinline__ CrackSums crack_eval_warp(const CrackParams &p, const T *w, int64_t P, const uint32_t *cut_v,
-                                                     const CrackState &S, int dir)
+// gets the sums.  tip, v_prev: the end's tip and previous speed; i_first,
+// i_last: the severed columns; fetch(i, above, below) reads the pair of
+// column i and tells whether its link is severed.  All 32 lanes of the warp
+// must call it.
+template <typename T, int G, typename F>
+__device__ __forceinline__ CrackSums crack_eval_pairs(const CrackParams &p, int64_t tip, double v_prev, int i_first,
+                                                      int i_last, int dir, F &&fetch)
 {
     const int lane = threadIdx.x & (G - 1);
-    const TipState &E = dir > 0 ? S.r : S.l;
-    const int64_t tip = E.tip_q;
-    const int i_first = S.i_first, i_last = S.i_last;
     // eq. r(v); the divisions are skipped where they are exact (v = 0, dh = 1):
     // FP64 instructions are few per cycle on GB300, and this chain is on
     // the crack step's critical path
-    const double r_min = p.r_min_fixed > 0.0 ? p.r_min_fixed : (E.v_prev == 0.0 ? p.r0 : p.r0 / (1.0 - E.v_prev));
+    const double r_min = p.r_min_fixed > 0.0 ? p.r_min_fixed : (v_prev == 0.0 ? p.r0 : p.r0 / (1.0 - v_prev));
     const double lo = p.dh == 1.0 ? r_min : r_min / p.dh;
     const double hi = p.dh == 1.0 ? r_min + p.fit_width : (r_min + p.fit_width) / p.dh;
     const double tip_h = (double)tip * kTwoM32;
@@ -85,16 +85,14 @@ __device__ __forceinline__ CrackSums crack_eval_warp(const CrackParams &p, const
     }
     c_lo = c_lo < i_first ? i_first : c_lo;
     c_hi = c_hi > i_last ? i_last : c_hi;
-    const int jc = p.jc;
     double num = 0.0, den = 0.0;
     int np = 0;
     for (int i = c_lo + lane; i <= c_hi; i += G) {
         // the pair's fields are loaded together with its mask word (the
         // columns lie in [i_first, i_last], inside the lattice), so the two
         // loads cost one round trip
-        const uint32_t word = cut_v[(int64_t)(jc - 1) * p.words + (i >> 5)];
-        const T above = w[(int64_t)jc * P + i], below = w[(int64_t)(jc - 1) * P + i];
-        if (!((word >> (i & 31)) & 1u)) continue;
+        T above, below;
+        if (!fetch(i, above, below)) continue;
         const int64_t xq = (int64_t)(2 * i + 1) << (kQBits - 1);
         const double r_h = (double)(dir > 0 ? tip - xq : xq - tip) * kTwoM32;
         if (!(r_h >= lo && r_h < hi)) continue;
@@ -108,9 +106,11 @@ __device__ __forceinline__ CrackSums crack_eval_warp(const CrackParams &p, const
     // with the pairs in one lane of the group (the one-pair window W = dh
     // always), that lane's sums are the group's: adding the other lanes'
     // zeros cannot change them, so one shuffle replaces the reduction tree
+    // (only where that holds for every group of the warp: the shuffles of
+    // both branches name all 32 lanes, so the warp takes one of them whole)
     const unsigned gmask = G == 32 ? 0xffffffffu : (0xffffu << (threadIdx.x & 16));
     const unsigned holders = __ballot_sync(0xffffffffu, np > 0) & gmask;
-    if (__popc(holders) <= 1) {
+    if (__all_sync(0xffffffffu, __popc(holders) <= 1)) {
         const int src = holders ? __ffs(holders) - 1 : (threadIdx.x & 31 & ~(G - 1));
         num = __shfl_sync(0xffffffffu, num, src);
         den = __shfl_sync(0xffffffffu, den, src);
@@ -124,6 +124,21 @@ __device__ __forceinline__ CrackSums crack_eval_warp(const CrackParams &p, const
         np += __shfl_xor_sync(0xffffffffu, np, o);
     }
     return CrackSums{num, den, r_min, np};
+}
+
+// The same with the fields in device memory.  Reads S only.
+template <typename T, int G = 32>
+__device__ __forceinline__ CrackSums crack_eval_warp(const CrackParams &p, const T *w, int64_t P, const uint32_t *cut_v,
+                                                     const CrackState &S, int dir)
+{
+    const TipState &E = dir > 0 ? S.r : S.l;
+    const int jc = p.jc;
+    return crack_eval_pairs<T, G>(p, E.tip_q, E.v_prev, S.i_first, S.i_last, dir, [&](int i, T &above, T &below) {
+        const uint32_t word = cut_v[(int64_t)(jc - 1) * p.words + (i >> 5)];
+        above = w[(int64_t)jc * P + i];
+        below = w[(int64_t)(jc - 1) * P + i];
+        return ((word >> (i & 31)) & 1u) != 0u;
+    });
 }
 
 // K from the sums (eq. sif; least squares when the window holds several
@@ -166,7 +181,8 @@ __device__ __forceinline__ CrackDecision crack_decide(const CrackParams &p, cons
 }
 
 // Step (3) for one end, by one thread: the advance, the severed links, this
-// end's fields of S and, if `commit`, its history record.
+// end's fields of S and, if `commit`, its history record.  cut_v may be null
+// (the caller sets the mask's bits).
 __device__ __forceinline__ void crack_commit(const CrackParams &p, uint32_t *cut_v, const History &hist, CrackState &S,
                                              int dir, bool commit, const CrackSums &c, const CrackDecision &d)
 {
@@ -191,7 +207,7 @@ __device__ __forceinline__ void crack_commit(const CrackParams &p, uint32_t *cut
                 int64_t last = (next - half) >> kQBits;   // largest i with x_i <= next
                 if (last > p.nx - 1) last = p.nx - 1;
                 for (int64_t i = (int64_t)i_last + 1; i <= last; ++i) {
-                    if (i < i_first) continue;
+                    if (i < i_first || !cut_v) continue;
                     atomicOr(&cut_v[(int64_t)jr * p.words + (i >> 5)], 1u << (i & 31));
                 }
                 if (last > i_last && last >= i_first) S.i_last = (int32_t)last;
@@ -205,7 +221,7 @@ __device__ __forceinline__ void crack_commit(const CrackParams &p, uint32_t *cut
                 int64_t first = (next - half + ((int64_t)1 << kQBits) - 1) >> kQBits;   // smallest i with x_i >= next
                 if (first < 0) first = 0;
                 for (int64_t i = first; i < (int64_t)i_first; ++i) {
-                    if (i > i_last) continue;
+                    if (i > i_last || !cut_v) continue;
                     atomicOr(&cut_v[(int64_t)jr * p.words + (i >> 5)], 1u << (i & 31));
                 }
                 if (first < i_first && first <= i_last) S.i_first = (int32_t)first;
