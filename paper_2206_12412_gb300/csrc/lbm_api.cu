@@ -59,6 +59,8 @@ void ChunkGraph::reset()
 
 namespace {
 
+// The largest scratch planes a handle takes for its passes (lattices of up to 1.4e9 FP32 sites, leapfrog 7e8).
+constexpr size_t kMaxPassScratch = (size_t)6 << 30;
 constexpr int64_t kDefaultHistCap = 65536;
 
 int64_t floor_div(int64_t a, int64_t b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
@@ -381,6 +383,27 @@ cudaError_t enqueue_step(const lbm_handle *h, int par, cudaStream_t s)
     }
 }
 
+// One pass of K steps; second: the second pass of a pair.
+template <typename T, typename D>
+cudaError_t enqueue_pass_t(const lbm_handle *h, const lbm::PassPlan &q, int par, bool second, cudaStream_t s)
+{
+    lbm::NvtxRange r("K1 pass");
+    lbm::PassArgs<T, D> a;
+    make_pass_args(h, par, second, q, a);
+    return launch_pass(a, h->pass_rpt, s);
+}
+
+cudaError_t enqueue_pass(const lbm_handle *h, const lbm::PassPlan &q, int par, bool second, cudaStream_t s)
+{
+    switch (h->lat.storage) {
+    case LBM_F32: return enqueue_pass_t<float, float>(h, q, par, second, s);
+    case LBM_F32_WD_BF16: return enqueue_pass_t<float, __nv_bfloat16>(h, q, par, second, s);
+    case LBM_F32_WD_F16: return enqueue_pass_t<float, __half>(h, q, par, second, s);
+    case LBM_F32_LEAPFROG: return enqueue_pass_t<float, Lf>(h, q, par, second, s);
+    default: return enqueue_pass_t<double, double>(h, q, par, second, s);
+    }
+}
+
 const void *step_kernel_for(int storage, bool bulk = false)
 {
     switch (storage) {
@@ -608,7 +631,11 @@ void free_host(lbm_handle *h)
     delete h;
 }
 
-void drop_graph(lbm_handle *h) { h->steps.reset(); }
+void drop_graph(lbm_handle *h)
+{
+    h->steps.reset();
+    h->passes.reset();
+}
 
 }  // namespace
 
@@ -874,6 +901,7 @@ lbm_status create_impl(const lbm_grid *grid, const lbm_lattice *lattice, const l
     h->stream = (cudaStream_t)stream;
     h->sticky = LBM_OK;
     h->steps.gen = -1;
+    h->passes.gen = -1;
     h->units_h = new (std::nothrow) std::vector<Unit>();
     h->init_cut = new (std::nothrow) std::vector<uint32_t>();
     if (!h->units_h || !h->init_cut) {
@@ -950,14 +978,32 @@ lbm_status create_impl(const lbm_grid *grid, const lbm_lattice *lattice, const l
     const size_t o_htyl = off; off = align256(off + (size_t)(line ? hcap_l : 1) * 8);
     size_t o_ser[4];
     for (int q = 0; q < 4; ++q) { o_ser[q] = off; off = align256(off + (size_t)h->load[q].n * 8); }
-    h->block_bytes = off;
-    h->block = dev_alloc(h, off);
+    h->state_bytes = off;
+    // scratch planes of the passes, for lattices that can take them and whose
+    // scratch is a small part of the device's memory
+    const size_t alt_bytes = h->esize_d ? plane_d : plane;
+    const size_t o_a0 = off; off = align256(off + alt_bytes);
+    const size_t o_a1 = off; if (!h->esize_d) off = align256(off + alt_bytes);
+    bool scratch = !line && !d2q9 && !slab && grid->edge[LBM_BOTTOM] != LBM_EDGE_PERIODIC &&
+                   off - h->state_bytes <= kMaxPassScratch;
+    h->block_bytes = scratch ? off : h->state_bytes;
+    h->block = dev_alloc(h, h->block_bytes);
+    if (!h->block && scratch) {
+        // no room for the scratch planes: single steps only
+        scratch = false;
+        h->block_bytes = h->state_bytes;
+        h->block = dev_alloc(h, h->block_bytes);
+    }
     if (!h->block) { free_host(h); return fail(LBM_ERR_OOM, "device allocation failed"); }
     char *base = static_cast<char *>(h->block);
     const size_t origin = ((size_t)h->pitch + (size_t)xoff) * h->esize;   // row 0, column 0
     h->w[0] = base + o_w0 + origin;
     h->w[1] = base + o_w1 + origin;
     h->wd = h->esize_d ? base + o_wd + ((size_t)h->pitch + (size_t)xoff) * h->esize_d : nullptr;
+    if (scratch) {
+        h->alt[0] = base + o_a0 + ((size_t)h->pitch + (size_t)xoff) * (h->esize_d ? h->esize_d : h->esize);
+        if (!h->esize_d) h->alt[1] = base + o_a1 + origin;
+    }
     h->wbase[0] = base + o_w0;
     h->wbase[1] = base + o_w1;
     h->wdbase = base + o_wd;
@@ -987,7 +1033,7 @@ lbm_status create_impl(const lbm_grid *grid, const lbm_lattice *lattice, const l
         free_host(h);
         return rc;
     };
-    e = cudaMemsetAsync(h->block, 0, h->block_bytes, s);
+    e = cudaMemsetAsync(h->block, 0, h->state_bytes, s);
     if (e != cudaSuccess) return bail(cuda_fail(e, "clearing device state"));
     for (int q = 0; q < 4; ++q) {
         if (h->load[q].kind != LBM_LOAD_SERIES) continue;
@@ -1103,6 +1149,7 @@ lbm_status create_impl(const lbm_grid *grid, const lbm_lattice *lattice, const l
 
     lbm_status rc = plan_bands(h, 0);
     if (rc != LBM_OK) return bail(rc);
+    choose_pass(h);
 
     // initial state: the initial crack's links (x_start <= x_i <= x_tip) severed
     CrackState hs;
@@ -1168,9 +1215,29 @@ lbm_status lbm_step(lbm_handle *h, int64_t n)
     if (n < 0) return fail(LBM_ERR_ARG, "n must be >= 0");
     if (n > 0 && h->cp.mode != CRACK_NONE) h->pending = true;
     if (!h->profiling) {
-        // runs of steps replay graphs of 64, 32, ..., 2 steps
         int par = h->parity;
-        const lbm_status rc = run_chunks(h->steps, h->gen, h->stream, h->cap_stream, n, par,
+        lbm_status rc = LBM_OK;
+        if (h->pass_k && !h->own_bands && !h->bulk) {
+            // as many pairs of passes as n holds, then a pair of shorter ones
+            // for what is left (a pair of K steps covers 2 K of them)
+            lbm::PassPlan q;
+            const int64_t pairs = n / (2 * h->pass_k);
+            const int base = par;
+            if (pairs > 0 && pass_plan(h, h->pass_k, h->pass_rpt, q)) {
+                rc = run_chunks(h->passes, h->gen, h->stream, h->cap_stream, 2 * pairs, par,
+                                [&](int p, cudaStream_t s) { return enqueue_pass(h, q, p, p != base, s); });
+                if (rc != LBM_OK) return rc;
+                n -= pairs * 2 * h->pass_k;
+            }
+            const int K = (int)std::min<int64_t>(n / 2, h->pass_k);
+            if (K >= 2 && pass_plan(h, K, h->pass_rpt, q)) {
+                LBM_CUDA(enqueue_pass(h, q, base, false, h->stream));
+                LBM_CUDA(enqueue_pass(h, q, base ^ 1, true, h->stream));
+                n -= 2 * K;
+            }
+        }
+        // runs of single steps replay graphs of 64, 32, ..., 2 steps
+        rc = run_chunks(h->steps, h->gen, h->stream, h->cap_stream, n, par,
                                          [&](int p, cudaStream_t s) { return enqueue_step(h, p, s); });
         h->parity = par;
         return rc;
@@ -1576,6 +1643,7 @@ lbm_status lbm_set_launch(lbm_handle *h, int32_t band_rows)
     if (band_rows < 0 || band_rows > (1 << 20)) return fail(LBM_ERR_ARG, "band_rows out of range");
     LBM_CUDA(cudaStreamSynchronize(h->stream));
     drop_graph(h);
+    h->own_bands = band_rows > 0;
     if (h->line) {
         // the march blocks of a crack in any direction: bands of band_rows
         // rows (every kernel computes its grid and its blocks' rows from it)
@@ -2630,7 +2698,7 @@ lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *threads, i
     std::vector<size_t> off;
     for (lbm_handle *h : b->hs) {
         off.push_back(total);
-        total = align256(total + h->block_bytes);
+        total = align256(total + h->state_bytes);
     }
     void *snap = batch_alloc(b, std::max<size_t>(total, 256));
     if (!snap) return fail(LBM_ERR_OOM, "device allocation failed (state snapshot for the trials)");
@@ -2648,7 +2716,7 @@ lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *threads, i
         lbm_handle *h = b->hs[i];
         par0.push_back(h->parity);
         pend0.push_back(h->pending);
-        cudaError_t e = cudaMemcpyAsync(static_cast<char *>(snap) + off[i], h->block, h->block_bytes,
+        cudaError_t e = cudaMemcpyAsync(static_cast<char *>(snap) + off[i], h->block, h->state_bytes,
                                         cudaMemcpyDeviceToDevice, b->stream);
         if (e != cudaSuccess) return done(cuda_fail(e, "saving the lattices' state"));
     }
@@ -2690,7 +2758,7 @@ lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *threads, i
             }
     for (size_t i = 0; i < b->hs.size(); ++i) {
         lbm_handle *h = b->hs[i];
-        cudaError_t e = cudaMemcpyAsync(h->block, static_cast<char *>(snap) + off[i], h->block_bytes,
+        cudaError_t e = cudaMemcpyAsync(h->block, static_cast<char *>(snap) + off[i], h->state_bytes,
                                         cudaMemcpyDeviceToDevice, b->stream);
         if (e != cudaSuccess) return done(cuda_fail(e, "restoring the lattices' state"));
         h->parity = par0[i];

@@ -105,6 +105,7 @@ struct lbm_handle {
     bool custom_alloc;
     void *block;
     size_t block_bytes;
+    size_t state_bytes;  // the leading part of the block that holds the state (the rest: scratch planes)
     void *w[2];          // element (0, 0) of each W buffer
     void *wd;
     void *wbase[2], *wdbase;   // first byte of each plane (halo row, pad)
@@ -125,6 +126,13 @@ struct lbm_handle {
     cudaStream_t stream;
     cudaStream_t cap_stream;
     lbm::host::ChunkGraph steps;   // graphs of runs of time steps (lbm_step)
+    // passes of several time steps (lbm_pass.cuh): always two at a time, so
+    // that the buffers end where an even number of single steps leaves them
+    lbm::host::ChunkGraph passes;  // graphs of runs of passes of pass_k steps
+    int32_t pass_k;      // steps of a pass (0: single steps only)
+    int32_t pass_rpt;    // rows per thread of its bulk tiles
+    bool own_bands;      // lbm_set_launch chose the bands of the single step: no passes
+    void *alt[2];        // scratch planes between two passes: wdot (leapfrog: w and the w before it)
     lbm_status sticky;
     // CUDA-event timing (lbm_set_profiling)
     int profiling;
@@ -196,6 +204,33 @@ inline void make_step_args(const lbm_handle *h, int par, StepArgs<T, D> &a)
     a.err = h->err;
     a.p = h->cp;
     a.hist = h->hist;
+}
+
+// The tiles of a pass of K steps of this lattice (lbm_pass_plan.cu); false
+// where a pass of K steps cannot be split so that every tile that needs a
+// crack decision holds what decides it.
+bool pass_plan(const lbm_handle *h, int K, int rpt, lbm::PassPlan &q);
+// Choose the pass of this lattice: h->pass_k, h->pass_rpt.
+void choose_pass(lbm_handle *h);
+
+// Arguments of pass number `second` of a pair (the first reads the state of
+// parity `par` in place, the second the scratch planes the first wrote; its
+// `par` is the other one).
+template <typename T, typename D>
+inline void make_pass_args(const lbm_handle *h, int par, bool second, const lbm::PassPlan &q, lbm::PassArgs<T, D> &a)
+{
+    make_step_args(h, par, a.s);
+    a.q = q;
+    if constexpr (std::is_same<D, lbm::Lf>::value) {
+        // (w_n, w_{n-1}): W[par], W[par ^ 1] -> the scratch planes -> back
+        a.s.w_in = static_cast<const T *>(second ? h->alt[0] : h->w[par]);
+        a.wd_in = static_cast<const D *>(second ? h->alt[1] : h->w[par ^ 1]);
+        a.s.w_out = static_cast<T *>(second ? h->w[par ^ 1] : h->alt[0]);
+        a.s.wd = static_cast<D *>(second ? h->w[par] : h->alt[1]);
+    } else {
+        a.wd_in = static_cast<const D *>(second ? h->alt[0] : h->wd);
+        a.s.wd = static_cast<D *>(second ? h->wd : h->alt[0]);
+    }
 }
 
 // Whether the single-lattice step launch adds the record CTA (StepArgs::k_cta)

@@ -203,6 +203,27 @@ struct FinalizeArgs {
     History hist;
 };
 
+// A pass of K time steps (lbm_pass.cuh): the static part of its split into
+// tiles.  Tiles are numbered ms crack-strip tiles first, then mx columns of
+// mb + mt row tiles.
+struct PassPlan {
+    int32_t K, hc;             // steps; halo columns on each side (K rounded up to whole vectors)
+    int32_t mx, px;            // column tiles of the bulk and their width
+    int32_t jb, mb, pb;        // rows [0, jb) below the strip: mb row tiles of pb rows
+    int32_t jt, mt, pt;        // rows [jt, ny) above it (a lattice without a crack: all rows)
+    int32_t ms, ps;            // column tiles of the strip and their nominal width
+    int32_t zb, za;            // strip: no tile boundary less than zb behind or up to za ahead of a tip
+    int32_t grow;              // strip: most columns an end can cut in a pass
+    int32_t tiles, edge_macro;
+};
+
+template <typename T, typename D>
+struct PassArgs {
+    StepArgs<T, D> s;          // w_in, w_out; s.wd: the wdot plane the pass writes (leapfrog: w of the step before last)
+    const D *wd_in;            // the wdot plane it reads (leapfrog: w_{n-1})
+    PassPlan q;
+};
+
 // One CTA of a batched step: column block cb of band `band` of lattice `inst`.
 struct BatchUnit {
     int32_t inst, cb, band, pad;
@@ -304,6 +325,8 @@ cudaError_t launch_batch_pieces(const StepArgs<T, D> *descs, const BatchPiece *p
                                 int par, cudaStream_t s, int threads, int lookahead, bool chained);
 template <typename T, typename D>
 cudaError_t launch_step(const StepArgs<T, D> &a, int bands, cudaStream_t s, bool bulk = false);
+// A pass of several time steps; rpt: rows per thread of the bulk tiles (4 or 8).
+template <typename T, typename D> cudaError_t launch_pass(const PassArgs<T, D> &a, int rpt, cudaStream_t s);
 template <typename T, typename D> cudaError_t launch_edge_rule(const StepArgs<T, D> &a, cudaStream_t s);
 template <typename T, typename D> int edge_rule_count(const StepArgs<T, D> &a);
 template <typename T, typename D>

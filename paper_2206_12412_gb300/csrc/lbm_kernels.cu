@@ -1192,28 +1192,6 @@ cudaError_t launch_wstar(CrackState *st, const LoadDesc *load, const int32_t *ed
 // the bottom / top one.  wdot_B = (w_B - w_B(t)) / dt, and the pad images
 // of the site are refreshed.
 
-template <typename T>
-struct EdgeRule {
-    const T *wn;          // the new fields
-    int64_t pitch;
-    int32_t dir[4];       // 1: Dirichlet edge
-    T ws[4];              // w* at the new time level
-    __device__ __forceinline__ T w(int i, int j) const { return wn[(int64_t)j * pitch + i]; }
-    __device__ __forceinline__ T rule(int e, T wI, T wII) const
-    {
-        if (dir[e])
-            return (T)(8.0 / 15.0) * ws[e] + (T)(2.0 / 3.0) * wI - (T)0.2 * wII;
-        return (T)1.5 * wI - (T)0.5 * wII;
-    }
-    // a non-corner point of edge e from its two sites along the inward normal
-    __device__ __forceinline__ T point(int e, int i, int j) const
-    {
-        const int dx = e == LEFT ? 1 : (e == RIGHT ? -1 : 0);
-        const int dy = e == BOTTOM ? 1 : (e == TOP ? -1 : 0);
-        return rule(e, w(i + dx, j + dy), w(i + 2 * dx, j + 2 * dy));
-    }
-};
-
 __host__ __device__ __forceinline__ bool ruled(int kind) { return kind == EDGE_FREE || kind == EDGE_DIRICHLET; }
 
 template <typename T, typename D>

@@ -1,0 +1,10 @@
+// lbm_pass16.cu -- the pass kernels (lbm_pass.cuh) of FP64 and of 16-bit wdot.
+#include "lbm_pass.cuh"
+
+namespace lbm {
+
+template cudaError_t launch_pass<double, double>(const PassArgs<double, double> &, int, cudaStream_t);
+template cudaError_t launch_pass<float, __nv_bfloat16>(const PassArgs<float, __nv_bfloat16> &, int, cudaStream_t);
+template cudaError_t launch_pass<float, __half>(const PassArgs<float, __half> &, int, cudaStream_t);
+
+}  // namespace lbm

@@ -1,0 +1,103 @@
+"""Passes of several time steps against single steps: the same arithmetic per
+site, so fields, masks, crack states and histories agree bit for bit.  A run
+of n steps in one call goes through passes (pairs of up to eight steps each,
+the rest single steps); n calls of one step never do."""
+import numpy as np
+import pytest
+
+from paper_2206_12412_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2206_12412_gb300 import lbm
+    lbm.load_library()
+    return lbm
+
+
+def _strip(nx, ny, mode="prescribed", bc="macroscopic", edges=("free", "free", "dirichlet", "dirichlet"), jc=None,
+           tip=None, start=0.0, u0=1e-3, **crack):
+    p = W.base_problem(nx, ny, bc_mode=bc, edges=edges)
+    p["hist_cap"] = 512
+    if mode:
+        p = W.with_crack(p, mode=mode, y=float(ny // 2 if jc is None else jc), x_start=start,
+                         x_tip=nx / 4 if tip is None else tip, **crack)
+    loads = []
+    for k, e in enumerate(("left", "right", "bottom", "top")):
+        if edges[k] == "dirichlet":
+            kind = ("linear", "sin2", "halfsine", "const")[k]
+            loads.append({"edge": e, "kind": kind, "amp": (-1) ** k * u0, "t": 25.0})
+    p["loads"] = loads
+    return p
+
+
+# sizes at which a tile is whole, one vector or one row over, and thin
+SIZES = [(24, 20), (97, 41), (128, 128), (129, 66), (240, 130), (241, 63), (352, 200), (1001, 97)]
+KC = 0.02 * 0.25 * 1e-3 * 2
+
+
+def cases():
+    out = []
+    for k, (nx, ny) in enumerate(SIZES):
+        out.append((f"prescribed_{nx}x{ny}", _strip(nx, ny, v_rel=0.6), "f32", 37 + k))
+        out.append((f"kcrit_{nx}x{ny}", _strip(nx, ny, mode="kcrit", K_C=KC), "f32", 50 - k))
+        out.append((f"bb_periodic_{nx}x{ny}", _strip(nx, ny, bc="bounceback", v_rel=0.5,
+                    edges=("periodic", "periodic", "dirichlet", "free"), start=nx * 0.7, tip=nx * 0.95), "f32", 48))
+    for st in ("f64", "f32_bf16", "f32_f16", "f32_lf"):
+        out.append((f"kcrit_{st}", _strip(300, 150, mode="kcrit", K_C=KC), st, 61))
+        out.append((f"two_{st}", _strip(500, 80, mode="kcrit", K_C=KC, start=200.0, tip=215.0, two_tips=True), st, 90))
+        out.append((f"edges_{st}", _strip(300, 150, mode="kcrit", bc="macroscopic_edges", K_C=KC), st, 50))
+    for tip in range(40, 140, 7):   # the tip at any place relative to the tiles' boundaries
+        out.append((f"tip_{tip}", _strip(331, 60, mode="kcrit", tip=tip + 0.3, K_C=KC), "f32", 64))
+        out.append((f"tips_{tip}", _strip(480, 60, mode="kcrit", start=tip + 0.2, tip=tip + 31.9, K_C=KC, two_tips=True),
+                    "f32", 64))
+    out += [
+        ("no_crack", _strip(300, 170, mode=None), "f32", 70),
+        ("no_crack_edges", _strip(300, 170, mode=None, bc="macroscopic_edges"), "f32", 70),
+        ("no_crack_small", _strip(33, 25, mode=None), "f64", 35),
+        ("stationary_two", _strip(260, 90, mode="stationary", start=100.0, tip=180.0, two_tips=True), "f32", 40),
+        ("crack_low", _strip(200, 120, mode="kcrit", jc=3, K_C=KC), "f32", 50),
+        ("crack_high", _strip(200, 120, mode="prescribed", jc=117, v_rel=0.4), "f32", 50),
+        ("dirichlet_all", _strip(270, 140, bc="bounceback", edges=("dirichlet",) * 4, v_rel=0.7, start=30.0), "f32", 50),
+        ("edges_dirichlet_sides", _strip(250, 110, mode="prescribed", bc="macroscopic_edges", start=20.0, v_rel=0.5,
+                                         edges=("dirichlet", "free", "free", "dirichlet")), "f32", 50),
+        ("edge_crack_edges_f64", _strip(150, 90, mode="prescribed", bc="macroscopic_edges", v_rel=0.5), "f64", 33),
+        ("clamped", _strip(200, 90, mode="prescribed", tip=180.0, v_rel=0.9), "f32", 100),
+        ("wide_window", _strip(400, 90, mode="kcrit", K_C=KC, tip=150.0, fit_width=9.0, r0=3.0), "f32", 64),
+        ("two_wide_windows", _strip(400, 90, mode="kcrit", K_C=KC, start=150.0, tip=158.0, two_tips=True, fit_width=5.0,
+                                    r0=1.0), "f32", 64),
+        ("far_window", _strip(400, 90, mode="kcrit", K_C=KC, tip=150.0, r_min=30.0), "f32", 64),
+        ("tall", _strip(120, 1500, mode="kcrit", K_C=KC), "f32", 40),
+        ("example", W.kcrit_centre_crack(), "f32", 200),
+    ]
+    return out
+
+
+@pytest.mark.parametrize("name,p,storage,n", cases(), ids=[c[0] for c in cases()])
+def test_passes_equal_single_steps(gpu, name, p, storage, n):
+    lbm = gpu
+    w0, wd0 = W.random_state(p["nx"], p["ny"], 11)
+    two = p["crack"].get("two_tips")
+    got = []
+    for chunks in ([n, 5, 19], [1] * (n + 24)):
+        lat = lbm.Lattice(p, storage)
+        lat.set_fields(w0, wd0)
+        for c in chunks:
+            lat.step(c)
+        h = [lat.history(n + 24)] + ([lat.history_left(n + 24)] if two else [])
+        st = [lat.crack_state()] + ([lat.crack_state_left()] if two else [])
+        got.append((lat.fields(), lat.cut_mask("v"), h, st))
+        lat.close()
+    (f, m, h, st), (f1, m1, h1, st1) = got
+    for a, b in zip(f, f1):
+        np.testing.assert_array_equal(a, b)
+    np.testing.assert_array_equal(m, m1)
+    for a, b in zip(h, h1):
+        for k in a:
+            np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+    assert st == st1
