@@ -20,9 +20,13 @@
 // step, for an eighth of its memory traffic and launches.
 //
 // Measured, one GB300, time per step of a run against one launch per step:
-// 4096 x 2048 FP32, K-criterion 20.0 -> 9.2 us; 8192 x 8192 BF16 wdot 161 ->
-// 75 us; 16384 x 16384 leapfrog 575 -> 238 us; 1001 x 777 FP16 wdot, periodic
-// sides 6.0 -> 3.3 us; 512 x 192 with the edge rule and two tips 10.7 -> 6.0 us.
+// 4096 x 2048 FP32, K-criterion 20.0 -> 8.6 us; 8192 x 8192 BF16 wdot 161 ->
+// 69 us; 16384 x 16384 leapfrog 575 -> 187 us; 1001 x 777 FP16 wdot, periodic
+// sides 6.0 -> 3.4 us; 512 x 192 with the edge rule and two tips 10.7 -> 5.3 us.
+// What bounds a bulk tile is instruction issue: with scalar FP32 and the rows
+// moved back after each step the leapfrog kernel issued 85.7 M instructions
+// per 4096^2 pass (120 us), without the moves 69.8 M (110 us), packed 50.7 M
+// (98 us; FP32 pipes 44 % busy, DRAM 27 %).
 //
 // The crack strip.  The rows within 16 - K of the crack line form tiles of
 // their own (32 rows, the line between warps 3 and 4), which apply the cuts
@@ -75,6 +79,70 @@ template <typename D, typename T> __device__ __forceinline__ void wd_put(D *p, T
 {
     if constexpr (std::is_same<D, Lf>::value) p->v = v;
     else WdIO<D>::put(p, v, scale);
+}
+
+// Two FP32 operations in one instruction (each rounded as the scalar one).
+// They do not raise the FP32 rate, but halve the instructions a row issues,
+// and a tile is bound by instruction issue.
+__device__ __forceinline__ uint64_t pk2(float a, float b)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void up2(uint64_t v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// The update of one row segment (site_update of each of its sites): cu the
+// row, up and dn the rows above and below, hs the sums of the east and west
+// neighbours; d: wdot, updated in place as storage rounds it (leapfrog: the
+// w before, left alone).
+template <typename T, typename D, int N>
+__device__ __forceinline__ void row_sites(const Row<T, N> &cu, const Row<T, N> &up, const Row<T, N> &dn, const Row<T, N> &hs,
+                                          Row<T, N> &d, T g, T dt, T wd_scale, T wd_inv, Row<T, N> &out)
+{
+    constexpr bool kLf = std::is_same<D, Lf>::value;
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int k = 0; k < N; k += 2) {
+            const uint64_t c = pk2(cu.v[k], cu.v[k + 1]);
+            const uint64_t v = add2(pk2(up.v[k], up.v[k + 1]), pk2(dn.v[k], dn.v[k + 1]));
+            const uint64_t lap = fma2(pk2(-4.0f, -4.0f), c, add2(v, pk2(hs.v[k], hs.v[k + 1])));
+            if constexpr (kLf) {
+                // w + ((w - w_{n-1}) + (g dt) lap)
+                const uint64_t e = fma2(pk2(-1.0f, -1.0f), pk2(d.v[k], d.v[k + 1]), c);
+                const float gd = g * dt;
+                up2(add2(c, fma2(pk2(gd, gd), lap, e)), out.v[k], out.v[k + 1]);
+            } else {
+                const uint64_t dn2 = fma2(pk2(g, g), lap, pk2(d.v[k], d.v[k + 1]));
+                up2(fma2(pk2(dt, dt), dn2, c), out.v[k], out.v[k + 1]);
+                float d0, d1;
+                up2(dn2, d0, d1);
+                d.v[k] = wd_round<D, T>(d0, wd_scale, wd_inv);
+                d.v[k + 1] = wd_round<D, T>(d1, wd_scale, wd_inv);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const T lap = ((up.v[k] + dn.v[k]) + hs.v[k]) - (T)4 * cu.v[k];
+            T wn, dn_;
+            site_update<T, D>(cu.v[k], d.v[k], lap, g, dt, wn, dn_);
+            d.v[k] = dn_;
+            out.v[k] = wn;
+        }
+    }
 }
 
 // Crack state in force during one step of a pass (modes whose decisions need
@@ -223,8 +291,308 @@ __device__ __forceinline__ int wrap_col(int c, int nx)
     return c < 0 ? c + nx : c;
 }
 
-// KIND: 0 a tile none of whose sites sees an edge or the crack, 1 with outer
-// edges, 2 a crack-strip tile (with edges where it meets them).
+// What a thread knows about its tile.
+struct PassCtx {
+    TileGeo g;
+    int lane, warp, x0, jb;
+    bool per;
+    bool is_l;                  // element 0 is column 0 (no periodic sides)
+    int kr;                     // the element that is column nx - 1, else -1
+    bool side;                  // the tile's warps hold column 0 or nx - 1
+    // strip tiles: whether the pass's decisions need no K; the ends this tile
+    // follows (a link it can see may be cut in this pass); the ends whose
+    // records it writes; the lattice column of its column 0 as seen from each
+    // end; the severed columns at the start
+    bool known, ev_r, ev_l, own_r, own_l, follow;
+    int org_r, org_l, f0, l0;
+};
+
+// The fields of a thread: RPT rows of one vector.  Each update writes the
+// new rows where the next one reads them, so that no register is copied from
+// step to step: leapfrog storage writes w_{n+1} over w_{n-1} and the two
+// planes change places; the other forms shift the rows of w by one slot, up
+// in one step (PH = 0, rows swept upwards) and down in the next (PH = 1).
+template <typename T, typename D, int RPT> struct PassRows {
+    static constexpr int N = Vec<T>::N;
+    typedef Row<T, N> R;
+    static constexpr bool kLf = std::is_same<D, Lf>::value;
+    R a[RPT + (kLf ? 0 : 1)];
+    R b[RPT];
+    // row r of w before a step of phase PH, and where the step writes it
+    template <int PH> __device__ __forceinline__ R &cur(int r)
+    {
+        if constexpr (kLf) return PH == 0 ? a[r] : b[r];
+        else return PH == 0 ? a[r + 1] : a[r];
+    }
+    template <int PH> __device__ __forceinline__ R &next(int r)
+    {
+        if constexpr (kLf) return PH == 0 ? b[r] : a[r];
+        else return PH == 0 ? a[r] : a[r + 1];
+    }
+    // row r of wdot (leapfrog: of the w before, which the step overwrites)
+    template <int PH> __device__ __forceinline__ R &rate(int r)
+    {
+        if constexpr (kLf) return PH == 0 ? b[r] : a[r];
+        else return b[r];
+    }
+};
+
+// One time step of a tile.
+template <typename T, typename D, int RPT, int KIND, int PH>
+__device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx &c, int s, PassRows<T, D, RPT> &F,
+                                          PassShared<T> &sh)
+{
+    constexpr int N = Vec<T>::N;
+    constexpr bool kLf = std::is_same<D, Lf>::value;
+    typedef Row<T, N> R;
+    const unsigned kFull = 0xffffffffu;
+    const StepArgs<T, D> &a = A.s;
+    const CrackParams &p = a.p;
+    const int lane = c.lane, warp = c.warp, x0 = c.x0, jb = c.jb, nx = a.nx, ny = a.ny;
+    const T gg = a.g, dt = a.dt, wd_inv = a.wd_inv, wd_scale = a.wd_scale;
+    const int b = s & 1;
+    stg_row(&sh.top[b][warp][lane * N], F.template cur<PH>(RPT - 1));
+    stg_row(&sh.bot[b][warp][lane * N], F.template cur<PH>(0));
+    if (KIND == 2 && c.known && warp == kBelowWarp) stg_row(&sh.pair[s][0][lane * N], F.template cur<PH>(RPT - 1));
+    if (KIND == 2 && c.known && warp == kBelowWarp + 1) stg_row(&sh.pair[s][1][lane * N], F.template cur<PH>(0));
+    __syncthreads();
+    if (KIND == 2 && c.follow) {
+        const bool reach = sh.reach[b] != 0;
+        if (warp == 0) {
+            pass_crack_step<T>(p, sh.top[b][kBelowWarp], sh.bot[b][kBelowWarp + 1], c.org_r, c.org_l, sh.S, a.hist, c.ev_r,
+                               c.ev_l, c.own_r, c.own_l);
+            if (lane == 0) sh.reach[b ^ 1] = crack_cut_in_reach(p, sh.S) ? 1 : 0;
+        }
+        // rows next to the crack wait for the decision only where it can cut a link
+        if (reach) __syncthreads();
+    }
+    R dnx, upx;
+    ld_row(&sh.top[b][warp > 0 ? warp - 1 : 0][lane * N], dnx);
+    ld_row(&sh.bot[b][warp < kPassWarps - 1 ? warp + 1 : warp][lane * N], upx);
+    uint32_t cut = 0u;
+    if (KIND == 2 && (warp == kBelowWarp || warp == kBelowWarp + 1)) {
+        const int f = c.known ? sh.log[s + 1].f : (c.ev_l ? sh.S.i_first : c.f0);
+        const int l = c.known ? sh.log[s + 1].l : (c.ev_r ? sh.S.i_last : c.l0);
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            int q = x0 + k;
+            if (c.per) q = wrap_col(q, nx);
+            if (q >= f && q <= l) cut |= 1u << k;
+        }
+    }
+    T tl = (T)0, tr = (T)0, tb = (T)0, tt = (T)0;
+    R first, last;                                         // the first and last rows before the update
+    T el[KIND != 0 ? RPT : 1], er[KIND != 0 ? RPT : 1];   // edge rule: the edge columns before the update
+    const bool em_side = KIND != 0 && A.q.edge_macro && c.side;
+    if (KIND != 0) {
+        tl = (T)2 * (T)sh.ws[LEFT][s];
+        tr = (T)2 * (T)sh.ws[RIGHT][s];
+        tb = (T)2 * (T)sh.ws[BOTTOM][s];
+        tt = (T)2 * (T)sh.ws[TOP][s];
+        first = F.template cur<PH>(0);
+        last = F.template cur<PH>(RPT - 1);
+        if (em_side) {
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) {
+                el[r] = F.template cur<PH>(r).v[0];
+#pragma unroll
+                for (int k = 0; k < N; ++k)
+                    if (k == 0 || k == c.kr) er[r] = F.template cur<PH>(r).v[k];
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+        const int r = PH == 0 ? q : RPT - 1 - q;
+        const R cu = F.template cur<PH>(r);
+        // the row whose slot this row's new values take is read first
+        R up = r + 1 < RPT ? F.template cur<PH>(r + 1 < RPT ? r + 1 : r) : upx;
+        R dn = r > 0 ? F.template cur<PH>(r > 0 ? r - 1 : r) : dnx;
+        T left0 = __shfl_up_sync(kFull, cu.v[N - 1], 1);
+        T rightN = __shfl_down_sync(kFull, cu.v[0], 1);
+        if (KIND != 0) {
+            const int j = jb + r;
+            if (j == ny - 1) {
+#pragma unroll
+                for (int k = 0; k < N; ++k) up.v[k] = a.edge[TOP] == EDGE_DIRICHLET ? tt - cu.v[k] : cu.v[k];
+            }
+            if (j == 0) {
+#pragma unroll
+                for (int k = 0; k < N; ++k) dn.v[k] = a.edge[BOTTOM] == EDGE_DIRICHLET ? tb - cu.v[k] : cu.v[k];
+            }
+            if (KIND == 2 && r == RPT - 1 && warp == kBelowWarp) {
+#pragma unroll
+                for (int k = 0; k < N; ++k)
+                    if ((cut >> k) & 1u) up.v[k] = cu.v[k];
+            }
+            if (KIND == 2 && r == 0 && warp == kBelowWarp + 1) {
+#pragma unroll
+                for (int k = 0; k < N; ++k)
+                    if ((cut >> k) & 1u) dn.v[k] = cu.v[k];
+            }
+            if (c.is_l) left0 = a.edge[LEFT] == EDGE_DIRICHLET ? tl - cu.v[0] : cu.v[0];
+        }
+        R hs;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const T wl = k == 0 ? left0 : cu.v[k - 1];
+            T wr = k == N - 1 ? rightN : cu.v[k + 1];
+            if (KIND != 0 && k == c.kr) wr = a.edge[RIGHT] == EDGE_DIRICHLET ? tr - cu.v[k] : cu.v[k];
+            hs.v[k] = wl + wr;
+        }
+        R out;
+        row_sites<T, D, N>(cu, up, dn, hs, F.template rate<PH>(r), gg, dt, wd_scale, wd_inv, out);
+        F.template next<PH>(r) = out;
+    }
+    if (KIND == 2 && p.macro && cut) {
+        // the crack-face rule: w_B from the two new values further from the crack
+        if (warp == kBelowWarp) {
+            R &w1 = F.template next<PH>(RPT - 1), &w2 = F.template next<PH>(RPT - 2), &w3 = F.template next<PH>(RPT - 3);
+#pragma unroll
+            for (int k = 0; k < N; ++k)
+                if ((cut >> k) & 1u) {
+                    const T wB = (T)1.5 * w2.v[k] - (T)0.5 * w3.v[k];
+                    if (!kLf) F.b[RPT - 1].v[k] = wd_round<D, T>((wB - last.v[k]) / dt, wd_scale, wd_inv);
+                    w1.v[k] = wB;
+                }
+        } else {
+            R &w1 = F.template next<PH>(0), &w2 = F.template next<PH>(1), &w3 = F.template next<PH>(2);
+#pragma unroll
+            for (int k = 0; k < N; ++k)
+                if ((cut >> k) & 1u) {
+                    const T wB = (T)1.5 * w2.v[k] - (T)0.5 * w3.v[k];
+                    if (!kLf) F.b[0].v[k] = wd_round<D, T>((wB - first.v[k]) / dt, wd_scale, wd_inv);
+                    w1.v[k] = wB;
+                }
+        }
+    }
+    if (KIND != 0 && A.q.edge_macro) {
+        // the macroscopic rule on the outer edges (the two levels of
+        // edge_rule_at): the edge columns, the crack-face points on
+        // them, then the bottom and top rows and the corners
+        const bool on_l = a.edge[LEFT] != EDGE_PERIODIC, on_r = a.edge[RIGHT] != EDGE_PERIODIC;
+        EdgeRule<T> E;
+        E.wn = nullptr;
+        E.pitch = 0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            E.dir[e] = a.edge[e] == EDGE_DIRICHLET;
+            E.ws[e] = (T)sh.ws[e][s + 1];
+        }
+        R in1, in2;         // rows 1, 2 (or ny-2, ny-3) before the edge columns
+        const bool has_b = jb == 0, has_t = jb + RPT == ny;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            in1.v[k] = has_t ? F.template next<PH>(RPT - 2).v[k] : F.template next<PH>(1).v[k];
+            in2.v[k] = has_t ? F.template next<PH>(RPT - 3).v[k] : F.template next<PH>(2).v[k];
+        }
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+            if (!em_side) break;
+            R &w = F.template next<PH>(r);
+            const int j = jb + r;
+            const T p1 = __shfl_up_sync(kFull, w.v[N - 1], 1), p2 = __shfl_up_sync(kFull, w.v[N - 2], 1);
+            const T n0 = __shfl_down_sync(kFull, w.v[0], 1);
+            if (j < 1 || j > ny - 2) continue;
+            if (c.is_l && on_l) {
+                const T v2 = N > 2 ? w.v[N > 2 ? 2 : 0] : n0;
+                w.v[0] = E.rule(LEFT, w.v[1], v2);
+            }
+            if (c.kr >= 0 && on_r) {
+                T wI = p1, wII = p2;
+#pragma unroll
+                for (int k = 1; k < N; ++k)
+                    if (k == c.kr) {
+                        wI = w.v[k - 1];
+                        wII = k >= 2 ? w.v[k >= 2 ? k - 2 : 0] : p1;
+                    }
+                const T v = E.rule(RIGHT, wI, wII);
+#pragma unroll
+                for (int k = 0; k < N; ++k)
+                    if (k == c.kr) w.v[k] = v;
+            }
+        }
+        if (KIND == 2 && em_side && p.macro && cut && (c.is_l || c.kr >= 0)) {
+            const bool be = warp == kBelowWarp;
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                if (!((cut >> k) & 1u) || !((c.is_l && on_l && k == 0) || (on_r && k == c.kr))) continue;
+                const T v1 = be ? F.template next<PH>(RPT - 2).v[k] : F.template next<PH>(1).v[k];
+                const T v2 = be ? F.template next<PH>(RPT - 3).v[k] : F.template next<PH>(2).v[k];
+                const T v = (T)1.5 * v1 - (T)0.5 * v2;
+                if (be) F.template next<PH>(RPT - 1).v[k] = v;
+                else F.template next<PH>(0).v[k] = v;
+            }
+        }
+        if (has_b || has_t) {
+            const int ev = has_t ? TOP : BOTTOM;
+            R e1, e2;   // the rows one and two from the edge, after the edge columns
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                e1.v[k] = has_t ? F.template next<PH>(RPT - 2).v[k] : F.template next<PH>(1).v[k];
+                e2.v[k] = has_t ? F.template next<PH>(RPT - 3).v[k] : F.template next<PH>(2).v[k];
+            }
+            R o;
+#pragma unroll
+            for (int k = 0; k < N; ++k) o.v[k] = E.rule(ev, in1.v[k], in2.v[k]);
+            // corners: along the bottom / top edge's normal from the edge
+            // columns, or (its side Dirichlet, ev not) along the row from
+            // the points of edge ev
+            const T q1 = __shfl_up_sync(kFull, o.v[N - 1], 1), q2 = __shfl_up_sync(kFull, o.v[N - 2], 1);
+            const T m0 = __shfl_down_sync(kFull, o.v[0], 1);
+            T cl = (T)0, cr = (T)0;
+            if (c.is_l && on_l)
+                cl = a.edge[LEFT] == EDGE_DIRICHLET && a.edge[ev] != EDGE_DIRICHLET
+                         ? E.rule(LEFT, o.v[1], N > 2 ? o.v[N > 2 ? 2 : 0] : m0)
+                         : E.rule(ev, e1.v[0], e2.v[0]);
+            if (c.kr >= 0 && on_r) {
+                T oI = q1, oII = q2, c1 = (T)0, c2 = (T)0;
+#pragma unroll
+                for (int k = 0; k < N; ++k)
+                    if (k == c.kr) {
+                        if (k >= 1) oI = o.v[k >= 1 ? k - 1 : 0];
+                        if (k >= 1) oII = k >= 2 ? o.v[k >= 2 ? k - 2 : 0] : q1;
+                        c1 = e1.v[k];
+                        c2 = e2.v[k];
+                    }
+                cr = a.edge[RIGHT] == EDGE_DIRICHLET && a.edge[ev] != EDGE_DIRICHLET ? E.rule(RIGHT, oI, oII)
+                                                                                   : E.rule(ev, c1, c2);
+            }
+            if (c.is_l && on_l) o.v[0] = cl;
+#pragma unroll
+            for (int k = 0; k < N; ++k)
+                if (on_r && k == c.kr) o.v[k] = cr;
+            if (has_t) F.template next<PH>(RPT - 1) = o;
+            else F.template next<PH>(0) = o;
+        }
+        if (!kLf && (em_side || has_b || has_t)) {
+            // wdot of the sites that took the rule
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) {
+                const R &w = F.template next<PH>(r);
+                const int j = jb + r;
+                if (j == 0 || j == ny - 1) {
+                    if ((r == 0 && has_b) || (r == RPT - 1 && has_t)) {
+#pragma unroll
+                        for (int k = 0; k < N; ++k)
+                            F.b[r].v[k] = wd_round<D, T>((w.v[k] - (r == 0 ? first.v[k] : last.v[k])) / dt, wd_scale, wd_inv);
+                    }
+                    continue;
+                }
+                if (!em_side) continue;
+                if (c.is_l && on_l) F.b[r].v[0] = wd_round<D, T>((w.v[0] - el[r]) / dt, wd_scale, wd_inv);
+                if (c.kr >= 0 && on_r) {
+#pragma unroll
+                    for (int k = 0; k < N; ++k)
+                        if (k == c.kr) F.b[r].v[k] = wd_round<D, T>((w.v[k] - er[r]) / dt, wd_scale, wd_inv);
+                }
+            }
+        }
+    }
+}
+
+// A tile.  KIND: 0 one none of whose sites sees an edge or the crack, 1 with
+// outer edges, 2 a crack-strip tile (with edges where it meets them).
 template <typename T, typename D, int RPT, int KIND>
 __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo g, PassShared<T> &sh)
 {
@@ -237,69 +605,78 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nx = a.nx, ny = a.ny, K = A.q.K;
     const int64_t P = a.pitch;
-    const int x0 = g.xl + lane * N;
-    const int jb = g.yl + warp * RPT;
-    const bool per = KIND != 0 && a.edge[LEFT] == EDGE_PERIODIC;
     const T wd_inv = a.wd_inv, wd_scale = a.wd_scale;
+    PassCtx c;
+    c.g = g;
+    c.lane = lane;
+    c.warp = warp;
+    c.x0 = g.xl + lane * N;
+    c.jb = g.yl + warp * RPT;
+    c.per = KIND != 0 && a.edge[LEFT] == EDGE_PERIODIC;
+    const int x0 = c.x0, jb = c.jb;
+    const bool per = c.per;
 
-    R w[RPT], d[RPT];
+    PassRows<T, D, RPT> F;
     {
         const T *wp = a.w_in + (int64_t)jb * P + x0;
         const D *dp = A.wd_in + (int64_t)jb * P + x0;
         const bool whole = KIND == 0 ? x0 < nx : (x0 >= 0 && x0 + N <= nx);
 #pragma unroll
         for (int r = 0; r < RPT; ++r) {
+            R &w = F.template cur<0>(r), &d = F.b[r];
 #pragma unroll
-            for (int k = 0; k < N; ++k) w[r].v[k] = d[r].v[k] = (T)0;
+            for (int k = 0; k < N; ++k) w.v[k] = d.v[k] = (T)0;
             const int j = jb + r;
             if (j < 0 || j >= ny) continue;
             if (whole) {
-                ldg_row(wp + (int64_t)r * P, w[r]);
-                WdIO<D>::load(dp + (int64_t)r * P, d[r], wd_inv);
+                ldg_row(wp + (int64_t)r * P, w);
+                WdIO<D>::load(dp + (int64_t)r * P, d, wd_inv);
             } else if (KIND != 0) {
 #pragma unroll
                 for (int k = 0; k < N; ++k) {
-                    int c = x0 + k;
-                    if (per) c = wrap_col(c, nx);
-                    if (c < 0 || c >= nx) continue;
-                    w[r].v[k] = a.w_in[(int64_t)j * P + c];
-                    d[r].v[k] = wd_get(A.wd_in + (int64_t)j * P + c, wd_inv);
+                    int q = x0 + k;
+                    if (per) q = wrap_col(q, nx);
+                    if (q < 0 || q >= nx) continue;
+                    w.v[k] = a.w_in[(int64_t)j * P + q];
+                    d.v[k] = wd_get(A.wd_in + (int64_t)j * P + q, wd_inv);
                 }
             }
         }
     }
 
-    // strip tiles: the ends this tile follows (a link it can see may be cut
-    // in this pass) and the one whose records it writes
-    bool known = true, ev_r = false, ev_l = false, own_r = false, own_l = false;
-    int org_r = g.xl, org_l = g.xl, rec0 = 0;
+    int rec0 = 0;
     int64_t hist0 = 0;
-    int f0 = 0, l0 = -1;
+    c.known = true;
+    c.ev_r = c.ev_l = c.own_r = c.own_l = c.follow = false;
+    c.org_r = c.org_l = g.xl;
+    c.f0 = 0;
+    c.l0 = -1;
     if (KIND == 2) {
-        known = p.mode != CRACK_KCRIT;
-        f0 = a.s_in->i_first;
-        l0 = a.s_in->i_last;
+        c.known = p.mode != CRACK_KCRIT;
+        c.f0 = a.s_in->i_first;
+        c.l0 = a.s_in->i_last;
         hist0 = a.s_in->hist_n;
         rec0 = a.s_in->r.decided ? 1 : 0;   // the first update whose crack step is still to run
-        const int cr = tip_col_r(f0, l0, nx), cl = tip_col_l(f0, l0, nx);
+        const int cr = tip_col_r(c.f0, c.l0, nx), cl = tip_col_l(c.f0, c.l0, nx);
         const int hc = A.q.hc, grow = A.q.grow;
         // (periodic sides: the column itself, then its images beyond either side)
         for (int q = 0; q < (per ? 3 : 1); ++q) {
             const int o = q == 0 ? 0 : (q == 1 ? -nx : nx);
-            if (cr + o >= g.x0 && cr + o < g.x1) own_r = true;
-            if (p.two_tips && cl + o >= g.x0 && cl + o < g.x1) own_l = true;
-            if (!ev_r && g.x0 - hc <= cr + o + grow && g.x1 + hc > cr + o) {
-                ev_r = true;
-                org_r = g.xl - o;
+            if (cr + o >= g.x0 && cr + o < g.x1) c.own_r = true;
+            if (p.two_tips && cl + o >= g.x0 && cl + o < g.x1) c.own_l = true;
+            if (!c.ev_r && g.x0 - hc <= cr + o + grow && g.x1 + hc > cr + o) {
+                c.ev_r = true;
+                c.org_r = g.xl - o;
             }
-            if (p.two_tips && !ev_l && g.x0 - hc <= cl + o && g.x1 + hc > cl + o - grow) {
-                ev_l = true;
-                org_l = g.xl - o;
+            if (p.two_tips && !c.ev_l && g.x0 - hc <= cl + o && g.x1 + hc > cl + o - grow) {
+                c.ev_l = true;
+                c.org_l = g.xl - o;
             }
         }
+        c.follow = !c.known && (c.ev_r || c.ev_l);
         if (tid == 0) {
             sh.S = *a.s_in;
-            if (known) pass_known_steps(p, a.hist, sh.S, sh.log, K);
+            if (c.known) pass_known_steps(p, a.hist, sh.S, sh.log, K);
             else sh.reach[0] = crack_cut_in_reach(p, sh.S) ? 1 : 0;
         }
     }
@@ -310,239 +687,32 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
             if (q <= K) sh.ws[e][q] = a.edge[e] == EDGE_DIRICHLET ? load_value(a.load[e], n + q, (double)p.dt) : 0.0;
         }
     }
-    const bool follow = KIND == 2 && !known && (ev_r || ev_l);
+    c.is_l = KIND != 0 && !per && x0 == 0;
+    c.kr = KIND != 0 && !per && nx - 1 - x0 >= 0 && nx - 1 - x0 < N ? nx - 1 - x0 : -1;
 
-    // this thread's edge columns: element 0 is column 0, element kr column nx - 1
-    const bool is_l = KIND != 0 && !per && x0 == 0;
-    const int kr = KIND != 0 && !per && nx - 1 - x0 >= 0 && nx - 1 - x0 < N ? nx - 1 - x0 : -1;
-    const T gg = a.g, dt = a.dt;
-
-    for (int s = 0; s < K; ++s) {
-        const int b = s & 1;
-        stg_row(&sh.top[b][warp][lane * N], w[RPT - 1]);
-        stg_row(&sh.bot[b][warp][lane * N], w[0]);
-        if (KIND == 2 && known && warp == kBelowWarp) stg_row(&sh.pair[s][0][lane * N], w[RPT - 1]);
-        if (KIND == 2 && known && warp == kBelowWarp + 1) stg_row(&sh.pair[s][1][lane * N], w[0]);
-        __syncthreads();
-        if (KIND == 2 && follow) {
-            const bool reach = sh.reach[b] != 0;
-            if (warp == 0) {
-                pass_crack_step<T>(p, sh.top[b][kBelowWarp], sh.bot[b][kBelowWarp + 1], org_r, org_l, sh.S, a.hist, ev_r,
-                                   ev_l, own_r, own_l);
-                if (lane == 0) sh.reach[b ^ 1] = crack_cut_in_reach(p, sh.S) ? 1 : 0;
-            }
-            // rows next to the crack wait for the decision only where it can cut a link
-            if (reach) __syncthreads();
+    c.side = KIND != 0 && __any_sync(kFull, c.is_l || c.kr >= 0);
+    // bulk tiles: two steps an iteration (PassRows); an odd last step leaves
+    // the rows where a step of phase 0 writes them.  The other tiles, whose
+    // step is far longer code, take every step in phase 0 and move the rows
+    // back: unrolled twice, it ran out of the instruction cache.
+    int s = 0;
+    if (KIND == 0) {
+        for (; s + 2 <= K; s += 2) {
+            pass_step<T, D, RPT, KIND, 0>(A, c, s, F, sh);
+            pass_step<T, D, RPT, KIND, 1>(A, c, s + 1, F, sh);
         }
-        R prev, upx;
-        ld_row(&sh.top[b][warp > 0 ? warp - 1 : 0][lane * N], prev);
-        ld_row(&sh.bot[b][warp < kPassWarps - 1 ? warp + 1 : warp][lane * N], upx);
-        uint32_t cut = 0u;
-        if (KIND == 2 && (warp == kBelowWarp || warp == kBelowWarp + 1)) {
-            const int f = known ? sh.log[s + 1].f : (ev_l ? sh.S.i_first : f0);
-            const int l = known ? sh.log[s + 1].l : (ev_r ? sh.S.i_last : l0);
+    }
+    for (; s < K; ++s) {
+        pass_step<T, D, RPT, KIND, 0>(A, c, s, F, sh);
 #pragma unroll
-            for (int k = 0; k < N; ++k) {
-                int c = x0 + k;
-                if (per) c = wrap_col(c, nx);
-                if (c >= f && c <= l) cut |= 1u << k;
-            }
-        }
-        T tl = (T)0, tr = (T)0, tb = (T)0, tt = (T)0;
-        if (KIND != 0) {
-            tl = (T)2 * (T)sh.ws[LEFT][s];
-            tr = (T)2 * (T)sh.ws[RIGHT][s];
-            tb = (T)2 * (T)sh.ws[BOTTOM][s];
-            tt = (T)2 * (T)sh.ws[TOP][s];
-        }
-        R first;   // the first row before the update (strip: row jc; edge rule: row 0)
-        if (KIND != 0) first = w[0];
-        T el[KIND != 0 ? RPT : 1], er[KIND != 0 ? RPT : 1];   // edge rule: the edge columns before the update
-        if (KIND != 0 && A.q.edge_macro) {
-#pragma unroll
-            for (int r = 0; r < RPT; ++r) {
-                el[r] = w[r].v[0];
-#pragma unroll
-                for (int k = 0; k < N; ++k)
-                    if (k == 0 || k == kr) er[r] = w[r].v[k];
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < RPT; ++r) {
-            const R cur = w[r];
-            R up = r + 1 < RPT ? w[r + 1] : upx;
-            R dn = prev;
-            T left0 = __shfl_up_sync(kFull, cur.v[N - 1], 1);
-            T rightN = __shfl_down_sync(kFull, cur.v[0], 1);
-            if (KIND != 0) {
-                const int j = jb + r;
-                if (j == ny - 1) {
-#pragma unroll
-                    for (int k = 0; k < N; ++k) up.v[k] = a.edge[TOP] == EDGE_DIRICHLET ? tt - cur.v[k] : cur.v[k];
-                }
-                if (j == 0) {
-#pragma unroll
-                    for (int k = 0; k < N; ++k) dn.v[k] = a.edge[BOTTOM] == EDGE_DIRICHLET ? tb - cur.v[k] : cur.v[k];
-                }
-                if (KIND == 2 && r == RPT - 1 && warp == kBelowWarp) {
-#pragma unroll
-                    for (int k = 0; k < N; ++k)
-                        if ((cut >> k) & 1u) up.v[k] = cur.v[k];
-                }
-                if (KIND == 2 && r == 0 && warp == kBelowWarp + 1) {
-#pragma unroll
-                    for (int k = 0; k < N; ++k)
-                        if ((cut >> k) & 1u) dn.v[k] = cur.v[k];
-                }
-                if (is_l) left0 = a.edge[LEFT] == EDGE_DIRICHLET ? tl - cur.v[0] : cur.v[0];
-            }
-#pragma unroll
-            for (int k = 0; k < N; ++k) {
-                const T wl = k == 0 ? left0 : cur.v[k - 1];
-                T wr = k == N - 1 ? rightN : cur.v[k + 1];
-                if (KIND != 0 && k == kr) wr = a.edge[RIGHT] == EDGE_DIRICHLET ? tr - cur.v[k] : cur.v[k];
-                const T lap = ((up.v[k] + dn.v[k]) + (wl + wr)) - (T)4 * cur.v[k];
-                T wn, dn_;
-                site_update<T, D>(cur.v[k], d[r].v[k], lap, gg, dt, wn, dn_);
-                w[r].v[k] = wn;
-                if (std::is_same<D, Lf>::value) d[r].v[k] = cur.v[k];
-                else d[r].v[k] = wd_round<D, T>(dn_, wd_scale, wd_inv);
-            }
-            prev = cur;
-        }
-        if (KIND == 2 && p.macro && cut) {
-            // the crack-face rule: w_B from the two new values further from the crack
-            if (warp == kBelowWarp) {
-#pragma unroll
-                for (int k = 0; k < N; ++k)
-                    if ((cut >> k) & 1u) {
-                        const T wB = (T)1.5 * w[RPT - 2].v[k] - (T)0.5 * w[RPT - 3].v[k];
-                        if (!std::is_same<D, Lf>::value)
-                            d[RPT - 1].v[k] = wd_round<D, T>((wB - prev.v[k]) / dt, wd_scale, wd_inv);
-                        w[RPT - 1].v[k] = wB;
-                    }
+        for (int q = 0; q < RPT; ++q) {
+            const int r = RPT - 1 - q;
+            if constexpr (std::is_same<D, Lf>::value) {
+                const R t = F.a[r];
+                F.a[r] = F.b[r];
+                F.b[r] = t;
             } else {
-#pragma unroll
-                for (int k = 0; k < N; ++k)
-                    if ((cut >> k) & 1u) {
-                        const T wB = (T)1.5 * w[1].v[k] - (T)0.5 * w[2].v[k];
-                        if (!std::is_same<D, Lf>::value)
-                            d[0].v[k] = wd_round<D, T>((wB - first.v[k]) / dt, wd_scale, wd_inv);
-                        w[0].v[k] = wB;
-                    }
-            }
-        }
-        if (KIND != 0 && A.q.edge_macro) {
-            // the macroscopic rule on the outer edges (the two levels of
-            // edge_rule_at): the edge columns, the crack-face points on
-            // them, then the bottom and top rows and the corners
-            const bool on_l = a.edge[LEFT] != EDGE_PERIODIC, on_r = a.edge[RIGHT] != EDGE_PERIODIC;
-            EdgeRule<T> E;
-            E.wn = nullptr;
-            E.pitch = 0;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                E.dir[e] = a.edge[e] == EDGE_DIRICHLET;
-                E.ws[e] = (T)sh.ws[e][s + 1];
-            }
-            R in[3];            // rows 0 .. 2 (or ny-1 .. ny-3) before the edge columns
-            const bool has_b = jb == 0, has_t = jb + RPT == ny;
-#pragma unroll
-            for (int q = 0; q < 3; ++q) in[q] = has_t ? w[RPT - 1 - q] : w[q];
-#pragma unroll
-            for (int r = 0; r < RPT; ++r) {
-                const int j = jb + r;
-                const T p1 = __shfl_up_sync(kFull, w[r].v[N - 1], 1), p2 = __shfl_up_sync(kFull, w[r].v[N - 2], 1);
-                const T n0 = __shfl_down_sync(kFull, w[r].v[0], 1);
-                if (j < 1 || j > ny - 2) continue;
-                if (is_l && on_l) {
-                    const T v2 = N > 2 ? w[r].v[N > 2 ? 2 : 0] : n0;
-                    w[r].v[0] = E.rule(LEFT, w[r].v[1], v2);
-                }
-                if (kr >= 0 && on_r) {
-                    T wI = p1, wII = p2;
-#pragma unroll
-                    for (int k = 1; k < N; ++k)
-                        if (k == kr) {
-                            wI = w[r].v[k - 1];
-                            wII = k >= 2 ? w[r].v[k >= 2 ? k - 2 : 0] : p1;
-                        }
-                    const T v = E.rule(RIGHT, wI, wII);
-#pragma unroll
-                    for (int k = 0; k < N; ++k)
-                        if (k == kr) w[r].v[k] = v;
-                }
-            }
-            if (KIND == 2 && p.macro && cut && (is_l || kr >= 0)) {
-#pragma unroll
-                for (int k = 0; k < N; ++k) {
-                    if (!((cut >> k) & 1u) || !((is_l && on_l && k == 0) || (on_r && k == kr))) continue;
-                    if (warp == kBelowWarp) w[RPT - 1].v[k] = (T)1.5 * w[RPT - 2].v[k] - (T)0.5 * w[RPT - 3].v[k];
-                    else w[0].v[k] = (T)1.5 * w[1].v[k] - (T)0.5 * w[2].v[k];
-                }
-            }
-            if (has_b || has_t) {
-                const int ev = has_t ? TOP : BOTTOM;
-                R e1, e2;   // the rows one and two from the edge, after the edge columns
-#pragma unroll
-                for (int k = 0; k < N; ++k) {
-                    e1.v[k] = has_t ? w[RPT - 2].v[k] : w[1].v[k];
-                    e2.v[k] = has_t ? w[RPT - 3].v[k] : w[2].v[k];
-                }
-                R o;
-#pragma unroll
-                for (int k = 0; k < N; ++k) o.v[k] = E.rule(ev, in[1].v[k], in[2].v[k]);
-                // corners: along the bottom / top edge's normal from the edge
-                // columns, or (its side Dirichlet, ev not) along the row from
-                // the points of edge ev
-                const T q1 = __shfl_up_sync(kFull, o.v[N - 1], 1), q2 = __shfl_up_sync(kFull, o.v[N - 2], 1);
-                const T m0 = __shfl_down_sync(kFull, o.v[0], 1);
-                T cl = (T)0, cr = (T)0;
-                if (is_l && on_l)
-                    cl = a.edge[LEFT] == EDGE_DIRICHLET && a.edge[ev] != EDGE_DIRICHLET
-                             ? E.rule(LEFT, o.v[1], N > 2 ? o.v[N > 2 ? 2 : 0] : m0)
-                             : E.rule(ev, e1.v[0], e2.v[0]);
-                if (kr >= 0 && on_r) {
-                    T oI = q1, oII = q2, c1 = (T)0, c2 = (T)0;
-#pragma unroll
-                    for (int k = 0; k < N; ++k)
-                        if (k == kr) {
-                            if (k >= 1) oI = o.v[k >= 1 ? k - 1 : 0];
-                            if (k >= 1) oII = k >= 2 ? o.v[k >= 2 ? k - 2 : 0] : q1;
-                            c1 = e1.v[k];
-                            c2 = e2.v[k];
-                        }
-                    cr = a.edge[RIGHT] == EDGE_DIRICHLET && a.edge[ev] != EDGE_DIRICHLET ? E.rule(RIGHT, oI, oII)
-                                                                                       : E.rule(ev, c1, c2);
-                }
-                if (is_l && on_l) o.v[0] = cl;
-#pragma unroll
-                for (int k = 0; k < N; ++k)
-                    if (on_r && k == kr) o.v[k] = cr;
-                if (has_t) w[RPT - 1] = o;
-                else w[0] = o;
-            }
-            if (!std::is_same<D, Lf>::value) {
-                // wdot of the sites that took the rule
-#pragma unroll
-                for (int r = 0; r < RPT; ++r) {
-                    const int j = jb + r;
-                    if (j == 0 || j == ny - 1) {
-                        if ((r == 0 && has_b) || (r == RPT - 1 && has_t)) {
-#pragma unroll
-                            for (int k = 0; k < N; ++k)
-                                d[r].v[k] = wd_round<D, T>((w[r].v[k] - (r == 0 ? first.v[k] : prev.v[k])) / dt, wd_scale,
-                                                           wd_inv);
-                        }
-                        continue;
-                    }
-                    if (is_l && on_l) d[r].v[0] = wd_round<D, T>((w[r].v[0] - el[r]) / dt, wd_scale, wd_inv);
-                    if (kr >= 0 && on_r) {
-#pragma unroll
-                        for (int k = 0; k < N; ++k)
-                            if (k == kr) d[r].v[k] = wd_round<D, T>((w[r].v[k] - er[r]) / dt, wd_scale, wd_inv);
-                    }
-                }
+                F.a[r + 1] = F.a[r];
             }
         }
     }
@@ -551,53 +721,54 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
     T acc = (T)0;
 #pragma unroll
     for (int r = 0; r < RPT; ++r) {
+        const R &w = F.template cur<0>(r), &d = F.b[r];
         const int j = jb + r;
         if (j < g.y0 || j >= g.y1) continue;
         if (x0 + N <= g.x0 || x0 >= g.x1) continue;
         const int64_t o = (int64_t)j * P + x0;
         if (KIND == 0 || (x0 >= g.x0 && x0 + N <= g.x1 && x0 >= 0 && x0 + N <= nx)) {
-            stg_row(a.w_out + o, w[r]);
-            wd_store(a.wd + o, d[r], wd_scale);
-            if (KIND != 0) write_pads(a, x0, j, w[r]);
-            acc += w[r].v[0];
+            stg_row(a.w_out + o, w);
+            wd_store(a.wd + o, d, wd_scale);
+            if (KIND != 0) write_pads(a, x0, j, w);
+            acc += w.v[0];
         } else {
 #pragma unroll
             for (int k = 0; k < N; ++k) {
-                int c = x0 + k;
-                if (c < g.x0 || c >= g.x1) continue;
-                if (per) c = wrap_col(c, nx);
-                if (c < 0 || c >= nx) continue;
+                int q = x0 + k;
+                if (q < g.x0 || q >= g.x1) continue;
+                if (per) q = wrap_col(q, nx);
+                if (q < 0 || q >= nx) continue;
                 T *row = a.w_out + (int64_t)j * P;
-                const T v = w[r].v[k];
-                row[c] = v;
-                wd_put(a.wd + (int64_t)j * P + c, d[r].v[k], wd_scale);
-                if (c == 0) {
+                const T v = w.v[k];
+                row[q] = v;
+                wd_put(a.wd + (int64_t)j * P + q, d.v[k], wd_scale);
+                if (q == 0) {
                     if (a.edge[LEFT] == EDGE_FREE) row[-1] = v;
                     else if (per) row[nx] = v;
                 }
-                if (c == nx - 1) {
+                if (q == nx - 1) {
                     if (a.edge[RIGHT] == EDGE_FREE) row[nx] = v;
                     else if (per) row[-1] = v;
                 }
-                if (j == 0 && a.edge[BOTTOM] == EDGE_FREE) row[c - P] = v;
-                if (j == ny - 1 && a.edge[TOP] == EDGE_FREE) row[c + P] = v;
+                if (j == 0 && a.edge[BOTTOM] == EDGE_FREE) row[q - P] = v;
+                if (j == ny - 1 && a.edge[TOP] == EDGE_FREE) row[q + P] = v;
                 acc += v;
             }
         }
     }
     if (__any_sync(kFull, !isfinite(acc)) && lane == 0) atomicOr(a.err, (uint32_t)ERR_NONFINITE);
 
-    if (KIND == 2 && (own_r || own_l)) {
-        if (known) {
+    if (KIND == 2 && (c.own_r || c.own_l)) {
+        if (c.known) {
             // the K fits of the pass's crack steps, one step per warp: their
             // decisions did not wait for them
             if (warp >= rec0 && warp < K) {
-                for (int dir = 1; dir >= (own_l ? -1 : 1); dir -= 2) {
-                    if (dir > 0 && !own_r) continue;
+                for (int dir = 1; dir >= (c.own_l ? -1 : 1); dir -= 2) {
+                    if (dir > 0 && !c.own_r) continue;
                     const PassTip &q = sh.log[warp], &q1 = sh.log[warp + 1];
-                    const int org = dir > 0 ? org_r : org_l;
+                    const int org = dir > 0 ? c.org_r : c.org_l;
                     const double v_prev = p.mode == CRACK_PRESCRIBED ? p.v_rel : 0.0;
-                    const CrackSums c = crack_eval_pairs<T, 32>(
+                    const CrackSums f = crack_eval_pairs<T, 32>(
                         p, dir > 0 ? q.tr : q.tl, v_prev, q.f, q.l, dir, [&](int i, T &ab, T &be) {
                             const int e = i - org;
                             if (e < 0 || e >= W) return false;
@@ -606,20 +777,20 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
                             return true;
                         });
                     if (lane == 0) {
-                        const double Kf = c.np > 0 ? p.mu / 4.0 * c.num / c.den : 0.0;
+                        const double Kf = f.np > 0 ? p.mu / 4.0 * f.num / f.den : 0.0;
                         if (!isfinite(Kf)) atomicOr(a.err, (uint32_t)ERR_NONFINITE);
                         if (p.hist_cap > 0) {
                             const int64_t h = (hist0 + (warp - rec0)) % p.hist_cap;
                             (dir > 0 ? a.hist.K : a.hist.Kl)[h] = Kf;
                             (dir > 0 ? a.hist.v : a.hist.vl)[h] = dir > 0 ? q1.vr : q1.vl;
                             (dir > 0 ? a.hist.tip : a.hist.tipl)[h] = dir > 0 ? q1.tr : q1.tl;
-                            (dir > 0 ? a.hist.np : a.hist.npl)[h] = c.np;
+                            (dir > 0 ? a.hist.np : a.hist.npl)[h] = f.np;
                         }
                         if (warp == K - 1) {
                             TipState &O = dir > 0 ? a.s_out->r : a.s_out->l;
                             O.K = Kf;
-                            O.r_min = c.r_min;
-                            O.npairs = c.np;
+                            O.r_min = f.r_min;
+                            O.npairs = f.np;
                         }
                     }
                 }
@@ -630,32 +801,32 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
         if (tid == 0) {
             CrackState *o = a.s_out;
             const CrackState &S = sh.S;
-            if (own_r) {
+            if (c.own_r) {
                 o->step = S.step + K;
                 o->hist_n = S.hist_n;
                 o->i_last = S.i_last;
                 if (!p.two_tips) o->i_first = S.i_first;
                 copy_tip_decision(o->r, S.r);
-                if (!known) {
+                if (!c.known) {
                     o->r.K = S.r.K;
                     o->r.r_min = S.r.r_min;
                     o->r.npairs = S.r.npairs;
                 }
                 o->r.decided = 0;
-                for (int i = l0 + 1; i <= S.i_last; ++i)
-                    if (i >= f0) atomicOr(&a.cut_v[(int64_t)(p.jc - 1) * p.words + (i >> 5)], 1u << (i & 31));
+                for (int i = c.l0 + 1; i <= S.i_last; ++i)
+                    if (i >= c.f0) atomicOr(&a.cut_v[(int64_t)(p.jc - 1) * p.words + (i >> 5)], 1u << (i & 31));
             }
-            if (own_l) {
+            if (c.own_l) {
                 o->i_first = S.i_first;
                 copy_tip_decision(o->l, S.l);
-                if (!known) {
+                if (!c.known) {
                     o->l.K = S.l.K;
                     o->l.r_min = S.l.r_min;
                     o->l.npairs = S.l.npairs;
                 }
                 o->l.decided = 0;
-                for (int i = S.i_first; i < f0; ++i)
-                    if (i <= l0) atomicOr(&a.cut_v[(int64_t)(p.jc - 1) * p.words + (i >> 5)], 1u << (i & 31));
+                for (int i = S.i_first; i < c.f0; ++i)
+                    if (i <= c.l0) atomicOr(&a.cut_v[(int64_t)(p.jc - 1) * p.words + (i >> 5)], 1u << (i & 31));
             }
         }
     }
