@@ -59,6 +59,8 @@ void ChunkGraph::reset()
 
 namespace {
 
+// Passes of one cooperative launch, at most (an even number).
+constexpr int64_t kMaxPasses = 1 << 16;
 // The largest scratch planes a handle takes for its passes (lattices of up to 1.4e9 FP32 sites, leapfrog 7e8).
 constexpr size_t kMaxPassScratch = (size_t)6 << 30;
 constexpr int64_t kDefaultHistCap = 65536;
@@ -383,24 +385,25 @@ cudaError_t enqueue_step(const lbm_handle *h, int par, cudaStream_t s)
     }
 }
 
-// One pass of K steps; second: the second pass of a pair.
+// n_pass passes of K steps (one, or an even number in one launch); second: the
+// second pass of a pair.
 template <typename T, typename D>
-cudaError_t enqueue_pass_t(const lbm_handle *h, const lbm::PassPlan &q, int par, bool second, cudaStream_t s)
+cudaError_t enqueue_pass_t(const lbm_handle *h, const lbm::PassPlan &q, int par, bool second, int n_pass, cudaStream_t s)
 {
     lbm::NvtxRange r("K1 pass");
     lbm::PassArgs<T, D> a;
     make_pass_args(h, par, second, q, a);
-    return launch_pass(a, h->pass_rpt, s);
+    return launch_pass(a, n_pass, s);
 }
 
-cudaError_t enqueue_pass(const lbm_handle *h, const lbm::PassPlan &q, int par, bool second, cudaStream_t s)
+cudaError_t enqueue_pass(const lbm_handle *h, const lbm::PassPlan &q, int par, bool second, int n_pass, cudaStream_t s)
 {
     switch (h->lat.storage) {
-    case LBM_F32: return enqueue_pass_t<float, float>(h, q, par, second, s);
-    case LBM_F32_WD_BF16: return enqueue_pass_t<float, __nv_bfloat16>(h, q, par, second, s);
-    case LBM_F32_WD_F16: return enqueue_pass_t<float, __half>(h, q, par, second, s);
-    case LBM_F32_LEAPFROG: return enqueue_pass_t<float, Lf>(h, q, par, second, s);
-    default: return enqueue_pass_t<double, double>(h, q, par, second, s);
+    case LBM_F32: return enqueue_pass_t<float, float>(h, q, par, second, n_pass, s);
+    case LBM_F32_WD_BF16: return enqueue_pass_t<float, __nv_bfloat16>(h, q, par, second, n_pass, s);
+    case LBM_F32_WD_F16: return enqueue_pass_t<float, __half>(h, q, par, second, n_pass, s);
+    case LBM_F32_LEAPFROG: return enqueue_pass_t<float, Lf>(h, q, par, second, n_pass, s);
+    default: return enqueue_pass_t<double, double>(h, q, par, second, n_pass, s);
     }
 }
 
@@ -517,7 +520,7 @@ lbm_status check_sticky(lbm_handle *h)
     }
     if (err & ERR_TIMEOUT) {
         h->sticky = LBM_ERR_TIMEOUT;
-        return fail(LBM_ERR_TIMEOUT, "a bounded device wait gave up (grid barrier of a persistent batched step)");
+        return fail(LBM_ERR_TIMEOUT, "a bounded device wait gave up (grid barrier of a persistent batched step or of a launch of several passes)");
     }
     if ((err & ERR_NONFINITE) || ((hs.r.flags | hs.l.flags) & FLAG_NONFINITE)) {
         h->sticky = LBM_ERR_UNSTABLE;
@@ -961,7 +964,7 @@ lbm_status create_impl(const lbm_grid *grid, const lbm_lattice *lattice, const l
     const size_t o_ch = off; off = align256(off + mask);
     const size_t o_cv = off; off = align256(off + mask_v);
     const size_t o_st = off; off = align256(off + 2 * sizeof(CrackState));
-    const size_t o_er = off; off = align256(off + sizeof(uint32_t));
+    const size_t o_er = off; off = align256(off + 64 + sizeof(lbm::GridBarrier));
     const size_t o_un = off; off = align256(off + (size_t)grid->ny * sizeof(Unit));
     const size_t o_hK = off; off = align256(off + (size_t)hcap * 8);
     const size_t o_hv = off; off = align256(off + (size_t)hcap * 8);
@@ -1014,6 +1017,7 @@ lbm_status create_impl(const lbm_grid *grid, const lbm_lattice *lattice, const l
     h->cut_v = reinterpret_cast<uint32_t *>(base + o_cv) + h->words;
     h->st = reinterpret_cast<CrackState *>(base + o_st);
     h->err = reinterpret_cast<uint32_t *>(base + o_er);
+    h->pass_bar = reinterpret_cast<lbm::GridBarrier *>(base + o_er + 64);
     h->units = reinterpret_cast<Unit *>(base + o_un);
     h->hist.K = reinterpret_cast<double *>(base + o_hK);
     h->hist.v = reinterpret_cast<double *>(base + o_hv);
@@ -1219,21 +1223,39 @@ lbm_status lbm_step(lbm_handle *h, int64_t n)
         lbm_status rc = LBM_OK;
         if (h->pass_k && !h->own_bands && !h->bulk) {
             // as many pairs of passes as n holds, then a pair of shorter ones
-            // for what is left (a pair of K steps covers 2 K of them)
-            lbm::PassPlan q;
-            const int64_t pairs = n / (2 * h->pass_k);
-            const int base = par;
-            if (pairs > 0 && pass_plan(h, h->pass_k, h->pass_rpt, q)) {
-                rc = run_chunks(h->passes, h->gen, h->stream, h->cap_stream, 2 * pairs, par,
-                                [&](int p, cudaStream_t s) { return enqueue_pass(h, q, p, p != base, s); });
-                if (rc != LBM_OK) return rc;
-                n -= pairs * 2 * h->pass_k;
-            }
-            const int K = (int)std::min<int64_t>(n / 2, h->pass_k);
-            if (K >= 2 && pass_plan(h, K, h->pass_rpt, q)) {
-                LBM_CUDA(enqueue_pass(h, q, base, false, h->stream));
-                LBM_CUDA(enqueue_pass(h, q, base ^ 1, true, h->stream));
-                n -= 2 * K;
+            // for what is left (a pair of K steps covers 2 K of them); or, for
+            // few steps, equally long passes where that leaves at most one step
+            while (n >= 4) {
+                int K = (int)std::min<int64_t>(n / 2, h->pass_k);
+                int64_t pairs = n / (2 * K);
+                if (n < 4 * h->pass_k) {
+                    const int64_t m = (n + 2 * h->pass_k - 1) / (2 * h->pass_k), k = n / (2 * m);
+                    if (k >= 2 && n - 2 * m * k <= 1) {
+                        K = (int)k;
+                        pairs = m;
+                    }
+                }
+                lbm::PassPlan q;
+                if (!pass_plan(h, K, h->pass_nw, h->pass_rpt, q)) break;
+                if (q.tiles <= h->pass_slots) {
+                    // every tile resident: the passes in one launch
+                    for (int64_t left = 2 * pairs; left > 0;) {
+                        const int m = (int)std::min<int64_t>(left, kMaxPasses);
+                        LBM_CUDA(enqueue_pass(h, q, par, false, m, h->stream));
+                        left -= m;
+                    }
+                } else if (K == h->pass_k) {
+                    const int base = par;
+                    rc = run_chunks(h->passes, h->gen, h->stream, h->cap_stream, 2 * pairs, par,
+                                    [&](int p, cudaStream_t s) { return enqueue_pass(h, q, p, p != base, 1, s); });
+                    if (rc != LBM_OK) return rc;
+                } else {
+                    for (int64_t m = 0; m < pairs; ++m) {
+                        LBM_CUDA(enqueue_pass(h, q, par, false, 1, h->stream));
+                        LBM_CUDA(enqueue_pass(h, q, par ^ 1, true, 1, h->stream));
+                    }
+                }
+                n -= pairs * 2 * K;
             }
         }
         // runs of single steps replay graphs of 64, 32, ..., 2 steps

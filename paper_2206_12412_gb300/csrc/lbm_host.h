@@ -130,7 +130,9 @@ struct lbm_handle {
     // that the buffers end where an even number of single steps leaves them
     lbm::host::ChunkGraph passes;  // graphs of runs of passes of pass_k steps
     int32_t pass_k;      // steps of a pass (0: single steps only)
-    int32_t pass_rpt;    // rows per thread of its bulk tiles
+    int32_t pass_slots;  // tiles resident at once
+    int32_t pass_nw, pass_rpt;   // warps of its tiles, rows per thread of the bulk ones
+    lbm::GridBarrier *pass_bar;  // of the cooperative launches of several passes, device
     bool own_bands;      // lbm_set_launch chose the bands of the single step: no passes
     void *alt[2];        // scratch planes between two passes: wdot (leapfrog: w and the w before it)
     lbm_status sticky;
@@ -209,8 +211,8 @@ inline void make_step_args(const lbm_handle *h, int par, StepArgs<T, D> &a)
 // The tiles of a pass of K steps of this lattice (lbm_pass_plan.cu); false
 // where a pass of K steps cannot be split so that every tile that needs a
 // crack decision holds what decides it.
-bool pass_plan(const lbm_handle *h, int K, int rpt, lbm::PassPlan &q);
-// Choose the pass of this lattice: h->pass_k, h->pass_rpt.
+bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, lbm::PassPlan &q);
+// Choose the pass of this lattice: h->pass_k, h->pass_nw, h->pass_rpt.
 void choose_pass(lbm_handle *h);
 
 // Arguments of pass number `second` of a pair (the first reads the state of
@@ -221,6 +223,8 @@ inline void make_pass_args(const lbm_handle *h, int par, bool second, const lbm:
 {
     make_step_args(h, par, a.s);
     a.q = q;
+    a.bar = h->pass_bar;
+    a.budget = (long long)1 << 31;
     if constexpr (std::is_same<D, lbm::Lf>::value) {
         // (w_n, w_{n-1}): W[par], W[par ^ 1] -> the scratch planes -> back
         a.s.w_in = static_cast<const T *>(second ? h->alt[0] : h->w[par]);
@@ -231,6 +235,11 @@ inline void make_pass_args(const lbm_handle *h, int par, bool second, const lbm:
         a.wd_in = static_cast<const D *>(second ? h->alt[0] : h->wd);
         a.s.wd = static_cast<D *>(second ? h->wd : h->alt[0]);
     }
+    // the other pass of the pair: back from where this one writes
+    a.w_in1 = a.s.w_out;
+    a.wd_in1 = a.s.wd;
+    a.w_out1 = const_cast<T *>(a.s.w_in);
+    a.wd1 = const_cast<D *>(a.wd_in);
 }
 
 // Whether the single-lattice step launch adds the record CTA (StepArgs::k_cta)

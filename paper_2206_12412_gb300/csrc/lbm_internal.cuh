@@ -208,6 +208,13 @@ struct FinalizeArgs {
 // mb + mt row tiles.
 struct PassPlan {
     int32_t K, hc;             // steps; halo columns on each side (K rounded up to whole vectors)
+    int32_t nw, rpt;           // warps of a tile; rows per thread of the bulk tiles
+    // the K window of an end at rest (prescribed growth: at its speed), in
+    // units of 2^-32 dh behind the tip; its r_min; at most one pair in any window
+    int64_t lo_q, hi_q;
+    double r_min;
+    int32_t one_pair;
+    float k_unit, k_rest;      // mu / 4 sqrt(2 pi / dh) 2^16; just below K_C
     int32_t mx, px;            // column tiles of the bulk and their width
     int32_t jb, mb, pb;        // rows [0, jb) below the strip: mb row tiles of pb rows
     int32_t jt, mt, pt;        // rows [jt, ny) above it (a lattice without a crack: all rows)
@@ -217,10 +224,23 @@ struct PassPlan {
     int32_t tiles, edge_macro;
 };
 
+// The grid barrier of the cooperative launches: arrivals of the current
+// round and the round number (zeroed before a launch).
+struct GridBarrier {
+    unsigned int count, gen;
+};
+
 template <typename T, typename D>
 struct PassArgs {
     StepArgs<T, D> s;          // w_in, w_out; s.wd: the wdot plane the pass writes (leapfrog: w of the step before last)
     const D *wd_in;            // the wdot plane it reads (leapfrog: w_{n-1})
+    // the buffers of every second pass of a launch of several, which swaps s.s_in and s.s_out
+    const T *w_in1;
+    const D *wd_in1;
+    T *w_out1;
+    D *wd1;
+    GridBarrier *bar;          // the barrier between its passes, a wait at most `budget` cycles
+    long long budget;
     PassPlan q;
 };
 
@@ -289,12 +309,6 @@ struct AdjArgs {
     int32_t slots, pad;
 };
 
-// The grid barrier of the persistent batched kernel: arrivals of the current
-// round and the round number (zeroed before a launch).
-struct GridBarrier {
-    unsigned int count, gen;
-};
-
 // One row copy of the halo exchange between row slabs (whole padded rows).
 struct RowCopy {
     const void *src;
@@ -325,8 +339,9 @@ cudaError_t launch_batch_pieces(const StepArgs<T, D> *descs, const BatchPiece *p
                                 int par, cudaStream_t s, int threads, int lookahead, bool chained);
 template <typename T, typename D>
 cudaError_t launch_step(const StepArgs<T, D> &a, int bands, cudaStream_t s, bool bulk = false);
-// A pass of several time steps; rpt: rows per thread of the bulk tiles (4 or 8).
-template <typename T, typename D> cudaError_t launch_pass(const PassArgs<T, D> &a, int rpt, cudaStream_t s);
+// n_pass passes of several time steps (more than one: one cooperative launch).
+template <typename T, typename D> cudaError_t launch_pass(const PassArgs<T, D> &a, int n_pass, cudaStream_t s);
+template <typename T, typename D> const void *pass_kernel_ptr(int nw, int rpt);
 template <typename T, typename D> cudaError_t launch_edge_rule(const StepArgs<T, D> &a, cudaStream_t s);
 template <typename T, typename D> int edge_rule_count(const StepArgs<T, D> &a);
 template <typename T, typename D>

@@ -11,7 +11,7 @@
 // of every site is the single step's, operation for operation, so a pass
 // gives the same bits as K single steps.
 //
-// Tile: 8 warps on top of one another, a warp spans 32 16-byte vectors of
+// Tile: 8 warps (small FP64 lattices: 4) on top of one another, a warp spans 32 16-byte vectors of
 // columns (128 FP32 columns), a thread holds RPT rows of one vector (w and
 // wdot: 64 registers at 8 rows).  East and west neighbours come by shuffles
 // within the warp, the rows between warps through shared memory (16-byte
@@ -38,6 +38,7 @@
 // owns the tip's column records it.
 #pragma once
 
+#include "lbm_barrier.cuh"
 #include "lbm_crack.cuh"
 #include "lbm_internal.cuh"
 #include "lbm_rows.cuh"
@@ -46,12 +47,8 @@
 
 namespace lbm {
 
-constexpr int kPassWarps = 8;
-constexpr int kPassThreads = 32 * kPassWarps;
-constexpr int kPassSteps = 8;     // most steps of a pass
+constexpr int kPassSteps = 8;     // most steps of a pass (and no more than a tile has warps)
 constexpr int kStripRpt = 4;      // rows per thread of a strip tile
-constexpr int kStripHalf = kPassWarps * kStripRpt / 2;   // rows of a strip tile on each side of the crack line
-constexpr int kBelowWarp = kPassWarps / 2 - 1;           // the warp whose last row is jc - 1; the next one's first is jc
 
 // One site's wdot as the next step reads it back from storage.
 template <typename D, typename T> __device__ __forceinline__ T wd_round(T v, T, T) { return v; }
@@ -62,12 +59,6 @@ template <> __device__ __forceinline__ float wd_round<__nv_bfloat16, float>(floa
 template <> __device__ __forceinline__ float wd_round<__half, float>(float v, float scale, float inv)
 {
     return __half2float(__float2half_rn(v * scale)) * inv;
-}
-template <typename D, typename T> __device__ __forceinline__ T wd_get(const D *p, T inv)
-{
-    if constexpr (std::is_same<D, Lf>::value) return p->v;
-    else if constexpr (sizeof(D) == 2) return WdIO<D>::get(p, inv);
-    else return *p;
 }
 template <typename D, typename T, int N>
 __device__ __forceinline__ void wd_store(D *p, const Row<T, N> &r, T scale)
@@ -102,6 +93,34 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
     uint64_t r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
+}
+
+// (new - old) / dt; exact without the division where dt = 1.  The division is
+// a call of its own, so that it is not computed and dropped there (inlined, it
+// was: with the slow path it takes for zeros, the crack-face rule of a strip
+// tile cost 850 cycles a step).
+template <typename T> static __device__ __noinline__ T div_dt(T d, T dt) { return d / dt; }
+template <typename T, int N> __device__ __forceinline__ Row<T, N> rate_of(const Row<T, N> &wn, const Row<T, N> &w0, T dt)
+{
+    Row<T, N> d;
+#pragma unroll
+    for (int k = 0; k < N; ++k) d.v[k] = wn.v[k] - w0.v[k];
+    if (dt != (T)1) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) d.v[k] = div_dt(d.v[k], dt);
+    }
+    return d;
+}
+
+// What the row next to an edge receives over it: its own values (free), 2 w* -
+// w (Dirichlet).
+template <typename T, int N>
+__device__ __forceinline__ Row<T, N> edge_image(const Row<T, N> &w, bool dirichlet, T two_ws)
+{
+    Row<T, N> o;
+#pragma unroll
+    for (int k = 0; k < N; ++k) o.v[k] = dirichlet ? two_ws - w.v[k] : w.v[k];
+    return o;
 }
 
 // The update of one row segment (site_update of each of its sites): cu the
@@ -145,22 +164,24 @@ __device__ __forceinline__ void row_sites(const Row<T, N> &cu, const Row<T, N> &
     }
 }
 
-// Crack state in force during one step of a pass (modes whose decisions need
-// no K: prescribed growth and stationary cracks).
+// The crack state in force during one update of a pass, and the records of
+// the crack step before it (lazy: its K and pairs are formed at the end).
 struct PassTip {
     int64_t tr, tl;
-    double vr, vl;       // speeds recorded by the crack step before the update
-    int32_t f, l;
+    double vr, vl, Kr, Kl;
+    int32_t f, l, npr, npl;
+    int32_t arr_r, arr_l, lazy, pad;
 };
 
-template <typename T>
+template <typename T, int NW>
 struct PassShared {
     static constexpr int W = 32 * Vec<T>::N;
-    alignas(16) T top[2][kPassWarps][W];    // each warp's last row, by step parity
-    alignas(16) T bot[2][kPassWarps][W];    // each warp's first row
+    alignas(16) T top[2][NW][W];    // each warp's last row, by step parity
+    alignas(16) T bot[2][NW][W];    // each warp's first row
     alignas(16) T pair[kPassSteps][2][W];   // rows jc - 1 and jc of a strip tile at each step
-    double ws[4][kPassSteps + 1];           // w* of the Dirichlet edges at t_n .. t_{n+K}
+    T ws[4][kPassSteps + 1], ws2[4][kPassSteps + 1];   // w* of the Dirichlet edges at t_n .. t_{n+K}, and twice that
     PassTip log[kPassSteps + 1];
+    CrackState in;                          // the state the pass starts from
     CrackState S;
     int32_t reach[2];
 };
@@ -209,38 +230,165 @@ __device__ __forceinline__ int pass_boundary(int b, int nx, bool per, int lo0, i
     return b;
 }
 
+// The one pair a K window of at most one spacing can hold: the nearest column
+// at least lo_q behind the tip, d its distance (units of 2^-32 dh).
+struct PassPair {
+    int32_t col, in;
+    int64_t d;
+};
+__device__ __forceinline__ PassPair pass_pair(int dir, int64_t tip, int64_t lo_q, int64_t hi_q, int f, int l)
+{
+    const int64_t half = (int64_t)1 << (kQBits - 1);
+    const int64_t i = dir > 0 ? (tip - lo_q - half) >> kQBits : (tip + lo_q - half + ((int64_t)1 << kQBits) - 1) >> kQBits;
+    const int64_t xq = (2 * i + 1) * half;
+    PassPair r;
+    r.d = dir > 0 ? tip - xq : xq - tip;
+    r.in = r.d >= lo_q && r.d < hi_q && i >= f && i <= l;
+    r.col = (int)i;
+    return r;
+}
+// sqrt(r / 2 pi) of a pair, and K from it (the sums of crack_eval_pairs over one pair).
+__device__ __forceinline__ double pass_sf(const CrackParams &p, int64_t d)
+{
+    const double r_h = (double)d * kTwoM32;
+    const double r = p.dh == 1.0 ? r_h : r_h * p.dh;
+    return sqrt(r / (2.0 * kPi));
+}
+template <typename T>
+__device__ __forceinline__ CrackSums pass_sums(double sf, T above, T below, double r_min)
+{
+    const double delta = (double)above - (double)below;
+    return CrackSums{delta * sf, sf * sf, r_min, 1};
+}
+__device__ __forceinline__ double pass_K(const CrackParams &p, const CrackSums &c)
+{
+    return c.np > 0 ? p.mu / 4.0 * c.num / c.den : 0.0;
+}
+
+// What a lane of warp 0 keeps to see that an end at rest stays at rest: the
+// column of its pair of the K window (lanes 0-15 the right end, 16-31 the
+// left; -1: none) and the pair's weight in K, in FP32.
+struct PassWindow {
+    int64_t tip;     // the tip they belong to
+    float coef;
+    int32_t col;
+};
+
+// The window of an end at rest (v = 0).  Its bounds are exact: r = d 2^-32
+// for the integer distance d between tip and column, and lo_q, hi_q are the
+// least integers with d 2^-32 >= r_min, >= r_min + W.
+__device__ __forceinline__ void pass_window(const PassPlan &q, const CrackState &S, int org, bool ev,
+                                            PassWindow &w)
+{
+    const int lane = threadIdx.x & 31, l = lane & 15;
+    const bool right = lane < 16;
+    const int64_t tip = right ? S.r.tip_q : S.l.tip_q, half = (int64_t)1 << (kQBits - 1);
+    const int64_t i = right ? ((tip - q.lo_q - half) >> kQBits) - l
+                            : ((tip + q.lo_q - half + ((int64_t)1 << kQBits) - 1) >> kQBits) + l;
+    const int64_t xq = (2 * i + 1) * half, d = right ? tip - xq : xq - tip;
+    const bool in = ev && d >= q.lo_q && d < q.hi_q && i >= S.i_first && i <= S.i_last;
+    const float r = in ? (float)d : 0.0f;
+    const float sf = sqrtf(r);
+    float den = r;
+    int np = in ? 1 : 0;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+        den += __shfl_xor_sync(0xffffffffu, den, o);
+        np += __shfl_xor_sync(0xffffffffu, np, o);
+    }
+    // |K| <= sum |coef delta| <= np max |coef delta|, K = mu / 4 sum(delta sf) / sum(sf^2), sf = sqrt(r / 2 pi)
+    w.tip = tip;
+    w.col = in ? (int)(i - org) : -1;
+    w.coef = in ? (float)np * q.k_unit * sf / den : 0.0f;
+}
+
 // One K-criterion crack step of a strip tile by warp 0 (all 32 lanes): the
 // ends this tile follows, from the pair rows of the current fields.  below /
 // above: rows jc - 1 and jc of the tile, column i at i - org (org_l for the
-// left end).
-template <typename T>
-__device__ __forceinline__ void pass_crack_step(const CrackParams &p, const T *below, const T *above, int org_r, int org_l,
-                                                CrackState &S, const History &hist, bool ev_r, bool ev_l, bool commit_r,
-                                                bool commit_l)
+// left end).  An end at rest whose K is below K_C by a margin far larger
+// than FP32 rounding stays at rest: that costs one product and a vote, and
+// its K, which decides nothing, is formed for the history at the end of the
+// pass (the exact step is a chain of FP64 divisions, roots and a tanh: 64
+// cycles per operation on GB300, 1.5 us at rest and 3.7 us growing).
+template <typename T, int W>
+__device__ __forceinline__ void pass_crack_step(const CrackParams &p, const PassPlan &q, const T *below, const T *above,
+                                                int org_r, int org_l, CrackState &S, PassTip &rec, bool ev_r, bool ev_l,
+                                                PassWindow &win)
 {
-    constexpr int W = PassShared<T>::W;
     const int lane = threadIdx.x & 31;
     const bool act_r = ev_r && !S.r.decided, act_l = ev_l && !S.l.decided;
     // lanes 0-15 the right end, 16-31 the left: both criteria on the state before either advances
     const int dir = lane < 16 ? +1 : -1;
     const TipState &E = dir > 0 ? S.r : S.l;
     const int org = dir > 0 ? org_r : org_l;
-    const CrackSums c = crack_eval_pairs<T, 16>(p, E.tip_q, E.v_prev, S.i_first, S.i_last, dir, [&](int i, T &a, T &b) {
-        const int q = i - org;
-        if (q < 0 || q >= W) return false;   // an end this tile does not follow
-        a = above[q];
-        b = below[q];
-        return true;
-    });
-    CrackDecision d = {};
-    if ((lane & 15) == 0 && (dir > 0 ? act_r : act_l)) d = crack_decide(p, S, dir, c);
-    __syncwarp();
+    const bool act = dir > 0 ? act_r : act_l;
+    if (__any_sync(0xffffffffu, act && E.tip_q != win.tip)) pass_window(q, S, org, dir > 0 ? ev_r : ev_l, win);
+    const bool rest = (__double_as_longlong(E.v_prev) << 1) == 0;   // v_prev = 0
+    float t = 0.0f;
+    if (win.col >= 0 && win.col < W) t = fabsf(win.coef * (float)(above[win.col] - below[win.col]));
+    const bool hot = act && !(rest && (E.arrested || t < q.k_rest));
     const bool pending = !S.r.decided;
-    if (lane == 0 && act_r) crack_commit(p, nullptr, hist, S, +1, commit_r, c, d);
-    __syncwarp();
-    if (lane == 16 && act_l) crack_commit(p, nullptr, hist, S, -1, commit_l, c, d);
-    __syncwarp();
+    if (!__any_sync(0xffffffffu, hot)) {
+        __syncwarp();
+        if (lane == 0) {
+            if (act_r) {
+                S.r.v = 0.0;
+                S.r.grew = 0;
+            }
+            if (act_l) {
+                S.l.v = 0.0;
+                S.l.grew = 0;
+            }
+            rec.lazy = 1;
+            rec.vr = rec.vl = 0.0;
+        }
+    } else {
+        CrackSums c = {0.0, 0.0, 0.0, 0};
+        bool many = !q.one_pair;
+        if (!many && (lane & 15) == 0 && act) {
+            // at most one pair: its column by integer distances
+            const double r_min = p.r_min_fixed > 0.0 ? p.r_min_fixed : (rest ? p.r0 : p.r0 / (1.0 - E.v_prev));
+            const double lo = p.dh == 1.0 ? r_min : r_min / p.dh;
+            const double hi = p.dh == 1.0 ? r_min + p.fit_width : (r_min + p.fit_width) / p.dh;
+            const int64_t lo_q = __double2ll_ru(lo * 4294967296.0), hi_q = __double2ll_ru(hi * 4294967296.0);
+            many = hi_q - lo_q > ((int64_t)1 << kQBits);   // by the rounding of hi
+            const PassPair w = pass_pair(dir, E.tip_q, lo_q, hi_q, S.i_first, S.i_last);
+            const int k = w.col - org;
+            c.r_min = r_min;
+            if (w.in && k >= 0 && k < W) c = pass_sums<T>(pass_sf(p, w.d), above[k], below[k], r_min);
+        }
+        if (__any_sync(0xffffffffu, many)) {
+            c = crack_eval_pairs<T, 16>(p, E.tip_q, E.v_prev, S.i_first, S.i_last, dir, [&](int i, T &a, T &b) {
+                const int k = i - org;
+                if (k < 0 || k >= W) return false;   // an end this tile does not follow
+                a = above[k];
+                b = below[k];
+                return true;
+            });
+        }
+        CrackDecision d = {};
+        if ((lane & 15) == 0 && act) d = crack_decide(p, S, dir, c);
+        const History none = {};
+        __syncwarp();
+        if (lane == 0 && act_r) crack_commit(p, nullptr, none, S, +1, false, c, d);
+        __syncwarp();
+        if (lane == 16 && act_l) crack_commit(p, nullptr, none, S, -1, false, c, d);
+        __syncwarp();
+        if (lane == 0) {
+            rec.lazy = 0;
+            rec.vr = S.r.v;
+            rec.vl = S.l.v;
+            rec.Kr = S.r.K;
+            rec.Kl = S.l.K;
+            rec.npr = S.r.npairs;
+            rec.npl = S.l.npairs;
+        }
+    }
     if (lane == 0) {
+        rec.tr = S.r.tip_q;
+        rec.tl = S.l.tip_q;
+        rec.f = S.i_first;
+        rec.l = S.i_last;
         S.hist_n += pending ? 1 : 0;
         S.r.decided = 0;
         S.l.decided = 0;
@@ -248,17 +396,22 @@ __device__ __forceinline__ void pass_crack_step(const CrackParams &p, const T *b
     __syncwarp();
 }
 
-// The crack steps of a pass whose decisions need no K, by one thread: the
-// state in force during each update.  S becomes the state after the last.
-__device__ __forceinline__ void pass_known_steps(const CrackParams &p, const History &hist, CrackState &S, PassTip *log,
-                                                 int K)
+// The crack steps of a pass whose decisions need no K, one after another by
+// one thread: the state in force during each update.
+static __device__ __noinline__ void pass_known_serial(const CrackParams &p, CrackState S, PassTip *log, int K)
 {
-    log[0].tr = S.r.tip_q;
-    log[0].tl = S.l.tip_q;
-    log[0].f = S.i_first;
-    log[0].l = S.i_last;
-    for (int s = 0; s < K; ++s) {
-        const bool pending = !S.r.decided;
+    const History none = {};
+    for (int s = 0; s <= K; ++s) {
+        log[s].tr = S.r.tip_q;
+        log[s].tl = S.l.tip_q;
+        log[s].vr = S.r.v;
+        log[s].vl = S.l.v;
+        log[s].f = S.i_first;
+        log[s].l = S.i_last;
+        log[s].arr_r = S.r.arrested;
+        log[s].arr_l = S.l.arrested;
+        log[s].lazy = 1;
+        if (s == K) break;
         const bool grow = p.mode == CRACK_PRESCRIBED;
         const CrackSums c = {0.0, 0.0, 0.0, 0};
         for (int dir = 1; dir >= (p.two_tips ? -1 : 1); dir -= 2) {
@@ -270,17 +423,48 @@ __device__ __forceinline__ void pass_known_steps(const CrackParams &p, const His
             d.dq = p.dq_prescribed;
             d.propagate = grow && !E.arrested ? 1 : 0;
             d.flags = E.flags;
-            crack_commit(p, nullptr, hist, S, dir, false, c, d);
+            crack_commit(p, nullptr, none, S, dir, false, c, d);
         }
-        S.hist_n += pending ? 1 : 0;
         S.r.decided = 0;
         S.l.decided = 0;
-        log[s + 1].tr = S.r.tip_q;
-        log[s + 1].tl = S.l.tip_q;
-        log[s + 1].vr = S.r.v;
-        log[s + 1].vl = S.l.v;
-        log[s + 1].f = S.i_first;
-        log[s + 1].l = S.i_last;
+    }
+}
+
+// The same in closed form, entry s by lane s of a warp (0 <= s <= K): an end
+// that grows has advanced s times by the prescribed distance or stopped at
+// the body's side.  For a crack that has links (first <= last): the ends do
+// not touch each other's columns.
+__device__ __forceinline__ void pass_known_lane(const CrackParams &p, const CrackState *st, int s, PassTip &t)
+{
+    const int64_t half = (int64_t)1 << (kQBits - 1);
+    const bool grow = p.mode == CRACK_PRESCRIBED;
+    t.f = st->i_first;
+    t.l = st->i_last;
+    t.lazy = 1;
+    {
+        const int64_t tip = st->r.tip_q, m = max(0, s - (st->r.decided ? 1 : 0)), dq = p.dq_prescribed;
+        const bool arr = st->r.arrested != 0, go = grow && !arr;
+        int64_t q = go ? tip + m * dq : tip;
+        const bool stop = go && m > 0 && q >= p.clamp_q, before = arr || (go && m > 1 && tip + (m - 1) * dq >= p.clamp_q);
+        if (stop) q = p.clamp_q;
+        t.tr = q;
+        t.arr_r = arr || stop;
+        t.vr = grow && !before ? p.v_rel : 0.0;
+        if (q > tip) t.l = max(t.l, min((int)((q - half) >> kQBits), p.nx - 1));
+    }
+    t.tl = st->l.tip_q;
+    t.arr_l = 0;
+    t.vl = 0.0;
+    if (p.two_tips) {
+        const int64_t tip = st->l.tip_q, m = max(0, s - (st->l.decided ? 1 : 0)), dq = p.dq_prescribed;
+        const bool arr = st->l.arrested != 0, go = grow && !arr;
+        int64_t q = go ? tip - m * dq : tip;
+        const bool stop = go && m > 0 && q <= 0, before = arr || (go && m > 1 && tip - (m - 1) * dq <= 0);
+        if (stop) q = 0;
+        t.tl = q;
+        t.arr_l = arr || stop;
+        t.vl = grow && !before ? p.v_rel : 0.0;
+        if (q < tip) t.f = min(t.f, max((int)((q - half + ((int64_t)1 << kQBits) - 1) >> kQBits), 0));
     }
 }
 
@@ -291,6 +475,51 @@ __device__ __forceinline__ int wrap_col(int c, int nx)
     return c < 0 ? c + nx : c;
 }
 
+// Rows and values that an earlier pass of the same launch may have written:
+// from L2, past the L1 caches.
+__device__ __forceinline__ void cg_row(const float *p, Row<float, 4> &r)
+{
+    const float4 q = __ldcg(reinterpret_cast<const float4 *>(p));
+    r.v[0] = q.x; r.v[1] = q.y; r.v[2] = q.z; r.v[3] = q.w;
+}
+__device__ __forceinline__ void cg_row(const double *p, Row<double, 2> &r)
+{
+    const double2 q = __ldcg(reinterpret_cast<const double2 *>(p));
+    r.v[0] = q.x; r.v[1] = q.y;
+}
+template <typename D, typename T, int N> __device__ __forceinline__ void cg_rate(const D *p, Row<T, N> &r, T inv)
+{
+    if constexpr (std::is_same<D, Lf>::value) cg_row(reinterpret_cast<const float *>(p), r);
+    else if constexpr (sizeof(D) == 2) WdIO<D>::unpack(__ldcg(reinterpret_cast<const uint2 *>(p)), r, inv);
+    else cg_row(p, r);
+}
+template <typename T> __device__ __forceinline__ T cg_get(const T *p) { return __ldcg(p); }
+template <typename D, typename T> __device__ __forceinline__ T cg_rate_get(const D *p, T inv)
+{
+    if constexpr (std::is_same<D, Lf>::value) return __ldcg(reinterpret_cast<const float *>(p));
+    else if constexpr (sizeof(D) == 2) {
+        const unsigned short u = __ldcg(reinterpret_cast<const unsigned short *>(p));
+        if constexpr (std::is_same<D, __half>::value) return __half2float(__ushort_as_half(u)) * inv;
+        else return __uint_as_float((uint32_t)u << 16);
+    } else return __ldcg(p);
+}
+
+// The buffers of one pass, and what write_pads reads of them.
+template <typename T, typename D> struct PassBuf {
+    const T *w_in;
+    const D *wd_in;
+    T *w_out;
+    D *wd;
+    const CrackState *s_in;
+    CrackState *s_out;
+};
+template <typename T> struct PassPads {
+    T *w_out;
+    int64_t pitch;
+    int32_t nx, ny;
+    int32_t edge[4];
+};
+
 // What a thread knows about its tile.
 struct PassCtx {
     TileGeo g;
@@ -298,7 +527,10 @@ struct PassCtx {
     bool per;
     bool is_l;                  // element 0 is column 0 (no periodic sides)
     int kr;                     // the element that is column nx - 1, else -1
-    bool side;                  // the tile's warps hold column 0 or nx - 1
+    bool side;                  // the warp holds column 0 or nx - 1
+    // the warp's rows: its last is ny - 1, its first 0; rows 0 or ny - 1 lie
+    // inside them, or nx - 1 inside a vector
+    bool has_t, has_b, odd;
     // strip tiles: whether the pass's decisions need no K; the ends this tile
     // follows (a link it can see may be cut in this pass); the ends whose
     // records it writes; the lattice column of its column 0 as seen from each
@@ -338,11 +570,12 @@ template <typename T, typename D, int RPT> struct PassRows {
 };
 
 // One time step of a tile.
-template <typename T, typename D, int RPT, int KIND, int PH>
+template <typename T, typename D, int NW, int RPT, int KIND, int PH>
 __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx &c, int s, PassRows<T, D, RPT> &F,
-                                          PassShared<T> &sh)
+                                          PassShared<T, NW> &sh, PassWindow &win)
 {
     constexpr int N = Vec<T>::N;
+    constexpr int kBelowWarp = NW / 2 - 1;   // strip: the warp whose last row is jc - 1; the next one's first is jc
     constexpr bool kLf = std::is_same<D, Lf>::value;
     typedef Row<T, N> R;
     const unsigned kFull = 0xffffffffu;
@@ -353,14 +586,91 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
     const int b = s & 1;
     stg_row(&sh.top[b][warp][lane * N], F.template cur<PH>(RPT - 1));
     stg_row(&sh.bot[b][warp][lane * N], F.template cur<PH>(0));
-    if (KIND == 2 && c.known && warp == kBelowWarp) stg_row(&sh.pair[s][0][lane * N], F.template cur<PH>(RPT - 1));
-    if (KIND == 2 && c.known && warp == kBelowWarp + 1) stg_row(&sh.pair[s][1][lane * N], F.template cur<PH>(0));
+    const bool face = KIND == 2 && (warp == kBelowWarp || warp == kBelowWarp + 1), below = warp == kBelowWarp;
+    if (KIND == 2 && face) stg_row(&sh.pair[s][below ? 0 : 1][lane * N], F.template cur<PH>(below ? RPT - 1 : 0));
+
+    const bool dir_l = KIND != 0 && a.edge[LEFT] == EDGE_DIRICHLET, dir_r = KIND != 0 && a.edge[RIGHT] == EDGE_DIRICHLET;
+    const bool em = KIND != 0 && A.q.edge_macro != 0, em_side = em && c.side;
+    const bool last_r = KIND != 0 && c.kr == N - 1;
+    T tl = (T)0, tr = (T)0;
+    R first, last;                                         // the first and last rows before the update
+    T el[KIND != 0 ? RPT : 1], er[KIND != 0 ? RPT : 1];   // edge rule: the edge columns before the update
+    if (KIND != 0) {
+        if (dir_l) tl = sh.ws2[LEFT][s];
+        if (dir_r) tr = sh.ws2[RIGHT][s];
+        first = F.template cur<PH>(0);
+        last = F.template cur<PH>(RPT - 1);
+        if (c.odd || em_side) {
+            // the images of edge sites inside a warp's rows or a thread's
+            // columns, as neighbours: the row update itself knows no edge
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) {
+                if (r + 1 < RPT && jb + r == ny - 1)
+                    F.template cur<PH>(r + 1 < RPT ? r + 1 : r) =
+                        edge_image<T, N>(F.template cur<PH>(r), a.edge[TOP] == EDGE_DIRICHLET, sh.ws2[TOP][s]);
+                if (r > 0 && jb + r == 0)
+                    F.template cur<PH>(r > 0 ? r - 1 : r) =
+                        edge_image<T, N>(F.template cur<PH>(r), a.edge[BOTTOM] == EDGE_DIRICHLET, sh.ws2[BOTTOM][s]);
+            }
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) {
+                R &w = F.template cur<PH>(r);
+#pragma unroll
+                for (int k = 0; k + 1 < N; ++k) w.v[k + 1] = k == c.kr ? (dir_r ? tr - w.v[k] : w.v[k]) : w.v[k + 1];
+                el[r] = w.v[0];
+                er[r] = el[r];
+#pragma unroll
+                for (int k = 1; k < N; ++k) er[r] = k == c.kr ? w.v[k] : er[r];
+            }
+        }
+    }
+    // the sums of a row's east and west neighbours, before the barrier
+    auto sides = [&](const R &cu) {
+        T left0 = __shfl_up_sync(kFull, cu.v[N - 1], 1);
+        T rightN = __shfl_down_sync(kFull, cu.v[0], 1);
+        if (KIND != 0) {
+            // no branches here: they would keep the rows' latencies from
+            // overlapping (FP64: two instructions of 64 cycles cost more)
+            if (sizeof(T) == 4 || c.side) {
+                T il = cu.v[0], ir = cu.v[N - 1];
+                if (dir_l) il = tl - il;
+                if (dir_r) ir = tr - ir;
+                left0 = c.is_l ? il : left0;
+                rightN = last_r ? ir : rightN;
+            }
+        }
+        R hs;
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            hs.v[k] = (k == 0 ? left0 : cu.v[k > 0 ? k - 1 : 0]) + (k == N - 1 ? rightN : cu.v[k < N - 1 ? k + 1 : k]);
+        return hs;
+    };
+    // Rows that need no other warp's: tiles of four rows a warp, which wait
+    // on latency more than on issue, update them before the barrier (row 1's
+    // new values take the slot of row 0, whose old values and neighbour are
+    // kept); larger ones sweep all rows after it.
+    constexpr bool kEarly = RPT <= 4;
+    R old0, old1, hs0, hsT;
+    if (kEarly && PH == 0) {
+        old0 = F.template cur<PH>(0);
+        old1 = F.template cur<PH>(1);
+        hs0 = sides(F.template cur<PH>(0));
+        hsT = sides(F.template cur<PH>(RPT - 1));
+#pragma unroll
+        for (int r = 1; r + 1 < RPT; ++r) {
+            const R cu = F.template cur<PH>(r), up = F.template cur<PH>(r + 1), dn = r == 1 ? old0 : F.template cur<PH>(r - 1);
+            const R hs = sides(cu);
+            R out;
+            row_sites<T, D, N>(cu, up, dn, hs, F.template rate<PH>(r), gg, dt, wd_scale, wd_inv, out);
+            F.template next<PH>(r) = out;
+        }
+    }
     __syncthreads();
     if (KIND == 2 && c.follow) {
         const bool reach = sh.reach[b] != 0;
         if (warp == 0) {
-            pass_crack_step<T>(p, sh.top[b][kBelowWarp], sh.bot[b][kBelowWarp + 1], c.org_r, c.org_l, sh.S, a.hist, c.ev_r,
-                               c.ev_l, c.own_r, c.own_l);
+            pass_crack_step<T, PassShared<T, NW>::W>(p, A.q, sh.top[b][kBelowWarp], sh.bot[b][kBelowWarp + 1], c.org_r,
+                                                     c.org_l, sh.S, sh.log[s + 1], c.ev_r, c.ev_l, win);
             if (lane == 0) sh.reach[b ^ 1] = crack_cut_in_reach(p, sh.S) ? 1 : 0;
         }
         // rows next to the crack wait for the decision only where it can cut a link
@@ -368,184 +678,167 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
     }
     R dnx, upx;
     ld_row(&sh.top[b][warp > 0 ? warp - 1 : 0][lane * N], dnx);
-    ld_row(&sh.bot[b][warp < kPassWarps - 1 ? warp + 1 : warp][lane * N], upx);
-    uint32_t cut = 0u;
-    if (KIND == 2 && (warp == kBelowWarp || warp == kBelowWarp + 1)) {
+    ld_row(&sh.bot[b][warp < NW - 1 ? warp + 1 : warp][lane * N], upx);
+    if (KIND != 0 && (c.has_t || c.has_b)) {
+        // the images beyond the bottom and top rows
+        if (c.has_t) upx = edge_image<T, N>(last, a.edge[TOP] == EDGE_DIRICHLET, sh.ws2[TOP][s]);
+        if (c.has_b) dnx = edge_image<T, N>(first, a.edge[BOTTOM] == EDGE_DIRICHLET, sh.ws2[BOTTOM][s]);
+    }
+    bool cut[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) cut[k] = false;
+    if (KIND == 2 && face) {
         const int f = c.known ? sh.log[s + 1].f : (c.ev_l ? sh.S.i_first : c.f0);
         const int l = c.known ? sh.log[s + 1].l : (c.ev_r ? sh.S.i_last : c.l0);
+        // a severed link sends the site's own value back
 #pragma unroll
         for (int k = 0; k < N; ++k) {
             int q = x0 + k;
-            if (c.per) q = wrap_col(q, nx);
-            if (q >= f && q <= l) cut |= 1u << k;
+            if (c.per) q = q < 0 ? q + nx : (q >= nx ? q - nx : q);
+            cut[k] = q >= f && q <= l;
+            upx.v[k] = cut[k] && below ? last.v[k] : upx.v[k];
+            dnx.v[k] = cut[k] && !below ? first.v[k] : dnx.v[k];
         }
     }
-    T tl = (T)0, tr = (T)0, tb = (T)0, tt = (T)0;
-    R first, last;                                         // the first and last rows before the update
-    T el[KIND != 0 ? RPT : 1], er[KIND != 0 ? RPT : 1];   // edge rule: the edge columns before the update
-    const bool em_side = KIND != 0 && A.q.edge_macro && c.side;
-    if (KIND != 0) {
-        tl = (T)2 * (T)sh.ws[LEFT][s];
-        tr = (T)2 * (T)sh.ws[RIGHT][s];
-        tb = (T)2 * (T)sh.ws[BOTTOM][s];
-        tt = (T)2 * (T)sh.ws[TOP][s];
-        first = F.template cur<PH>(0);
-        last = F.template cur<PH>(RPT - 1);
-        if (em_side) {
+    if (kEarly && PH == 0) {
+        R out;
+        row_sites<T, D, N>(old0, old1, dnx, hs0, F.template rate<PH>(0), gg, dt, wd_scale, wd_inv, out);
+        // the last row: its old values and its neighbour's are still in place
+        const R cuT = F.template cur<PH>(RPT - 1), dnT = std::is_same<D, Lf>::value || RPT > 2 ? F.template cur<PH>(RPT - 2) : old0;
+        R outT;
+        row_sites<T, D, N>(cuT, upx, dnT, hsT, F.template rate<PH>(RPT - 1), gg, dt, wd_scale, wd_inv, outT);
+        F.template next<PH>(0) = out;
+        F.template next<PH>(RPT - 1) = outT;
+    } else {
 #pragma unroll
-            for (int r = 0; r < RPT; ++r) {
-                el[r] = F.template cur<PH>(r).v[0];
-#pragma unroll
-                for (int k = 0; k < N; ++k)
-                    if (k == 0 || k == c.kr) er[r] = F.template cur<PH>(r).v[k];
-            }
+        for (int q = 0; q < RPT; ++q) {
+            const int r = PH == 0 ? q : RPT - 1 - q;
+            const R cu = F.template cur<PH>(r);
+            // the row whose slot this row's new values take is read first
+            const R up = r + 1 < RPT ? F.template cur<PH>(r + 1 < RPT ? r + 1 : r) : upx;
+            const R dn = r > 0 ? F.template cur<PH>(r > 0 ? r - 1 : r) : dnx;
+            const R hs = sides(cu);
+            R out;
+            row_sites<T, D, N>(cu, up, dn, hs, F.template rate<PH>(r), gg, dt, wd_scale, wd_inv, out);
+            F.template next<PH>(r) = out;
         }
     }
-#pragma unroll
-    for (int q = 0; q < RPT; ++q) {
-        const int r = PH == 0 ? q : RPT - 1 - q;
-        const R cu = F.template cur<PH>(r);
-        // the row whose slot this row's new values take is read first
-        R up = r + 1 < RPT ? F.template cur<PH>(r + 1 < RPT ? r + 1 : r) : upx;
-        R dn = r > 0 ? F.template cur<PH>(r > 0 ? r - 1 : r) : dnx;
-        T left0 = __shfl_up_sync(kFull, cu.v[N - 1], 1);
-        T rightN = __shfl_down_sync(kFull, cu.v[0], 1);
-        if (KIND != 0) {
-            const int j = jb + r;
-            if (j == ny - 1) {
-#pragma unroll
-                for (int k = 0; k < N; ++k) up.v[k] = a.edge[TOP] == EDGE_DIRICHLET ? tt - cu.v[k] : cu.v[k];
-            }
-            if (j == 0) {
-#pragma unroll
-                for (int k = 0; k < N; ++k) dn.v[k] = a.edge[BOTTOM] == EDGE_DIRICHLET ? tb - cu.v[k] : cu.v[k];
-            }
-            if (KIND == 2 && r == RPT - 1 && warp == kBelowWarp) {
-#pragma unroll
-                for (int k = 0; k < N; ++k)
-                    if ((cut >> k) & 1u) up.v[k] = cu.v[k];
-            }
-            if (KIND == 2 && r == 0 && warp == kBelowWarp + 1) {
-#pragma unroll
-                for (int k = 0; k < N; ++k)
-                    if ((cut >> k) & 1u) dn.v[k] = cu.v[k];
-            }
-            if (c.is_l) left0 = a.edge[LEFT] == EDGE_DIRICHLET ? tl - cu.v[0] : cu.v[0];
-        }
-        R hs;
+    if (KIND == 2 && p.macro && face) {
+        // the crack-face rule: w_B from the two new values further from the crack
+        R wB, w0;
 #pragma unroll
         for (int k = 0; k < N; ++k) {
-            const T wl = k == 0 ? left0 : cu.v[k - 1];
-            T wr = k == N - 1 ? rightN : cu.v[k + 1];
-            if (KIND != 0 && k == c.kr) wr = a.edge[RIGHT] == EDGE_DIRICHLET ? tr - cu.v[k] : cu.v[k];
-            hs.v[k] = wl + wr;
+            const T w2 = below ? F.template next<PH>(RPT - 2).v[k] : F.template next<PH>(1).v[k];
+            const T w3 = below ? F.template next<PH>(RPT - 3).v[k] : F.template next<PH>(2).v[k];
+            wB.v[k] = (T)1.5 * w2 - (T)0.5 * w3;
+            w0.v[k] = below ? last.v[k] : first.v[k];
         }
-        R out;
-        row_sites<T, D, N>(cu, up, dn, hs, F.template rate<PH>(r), gg, dt, wd_scale, wd_inv, out);
-        F.template next<PH>(r) = out;
-    }
-    if (KIND == 2 && p.macro && cut) {
-        // the crack-face rule: w_B from the two new values further from the crack
-        if (warp == kBelowWarp) {
-            R &w1 = F.template next<PH>(RPT - 1), &w2 = F.template next<PH>(RPT - 2), &w3 = F.template next<PH>(RPT - 3);
+        const R rt = kLf ? wB : rate_of(wB, w0, dt);
 #pragma unroll
-            for (int k = 0; k < N; ++k)
-                if ((cut >> k) & 1u) {
-                    const T wB = (T)1.5 * w2.v[k] - (T)0.5 * w3.v[k];
-                    if (!kLf) F.b[RPT - 1].v[k] = wd_round<D, T>((wB - last.v[k]) / dt, wd_scale, wd_inv);
-                    w1.v[k] = wB;
-                }
-        } else {
-            R &w1 = F.template next<PH>(0), &w2 = F.template next<PH>(1), &w3 = F.template next<PH>(2);
-#pragma unroll
-            for (int k = 0; k < N; ++k)
-                if ((cut >> k) & 1u) {
-                    const T wB = (T)1.5 * w2.v[k] - (T)0.5 * w3.v[k];
-                    if (!kLf) F.b[0].v[k] = wd_round<D, T>((wB - first.v[k]) / dt, wd_scale, wd_inv);
-                    w1.v[k] = wB;
-                }
+        for (int k = 0; k < N; ++k) {
+            if (!kLf) {
+                const T v = wd_round<D, T>(rt.v[k], wd_scale, wd_inv);
+                F.b[RPT - 1].v[k] = cut[k] && below ? v : F.b[RPT - 1].v[k];
+                F.b[0].v[k] = cut[k] && !below ? v : F.b[0].v[k];
+            }
+            T &oT = F.template next<PH>(RPT - 1).v[k], &oB = F.template next<PH>(0).v[k];
+            oT = cut[k] && below ? wB.v[k] : oT;
+            oB = cut[k] && !below ? wB.v[k] : oB;
         }
     }
     if (KIND != 0 && A.q.edge_macro) {
         // the macroscopic rule on the outer edges (the two levels of
         // edge_rule_at): the edge columns, the crack-face points on
         // them, then the bottom and top rows and the corners
-        const bool on_l = a.edge[LEFT] != EDGE_PERIODIC, on_r = a.edge[RIGHT] != EDGE_PERIODIC;
+        const bool on_l = a.edge[LEFT] != EDGE_PERIODIC && c.is_l, on_r = a.edge[RIGHT] != EDGE_PERIODIC && c.kr >= 0;
         EdgeRule<T> E;
         E.wn = nullptr;
         E.pitch = 0;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             E.dir[e] = a.edge[e] == EDGE_DIRICHLET;
-            E.ws[e] = (T)sh.ws[e][s + 1];
+            E.ws[e] = E.dir[e] ? sh.ws[e][s + 1] : (T)0;
         }
         R in1, in2;         // rows 1, 2 (or ny-2, ny-3) before the edge columns
-        const bool has_b = jb == 0, has_t = jb + RPT == ny;
+        const bool has_b = c.has_b, has_t = c.has_t;
 #pragma unroll
         for (int k = 0; k < N; ++k) {
             in1.v[k] = has_t ? F.template next<PH>(RPT - 2).v[k] : F.template next<PH>(1).v[k];
             in2.v[k] = has_t ? F.template next<PH>(RPT - 3).v[k] : F.template next<PH>(2).v[k];
         }
+        if (em_side) {
 #pragma unroll
-        for (int r = 0; r < RPT; ++r) {
-            if (!em_side) break;
-            R &w = F.template next<PH>(r);
-            const int j = jb + r;
-            const T p1 = __shfl_up_sync(kFull, w.v[N - 1], 1), p2 = __shfl_up_sync(kFull, w.v[N - 2], 1);
-            const T n0 = __shfl_down_sync(kFull, w.v[0], 1);
-            if (j < 1 || j > ny - 2) continue;
-            if (c.is_l && on_l) {
-                const T v2 = N > 2 ? w.v[N > 2 ? 2 : 0] : n0;
-                w.v[0] = E.rule(LEFT, w.v[1], v2);
-            }
-            if (c.kr >= 0 && on_r) {
+            for (int r = 0; r < RPT; ++r) {
+                R &w = F.template next<PH>(r);
+                const int j = jb + r;
+                const bool row = j >= 1 && j <= ny - 2;
+                const T p1 = __shfl_up_sync(kFull, w.v[N - 1], 1), p2 = __shfl_up_sync(kFull, w.v[N - 2], 1);
+                const T n0 = __shfl_down_sync(kFull, w.v[0], 1);
+                const T vl = E.rule(LEFT, w.v[1], N > 2 ? w.v[N > 2 ? 2 : 0] : n0);
                 T wI = p1, wII = p2;
 #pragma unroll
-                for (int k = 1; k < N; ++k)
-                    if (k == c.kr) {
-                        wI = w.v[k - 1];
-                        wII = k >= 2 ? w.v[k >= 2 ? k - 2 : 0] : p1;
-                    }
-                const T v = E.rule(RIGHT, wI, wII);
+                for (int k = 1; k < N; ++k) {
+                    wI = k == c.kr ? w.v[k - 1] : wI;
+                    wII = k == c.kr ? (k >= 2 ? w.v[k >= 2 ? k - 2 : 0] : p1) : wII;
+                }
+                const T vr = E.rule(RIGHT, wI, wII);
+                Row<T, 2> wn, wo;
+                wn.v[0] = vl;
+                wn.v[1] = vr;
+                wo.v[0] = el[r];
+                wo.v[1] = er[r];
+                w.v[0] = row && on_l ? vl : w.v[0];
 #pragma unroll
-                for (int k = 0; k < N; ++k)
-                    if (k == c.kr) w.v[k] = v;
+                for (int k = 0; k < N; ++k) w.v[k] = row && on_r && k == c.kr ? vr : w.v[k];
+                if (!kLf) {
+                    // wdot of the sites that took the rule (crack-face points again below)
+                    const Row<T, 2> rt = rate_of(wn, wo, dt);
+                    const T rl = wd_round<D, T>(rt.v[0], wd_scale, wd_inv), rr = wd_round<D, T>(rt.v[1], wd_scale, wd_inv);
+                    F.b[r].v[0] = row && on_l ? rl : F.b[r].v[0];
+#pragma unroll
+                    for (int k = 0; k < N; ++k) F.b[r].v[k] = row && on_r && k == c.kr ? rr : F.b[r].v[k];
+                }
             }
-        }
-        if (KIND == 2 && em_side && p.macro && cut && (c.is_l || c.kr >= 0)) {
-            const bool be = warp == kBelowWarp;
+            if (KIND == 2 && face && p.macro) {
 #pragma unroll
-            for (int k = 0; k < N; ++k) {
-                if (!((cut >> k) & 1u) || !((c.is_l && on_l && k == 0) || (on_r && k == c.kr))) continue;
-                const T v1 = be ? F.template next<PH>(RPT - 2).v[k] : F.template next<PH>(1).v[k];
-                const T v2 = be ? F.template next<PH>(RPT - 3).v[k] : F.template next<PH>(2).v[k];
-                const T v = (T)1.5 * v1 - (T)0.5 * v2;
-                if (be) F.template next<PH>(RPT - 1).v[k] = v;
-                else F.template next<PH>(0).v[k] = v;
+                for (int k = 0; k < N; ++k) {
+                    if (!(cut[k] && ((on_l && k == 0) || (on_r && k == c.kr)))) continue;
+                    const T v1 = below ? F.template next<PH>(RPT - 2).v[k] : F.template next<PH>(1).v[k];
+                    const T v2 = below ? F.template next<PH>(RPT - 3).v[k] : F.template next<PH>(2).v[k];
+                    const T v = (T)1.5 * v1 - (T)0.5 * v2;
+                    Row<T, 1> wn, wo;
+                    wn.v[0] = v;
+                    wo.v[0] = below ? last.v[k] : first.v[k];
+                    const T rt = wd_round<D, T>(rate_of(wn, wo, dt).v[0], wd_scale, wd_inv);
+                    if (below) {
+                        F.template next<PH>(RPT - 1).v[k] = v;
+                        if (!kLf) F.b[RPT - 1].v[k] = rt;
+                    } else {
+                        F.template next<PH>(0).v[k] = v;
+                        if (!kLf) F.b[0].v[k] = rt;
+                    }
+                }
             }
         }
         if (has_b || has_t) {
             const int ev = has_t ? TOP : BOTTOM;
-            R e1, e2;   // the rows one and two from the edge, after the edge columns
-#pragma unroll
-            for (int k = 0; k < N; ++k) {
-                e1.v[k] = has_t ? F.template next<PH>(RPT - 2).v[k] : F.template next<PH>(1).v[k];
-                e2.v[k] = has_t ? F.template next<PH>(RPT - 3).v[k] : F.template next<PH>(2).v[k];
-            }
             R o;
 #pragma unroll
             for (int k = 0; k < N; ++k) o.v[k] = E.rule(ev, in1.v[k], in2.v[k]);
-            // corners: along the bottom / top edge's normal from the edge
-            // columns, or (its side Dirichlet, ev not) along the row from
-            // the points of edge ev
-            const T q1 = __shfl_up_sync(kFull, o.v[N - 1], 1), q2 = __shfl_up_sync(kFull, o.v[N - 2], 1);
-            const T m0 = __shfl_down_sync(kFull, o.v[0], 1);
-            T cl = (T)0, cr = (T)0;
-            if (c.is_l && on_l)
-                cl = a.edge[LEFT] == EDGE_DIRICHLET && a.edge[ev] != EDGE_DIRICHLET
-                         ? E.rule(LEFT, o.v[1], N > 2 ? o.v[N > 2 ? 2 : 0] : m0)
-                         : E.rule(ev, e1.v[0], e2.v[0]);
-            if (c.kr >= 0 && on_r) {
+            if (em_side) {
+                // corners: along the bottom / top edge's normal from the edge
+                // columns, or (its side Dirichlet, ev not) along the row from
+                // the points of edge ev
+                const T q1 = __shfl_up_sync(kFull, o.v[N - 1], 1), q2 = __shfl_up_sync(kFull, o.v[N - 2], 1);
+                const T m0 = __shfl_down_sync(kFull, o.v[0], 1);
+                R e1, e2;   // the rows one and two from the edge, after the edge columns
+#pragma unroll
+                for (int k = 0; k < N; ++k) {
+                    e1.v[k] = has_t ? F.template next<PH>(RPT - 2).v[k] : F.template next<PH>(1).v[k];
+                    e2.v[k] = has_t ? F.template next<PH>(RPT - 3).v[k] : F.template next<PH>(2).v[k];
+                }
+                const T cl = E.dir[LEFT] && !E.dir[ev] ? E.rule(LEFT, o.v[1], N > 2 ? o.v[N > 2 ? 2 : 0] : m0)
+                                                       : E.rule(ev, e1.v[0], e2.v[0]);
                 T oI = q1, oII = q2, c1 = (T)0, c2 = (T)0;
 #pragma unroll
                 for (int k = 0; k < N; ++k)
@@ -555,36 +848,24 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
                         c1 = e1.v[k];
                         c2 = e2.v[k];
                     }
-                cr = a.edge[RIGHT] == EDGE_DIRICHLET && a.edge[ev] != EDGE_DIRICHLET ? E.rule(RIGHT, oI, oII)
-                                                                                   : E.rule(ev, c1, c2);
+                const T cr = E.dir[RIGHT] && !E.dir[ev] ? E.rule(RIGHT, oI, oII) : E.rule(ev, c1, c2);
+                o.v[0] = on_l ? cl : o.v[0];
+#pragma unroll
+                for (int k = 0; k < N; ++k) o.v[k] = on_r && k == c.kr ? cr : o.v[k];
             }
-            if (c.is_l && on_l) o.v[0] = cl;
+            R w0;
 #pragma unroll
-            for (int k = 0; k < N; ++k)
-                if (on_r && k == c.kr) o.v[k] = cr;
-            if (has_t) F.template next<PH>(RPT - 1) = o;
-            else F.template next<PH>(0) = o;
-        }
-        if (!kLf && (em_side || has_b || has_t)) {
-            // wdot of the sites that took the rule
+            for (int k = 0; k < N; ++k) w0.v[k] = has_t ? last.v[k] : first.v[k];
+            const R rt = kLf ? o : rate_of(o, w0, dt);
 #pragma unroll
-            for (int r = 0; r < RPT; ++r) {
-                const R &w = F.template next<PH>(r);
-                const int j = jb + r;
-                if (j == 0 || j == ny - 1) {
-                    if ((r == 0 && has_b) || (r == RPT - 1 && has_t)) {
-#pragma unroll
-                        for (int k = 0; k < N; ++k)
-                            F.b[r].v[k] = wd_round<D, T>((w.v[k] - (r == 0 ? first.v[k] : last.v[k])) / dt, wd_scale, wd_inv);
-                    }
-                    continue;
-                }
-                if (!em_side) continue;
-                if (c.is_l && on_l) F.b[r].v[0] = wd_round<D, T>((w.v[0] - el[r]) / dt, wd_scale, wd_inv);
-                if (c.kr >= 0 && on_r) {
-#pragma unroll
-                    for (int k = 0; k < N; ++k)
-                        if (k == c.kr) F.b[r].v[k] = wd_round<D, T>((w.v[k] - er[r]) / dt, wd_scale, wd_inv);
+            for (int k = 0; k < N; ++k) {
+                const T v = kLf ? rt.v[k] : wd_round<D, T>(rt.v[k], wd_scale, wd_inv);
+                if (has_t) {
+                    F.template next<PH>(RPT - 1).v[k] = o.v[k];
+                    if (!kLf) F.b[RPT - 1].v[k] = v;
+                } else {
+                    F.template next<PH>(0).v[k] = o.v[k];
+                    if (!kLf) F.b[0].v[k] = v;
                 }
             }
         }
@@ -593,11 +874,12 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
 
 // A tile.  KIND: 0 one none of whose sites sees an edge or the crack, 1 with
 // outer edges, 2 a crack-strip tile (with edges where it meets them).
-template <typename T, typename D, int RPT, int KIND>
-__device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo g, PassShared<T> &sh)
+template <typename T, typename D, int NW, int RPT, int KIND>
+__device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf<T, D> &B, const TileGeo g,
+                                          PassShared<T, NW> &sh)
 {
     constexpr int N = Vec<T>::N;
-    constexpr int W = PassShared<T>::W;
+    constexpr int W = PassShared<T, NW>::W;
     typedef Row<T, N> R;
     const unsigned kFull = 0xffffffffu;
     const StepArgs<T, D> &a = A.s;
@@ -618,8 +900,8 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
 
     PassRows<T, D, RPT> F;
     {
-        const T *wp = a.w_in + (int64_t)jb * P + x0;
-        const D *dp = A.wd_in + (int64_t)jb * P + x0;
+        const T *wp = B.w_in + (int64_t)jb * P + x0;
+        const D *dp = B.wd_in + (int64_t)jb * P + x0;
         const bool whole = KIND == 0 ? x0 < nx : (x0 >= 0 && x0 + N <= nx);
 #pragma unroll
         for (int r = 0; r < RPT; ++r) {
@@ -629,16 +911,16 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
             const int j = jb + r;
             if (j < 0 || j >= ny) continue;
             if (whole) {
-                ldg_row(wp + (int64_t)r * P, w);
-                WdIO<D>::load(dp + (int64_t)r * P, d, wd_inv);
+                cg_row(wp + (int64_t)r * P, w);
+                cg_rate(dp + (int64_t)r * P, d, wd_inv);
             } else if (KIND != 0) {
 #pragma unroll
                 for (int k = 0; k < N; ++k) {
                     int q = x0 + k;
                     if (per) q = wrap_col(q, nx);
                     if (q < 0 || q >= nx) continue;
-                    w.v[k] = a.w_in[(int64_t)j * P + q];
-                    d.v[k] = wd_get(A.wd_in + (int64_t)j * P + q, wd_inv);
+                    w.v[k] = cg_get(B.w_in + (int64_t)j * P + q);
+                    d.v[k] = cg_rate_get(B.wd_in + (int64_t)j * P + q, wd_inv);
                 }
             }
         }
@@ -651,12 +933,16 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
     c.org_r = c.org_l = g.xl;
     c.f0 = 0;
     c.l0 = -1;
+    PassWindow win = {-1, 0.0f, -1};
+    int64_t fit_tip = 0;
+    PassPair fit_pair = {0, 0, 0};
+    double fit_sf = 0.0;
     if (KIND == 2) {
         c.known = p.mode != CRACK_KCRIT;
-        c.f0 = a.s_in->i_first;
-        c.l0 = a.s_in->i_last;
-        hist0 = a.s_in->hist_n;
-        rec0 = a.s_in->r.decided ? 1 : 0;   // the first update whose crack step is still to run
+        c.f0 = sh.in.i_first;
+        c.l0 = sh.in.i_last;
+        hist0 = p.hist_cap > 0 ? sh.in.hist_n % p.hist_cap : 0;   // the ring slot of the first record
+        rec0 = sh.in.r.decided ? 1 : 0;   // the first update whose crack step is still to run
         const int cr = tip_col_r(c.f0, c.l0, nx), cl = tip_col_l(c.f0, c.l0, nx);
         const int hc = A.q.hc, grow = A.q.grow;
         // (periodic sides: the column itself, then its images beyond either side)
@@ -674,23 +960,71 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
             }
         }
         c.follow = !c.known && (c.ev_r || c.ev_l);
-        if (tid == 0) {
-            sh.S = *a.s_in;
-            if (c.known) pass_known_steps(p, a.hist, sh.S, sh.log, K);
-            else sh.reach[0] = crack_cut_in_reach(p, sh.S) ? 1 : 0;
+        if (c.known) {
+            // every tile of the strip forms the cuts of the whole pass
+            if (c.f0 <= c.l0) {
+                if (tid <= K) pass_known_lane(p, &sh.in, tid, sh.log[tid]);
+            } else if (tid == 0) {
+                pass_known_serial(p, sh.in, sh.log, K);
+            }
+        } else {
+            if (tid == 0) {
+                sh.S = sh.in;
+                sh.reach[0] = crack_cut_in_reach(p, sh.S) ? 1 : 0;
+                sh.log[0].tr = sh.S.r.tip_q;
+                sh.log[0].tl = sh.S.l.tip_q;
+                sh.log[0].f = c.f0;
+                sh.log[0].l = c.l0;
+            }
+            if (c.follow && warp == 0) {
+                __syncwarp();
+                pass_window(A.q, sh.S, lane < 16 ? c.org_r : c.org_l, lane < 16 ? c.ev_r : c.ev_l, win);
+            }
+        }
+        if ((c.own_r || c.own_l) && A.q.one_pair && warp == 1 && lane < 2 * kPassSteps) {
+            // the part of the K fits that needs no fields (an FP64 root and
+            // division), while the loads are under way: lane st of the right
+            // end, st + 8 of the left, for the tip before update st (K-
+            // criterion: the tip at rest where it starts)
+            const int st = lane & (kPassSteps - 1), dir = lane < kPassSteps ? +1 : -1;
+            PassTip t;
+            if (c.known && c.f0 <= c.l0) {
+                pass_known_lane(p, &sh.in, st, t);
+            } else {
+                t.tr = sh.in.r.tip_q;
+                t.tl = sh.in.l.tip_q;
+                t.f = c.f0;
+                t.l = c.l0;
+            }
+            fit_tip = dir > 0 ? t.tr : t.tl;
+            fit_pair = pass_pair(dir, fit_tip, A.q.lo_q, A.q.hi_q, t.f, t.l);
+            fit_sf = fit_pair.in ? pass_sf(p, fit_pair.d) : 0.0;
         }
     }
     if (KIND != 0) {
-        const int64_t n = a.s_in->step;
+        // w* of the Dirichlet edges this tile meets, in the arithmetic's
+        // precision once (a conversion from FP64 costs a warp 64 cycles)
         if (tid < 4 * (kPassSteps + 1)) {
             const int e = tid / (kPassSteps + 1), q = tid % (kPassSteps + 1);
-            if (q <= K) sh.ws[e][q] = a.edge[e] == EDGE_DIRICHLET ? load_value(a.load[e], n + q, (double)p.dt) : 0.0;
+            const bool meets = e == LEFT ? g.xl <= 0 : e == RIGHT ? g.xl + W >= nx : e == BOTTOM ? g.yl <= 0 : g.yl + NW * RPT >= ny;
+            if (q <= K && meets && a.edge[e] == EDGE_DIRICHLET) {
+                const T v = a.load[e].kind == LOAD_CONST ? (T)a.load[e].amp
+                          : a.load[e].kind == LOAD_ZERO  ? (T)0
+                                                         : (T)load_value(a.load[e], __ldcg(&B.s_in->step) + q, (double)p.dt);
+                sh.ws[e][q] = v;
+                sh.ws2[e][q] = (T)2 * v;
+            }
         }
     }
     c.is_l = KIND != 0 && !per && x0 == 0;
     c.kr = KIND != 0 && !per && nx - 1 - x0 >= 0 && nx - 1 - x0 < N ? nx - 1 - x0 : -1;
 
     c.side = KIND != 0 && __any_sync(kFull, c.is_l || c.kr >= 0);
+    c.has_t = KIND != 0 && jb + RPT == ny;
+    c.has_b = KIND != 0 && jb == 0;
+    c.odd = KIND != 0 && ((jb < 0 && jb + RPT > 0) || (jb < ny && jb + RPT > ny) ||
+                          __any_sync(kFull, c.kr >= 0 && c.kr < N - 1));
+    if (KIND != 0) __syncthreads();   // w* and the cuts of the pass
     // bulk tiles: two steps an iteration (PassRows); an odd last step leaves
     // the rows where a step of phase 0 writes them.  The other tiles, whose
     // step is far longer code, take every step in phase 0 and move the rows
@@ -698,12 +1032,12 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
     int s = 0;
     if (KIND == 0) {
         for (; s + 2 <= K; s += 2) {
-            pass_step<T, D, RPT, KIND, 0>(A, c, s, F, sh);
-            pass_step<T, D, RPT, KIND, 1>(A, c, s + 1, F, sh);
+            pass_step<T, D, NW, RPT, KIND, 0>(A, c, s, F, sh, win);
+            pass_step<T, D, NW, RPT, KIND, 1>(A, c, s + 1, F, sh, win);
         }
     }
     for (; s < K; ++s) {
-        pass_step<T, D, RPT, KIND, 0>(A, c, s, F, sh);
+        pass_step<T, D, NW, RPT, KIND, 0>(A, c, s, F, sh, win);
 #pragma unroll
         for (int q = 0; q < RPT; ++q) {
             const int r = RPT - 1 - q;
@@ -718,6 +1052,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
     }
 
     // the tile's own sites
+    const PassPads<T> pads = {B.w_out, P, nx, ny, {a.edge[0], a.edge[1], a.edge[2], a.edge[3]}};
     T acc = (T)0;
 #pragma unroll
     for (int r = 0; r < RPT; ++r) {
@@ -727,9 +1062,9 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
         if (x0 + N <= g.x0 || x0 >= g.x1) continue;
         const int64_t o = (int64_t)j * P + x0;
         if (KIND == 0 || (x0 >= g.x0 && x0 + N <= g.x1 && x0 >= 0 && x0 + N <= nx)) {
-            stg_row(a.w_out + o, w);
-            wd_store(a.wd + o, d, wd_scale);
-            if (KIND != 0) write_pads(a, x0, j, w);
+            stg_row(B.w_out + o, w);
+            wd_store(B.wd + o, d, wd_scale);
+            if (KIND != 0) write_pads(pads, x0, j, w);
             acc += w.v[0];
         } else {
 #pragma unroll
@@ -738,10 +1073,10 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
                 if (q < g.x0 || q >= g.x1) continue;
                 if (per) q = wrap_col(q, nx);
                 if (q < 0 || q >= nx) continue;
-                T *row = a.w_out + (int64_t)j * P;
+                T *row = B.w_out + (int64_t)j * P;
                 const T v = w.v[k];
                 row[q] = v;
-                wd_put(a.wd + (int64_t)j * P + q, d.v[k], wd_scale);
+                wd_put(B.wd + (int64_t)j * P + q, d.v[k], wd_scale);
                 if (q == 0) {
                     if (a.edge[LEFT] == EDGE_FREE) row[-1] = v;
                     else if (per) row[nx] = v;
@@ -759,73 +1094,129 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
     if (__any_sync(kFull, !isfinite(acc)) && lane == 0) atomicOr(a.err, (uint32_t)ERR_NONFINITE);
 
     if (KIND == 2 && (c.own_r || c.own_l)) {
-        if (c.known) {
-            // the K fits of the pass's crack steps, one step per warp: their
-            // decisions did not wait for them
-            if (warp >= rec0 && warp < K) {
-                for (int dir = 1; dir >= (c.own_l ? -1 : 1); dir -= 2) {
-                    if (dir > 0 && !c.own_r) continue;
-                    const PassTip &q = sh.log[warp], &q1 = sh.log[warp + 1];
-                    const int org = dir > 0 ? c.org_r : c.org_l;
-                    const double v_prev = p.mode == CRACK_PRESCRIBED ? p.v_rel : 0.0;
-                    const CrackSums f = crack_eval_pairs<T, 32>(
-                        p, dir > 0 ? q.tr : q.tl, v_prev, q.f, q.l, dir, [&](int i, T &ab, T &be) {
-                            const int e = i - org;
-                            if (e < 0 || e >= W) return false;
-                            ab = sh.pair[warp][1][e];
-                            be = sh.pair[warp][0][e];
-                            return true;
-                        });
-                    if (lane == 0) {
-                        const double Kf = f.np > 0 ? p.mu / 4.0 * f.num / f.den : 0.0;
-                        if (!isfinite(Kf)) atomicOr(a.err, (uint32_t)ERR_NONFINITE);
-                        if (p.hist_cap > 0) {
-                            const int64_t h = (hist0 + (warp - rec0)) % p.hist_cap;
-                            (dir > 0 ? a.hist.K : a.hist.Kl)[h] = Kf;
-                            (dir > 0 ? a.hist.v : a.hist.vl)[h] = dir > 0 ? q1.vr : q1.vl;
-                            (dir > 0 ? a.hist.tip : a.hist.tipl)[h] = dir > 0 ? q1.tr : q1.tl;
-                            (dir > 0 ? a.hist.np : a.hist.npl)[h] = f.np;
-                        }
-                        if (warp == K - 1) {
-                            TipState &O = dir > 0 ? a.s_out->r : a.s_out->l;
-                            O.K = Kf;
-                            O.r_min = f.r_min;
-                            O.npairs = f.np;
-                        }
+        __syncthreads();   // the last crack step
+        // the records of the pass's crack steps, and the K fits their decisions
+        // did not wait for.  A window of one spacing holds at most one pair, so
+        // one warp forms the fits of all steps, a lane each (an FP64
+        // instruction takes a warp 64 cycles whatever its active lanes); a
+        // wider one takes a warp per step.
+        auto fit = [&](int st, int dir, double v_prev, double &Kf, int &np, double &r_min, auto group) {
+            const PassTip &q = sh.log[st];
+            const int org = dir > 0 ? c.org_r : c.org_l;
+            const CrackSums f = crack_eval_pairs<T, decltype(group)::value>(
+                p, dir > 0 ? q.tr : q.tl, v_prev, q.f, q.l, dir, [&](int i, T &ab, T &be) {
+                    const int e = i - org;
+                    if (e < 0 || e >= W) return false;
+                    ab = sh.pair[st][1][e];
+                    be = sh.pair[st][0][e];
+                    return true;
+                });
+            np = f.np;
+            Kf = np > 0 ? p.mu / 4.0 * f.num / f.den : 0.0;
+            r_min = f.r_min;
+        };
+        auto record = [&](int st, int dir, double Kf, int np, double r_min) {
+            const PassTip &q1 = sh.log[st + 1];
+            if (q1.lazy) {
+                if (!isfinite(Kf)) atomicOr(a.err, (uint32_t)ERR_NONFINITE);
+                if (st == K - 1) {
+                    TipState &O = dir > 0 ? B.s_out->r : B.s_out->l;
+                    O.K = Kf;
+                    O.r_min = r_min;
+                    O.npairs = np;
+                }
+            } else {
+                Kf = dir > 0 ? q1.Kr : q1.Kl;
+                np = dir > 0 ? q1.npr : q1.npl;
+            }
+            if (p.hist_cap > 0) {
+                int64_t h = hist0 + (st - rec0);   // the ring slot
+                h -= h >= p.hist_cap ? p.hist_cap : 0;
+                (dir > 0 ? a.hist.K : a.hist.Kl)[h] = Kf;
+                (dir > 0 ? a.hist.v : a.hist.vl)[h] = dir > 0 ? q1.vr : q1.vl;
+                (dir > 0 ? a.hist.tip : a.hist.tipl)[h] = dir > 0 ? q1.tr : q1.tl;
+                (dir > 0 ? a.hist.np : a.hist.npl)[h] = np;
+            }
+        };
+        const double v_prev = p.mode == CRACK_PRESCRIBED ? p.v_rel : 0.0;
+        if (A.q.one_pair) {
+            const int st = lane & (kPassSteps - 1), dir = lane < kPassSteps ? +1 : -1;
+            if (warp == 1 && lane < 2 * kPassSteps && st >= rec0 && st < K && (dir > 0 ? c.own_r : c.own_l)) {
+                double Kf = 0.0;
+                int np = 0;
+                if (sh.log[st + 1].lazy) {
+                    const PassTip &q = sh.log[st];
+                    const int64_t tip = dir > 0 ? q.tr : q.tl;
+                    PassPair w = pass_pair(dir, tip, A.q.lo_q, A.q.hi_q, q.f, q.l);
+                    if (tip != fit_tip || w.in != fit_pair.in) fit_sf = w.in ? pass_sf(p, w.d) : 0.0;   // it has moved since
+                    const int e = w.col - (dir > 0 ? c.org_r : c.org_l);
+                    if (w.in && e >= 0 && e < W) {
+                        const CrackSums f = pass_sums<T>(fit_sf, sh.pair[st][1][e], sh.pair[st][0][e], 0.0);
+                        Kf = pass_K(p, f);
+                        np = 1;
                     }
                 }
+                record(st, dir, Kf, np, A.q.r_min);
             }
-        } else {
-            __syncthreads();   // the last crack step
+        } else if (warp >= rec0 && warp < K) {
+            for (int dir = 1; dir >= (c.own_l ? -1 : 1); dir -= 2) {
+                if (dir > 0 && !c.own_r) continue;
+                double Kf = 0.0, r_min = 0.0;
+                int np = 0;
+                if (sh.log[warp + 1].lazy) fit(warp, dir, v_prev, Kf, np, r_min, std::integral_constant<int, 32>());
+                if (lane == 0) record(warp, dir, Kf, np, r_min);
+            }
         }
         if (tid == 0) {
-            CrackState *o = a.s_out;
-            const CrackState &S = sh.S;
+            CrackState *o = B.s_out;
+            const PassTip &e = sh.log[K], &e1 = sh.log[K - 1];
+            // an end's decision after the pass (modes that need no K)
+            auto known_end = [&](const TipState &s0, int64_t tip, int64_t tip1, int arr, double v, TipState &t) {
+                t = s0;
+                t.flags |= arr && !s0.arrested ? FLAG_CLAMPED : 0;
+                t.tip_q = tip;
+                t.arrested = arr;
+                t.grew = tip != tip1;
+                t.v = v;
+                t.v_prev = p.mode == CRACK_PRESCRIBED ? p.v_rel : 0.0;
+            };
             if (c.own_r) {
-                o->step = S.step + K;
-                o->hist_n = S.hist_n;
-                o->i_last = S.i_last;
-                if (!p.two_tips) o->i_first = S.i_first;
-                copy_tip_decision(o->r, S.r);
-                if (!c.known) {
-                    o->r.K = S.r.K;
-                    o->r.r_min = S.r.r_min;
-                    o->r.npairs = S.r.npairs;
+                o->step = sh.in.step + K;
+                o->hist_n = sh.in.hist_n + K - rec0;
+                o->i_last = e.l;
+                if (!p.two_tips) o->i_first = e.f;
+                if (c.known) {
+                    TipState t;
+                    known_end(sh.in.r, e.tr, e1.tr, e.arr_r, e.vr, t);
+                    copy_tip_decision(o->r, t);
+                } else {
+                    copy_tip_decision(o->r, sh.S.r);
+                }
+                if (!e.lazy) {
+                    o->r.K = sh.S.r.K;
+                    o->r.r_min = sh.S.r.r_min;
+                    o->r.npairs = sh.S.r.npairs;
                 }
                 o->r.decided = 0;
-                for (int i = c.l0 + 1; i <= S.i_last; ++i)
+                for (int i = c.l0 + 1; i <= e.l; ++i)
                     if (i >= c.f0) atomicOr(&a.cut_v[(int64_t)(p.jc - 1) * p.words + (i >> 5)], 1u << (i & 31));
             }
             if (c.own_l) {
-                o->i_first = S.i_first;
-                copy_tip_decision(o->l, S.l);
-                if (!c.known) {
-                    o->l.K = S.l.K;
-                    o->l.r_min = S.l.r_min;
-                    o->l.npairs = S.l.npairs;
+                o->i_first = e.f;
+                if (c.known) {
+                    TipState t;
+                    known_end(sh.in.l, e.tl, e1.tl, e.arr_l, e.vl, t);
+                    copy_tip_decision(o->l, t);
+                } else {
+                    copy_tip_decision(o->l, sh.S.l);
+                }
+                if (!e.lazy) {
+                    o->l.K = sh.S.l.K;
+                    o->l.r_min = sh.S.l.r_min;
+                    o->l.npairs = sh.S.l.npairs;
                 }
                 o->l.decided = 0;
-                for (int i = S.i_first; i < c.f0; ++i)
+                for (int i = e.f; i < c.f0; ++i)
                     if (i <= c.l0) atomicOr(&a.cut_v[(int64_t)(p.jc - 1) * p.words + (i >> 5)], 1u << (i & 31));
             }
         }
@@ -833,8 +1224,8 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const TileGeo
 }
 
 // Tile t of a pass.
-template <typename T, typename D, int RPT>
-__device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, int t, PassShared<T> &sh)
+template <typename T, typename D, int NW, int RPT>
+__device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<T, D> &B, int t, PassShared<T, NW> &sh)
 {
     constexpr int N = Vec<T>::N;
     const StepArgs<T, D> &a = A.s;
@@ -842,24 +1233,33 @@ __device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, int t, PassSha
     const int nx = a.nx, ny = a.ny;
     const bool per = a.edge[LEFT] == EDGE_PERIODIC;
     const int tid = threadIdx.x;
-    // the next pass's Dirichlet values (and, without a crack, its state): the last tile
-    if (t == q.tiles - 1 && tid < 4) {
-        const int64_t n1 = a.s_in->step + q.K;
-        if (tid == 0 && a.p.mode == CRACK_NONE) {
-            CrackState S = *a.s_in;
-            S.step = n1;
+    auto read_state = [&](CrackState &S) {
+        constexpr int kWords = (int)(sizeof(CrackState) / 4);
+        for (int k = tid; k < kWords; k += 32 * NW)
+            reinterpret_cast<uint32_t *>(&S)[k] = __ldcg(reinterpret_cast<const uint32_t *>(B.s_in) + k);
+        __syncthreads();
+    };
+    if (t == q.tiles - 1 && a.p.mode == CRACK_NONE) {
+        // without a crack, the state only counts steps
+        read_state(sh.in);
+        if (tid == 0) {
+            CrackState S = sh.in;
+            S.step += q.K;
             S.r.decided = 1;
             S.l.decided = 1;
             for (int e = 0; e < 4; ++e)
-                S.wstar[e] = a.edge[e] == EDGE_DIRICHLET ? load_value(a.load[e], n1, (double)a.p.dt) : 0.0;
-            *a.s_out = S;
-        } else if (a.p.mode != CRACK_NONE) {
-            a.s_out->wstar[tid] = a.edge[tid] == EDGE_DIRICHLET ? load_value(a.load[tid], n1, (double)a.p.dt) : 0.0;
+                S.wstar[e] = a.edge[e] == EDGE_DIRICHLET ? load_value(a.load[e], S.step, (double)a.p.dt) : 0.0;
+            *B.s_out = S;
         }
+    } else if (t == q.tiles - 1 && tid < 4) {
+        // the Dirichlet values after the pass (single steps read them)
+        const int64_t n1 = __ldcg(&B.s_in->step) + q.K;
+        B.s_out->wstar[tid] = a.edge[tid] == EDGE_DIRICHLET ? load_value(a.load[tid], n1, (double)a.p.dt) : 0.0;
     }
     TileGeo g;
     if (t < q.ms) {
-        const int f = a.s_in->i_first, l = a.s_in->i_last;
+        read_state(sh.in);
+        const int f = sh.in.i_first, l = sh.in.i_last;
         const int cr = tip_col_r(f, l, nx), cl = tip_col_l(f, l, nx);
         int lo0 = cr - q.zb, hi0 = cr + q.za, lo1 = cl + 1 - q.za, hi1 = cl + q.zb;
         bool two = a.p.two_tips != 0;
@@ -877,10 +1277,10 @@ __device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, int t, PassSha
         }
         if (g.x0 >= g.x1) return;
         g.xl = g.x0 == 0 && !per ? 0 : g.x0 - q.hc;
-        g.yl = a.p.jc - kStripHalf;
+        g.yl = a.p.jc - NW * kStripRpt / 2;
         g.y0 = q.jb;
         g.y1 = q.jt;
-        pass_tile<T, D, kStripRpt, 2>(A, g, sh);
+        pass_tile<T, D, NW, kStripRpt, 2>(A, B, g, sh);
         return;
     }
     t -= q.ms;
@@ -895,27 +1295,65 @@ __device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, int t, PassSha
         g.y1 = min(g.y0 + q.pt, ny);
     }
     g.xl = g.x0 == 0 && !per ? 0 : g.x0 - q.hc;
-    g.yl = g.y0 == 0 ? 0 : (g.y1 == ny ? ny - kPassWarps * RPT : g.y0 - q.K);
+    g.yl = g.y0 == 0 ? 0 : (g.y1 == ny ? ny - NW * RPT : g.y0 - q.K);
     const bool plain = g.x0 >= q.K && g.x1 + q.K <= nx && g.y0 >= q.K && g.y1 + q.K <= ny && g.xl >= 0;
-    if (plain) pass_tile<T, D, RPT, 0>(A, g, sh);
-    else pass_tile<T, D, RPT, 1>(A, g, sh);
+    if (plain) pass_tile<T, D, NW, RPT, 0>(A, B, g, sh);
+    else pass_tile<T, D, NW, RPT, 1>(A, B, g, sh);
 }
 
-template <typename T, typename D, int RPT>
-__global__ void __launch_bounds__(kPassThreads, 2) pass_kernel(const __grid_constant__ PassArgs<T, D> a)
+// n_pass passes, alternating between the two buffer sets.  One pass is a
+// plain launch with a CTA per tile.  Several are one cooperative launch (every
+// tile resident at once) with a grid barrier between passes: on lattices of a
+// few hundred tiles a pass takes about as long as the launch gap plus the
+// instruction fetches of a cold start.
+template <typename T, typename D, int NW, int RPT>
+__global__ void __launch_bounds__(32 * NW, 16 / NW)
+    pass_kernel(const __grid_constant__ PassArgs<T, D> a, int n_pass)
 {
-    __shared__ PassShared<T> sh;
+    __shared__ PassShared<T, NW> sh;
     pdl_wait();
     pdl_trigger();
-    pass_cta<T, D, RPT>(a, blockIdx.x, sh);
+    for (int it = 0; it < n_pass; ++it) {
+        const bool odd = (it & 1) != 0;
+        PassBuf<T, D> B;
+        B.w_in = odd ? a.w_in1 : a.s.w_in;
+        B.wd_in = odd ? a.wd_in1 : a.wd_in;
+        B.w_out = odd ? a.w_out1 : a.s.w_out;
+        B.wd = odd ? a.wd1 : a.s.wd;
+        B.s_in = odd ? a.s.s_out : a.s.s_in;
+        B.s_out = odd ? const_cast<CrackState *>(a.s.s_in) : a.s.s_out;
+        pass_cta<T, D, NW, RPT>(a, B, blockIdx.x, sh);
+        if (it + 1 < n_pass && !grid_barrier(a.bar, gridDim.x, a.budget, a.s.err)) return;
+    }
 }
 
-template <typename T, typename D> cudaError_t launch_pass(const PassArgs<T, D> &a, int rpt, cudaStream_t s)
+template <typename T, typename D> const void *pass_kernel_ptr(int nw, int rpt)
 {
-    const dim3 grid((unsigned)a.q.tiles), block(kPassThreads);
-    const bool ch = a.s.chained != 0;
-    return rpt == 8 ? launch_chained(pass_kernel<T, D, 8>, grid, block, 0, s, ch, a)
-                    : launch_chained(pass_kernel<T, D, 4>, grid, block, 0, s, ch, a);
+    if constexpr (sizeof(T) == 8)
+        if (nw == 4) return reinterpret_cast<const void *>(&pass_kernel<T, D, 4, 4>);
+    if constexpr (sizeof(T) == 4)
+        if (rpt == 4) return reinterpret_cast<const void *>(&pass_kernel<T, D, 8, 4>);
+    return reinterpret_cast<const void *>(&pass_kernel<T, D, 8, 8>);
+}
+
+template <typename T, typename D> cudaError_t launch_pass(const PassArgs<T, D> &a, int n_pass, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)a.q.tiles);
+    cfg.blockDim = dim3(32u * (unsigned)a.q.nw);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    if (n_pass > 1) {
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+    } else {
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = n_pass > 1 || a.s.chained ? 1 : 0;
+    void *args[] = {(void *)&a, (void *)&n_pass};
+    return cudaLaunchKernelExC(&cfg, pass_kernel_ptr<T, D>(a.q.nw, a.q.rpt), args);
 }
 
 }  // namespace lbm

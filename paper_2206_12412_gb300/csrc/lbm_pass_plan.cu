@@ -11,10 +11,12 @@ namespace host {
 
 namespace {
 
-constexpr int kWarps = 8, kStripHalfRows = 16;
-
 int ceil_div(int a, int b) { return (a + b - 1) / b; }
 int round_up(int a, int n) { return ceil_div(a, n) * n; }
+
+// FP64 lattices up to kPass64Sites sites are stepped in passes, those up to
+// kPass64Small in tiles of four warps.
+constexpr int64_t kPass64Sites = (int64_t)1 << 19, kPass64Small = (int64_t)1 << 17;
 
 // Row tiles of H held rows, K of them halo on each side that is no lattice
 // edge, over a region of `len` rows; at least `least` tiles.
@@ -36,16 +38,20 @@ void split_rows(int len, int H, int K, bool edge0, bool edge1, int least, int &m
 
 }  // namespace
 
-bool pass_plan(const lbm_handle *h, int K, int rpt, PassPlan &q)
+bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q)
 {
     const int nx = h->grid.nx, ny = h->grid.ny;
-    const int N = (int)(16 / h->esize), W = 32 * N, H = kWarps * rpt;
+    const int N = (int)(16 / h->esize), W = 32 * N, H = nw * rpt;
+    const int strip_half = nw * 4 / 2;   // kStripRpt rows a warp
     const bool per = h->grid.edge[LBM_LEFT] == LBM_EDGE_PERIODIC;
     const bool crack = h->cp.mode != CRACK_NONE;
     const CrackParams &p = h->cp;
-    if (K < 2 || K > 8) return false;
+    if (K < 2 || K > nw || 2 * K > strip_half) return false;
+    if (crack && p.hist_cap > 0 && p.hist_cap < K) return false;   // a pass's records go around the ring once at most
     std::memset(&q, 0, sizeof q);
     q.K = K;
+    q.nw = nw;
+    q.rpt = rpt;
     q.hc = round_up(K, N);
     q.edge_macro = h->edge_macro ? 1 : 0;
 
@@ -63,7 +69,7 @@ bool pass_plan(const lbm_handle *h, int K, int rpt, PassPlan &q)
     }
 
     // rows: the crack strip, and the bulk below and above it (all of it without a crack)
-    const int so = kStripHalfRows - K;
+    const int so = strip_half - K;
     int region0 = 0, region1 = ny;
     if (crack) {
         region0 = std::max(0, p.jc - so);
@@ -77,7 +83,7 @@ bool pass_plan(const lbm_handle *h, int K, int rpt, PassPlan &q)
     }
     // the edge rule is applied by tiles whose rows 0 .. 2 (or ny-1 .. ny-3) lie
     // in one thread: tiles held from row 0 or up to row ny - 1, not the strip
-    if (h->edge_macro && (crack ? p.jc < kStripHalfRows + 3 || ny - p.jc < kStripHalfRows + 3 : ny < 64)) return false;
+    if (h->edge_macro && (crack ? p.jc < strip_half + 3 || ny - p.jc < strip_half + 3 : ny < 64)) return false;
     if (h->edge_macro && nx < 4) return false;
 
     if (crack) {
@@ -87,6 +93,17 @@ bool pass_plan(const lbm_handle *h, int K, int rpt, PassPlan &q)
         const double v = p.mode == CRACK_KCRIT ? p.v_max : p.mode == CRACK_PRESCRIBED ? p.v_rel : 0.0;
         const double r_min = p.r_min_fixed > 0.0 ? p.r_min_fixed : p.r0 / (1.0 - v);
         const double reach = (r_min + p.fit_width) / p.dh;
+        // the window of an end at rest (prescribed growth: at its speed), as
+        // crack_eval_pairs bounds it, in whole units
+        const double v0 = p.mode == CRACK_PRESCRIBED ? p.v_rel : 0.0;
+        q.r_min = p.r_min_fixed > 0.0 ? p.r_min_fixed : (v0 == 0.0 ? p.r0 : p.r0 / (1.0 - v0));
+        const double lo = p.dh == 1.0 ? q.r_min : q.r_min / p.dh;
+        const double hi = p.dh == 1.0 ? q.r_min + p.fit_width : (q.r_min + p.fit_width) / p.dh;
+        q.lo_q = (int64_t)std::ceil(std::min(lo, 1e6) * 4294967296.0);
+        q.hi_q = (int64_t)std::ceil(std::min(hi, 1e6) * 4294967296.0);
+        q.one_pair = p.fit_width <= p.dh && q.hi_q - q.lo_q <= ((int64_t)1 << kQBits);
+        q.k_unit = (float)(p.mu / 4.0 * std::sqrt(2.0 * kPi / p.dh) * 65536.0);
+        q.k_rest = (float)(p.K_C * 0.999);
         // both ends are fitted at once by half a warp each: at most 16 columns
         if (!(p.fit_width / p.dh <= 12.0)) return false;
         if (nx + (per ? 2 * q.hc : 0) <= W) {
@@ -118,13 +135,28 @@ void choose_pass(lbm_handle *h)
 {
     h->pass_k = 0;
     if (!h->alt[0]) return;
+    const int64_t sites = (int64_t)h->grid.nx * h->grid.ny;
+    // FP64: two results per cycle and SM, so recomputed halos cost more than
+    // launches save on large lattices, and on small ones the tiles have to be
+    // many and small (see kPass64*)
+    if (h->esize == 8 && sites > kPass64Sites) return;
+    h->pass_nw = h->esize == 8 && sites <= kPass64Small ? 4 : 8;
     const int kmax = h->esize == 8 ? 4 : 8;
     for (int K = kmax; K >= 2; --K) {
         PassPlan q;
-        h->pass_rpt = 8;
-        if (!pass_plan(h, K, 8, q)) continue;
-        if (q.tiles < 2 * h->sms) h->pass_rpt = 4;
-        if (!pass_plan(h, K, h->pass_rpt, q)) continue;
+        h->pass_rpt = h->pass_nw == 4 ? 4 : 8;
+        if (!pass_plan(h, K, h->pass_nw, h->pass_rpt, q)) continue;
+        if (h->esize == 4 && q.tiles < 2 * h->sms) h->pass_rpt = 4;
+        if (!pass_plan(h, K, h->pass_nw, h->pass_rpt, q)) continue;
+        const void *fn = h->lat.storage == LBM_F64           ? pass_kernel_ptr<double, double>(h->pass_nw, h->pass_rpt)
+                         : h->lat.storage == LBM_F32_WD_BF16 ? pass_kernel_ptr<float, __nv_bfloat16>(h->pass_nw, h->pass_rpt)
+                         : h->lat.storage == LBM_F32_WD_F16  ? pass_kernel_ptr<float, __half>(h->pass_nw, h->pass_rpt)
+                         : h->lat.storage == LBM_F32_LEAPFROG ? pass_kernel_ptr<float, Lf>(h->pass_nw, h->pass_rpt)
+                                                              : pass_kernel_ptr<float, float>(h->pass_nw, h->pass_rpt);
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * h->pass_nw, 0) != cudaSuccess || per_sm < 1)
+            return;
+        h->pass_slots = per_sm * h->sms;
         h->pass_k = K;
         return;
     }

@@ -56,6 +56,11 @@ def cases():
         out.append((f"tip_{tip}", _strip(331, 60, mode="kcrit", tip=tip + 0.3, K_C=KC), "f32", 64))
         out.append((f"tips_{tip}", _strip(480, 60, mode="kcrit", start=tip + 0.2, tip=tip + 31.9, K_C=KC, two_tips=True),
                     "f32", 64))
+    for k, kc in enumerate((3e-5, 6e-5, 1.2e-4, 2.4e-4)):   # ends that rest, grow and rest again
+        out.append((f"rest_{k}", _strip(300, 150, mode="kcrit", K_C=kc), "f32", 91))
+        out.append((f"rest_two_{k}", _strip(300, 150, mode="kcrit", K_C=kc, start=140.2, tip=143.9, two_tips=True), "f32", 91))
+        out.append((f"rest_wide_{k}", _strip(700, 300, mode="kcrit", K_C=kc, start=140.0, tip=181.0, two_tips=True,
+                                             fit_width=3.5), "f64", 60))
     out += [
         ("no_crack", _strip(300, 170, mode=None), "f32", 70),
         ("no_crack_edges", _strip(300, 170, mode=None, bc="macroscopic_edges"), "f32", 70),
