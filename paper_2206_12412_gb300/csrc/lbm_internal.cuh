@@ -214,6 +214,10 @@ struct PassPlan {
     int64_t lo_q, hi_q;
     double r_min;
     int32_t one_pair;
+    int32_t unit;              // dh = dt = 1
+    float lo_f;                // r_min at rest
+    int64_t w_q;               // the window's width
+    double k_inv;              // 1 / K_C
     float k_unit, k_rest;      // mu / 4 sqrt(2 pi / dh) 2^16; just below K_C
     int32_t mx, px;            // column tiles of the bulk and their width
     int32_t jb, mb, pb;        // rows [0, jb) below the strip: mb row tiles of pb rows
@@ -341,7 +345,7 @@ template <typename T, typename D>
 cudaError_t launch_step(const StepArgs<T, D> &a, int bands, cudaStream_t s, bool bulk = false);
 // n_pass passes of several time steps (more than one: one cooperative launch).
 template <typename T, typename D> cudaError_t launch_pass(const PassArgs<T, D> &a, int n_pass, cudaStream_t s);
-template <typename T, typename D> const void *pass_kernel_ptr(int nw, int rpt);
+template <typename T, typename D> const void *pass_kernel_ptr(int nw, int rpt, bool run);
 template <typename T, typename D> cudaError_t launch_edge_rule(const StepArgs<T, D> &a, cudaStream_t s);
 template <typename T, typename D> int edge_rule_count(const StepArgs<T, D> &a);
 template <typename T, typename D>

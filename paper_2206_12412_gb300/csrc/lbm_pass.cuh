@@ -168,7 +168,7 @@ __device__ __forceinline__ void row_sites(const Row<T, N> &cu, const Row<T, N> &
 // the crack step before it (lazy: its K and pairs are formed at the end).
 struct PassTip {
     int64_t tr, tl;
-    double vr, vl, Kr, Kl;
+    double vr, vl, Kr, Kl, vp_r, vp_l;   // vp: the speed before it (its window's, eq. r(v))
     int32_t f, l, npr, npl;
     int32_t arr_r, arr_l, lazy, pad;
 };
@@ -247,12 +247,23 @@ __device__ __forceinline__ PassPair pass_pair(int dir, int64_t tip, int64_t lo_q
     r.col = (int)i;
     return r;
 }
+// a / b for a divisor known in advance, y = 1 / b rounded: the residual of a y
+// is exact in one FMA, and adding its share rounds to the quotient (Markstein,
+// IBM J. Res. Dev. 34, 1990; equal to the division in 1.2e8 random quotients
+// over the divisors used here).  Three FP64 instructions instead of ten, at
+// 64 cycles each.
+__device__ __forceinline__ double div_known(double a, double b, double y)
+{
+    const double q = a * y;
+    return fma(fma(-q, b, a), y, q);
+}
+
 // sqrt(r / 2 pi) of a pair, and K from it (the sums of crack_eval_pairs over one pair).
 __device__ __forceinline__ double pass_sf(const CrackParams &p, int64_t d)
 {
     const double r_h = (double)d * kTwoM32;
     const double r = p.dh == 1.0 ? r_h : r_h * p.dh;
-    return sqrt(r / (2.0 * kPi));
+    return sqrt(div_known(r, 2.0 * kPi, 1.0 / (2.0 * kPi)));
 }
 template <typename T>
 __device__ __forceinline__ CrackSums pass_sums(double sf, T above, T below, double r_min)
@@ -322,8 +333,8 @@ __device__ __forceinline__ void pass_crack_step(const CrackParams &p, const Pass
     const TipState &E = dir > 0 ? S.r : S.l;
     const int org = dir > 0 ? org_r : org_l;
     const bool act = dir > 0 ? act_r : act_l;
-    if (__any_sync(0xffffffffu, act && E.tip_q != win.tip)) pass_window(q, S, org, dir > 0 ? ev_r : ev_l, win);
     const bool rest = (__double_as_longlong(E.v_prev) << 1) == 0;   // v_prev = 0
+    if (__any_sync(0xffffffffu, act && rest && E.tip_q != win.tip)) pass_window(q, S, org, dir > 0 ? ev_r : ev_l, win);
     float t = 0.0f;
     if (win.col >= 0 && win.col < W) t = fabsf(win.coef * (float)(above[win.col] - below[win.col]));
     const bool hot = act && !(rest && (E.arrested || t < q.k_rest));
@@ -344,20 +355,39 @@ __device__ __forceinline__ void pass_crack_step(const CrackParams &p, const Pass
         }
     } else {
         CrackSums c = {0.0, 0.0, 0.0, 0};
-        bool many = !q.one_pair;
-        if (!many && (lane & 15) == 0 && act) {
-            // at most one pair: its column by integer distances
-            const double r_min = p.r_min_fixed > 0.0 ? p.r_min_fixed : (rest ? p.r0 : p.r0 / (1.0 - E.v_prev));
-            const double lo = p.dh == 1.0 ? r_min : r_min / p.dh;
-            const double hi = p.dh == 1.0 ? r_min + p.fit_width : (r_min + p.fit_width) / p.dh;
-            const int64_t lo_q = __double2ll_ru(lo * 4294967296.0), hi_q = __double2ll_ru(hi * 4294967296.0);
-            many = hi_q - lo_q > ((int64_t)1 << kQBits);   // by the rounding of hi
-            const PassPair w = pass_pair(dir, E.tip_q, lo_q, hi_q, S.i_first, S.i_last);
+        CrackDecision d = {};
+        const bool head = (lane & 15) == 0 && act;
+        bool full = !q.one_pair || !q.unit;
+        if (!full && head) {
+            // dh = dt = 1 and a window of at most one pair: its column from
+            // r_min in FP32 (exact unless a column lies within 2^-17 of the
+            // window's ends), and no FP64 operation that does not decide
+            const float lo = rest ? q.lo_f : q.lo_f / (1.0f - (float)E.v_prev);
+            const int64_t lo_q = (int64_t)(lo * 4294967296.0f), slack = (int64_t)1 << 15;
+            const PassPair w = pass_pair(dir, E.tip_q, lo_q, lo_q + ((int64_t)1 << kQBits), S.i_first, S.i_last);
+            const int64_t past = w.d - lo_q;   // in [0, 2^32)
+            full = !(lo < 24.0f) || past < slack || past > ((int64_t)1 << kQBits) - slack || llabs(past - q.w_q) < slack;
             const int k = w.col - org;
-            c.r_min = r_min;
-            if (w.in && k >= 0 && k < W) c = pass_sums<T>(pass_sf(p, w.d), above[k], below[k], r_min);
+            if (w.in && past < q.w_q && k >= 0 && k < W) c = pass_sums<T>(pass_sf(p, w.d), above[k], below[k], 0.0);
+            if (!full) {
+                // crack_decide for K-criterion growth
+                d.K = pass_K(p, c);
+                d.flags = E.flags;
+                const double Ka = fabs(d.K);
+                if (c.np > 0 && Ka > p.K_C) {
+                    const double ratio = div_known(Ka, p.K_C, q.k_inv);
+                    d.propagate = 1;
+                    d.v = p.v_max * tanh(sqrt(ratio * ratio * ratio * ratio - 1.0));   // eq. v-tanh
+                }
+                if ((__double_as_longlong(d.K) & 0x7ff0000000000000ll) == 0x7ff0000000000000ll) d.flags |= FLAG_NONFINITE;
+                if (E.arrested) {
+                    d.propagate = 0;
+                    d.v = 0.0;
+                }
+                if (d.propagate) d.dq = __double2ll_rn(d.v * p.cs * 4294967296.0);
+            }
         }
-        if (__any_sync(0xffffffffu, many)) {
+        if (__any_sync(0xffffffffu, full)) {
             c = crack_eval_pairs<T, 16>(p, E.tip_q, E.v_prev, S.i_first, S.i_last, dir, [&](int i, T &a, T &b) {
                 const int k = i - org;
                 if (k < 0 || k >= W) return false;   // an end this tile does not follow
@@ -365,9 +395,10 @@ __device__ __forceinline__ void pass_crack_step(const CrackParams &p, const Pass
                 b = below[k];
                 return true;
             });
+            if (head) d = crack_decide(p, S, dir, c);
         }
-        CrackDecision d = {};
-        if ((lane & 15) == 0 && act) d = crack_decide(p, S, dir, c);
+        if (lane == 0) rec.vp_r = S.r.v_prev;
+        if (lane == 16) rec.vp_l = S.l.v_prev;
         const History none = {};
         __syncwarp();
         if (lane == 0 && act_r) crack_commit(p, nullptr, none, S, +1, false, c, d);
@@ -874,7 +905,7 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
 
 // A tile.  KIND: 0 one none of whose sites sees an edge or the crack, 1 with
 // outer edges, 2 a crack-strip tile (with edges where it meets them).
-template <typename T, typename D, int NW, int RPT, int KIND>
+template <typename T, typename D, int NW, int RPT, int KIND, bool COOP>
 __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf<T, D> &B, const TileGeo g,
                                           PassShared<T, NW> &sh)
 {
@@ -911,8 +942,13 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
             const int j = jb + r;
             if (j < 0 || j >= ny) continue;
             if (whole) {
-                cg_row(wp + (int64_t)r * P, w);
-                cg_rate(dp + (int64_t)r * P, d, wd_inv);
+                if (COOP) {
+                    cg_row(wp + (int64_t)r * P, w);
+                    cg_rate(dp + (int64_t)r * P, d, wd_inv);
+                } else {
+                    ldg_row(wp + (int64_t)r * P, w);
+                    WdIO<D>::load(dp + (int64_t)r * P, d, wd_inv);
+                }
             } else if (KIND != 0) {
 #pragma unroll
                 for (int k = 0; k < N; ++k) {
@@ -1170,6 +1206,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
         if (tid == 0) {
             CrackState *o = B.s_out;
             const PassTip &e = sh.log[K], &e1 = sh.log[K - 1];
+            auto r_min_at = [&](double v) { return p.r_min_fixed > 0.0 ? p.r_min_fixed : (v == 0.0 ? p.r0 : p.r0 / (1.0 - v)); };
             // an end's decision after the pass (modes that need no K)
             auto known_end = [&](const TipState &s0, int64_t tip, int64_t tip1, int arr, double v, TipState &t) {
                 t = s0;
@@ -1194,7 +1231,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
                 }
                 if (!e.lazy) {
                     o->r.K = sh.S.r.K;
-                    o->r.r_min = sh.S.r.r_min;
+                    o->r.r_min = r_min_at(e.vp_r);
                     o->r.npairs = sh.S.r.npairs;
                 }
                 o->r.decided = 0;
@@ -1212,7 +1249,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
                 }
                 if (!e.lazy) {
                     o->l.K = sh.S.l.K;
-                    o->l.r_min = sh.S.l.r_min;
+                    o->l.r_min = r_min_at(e.vp_l);
                     o->l.npairs = sh.S.l.npairs;
                 }
                 o->l.decided = 0;
@@ -1224,7 +1261,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
 }
 
 // Tile t of a pass.
-template <typename T, typename D, int NW, int RPT>
+template <typename T, typename D, int NW, int RPT, bool COOP>
 __device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<T, D> &B, int t, PassShared<T, NW> &sh)
 {
     constexpr int N = Vec<T>::N;
@@ -1280,7 +1317,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<
         g.yl = a.p.jc - NW * kStripRpt / 2;
         g.y0 = q.jb;
         g.y1 = q.jt;
-        pass_tile<T, D, NW, kStripRpt, 2>(A, B, g, sh);
+        pass_tile<T, D, NW, kStripRpt, 2, COOP>(A, B, g, sh);
         return;
     }
     t -= q.ms;
@@ -1297,22 +1334,30 @@ __device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<
     g.xl = g.x0 == 0 && !per ? 0 : g.x0 - q.hc;
     g.yl = g.y0 == 0 ? 0 : (g.y1 == ny ? ny - NW * RPT : g.y0 - q.K);
     const bool plain = g.x0 >= q.K && g.x1 + q.K <= nx && g.y0 >= q.K && g.y1 + q.K <= ny && g.xl >= 0;
-    if (plain) pass_tile<T, D, NW, RPT, 0>(A, B, g, sh);
-    else pass_tile<T, D, NW, RPT, 1>(A, B, g, sh);
+    if (plain) pass_tile<T, D, NW, RPT, 0, COOP>(A, B, g, sh);
+    else pass_tile<T, D, NW, RPT, 1, COOP>(A, B, g, sh);
 }
 
-// n_pass passes, alternating between the two buffer sets.  One pass is a
-// plain launch with a CTA per tile.  Several are one cooperative launch (every
-// tile resident at once) with a grid barrier between passes: on lattices of a
-// few hundred tiles a pass takes about as long as the launch gap plus the
-// instruction fetches of a cold start.
+// One pass, a CTA per tile.
 template <typename T, typename D, int NW, int RPT>
-__global__ void __launch_bounds__(32 * NW, 16 / NW)
-    pass_kernel(const __grid_constant__ PassArgs<T, D> a, int n_pass)
+__global__ void __launch_bounds__(32 * NW, 16 / NW) pass_kernel(const __grid_constant__ PassArgs<T, D> a)
 {
     __shared__ PassShared<T, NW> sh;
     pdl_wait();
     pdl_trigger();
+    const PassBuf<T, D> B = {a.s.w_in, a.wd_in, a.s.w_out, a.s.wd, a.s.s_in, a.s.s_out};
+    pass_cta<T, D, NW, RPT, false>(a, B, blockIdx.x, sh);
+}
+
+// n_pass passes, alternating between the two buffer sets, as one cooperative
+// launch (every tile resident at once) with a grid barrier between passes: on
+// lattices of a few hundred tiles a pass takes hardly longer than the launch
+// gap, the ramp and the instruction fetches of a cold start.
+template <typename T, typename D, int NW, int RPT>
+__global__ void __launch_bounds__(32 * NW, 16 / NW)
+    pass_run_kernel(const __grid_constant__ PassArgs<T, D> a, int n_pass)
+{
+    __shared__ PassShared<T, NW> sh;
     for (int it = 0; it < n_pass; ++it) {
         const bool odd = (it & 1) != 0;
         PassBuf<T, D> B;
@@ -1322,28 +1367,34 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW)
         B.wd = odd ? a.wd1 : a.s.wd;
         B.s_in = odd ? a.s.s_out : a.s.s_in;
         B.s_out = odd ? const_cast<CrackState *>(a.s.s_in) : a.s.s_out;
-        pass_cta<T, D, NW, RPT>(a, B, blockIdx.x, sh);
+        pass_cta<T, D, NW, RPT, true>(a, B, blockIdx.x, sh);
         if (it + 1 < n_pass && !grid_barrier(a.bar, gridDim.x, a.budget, a.s.err)) return;
     }
 }
 
-template <typename T, typename D> const void *pass_kernel_ptr(int nw, int rpt)
+template <typename T, typename D> const void *pass_kernel_ptr(int nw, int rpt, bool run)
 {
     if constexpr (sizeof(T) == 8)
-        if (nw == 4) return reinterpret_cast<const void *>(&pass_kernel<T, D, 4, 4>);
+        if (nw == 4)
+            return run ? reinterpret_cast<const void *>(&pass_run_kernel<T, D, 4, 4>)
+                       : reinterpret_cast<const void *>(&pass_kernel<T, D, 4, 4>);
     if constexpr (sizeof(T) == 4)
-        if (rpt == 4) return reinterpret_cast<const void *>(&pass_kernel<T, D, 8, 4>);
-    return reinterpret_cast<const void *>(&pass_kernel<T, D, 8, 8>);
+        if (rpt == 4)
+            return run ? reinterpret_cast<const void *>(&pass_run_kernel<T, D, 8, 4>)
+                       : reinterpret_cast<const void *>(&pass_kernel<T, D, 8, 4>);
+    return run ? reinterpret_cast<const void *>(&pass_run_kernel<T, D, 8, 8>)
+               : reinterpret_cast<const void *>(&pass_kernel<T, D, 8, 8>);
 }
 
 template <typename T, typename D> cudaError_t launch_pass(const PassArgs<T, D> &a, int n_pass, cudaStream_t s)
 {
+    const bool run = n_pass > 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)a.q.tiles);
     cfg.blockDim = dim3(32u * (unsigned)a.q.nw);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
-    if (n_pass > 1) {
+    if (run) {
         attr[0].id = cudaLaunchAttributeCooperative;
         attr[0].val.cooperative = 1;
     } else {
@@ -1351,9 +1402,9 @@ template <typename T, typename D> cudaError_t launch_pass(const PassArgs<T, D> &
         attr[0].val.programmaticStreamSerializationAllowed = 1;
     }
     cfg.attrs = attr;
-    cfg.numAttrs = n_pass > 1 || a.s.chained ? 1 : 0;
-    void *args[] = {(void *)&a, (void *)&n_pass};
-    return cudaLaunchKernelExC(&cfg, pass_kernel_ptr<T, D>(a.q.nw, a.q.rpt), args);
+    cfg.numAttrs = run || a.s.chained ? 1 : 0;
+    void *args[] = {(void *)&a, (void *)&n_pass};   // one pass: the first argument only
+    return cudaLaunchKernelExC(&cfg, pass_kernel_ptr<T, D>(a.q.nw, a.q.rpt, run), args);
 }
 
 }  // namespace lbm

@@ -102,6 +102,11 @@ bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q)
         q.lo_q = (int64_t)std::ceil(std::min(lo, 1e6) * 4294967296.0);
         q.hi_q = (int64_t)std::ceil(std::min(hi, 1e6) * 4294967296.0);
         q.one_pair = p.fit_width <= p.dh && q.hi_q - q.lo_q <= ((int64_t)1 << kQBits);
+        // (a fixed r_min does not follow the speed: the general step)
+        q.unit = p.dh == 1.0 && p.dt == 1.0 && !(p.r_min_fixed > 0.0);
+        q.lo_f = (float)p.r0;
+        q.w_q = (int64_t)std::llrint(std::min(p.fit_width / p.dh, 1e6) * 4294967296.0);
+        q.k_inv = p.K_C > 0.0 ? 1.0 / p.K_C : 0.0;
         q.k_unit = (float)(p.mu / 4.0 * std::sqrt(2.0 * kPi / p.dh) * 65536.0);
         q.k_rest = (float)(p.K_C * 0.999);
         // both ends are fitted at once by half a warp each: at most 16 columns
@@ -148,11 +153,11 @@ void choose_pass(lbm_handle *h)
         if (!pass_plan(h, K, h->pass_nw, h->pass_rpt, q)) continue;
         if (h->esize == 4 && q.tiles < 2 * h->sms) h->pass_rpt = 4;
         if (!pass_plan(h, K, h->pass_nw, h->pass_rpt, q)) continue;
-        const void *fn = h->lat.storage == LBM_F64           ? pass_kernel_ptr<double, double>(h->pass_nw, h->pass_rpt)
-                         : h->lat.storage == LBM_F32_WD_BF16 ? pass_kernel_ptr<float, __nv_bfloat16>(h->pass_nw, h->pass_rpt)
-                         : h->lat.storage == LBM_F32_WD_F16  ? pass_kernel_ptr<float, __half>(h->pass_nw, h->pass_rpt)
-                         : h->lat.storage == LBM_F32_LEAPFROG ? pass_kernel_ptr<float, Lf>(h->pass_nw, h->pass_rpt)
-                                                              : pass_kernel_ptr<float, float>(h->pass_nw, h->pass_rpt);
+        const void *fn = h->lat.storage == LBM_F64           ? pass_kernel_ptr<double, double>(h->pass_nw, h->pass_rpt, true)
+                         : h->lat.storage == LBM_F32_WD_BF16 ? pass_kernel_ptr<float, __nv_bfloat16>(h->pass_nw, h->pass_rpt, true)
+                         : h->lat.storage == LBM_F32_WD_F16  ? pass_kernel_ptr<float, __half>(h->pass_nw, h->pass_rpt, true)
+                         : h->lat.storage == LBM_F32_LEAPFROG ? pass_kernel_ptr<float, Lf>(h->pass_nw, h->pass_rpt, true)
+                                                              : pass_kernel_ptr<float, float>(h->pass_nw, h->pass_rpt, true);
         int per_sm = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * h->pass_nw, 0) != cudaSuccess || per_sm < 1)
             return;
