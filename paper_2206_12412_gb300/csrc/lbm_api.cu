@@ -1222,41 +1222,31 @@ lbm_status lbm_step(lbm_handle *h, int64_t n)
         int par = h->parity;
         lbm_status rc = LBM_OK;
         if (h->pass_k && !h->own_bands && !h->bulk) {
-            // as many pairs of passes as n holds, then a pair of shorter ones
-            // for what is left (a pair of K steps covers 2 K of them); or, for
-            // few steps, equally long passes where that leaves at most one step
-            while (n >= 4) {
-                int K = (int)std::min<int64_t>(n / 2, h->pass_k);
-                int64_t pairs = n / (2 * K);
-                if (n < 4 * h->pass_k) {
-                    const int64_t m = (n + 2 * h->pass_k - 1) / (2 * h->pass_k), k = n / (2 * m);
-                    if (k >= 2 && n - 2 * m * k <= 1) {
-                        K = (int)k;
-                        pairs = m;
-                    }
-                }
+            auto go = [&](int K, int64_t m) -> lbm_status {
                 lbm::PassPlan q;
-                if (!pass_plan(h, K, h->pass_nw, h->pass_rpt, q)) break;
+                if (!pass_plan(h, K, h->pass_nw, h->pass_rpt, q)) return fail(LBM_ERR_ARG, "no plan of a pass");
                 if (q.tiles <= h->pass_slots) {
                     // every tile resident: the passes in one launch
-                    for (int64_t left = 2 * pairs; left > 0;) {
-                        const int m = (int)std::min<int64_t>(left, kMaxPasses);
-                        LBM_CUDA(enqueue_pass(h, q, par, false, m, h->stream));
-                        left -= m;
-                    }
-                } else if (K == h->pass_k) {
-                    const int base = par;
-                    rc = run_chunks(h->passes, h->gen, h->stream, h->cap_stream, 2 * pairs, par,
-                                    [&](int p, cudaStream_t s) { return enqueue_pass(h, q, p, p != base, 1, s); });
-                    if (rc != LBM_OK) return rc;
-                } else {
-                    for (int64_t m = 0; m < pairs; ++m) {
-                        LBM_CUDA(enqueue_pass(h, q, par, false, 1, h->stream));
-                        LBM_CUDA(enqueue_pass(h, q, par ^ 1, true, 1, h->stream));
-                    }
+                    for (; m > 0; m -= std::min(m, kMaxPasses))
+                        LBM_CUDA(enqueue_pass(h, q, par, false, (int)std::min(m, kMaxPasses), h->stream));
+                    return LBM_OK;
                 }
-                n -= pairs * 2 * K;
-            }
+                const int base = par;
+                auto one = [&](int p, cudaStream_t s) { return enqueue_pass(h, q, p, p != base, 1, s); };
+                if (K == h->pass_k) return run_chunks(h->passes, h->gen, h->stream, h->cap_stream, m, par, one);
+                for (; m > 0; --m, par ^= 1) LBM_CUDA(one(par, h->stream));
+                return LBM_OK;
+            };
+            auto pair = [&](int Ka, int Kb) -> lbm_status {
+                lbm::PassPlan qa, qb;
+                if (!pass_plan(h, Ka, h->pass_nw, h->pass_rpt, qa) || !pass_plan(h, Kb, h->pass_nw, h->pass_rpt, qb))
+                    return fail(LBM_ERR_ARG, "no plan of a pass");
+                LBM_CUDA(enqueue_pass(h, qa, par, false, 1, h->stream));
+                LBM_CUDA(enqueue_pass(h, qb, par ^ 1, true, 1, h->stream));
+                return LBM_OK;
+            };
+            rc = split_passes(n, h->pass_k, go, pair);
+            if (rc != LBM_OK) return rc;
         }
         // runs of single steps replay graphs of 64, 32, ..., 2 steps
         rc = run_chunks(h->steps, h->gen, h->stream, h->cap_stream, n, par,

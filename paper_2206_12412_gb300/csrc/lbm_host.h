@@ -211,7 +211,8 @@ inline void make_step_args(const lbm_handle *h, int par, StepArgs<T, D> &a)
 // The tiles of a pass of K steps of this lattice (lbm_pass_plan.cu); false
 // where a pass of K steps cannot be split so that every tile that needs a
 // crack decision holds what decides it.
-bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, lbm::PassPlan &q);
+// adjoint: the plan of the sweep's transposed steps.
+bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, lbm::PassPlan &q, bool adjoint = false);
 // Choose the pass of this lattice: h->pass_k, h->pass_nw, h->pass_rpt.
 void choose_pass(lbm_handle *h);
 
@@ -240,6 +241,37 @@ inline void make_pass_args(const lbm_handle *h, int par, bool second, const lbm:
     a.wd_in1 = a.s.wd;
     a.w_out1 = const_cast<T *>(a.s.w_in);
     a.wd1 = const_cast<D *>(a.wd_in);
+}
+
+// Split n steps into passes of at most kmax, always an even number of them:
+// go(K, m) runs m (even) passes of K steps, pair(Ka, Kb) one of Ka and one of
+// Kb.  As many of kmax as leave enough, then about equal ones; n < 4 is left
+// to single steps.  Returns with n the steps left.
+template <typename G, typename P>
+inline lbm_status split_passes(int64_t &n, int kmax, G &&go, P &&pair)
+{
+    lbm_status rc = LBM_OK;
+    const int64_t two = 2 * (int64_t)kmax;
+    if (n >= 2 * two || (n >= two && n % two == 0)) {
+        const int64_t pairs = n % two == 0 ? n / two : n / two - 1;
+        if ((rc = go(kmax, 2 * pairs)) != LBM_OK) return rc;
+        n -= pairs * two;
+    }
+    if (n < 4) return rc;
+    int64_t m = (n + two - 1) / two;
+    if (n < 4 * m) {   // too few for m pairs of two steps or more
+        m -= 1;
+        if ((rc = go(kmax, 2 * m)) != LBM_OK) return rc;
+        n -= m * two;
+        return rc;
+    }
+    const int64_t k = n / (2 * m), r = n - 2 * m * k;   // r passes of k + 1, the rest of k
+    if (r >= 2 && (rc = go((int)k + 1, r / 2 * 2)) != LBM_OK) return rc;
+    if (r % 2 != 0 && (rc = pair((int)k + 1, (int)k)) != LBM_OK) return rc;
+    const int64_t left = 2 * m - r / 2 * 2 - (r % 2 != 0 ? 2 : 0);
+    if (left > 0 && (rc = go((int)k, left)) != LBM_OK) return rc;
+    n = 0;
+    return rc;
 }
 
 // Whether the single-lattice step launch adds the record CTA (StepArgs::k_cta)

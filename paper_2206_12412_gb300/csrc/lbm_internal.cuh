@@ -234,6 +234,44 @@ struct GridBarrier {
     unsigned int count, gen;
 };
 
+// Recording of a forward run for the adjoint (see the adjoint kernel).  The
+// sensors of each unit (CTA of the step kernel: band * ncb + cb) are the
+// entries s_off[u] .. s_off[u+1]-1 of s_ent, each an index k into s_i / s_j.
+// Step t of the recording (t = step - *n0, 0 <= t < n_steps) stores the misfit
+// r = w(x_k) - target[t][k] of the state it produces in resid[t % ring][k],
+// adds r^2 to loss[k] if acc_loss, and stores the first and last severed
+// crack columns in force during step t in i_first[t], i_last[t].
+struct RecArgs {
+    const int32_t *s_off, *s_ent, *s_i, *s_j;
+    const double *target;
+    double *resid;
+    double *loss;
+    int32_t *i_first, *i_last;
+    const int64_t *n0;
+    int64_t n_steps, ring;
+    int32_t ns, acc_loss;
+};
+
+// What a pass does besides stepping: nothing, the adjoint's recording, or the
+// transposed steps of its sweep (m and a in place of w and wdot).
+enum { kForward = 0, kRecord = 1, kAdjoint = 2 };
+constexpr int kPassSensors = 64;   // most sensors of a recording or sweep in passes
+
+// The sweep's part of a pass's arguments (see AdjArgs); edge_m: the values of m
+// next to the Dirichlet edges at each step, edge_ring steps x 4 edges x
+// edge_len.
+template <typename T>
+struct PassAdj {
+    const int32_t *i_first, *i_last;
+    const int64_t *cnt_in;
+    int64_t *cnt_out;
+    int64_t n_steps, ring, edge_ring, edge_len;
+    const int32_t *s_i, *s_j;
+    const double *resid;
+    T *edge_m;
+    int32_t ns, pad;
+};
+
 template <typename T, typename D>
 struct PassArgs {
     StepArgs<T, D> s;          // w_in, w_out; s.wd: the wdot plane the pass writes (leapfrog: w of the step before last)
@@ -246,6 +284,8 @@ struct PassArgs {
     GridBarrier *bar;          // the barrier between its passes, a wait at most `budget` cycles
     long long budget;
     PassPlan q;
+    RecArgs rec;               // kRecord
+    PassAdj<T> adj;            // kAdjoint
 };
 
 // One CTA of a batched step: column block cb of band `band` of lattice `inst`.
@@ -265,24 +305,6 @@ struct BatchPiece {
     int32_t inst;
     int16_t cb, duty;
     int32_t j0, j1;
-};
-
-// Recording of a forward run for the adjoint (see the adjoint kernel).  The
-// sensors of each unit (CTA of the step kernel: band * ncb + cb) are the
-// entries s_off[u] .. s_off[u+1]-1 of s_ent, each an index k into s_i / s_j.
-// Step t of the recording (t = step - *n0, 0 <= t < n_steps) stores the misfit
-// r = w(x_k) - target[t][k] of the state it produces in resid[t % ring][k],
-// adds r^2 to loss[k] if acc_loss, and stores the first and last severed
-// crack columns in force during step t in i_first[t], i_last[t].
-struct RecArgs {
-    const int32_t *s_off, *s_ent, *s_i, *s_j;
-    const double *target;
-    double *resid;
-    double *loss;
-    int32_t *i_first, *i_last;
-    const int64_t *n0;
-    int64_t n_steps, ring;
-    int32_t ns, acc_loss;
 };
 
 // One step of the adjoint sweep (see lbm_adjoint.cu).  The adjoint state is
@@ -308,9 +330,9 @@ struct AdjArgs {
     int64_t n_steps, ring;
     const int32_t *s_off, *s_ent, *s_i, *s_j;
     const double *resid;       // [ring][ns] misfits of the recorded states
-    double *part;              // [n_steps][4][slots] per-CTA sums of m along the Dirichlet edges
+    T *edge_m;                 // [edge_ring][4][edge_len] values of m along the Dirichlet edges
+    int64_t edge_ring, edge_len;
     uint32_t *err;
-    int32_t slots, pad;
 };
 
 // One row copy of the halo exchange between row slabs (whole padded rows).
@@ -344,8 +366,9 @@ cudaError_t launch_batch_pieces(const StepArgs<T, D> *descs, const BatchPiece *p
 template <typename T, typename D>
 cudaError_t launch_step(const StepArgs<T, D> &a, int bands, cudaStream_t s, bool bulk = false);
 // n_pass passes of several time steps (more than one: one cooperative launch).
-template <typename T, typename D> cudaError_t launch_pass(const PassArgs<T, D> &a, int n_pass, cudaStream_t s);
-template <typename T, typename D> const void *pass_kernel_ptr(int nw, int rpt, bool run);
+template <typename T, typename D, int MODE = kForward>
+cudaError_t launch_pass(const PassArgs<T, D> &a, int n_pass, cudaStream_t s);
+template <typename T, typename D, int MODE = kForward> const void *pass_kernel_ptr(int nw, int rpt, bool run);
 template <typename T, typename D> cudaError_t launch_edge_rule(const StepArgs<T, D> &a, cudaStream_t s);
 template <typename T, typename D> int edge_rule_count(const StepArgs<T, D> &a);
 template <typename T, typename D>
@@ -367,8 +390,10 @@ template <typename T> cudaError_t launch_step_rec(const StepArgs<T, T> &a, const
 template <typename T> const void *adjoint_kernel_ptr();
 template <typename T> cudaError_t launch_adjoint(const AdjArgs<T> &a, int bands, cudaStream_t s);
 cudaError_t launch_loss_sum(const double *acc, int ns, double *out, cudaStream_t s);
-cudaError_t launch_grad_sum(const double *part, int64_t T, int slots, int dir_mask, double g, double *grad,
-                            cudaStream_t s);
+// grad[e][n] for n0 <= n < n0 + n_count from the values of m next to edge e at step n.
+template <typename T>
+cudaError_t launch_grad_sum(const T *edge, int64_t edge_ring, int64_t edge_len, int64_t n0, int64_t n_count, int64_t n_steps,
+                            int nx, int ny, int dir_mask, double g, double *grad, cudaStream_t s);
 template <typename T>
 cudaError_t launch_adjoint_out(const T *a, const T *m, int64_t pitch, int nx, int ny, T dt, T *dw, T *dwd, cudaStream_t s);
 template <typename D>

@@ -3,9 +3,9 @@
 
 namespace lbm {
 
-template const void *pass_kernel_ptr<float, float>(int, int, bool);
-template cudaError_t launch_pass<float, float>(const PassArgs<float, float> &, int, cudaStream_t);
-template const void *pass_kernel_ptr<float, Lf>(int, int, bool);
-template cudaError_t launch_pass<float, Lf>(const PassArgs<float, Lf> &, int, cudaStream_t);
+template const void *pass_kernel_ptr<float, float, kForward>(int, int, bool);
+template cudaError_t launch_pass<float, float, kForward>(const PassArgs<float, float> &, int, cudaStream_t);
+template const void *pass_kernel_ptr<float, Lf, kForward>(int, int, bool);
+template cudaError_t launch_pass<float, Lf, kForward>(const PassArgs<float, Lf> &, int, cudaStream_t);
 
 }  // namespace lbm

@@ -186,6 +186,16 @@ struct PassShared {
     int32_t reach[2];
 };
 
+// What a pass of the adjoint's recording (kRecord) or sweep (kAdjoint) keeps
+// besides: the tile's sensors, in ascending order, and their values at each
+// step (recording: w; sweep: the sources 2 r).
+template <typename T, int MODE> struct PassSensors {
+    int32_t n;
+    int32_t i[2 * kPassSensors], j[2 * kPassSensors], k[2 * kPassSensors];
+    T v[kPassSteps][2 * kPassSensors];
+};
+template <typename T> struct PassSensors<T, kForward> {};
+
 struct TileGeo {
     int xl, x0, x1, yl, y0, y1;   // first column held, own columns [x0, x1); first row held, own rows [y0, y1)
 };
@@ -543,6 +553,8 @@ template <typename T, typename D> struct PassBuf {
     D *wd;
     const CrackState *s_in;
     CrackState *s_out;
+    const int64_t *cnt_in;   // adjoint: the step counter
+    int64_t *cnt_out;
 };
 template <typename T> struct PassPads {
     T *w_out;
@@ -568,6 +580,9 @@ struct PassCtx {
     // end; the severed columns at the start
     bool known, ev_r, ev_l, own_r, own_l, follow;
     int org_r, org_l, f0, l0;
+    bool senses;                // a sensor of the tile's list lies on one of the thread's sites
+    bool on_edge;               // adjoint: the warp holds row 0 or ny - 1
+    int64_t n;                  // adjoint: the transposed step the pass starts with
 };
 
 // The fields of a thread: RPT rows of one vector.  Each update writes the
@@ -600,10 +615,49 @@ template <typename T, typename D, int RPT> struct PassRows {
     }
 };
 
+// Adjoint: the values of m next to the Dirichlet edges before step s, which a
+// reduction over all steps turns into the load gradient (summed here, in FP64,
+// they would cost the tiles along an edge as much as a step).
+template <typename T, typename D, int RPT, typename F>
+__device__ __forceinline__ void pass_edge_rows(const PassArgs<T, D> &A, const PassCtx &c, int s, F &&row)
+{
+    constexpr int N = Vec<T>::N;
+    const PassAdj<T> &d = A.adj;
+    const int64_t n = c.n - s;
+    if (n < 0 || n >= d.n_steps || !(c.on_edge || c.side)) return;
+    const StepArgs<T, D> &a = A.s;
+    T *at = d.edge_m + (n % d.edge_ring) * 4 * d.edge_len;
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) {
+        const int j = c.jb + r;
+        if (j < c.g.y0 || j >= c.g.y1) continue;
+        const Row<T, N> w = row(r);
+        if (c.on_edge) {
+#pragma unroll
+            for (int e = BOTTOM; e <= TOP; ++e) {
+                if (j != (e == BOTTOM ? 0 : a.ny - 1) || a.edge[e] != EDGE_DIRICHLET) continue;
+#pragma unroll
+                for (int k = 0; k < N; ++k) {
+                    int q = c.x0 + k;
+                    if (q < c.g.x0 || q >= c.g.x1) continue;
+                    if (c.per) q = wrap_col(q, a.nx);
+                    at[e * d.edge_len + q] = w.v[k];
+                }
+            }
+        }
+        if (c.is_l && a.edge[LEFT] == EDGE_DIRICHLET && c.g.x0 == 0) at[LEFT * d.edge_len + j] = w.v[0];
+        if (c.kr >= 0 && a.edge[RIGHT] == EDGE_DIRICHLET && c.g.x1 == a.nx) {
+#pragma unroll
+            for (int k = 0; k < N; ++k)
+                if (k == c.kr) at[RIGHT * d.edge_len + j] = w.v[k];
+        }
+    }
+}
+
 // One time step of a tile.
-template <typename T, typename D, int NW, int RPT, int KIND, int PH>
+template <typename T, typename D, int NW, int RPT, int KIND, int PH, int MODE>
 __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx &c, int s, PassRows<T, D, RPT> &F,
-                                          PassShared<T, NW> &sh, PassWindow &win)
+                                          PassShared<T, NW> &sh, PassSensors<T, MODE> &sen, PassWindow &win)
 {
     constexpr int N = Vec<T>::N;
     constexpr int kBelowWarp = NW / 2 - 1;   // strip: the warp whose last row is jc - 1; the next one's first is jc
@@ -618,10 +672,11 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
     stg_row(&sh.top[b][warp][lane * N], F.template cur<PH>(RPT - 1));
     stg_row(&sh.bot[b][warp][lane * N], F.template cur<PH>(0));
     const bool face = KIND == 2 && (warp == kBelowWarp || warp == kBelowWarp + 1), below = warp == kBelowWarp;
-    if (KIND == 2 && face) stg_row(&sh.pair[s][below ? 0 : 1][lane * N], F.template cur<PH>(below ? RPT - 1 : 0));
+    if (MODE == kAdjoint && KIND != 0) pass_edge_rows<T, D, RPT>(A, c, s, [&](int r) { return F.template cur<PH>(r); });
+    if (MODE != kAdjoint && KIND == 2 && face) stg_row(&sh.pair[s][below ? 0 : 1][lane * N], F.template cur<PH>(below ? RPT - 1 : 0));
 
     const bool dir_l = KIND != 0 && a.edge[LEFT] == EDGE_DIRICHLET, dir_r = KIND != 0 && a.edge[RIGHT] == EDGE_DIRICHLET;
-    const bool em = KIND != 0 && A.q.edge_macro != 0, em_side = em && c.side;
+    const bool em = MODE == kForward && KIND != 0 && A.q.edge_macro != 0, em_side = em && c.side;
     const bool last_r = KIND != 0 && c.kr == N - 1;
     T tl = (T)0, tr = (T)0;
     R first, last;                                         // the first and last rows before the update
@@ -697,7 +752,7 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
         }
     }
     __syncthreads();
-    if (KIND == 2 && c.follow) {
+    if (MODE != kAdjoint && KIND == 2 && c.follow) {
         const bool reach = sh.reach[b] != 0;
         if (warp == 0) {
             pass_crack_step<T, PassShared<T, NW>::W>(p, A.q, sh.top[b][kBelowWarp], sh.bot[b][kBelowWarp + 1], c.org_r,
@@ -715,18 +770,21 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
         if (c.has_t) upx = edge_image<T, N>(last, a.edge[TOP] == EDGE_DIRICHLET, sh.ws2[TOP][s]);
         if (c.has_b) dnx = edge_image<T, N>(first, a.edge[BOTTOM] == EDGE_DIRICHLET, sh.ws2[BOTTOM][s]);
     }
-    bool cut[N];
+    bool cut[N], cutp[N];   // cutp (adjoint): severed in the forward step before
 #pragma unroll
-    for (int k = 0; k < N; ++k) cut[k] = false;
+    for (int k = 0; k < N; ++k) cut[k] = cutp[k] = false;
     if (KIND == 2 && face) {
-        const int f = c.known ? sh.log[s + 1].f : (c.ev_l ? sh.S.i_first : c.f0);
-        const int l = c.known ? sh.log[s + 1].l : (c.ev_r ? sh.S.i_last : c.l0);
+        const int e = MODE == kAdjoint ? s : s + 1;
+        const int f = c.known ? sh.log[e].f : (c.ev_l ? sh.S.i_first : c.f0);
+        const int l = c.known ? sh.log[e].l : (c.ev_r ? sh.S.i_last : c.l0);
+        const int fp = MODE == kAdjoint ? sh.log[s + 1].f : 0, lp = MODE == kAdjoint ? sh.log[s + 1].l : -1;
         // a severed link sends the site's own value back
 #pragma unroll
         for (int k = 0; k < N; ++k) {
             int q = x0 + k;
             if (c.per) q = q < 0 ? q + nx : (q >= nx ? q - nx : q);
             cut[k] = q >= f && q <= l;
+            cutp[k] = q >= fp && q <= lp;
             upx.v[k] = cut[k] && below ? last.v[k] : upx.v[k];
             dnx.v[k] = cut[k] && !below ? first.v[k] : dnx.v[k];
         }
@@ -754,7 +812,51 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
             F.template next<PH>(r) = out;
         }
     }
-    if (KIND == 2 && p.macro && face) {
+    if constexpr (MODE == kAdjoint) {
+        // the sensor sources of the state this step belongs to
+        if (c.senses)
+            for (int e = 0; e < sen.n; ++e) {
+                const int r0 = sen.j[e] - jb, k0 = sen.i[e] - x0;
+                const T v = sen.v[s][e];
+#pragma unroll
+                for (int r = 0; r < RPT; ++r)
+#pragma unroll
+                    for (int k = 0; k < N; ++k)
+                        if (r == r0 && k == k0) {
+                            F.template rate<PH>(r).v[k] += v;
+                            F.template next<PH>(r).v[k] += dt * v;
+                        }
+            }
+        if (KIND == 2 && p.macro && face) {
+            // the transposed crack-face rule of the columns severed before
+            const T inv_dt = dt == (T)1 ? (T)1 : div_dt((T)1, dt);
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                const T mB = below ? F.template next<PH>(RPT - 1).v[k] : F.template next<PH>(0).v[k];
+                T &oT = F.template next<PH>(RPT - 1).v[k], &oT1 = F.template next<PH>(RPT - 2).v[k], &oT2 = F.template next<PH>(RPT - 3).v[k];
+                T &oB = F.template next<PH>(0).v[k], &oB1 = F.template next<PH>(1).v[k], &oB2 = F.template next<PH>(2).v[k];
+                T &aT = F.b[RPT - 1].v[k], &aT1 = F.b[RPT - 2].v[k], &aT2 = F.b[RPT - 3].v[k];
+                T &aB = F.b[0].v[k], &aB1 = F.b[1].v[k], &aB2 = F.b[2].v[k];
+                if (cutp[k] && below) {
+                    aT -= mB * inv_dt;
+                    oT = (T)0;
+                    aT1 += (T)1.5 * mB * inv_dt;
+                    oT1 += (T)1.5 * mB;
+                    aT2 -= (T)0.5 * mB * inv_dt;
+                    oT2 -= (T)0.5 * mB;
+                }
+                if (cutp[k] && !below) {
+                    aB -= mB * inv_dt;
+                    oB = (T)0;
+                    aB1 += (T)1.5 * mB * inv_dt;
+                    oB1 += (T)1.5 * mB;
+                    aB2 -= (T)0.5 * mB * inv_dt;
+                    oB2 -= (T)0.5 * mB;
+                }
+            }
+        }
+    }
+    if (MODE != kAdjoint && KIND == 2 && p.macro && face) {
         // the crack-face rule: w_B from the two new values further from the crack
         R wB, w0;
 #pragma unroll
@@ -777,7 +879,7 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
             oB = cut[k] && !below ? wB.v[k] : oB;
         }
     }
-    if (KIND != 0 && A.q.edge_macro) {
+    if (em) {
         // the macroscopic rule on the outer edges (the two levels of
         // edge_rule_at): the edge columns, the crack-face points on
         // them, then the bottom and top rows and the corners
@@ -901,13 +1003,100 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
             }
         }
     }
+    if constexpr (MODE == kRecord)
+        for (int e = 0; c.senses && e < sen.n; ++e) {
+            const int r0 = sen.j[e] - jb, k0 = sen.i[e] - x0;
+            if (r0 < 0 || r0 >= RPT || k0 < 0 || k0 >= N) continue;
+            T v = (T)0;
+#pragma unroll
+            for (int r = 0; r < RPT; ++r)
+#pragma unroll
+                for (int k = 0; k < N; ++k) v = r == r0 && k == k0 ? F.template next<PH>(r).v[k] : v;
+            sen.v[s][e] = v;
+        }
+}
+
+// The sensors of a tile, in ascending order (warp 0): recording, those among
+// its own sites; adjoint, those among all the sites it holds (a halo site's
+// source reaches the tile's own sites) and their sources at each step.
+template <typename T, typename D, int NW, int RPT, int MODE>
+__device__ __forceinline__ void pass_sensors(const PassArgs<T, D> &A, const PassBuf<T, D> &B, const TileGeo &g, int64_t n,
+                                             PassSensors<T, MODE> &sen)
+{
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int ns = MODE == kRecord ? A.rec.ns : A.adj.ns;
+    const int32_t *si = MODE == kRecord ? A.rec.s_i : A.adj.s_i, *sj = MODE == kRecord ? A.rec.s_j : A.adj.s_j;
+    const int nx = A.s.nx;
+    const int i0 = MODE == kRecord ? g.x0 : g.xl, i1 = MODE == kRecord ? g.x1 : g.x1 + A.q.hc;
+    const int j0 = MODE == kRecord ? g.y0 : g.yl, j1 = MODE == kRecord ? g.y1 : g.yl + NW * RPT;
+    const bool per = A.s.edge[LEFT] == EDGE_PERIODIC;
+    if (tid < 32) {
+        int cnt = 0;
+        for (int img = 0; img < (per ? 3 : 1); ++img) {   // (periodic sides: the columns' images too)
+            const int o = img == 0 ? 0 : (img == 1 ? -nx : nx);
+            for (int q0 = 0; q0 < ns; q0 += 32) {
+                const int q = q0 + lane;
+                int i = 0, j = -1;
+                if (q < ns) {
+                    i = si[q] + o;
+                    j = sj[q];
+                }
+                const bool mine = q < ns && j >= j0 && j < j1 && i >= i0 && i < i1;
+                const unsigned m = __ballot_sync(0xffffffffu, mine);
+                const int at = cnt + __popc(m & ((1u << lane) - 1u));
+                if (mine && at < 2 * kPassSensors) {
+                    sen.i[at] = i;
+                    sen.j[at] = j;
+                    sen.k[at] = q;
+                }
+                cnt += __popc(m);
+            }
+        }
+        __syncwarp();
+        cnt = min(cnt, 2 * kPassSensors);   // (with images; a tile of a narrow lattice holds at most two of a column)
+        if (lane == 0) sen.n = cnt;
+        if (MODE == kAdjoint) {
+            for (int q = lane; q < cnt * A.q.K; q += 32) {
+                const int e = q % cnt, s = q / cnt;
+                // step n - s adds the sources of state n - s (none before the first)
+                const int64_t t = n - s - 1;
+                sen.v[s][e] = t >= 0 ? (T)(2.0 * A.adj.resid[(t % A.adj.ring) * ns + sen.k[e]]) : (T)0;
+            }
+        }
+    }
+}
+
+// The misfits of a recording pass's states, and their squares added to the
+// loss step by step.
+template <typename T, typename D, int NW>
+__device__ __forceinline__ void pass_misfits(const PassArgs<T, D> &A, const PassBuf<T, D> &B, PassSensors<T, kRecord> &sen)
+{
+    __syncthreads();
+    const RecArgs &r = A.rec;
+    const int64_t t0 = __ldcg(&B.s_in->step) - *r.n0;
+    for (int e = threadIdx.x; e < sen.n; e += 32 * NW) {
+        const int k = sen.k[e];
+        double sum = r.acc_loss ? __ldcg(&r.loss[k]) : 0.0;
+        double tg[kPassSteps];
+#pragma unroll
+        for (int s = 0; s < kPassSteps; ++s) tg[s] = s < A.q.K && t0 + s < r.n_steps ? r.target[(t0 + s) * r.ns + k] : 0.0;
+#pragma unroll
+        for (int s = 0; s < kPassSteps; ++s) {
+            const int64_t t = t0 + s;
+            if (s >= A.q.K || t < 0 || t >= r.n_steps) continue;
+            const double res = (double)sen.v[s][e] - tg[s];
+            r.resid[(t % r.ring) * r.ns + k] = res;
+            sum += res * res;
+        }
+        if (r.acc_loss) __stcg(&r.loss[k], sum);
+    }
 }
 
 // A tile.  KIND: 0 one none of whose sites sees an edge or the crack, 1 with
 // outer edges, 2 a crack-strip tile (with edges where it meets them).
-template <typename T, typename D, int NW, int RPT, int KIND, bool COOP>
+template <typename T, typename D, int NW, int RPT, int KIND, bool COOP, int MODE>
 __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf<T, D> &B, const TileGeo g,
-                                          PassShared<T, NW> &sh)
+                                          PassShared<T, NW> &sh, PassSensors<T, MODE> &sen)
 {
     constexpr int N = Vec<T>::N;
     constexpr int W = PassShared<T, NW>::W;
@@ -973,7 +1162,19 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
     int64_t fit_tip = 0;
     PassPair fit_pair = {0, 0, 0};
     double fit_sf = 0.0;
-    if (KIND == 2) {
+    c.senses = false;
+    c.n = 0;
+    if (MODE == kAdjoint) {
+        c.n = __ldcg(B.cnt_in);
+        if (KIND == 2 && tid <= K) {
+            // the columns severed in forward step n - tid
+            const int64_t q = c.n - tid, qc = q < A.adj.n_steps ? q : A.adj.n_steps - 1;
+            sh.log[tid].f = q >= 0 ? A.adj.i_first[qc] : 1;
+            sh.log[tid].l = q >= 0 ? A.adj.i_last[qc] : 0;
+        }
+    }
+    if constexpr (MODE != kForward) pass_sensors<T, D, NW, RPT, MODE>(A, B, g, c.n, sen);
+    if (MODE != kAdjoint && KIND == 2) {
         c.known = p.mode != CRACK_KCRIT;
         c.f0 = sh.in.i_first;
         c.l0 = sh.in.i_last;
@@ -1037,7 +1238,8 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
             fit_sf = fit_pair.in ? pass_sf(p, fit_pair.d) : 0.0;
         }
     }
-    if (KIND != 0) {
+    if (MODE == kAdjoint && KIND != 0 && tid < 4 * (kPassSteps + 1)) sh.ws2[tid / (kPassSteps + 1)][tid % (kPassSteps + 1)] = (T)0;
+    if (MODE != kAdjoint && KIND != 0) {
         // w* of the Dirichlet edges this tile meets, in the arithmetic's
         // precision once (a conversion from FP64 costs a warp 64 cycles)
         if (tid < 4 * (kPassSteps + 1)) {
@@ -1060,7 +1262,14 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
     c.has_b = KIND != 0 && jb == 0;
     c.odd = KIND != 0 && ((jb < 0 && jb + RPT > 0) || (jb < ny && jb + RPT > ny) ||
                           __any_sync(kFull, c.kr >= 0 && c.kr < N - 1));
-    if (KIND != 0) __syncthreads();   // w* and the cuts of the pass
+    if (KIND != 0 || MODE != kForward) __syncthreads();   // w*, the cuts of the pass, the sensors
+    if constexpr (MODE != kForward) {
+        for (int e = 0; e < sen.n; ++e) {
+            const int r0 = sen.j[e] - jb, k0 = sen.i[e] - x0;
+            c.senses |= r0 >= 0 && r0 < RPT && k0 >= 0 && k0 < N;
+        }
+    }
+    c.on_edge = KIND != 0 && ((jb <= 0 && jb + RPT > 0) || (jb <= ny - 1 && jb + RPT > ny - 1));
     // bulk tiles: two steps an iteration (PassRows); an odd last step leaves
     // the rows where a step of phase 0 writes them.  The other tiles, whose
     // step is far longer code, take every step in phase 0 and move the rows
@@ -1068,12 +1277,12 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
     int s = 0;
     if (KIND == 0) {
         for (; s + 2 <= K; s += 2) {
-            pass_step<T, D, NW, RPT, KIND, 0>(A, c, s, F, sh, win);
-            pass_step<T, D, NW, RPT, KIND, 1>(A, c, s + 1, F, sh, win);
+            pass_step<T, D, NW, RPT, KIND, 0, MODE>(A, c, s, F, sh, sen, win);
+            pass_step<T, D, NW, RPT, KIND, 1, MODE>(A, c, s + 1, F, sh, sen, win);
         }
     }
     for (; s < K; ++s) {
-        pass_step<T, D, NW, RPT, KIND, 0>(A, c, s, F, sh, win);
+        pass_step<T, D, NW, RPT, KIND, 0, MODE>(A, c, s, F, sh, sen, win);
 #pragma unroll
         for (int q = 0; q < RPT; ++q) {
             const int r = RPT - 1 - q;
@@ -1129,7 +1338,8 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
     }
     if (__any_sync(kFull, !isfinite(acc)) && lane == 0) atomicOr(a.err, (uint32_t)ERR_NONFINITE);
 
-    if (KIND == 2 && (c.own_r || c.own_l)) {
+    if constexpr (MODE == kRecord) pass_misfits<T, D, NW>(A, B, sen);
+    if (MODE != kAdjoint && KIND == 2 && (c.own_r || c.own_l)) {
         __syncthreads();   // the last crack step
         // the records of the pass's crack steps, and the K fits their decisions
         // did not wait for.  A window of one spacing holds at most one pair, so
@@ -1203,6 +1413,14 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
                 if (lane == 0) record(warp, dir, Kf, np, r_min);
             }
         }
+        if (MODE == kRecord && tid < K) {
+            // the columns severed in each step, for the adjoint
+            const int64_t t = sh.in.step + tid - *A.rec.n0;
+            if (t >= 0 && t < A.rec.n_steps) {
+                if (c.own_r) A.rec.i_last[t] = sh.log[tid + 1].l;
+                if (c.own_l || (c.own_r && !p.two_tips)) A.rec.i_first[t] = sh.log[tid + 1].f;
+            }
+        }
         if (tid == 0) {
             CrackState *o = B.s_out;
             const PassTip &e = sh.log[K], &e1 = sh.log[K - 1];
@@ -1261,8 +1479,9 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
 }
 
 // Tile t of a pass.
-template <typename T, typename D, int NW, int RPT, bool COOP>
-__device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<T, D> &B, int t, PassShared<T, NW> &sh)
+template <typename T, typename D, int NW, int RPT, bool COOP, int MODE>
+__device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<T, D> &B, int t, PassShared<T, NW> &sh,
+                                         PassSensors<T, MODE> &sen)
 {
     constexpr int N = Vec<T>::N;
     const StepArgs<T, D> &a = A.s;
@@ -1276,7 +1495,9 @@ __device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<
             reinterpret_cast<uint32_t *>(&S)[k] = __ldcg(reinterpret_cast<const uint32_t *>(B.s_in) + k);
         __syncthreads();
     };
-    if (t == q.tiles - 1 && a.p.mode == CRACK_NONE) {
+    if (MODE == kAdjoint) {
+        if (t == q.tiles - 1 && tid == 0) __stcg(B.cnt_out, __ldcg(B.cnt_in) - q.K);
+    } else if (t == q.tiles - 1 && a.p.mode == CRACK_NONE) {
         // without a crack, the state only counts steps
         read_state(sh.in);
         if (tid == 0) {
@@ -1294,7 +1515,18 @@ __device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<
         B.s_out->wstar[tid] = a.edge[tid] == EDGE_DIRICHLET ? load_value(a.load[tid], n1, (double)a.p.dt) : 0.0;
     }
     TileGeo g;
-    if (t < q.ms) {
+    if (MODE == kAdjoint && t < q.ms) {
+        // the recorded cuts need no tips: columns as the bulk splits them
+        g.x0 = t * q.ps;
+        g.x1 = min(g.x0 + q.ps, nx);
+        g.xl = g.x0 == 0 && !per ? 0 : g.x0 - q.hc;
+        g.yl = a.p.jc - NW * kStripRpt / 2;
+        g.y0 = q.jb;
+        g.y1 = q.jt;
+        pass_tile<T, D, NW, kStripRpt, 2, COOP, MODE>(A, B, g, sh, sen);
+        return;
+    }
+    if (MODE != kAdjoint && t < q.ms) {
         read_state(sh.in);
         const int f = sh.in.i_first, l = sh.in.i_last;
         const int cr = tip_col_r(f, l, nx), cl = tip_col_l(f, l, nx);
@@ -1317,7 +1549,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<
         g.yl = a.p.jc - NW * kStripRpt / 2;
         g.y0 = q.jb;
         g.y1 = q.jt;
-        pass_tile<T, D, NW, kStripRpt, 2, COOP>(A, B, g, sh);
+        pass_tile<T, D, NW, kStripRpt, 2, COOP, MODE>(A, B, g, sh, sen);
         return;
     }
     t -= q.ms;
@@ -1334,30 +1566,32 @@ __device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<
     g.xl = g.x0 == 0 && !per ? 0 : g.x0 - q.hc;
     g.yl = g.y0 == 0 ? 0 : (g.y1 == ny ? ny - NW * RPT : g.y0 - q.K);
     const bool plain = g.x0 >= q.K && g.x1 + q.K <= nx && g.y0 >= q.K && g.y1 + q.K <= ny && g.xl >= 0;
-    if (plain) pass_tile<T, D, NW, RPT, 0, COOP>(A, B, g, sh);
-    else pass_tile<T, D, NW, RPT, 1, COOP>(A, B, g, sh);
+    if (plain) pass_tile<T, D, NW, RPT, 0, COOP, MODE>(A, B, g, sh, sen);
+    else pass_tile<T, D, NW, RPT, 1, COOP, MODE>(A, B, g, sh, sen);
 }
 
 // One pass, a CTA per tile.
-template <typename T, typename D, int NW, int RPT>
+template <typename T, typename D, int NW, int RPT, int MODE>
 __global__ void __launch_bounds__(32 * NW, 16 / NW) pass_kernel(const __grid_constant__ PassArgs<T, D> a)
 {
     __shared__ PassShared<T, NW> sh;
+    __shared__ PassSensors<T, MODE> sen;
     pdl_wait();
     pdl_trigger();
-    const PassBuf<T, D> B = {a.s.w_in, a.wd_in, a.s.w_out, a.s.wd, a.s.s_in, a.s.s_out};
-    pass_cta<T, D, NW, RPT, false>(a, B, blockIdx.x, sh);
+    const PassBuf<T, D> B = {a.s.w_in, a.wd_in, a.s.w_out, a.s.wd, a.s.s_in, a.s.s_out, a.adj.cnt_in, a.adj.cnt_out};
+    pass_cta<T, D, NW, RPT, false, MODE>(a, B, blockIdx.x, sh, sen);
 }
 
 // n_pass passes, alternating between the two buffer sets, as one cooperative
 // launch (every tile resident at once) with a grid barrier between passes: on
 // lattices of a few hundred tiles a pass takes hardly longer than the launch
 // gap, the ramp and the instruction fetches of a cold start.
-template <typename T, typename D, int NW, int RPT>
+template <typename T, typename D, int NW, int RPT, int MODE>
 __global__ void __launch_bounds__(32 * NW, 16 / NW)
     pass_run_kernel(const __grid_constant__ PassArgs<T, D> a, int n_pass)
 {
     __shared__ PassShared<T, NW> sh;
+    __shared__ PassSensors<T, MODE> sen;
     for (int it = 0; it < n_pass; ++it) {
         const bool odd = (it & 1) != 0;
         PassBuf<T, D> B;
@@ -1367,26 +1601,28 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW)
         B.wd = odd ? a.wd1 : a.s.wd;
         B.s_in = odd ? a.s.s_out : a.s.s_in;
         B.s_out = odd ? const_cast<CrackState *>(a.s.s_in) : a.s.s_out;
-        pass_cta<T, D, NW, RPT, true>(a, B, blockIdx.x, sh);
+        B.cnt_in = odd ? a.adj.cnt_out : a.adj.cnt_in;
+        B.cnt_out = odd ? const_cast<int64_t *>(a.adj.cnt_in) : a.adj.cnt_out;
+        pass_cta<T, D, NW, RPT, true, MODE>(a, B, blockIdx.x, sh, sen);
         if (it + 1 < n_pass && !grid_barrier(a.bar, gridDim.x, a.budget, a.s.err)) return;
     }
 }
 
-template <typename T, typename D> const void *pass_kernel_ptr(int nw, int rpt, bool run)
+template <typename T, typename D, int MODE> const void *pass_kernel_ptr(int nw, int rpt, bool run)
 {
     if constexpr (sizeof(T) == 8)
         if (nw == 4)
-            return run ? reinterpret_cast<const void *>(&pass_run_kernel<T, D, 4, 4>)
-                       : reinterpret_cast<const void *>(&pass_kernel<T, D, 4, 4>);
+            return run ? reinterpret_cast<const void *>(&pass_run_kernel<T, D, 4, 4, MODE>)
+                       : reinterpret_cast<const void *>(&pass_kernel<T, D, 4, 4, MODE>);
     if constexpr (sizeof(T) == 4)
         if (rpt == 4)
-            return run ? reinterpret_cast<const void *>(&pass_run_kernel<T, D, 8, 4>)
-                       : reinterpret_cast<const void *>(&pass_kernel<T, D, 8, 4>);
-    return run ? reinterpret_cast<const void *>(&pass_run_kernel<T, D, 8, 8>)
-               : reinterpret_cast<const void *>(&pass_kernel<T, D, 8, 8>);
+            return run ? reinterpret_cast<const void *>(&pass_run_kernel<T, D, 8, 4, MODE>)
+                       : reinterpret_cast<const void *>(&pass_kernel<T, D, 8, 4, MODE>);
+    return run ? reinterpret_cast<const void *>(&pass_run_kernel<T, D, 8, 8, MODE>)
+               : reinterpret_cast<const void *>(&pass_kernel<T, D, 8, 8, MODE>);
 }
 
-template <typename T, typename D> cudaError_t launch_pass(const PassArgs<T, D> &a, int n_pass, cudaStream_t s)
+template <typename T, typename D, int MODE> cudaError_t launch_pass(const PassArgs<T, D> &a, int n_pass, cudaStream_t s)
 {
     const bool run = n_pass > 1;
     cudaLaunchConfig_t cfg = {};
@@ -1404,7 +1640,7 @@ template <typename T, typename D> cudaError_t launch_pass(const PassArgs<T, D> &
     cfg.attrs = attr;
     cfg.numAttrs = run || a.s.chained ? 1 : 0;
     void *args[] = {(void *)&a, (void *)&n_pass};   // one pass: the first argument only
-    return cudaLaunchKernelExC(&cfg, pass_kernel_ptr<T, D>(a.q.nw, a.q.rpt, run), args);
+    return cudaLaunchKernelExC(&cfg, pass_kernel_ptr<T, D, MODE>(a.q.nw, a.q.rpt, run), args);
 }
 
 }  // namespace lbm

@@ -3,11 +3,11 @@
 
 namespace lbm {
 
-template const void *pass_kernel_ptr<double, double>(int, int, bool);
-template cudaError_t launch_pass<double, double>(const PassArgs<double, double> &, int, cudaStream_t);
-template const void *pass_kernel_ptr<float, __nv_bfloat16>(int, int, bool);
-template cudaError_t launch_pass<float, __nv_bfloat16>(const PassArgs<float, __nv_bfloat16> &, int, cudaStream_t);
-template const void *pass_kernel_ptr<float, __half>(int, int, bool);
-template cudaError_t launch_pass<float, __half>(const PassArgs<float, __half> &, int, cudaStream_t);
+template const void *pass_kernel_ptr<double, double, kForward>(int, int, bool);
+template cudaError_t launch_pass<double, double, kForward>(const PassArgs<double, double> &, int, cudaStream_t);
+template const void *pass_kernel_ptr<float, __nv_bfloat16, kForward>(int, int, bool);
+template cudaError_t launch_pass<float, __nv_bfloat16, kForward>(const PassArgs<float, __nv_bfloat16> &, int, cudaStream_t);
+template const void *pass_kernel_ptr<float, __half, kForward>(int, int, bool);
+template cudaError_t launch_pass<float, __half, kForward>(const PassArgs<float, __half> &, int, cudaStream_t);
 
 }  // namespace lbm

@@ -38,7 +38,7 @@ void split_rows(int len, int H, int K, bool edge0, bool edge1, int least, int &m
 
 }  // namespace
 
-bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q)
+bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q, bool adjoint)
 {
     const int nx = h->grid.nx, ny = h->grid.ny;
     const int N = (int)(16 / h->esize), W = 32 * N, H = nw * rpt;
@@ -47,6 +47,7 @@ bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q)
     const bool crack = h->cp.mode != CRACK_NONE;
     const CrackParams &p = h->cp;
     if (K < 2 || K > nw || 2 * K > strip_half) return false;
+    if (per && nx < 16) return false;   // a halo holds at most one image of a column
     if (crack && p.hist_cap > 0 && p.hist_cap < K) return false;   // a pass's records go around the ring once at most
     std::memset(&q, 0, sizeof q);
     q.K = K;
@@ -70,6 +71,8 @@ bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q)
 
     // rows: the crack strip, and the bulk below and above it (all of it without a crack)
     const int so = strip_half - K;
+    // the transposed crack-face rule reaches two rows further from the crack
+    if (adjoint && crack && p.macro && so < K + 2) return false;
     int region0 = 0, region1 = ny;
     if (crack) {
         region0 = std::max(0, p.jc - so);
@@ -86,7 +89,10 @@ bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q)
     if (h->edge_macro && (crack ? p.jc < strip_half + 3 || ny - p.jc < strip_half + 3 : ny < 64)) return false;
     if (h->edge_macro && nx < 4) return false;
 
-    if (crack) {
+    if (crack && adjoint) {
+        q.ms = q.mx;
+        q.ps = q.px;
+    } else if (crack) {
         // columns an end can cut in a pass, and the reach of its K window
         const int64_t dq = p.mode == CRACK_KCRIT ? p.dq_max : p.mode == CRACK_PRESCRIBED ? p.dq_prescribed : 0;
         q.grow = (int)((dq * K) >> kQBits) + 2;
@@ -152,7 +158,9 @@ void choose_pass(lbm_handle *h)
         h->pass_rpt = h->pass_nw == 4 ? 4 : 8;
         if (!pass_plan(h, K, h->pass_nw, h->pass_rpt, q)) continue;
         if (h->esize == 4 && q.tiles < 2 * h->sms) h->pass_rpt = 4;
-        if (!pass_plan(h, K, h->pass_nw, h->pass_rpt, q)) continue;
+        bool shorter = true;   // every shorter pass too: a call's last passes
+        for (int k = K; k >= 2; --k) shorter = shorter && pass_plan(h, k, h->pass_nw, h->pass_rpt, q);
+        if (!shorter) continue;
         const void *fn = h->lat.storage == LBM_F64           ? pass_kernel_ptr<double, double>(h->pass_nw, h->pass_rpt, true)
                          : h->lat.storage == LBM_F32_WD_BF16 ? pass_kernel_ptr<float, __nv_bfloat16>(h->pass_nw, h->pass_rpt, true)
                          : h->lat.storage == LBM_F32_WD_F16  ? pass_kernel_ptr<float, __half>(h->pass_nw, h->pass_rpt, true)

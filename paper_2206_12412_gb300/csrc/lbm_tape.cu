@@ -27,7 +27,7 @@ struct lbm_tape {
     int32_t every;        // snapshot interval (0: keep the misfits of all steps)
     int64_t ring;         // rows of the misfit buffer
     int64_t n_ckpt;
-    int32_t slots;        // partial sums per (step, edge)
+    int32_t slots;        // bands and column blocks of the handle's steps when the tape was created
     int32_t units_cap;
     lbm_allocator alloc;
     bool custom_alloc;
@@ -35,7 +35,10 @@ struct lbm_tape {
     size_t block_bytes;
     // device memory
     int32_t *s_i, *s_j, *s_off, *s_ent;
-    double *target, *resid, *loss_acc, *loss, *part, *grad;
+    double *target, *resid, *loss_acc, *loss, *grad;
+    void *edge_m;         // values of m next to the Dirichlet edges, edge_ring steps of them
+    int64_t edge_ring, edge_len;
+    int64_t edge_hi, edge_count;   // steps edge_hi - edge_count + 1 .. edge_hi are in it, not yet summed
     int32_t *i_first, *i_last;
     int64_t *n0, *cnt;
     void *m[2], *a;       // adjoint planes, element (0, 0)
@@ -53,6 +56,9 @@ struct lbm_tape {
     ChunkGraph g_rec[2];  // recording steps without / with loss accumulation
     ChunkGraph g_adj;
     cudaStream_t cap;
+    // passes of several steps (lbm_pass.cuh): the sweep's (0: single steps)
+    int32_t adj_k, adj_nw, adj_rpt;
+    int32_t rec_slots, adj_slots;   // tiles resident at once
 };
 
 namespace {
@@ -110,10 +116,84 @@ void make_adj_args(const lbm_tape *t, int par, AdjArgs<T> &a)
     a.s_i = t->s_i;
     a.s_j = t->s_j;
     a.resid = t->resid;
-    a.part = t->part;
+    a.edge_m = static_cast<T *>(t->edge_m);
+    a.edge_ring = t->edge_ring;
+    a.edge_len = t->edge_len;
     a.err = h->err;
-    a.slots = t->slots;
-    a.pad = 0;
+}
+
+// n_pass recording passes (one, or an even number in one launch); second:
+// the second pass of a pair.
+template <typename T>
+cudaError_t enqueue_record(const lbm_tape *t, const PassPlan &q, int par, bool second, int n_pass, int acc_loss)
+{
+    const lbm_handle *h = t->h;
+    PassArgs<T, T> a;
+    make_pass_args(h, par, second, q, a);
+    a.rec = rec_args(t, acc_loss);
+    return launch_pass<T, T, kRecord>(a, n_pass, h->stream);
+}
+
+// n_pass passes of transposed steps from adjoint parity par; a ping-pongs
+// with the handle's scratch plane (free between the handle's own passes).
+template <typename T>
+cudaError_t enqueue_sweep(const lbm_tape *t, const PassPlan &q, int par, bool second, int n_pass)
+{
+    const lbm_handle *h = t->h;
+    PassArgs<T, T> a;
+    make_pass_args(h, 0, second, q, a);
+    a.s.w_in = static_cast<const T *>(t->m[par]);
+    a.s.w_out = static_cast<T *>(t->m[par ^ 1]);
+    a.wd_in = static_cast<const T *>(second ? h->alt[0] : t->a);
+    a.s.wd = static_cast<T *>(second ? t->a : h->alt[0]);
+    a.w_in1 = a.s.w_out;
+    a.wd_in1 = a.s.wd;
+    a.w_out1 = const_cast<T *>(a.s.w_in);
+    a.wd1 = const_cast<T *>(a.wd_in);
+    PassAdj<T> &d = a.adj;
+    d.i_first = t->i_first;
+    d.i_last = t->i_last;
+    d.cnt_in = t->cnt + par;
+    d.cnt_out = t->cnt + (par ^ 1);
+    d.n_steps = t->T;
+    d.ring = t->ring;
+    d.edge_ring = t->edge_ring;
+    d.edge_len = t->edge_len;
+    d.s_i = t->s_i;
+    d.s_j = t->s_j;
+    d.resid = t->resid;
+    d.edge_m = static_cast<T *>(t->edge_m);
+    d.ns = t->ns;
+    return launch_pass<T, T, kAdjoint>(a, n_pass, h->stream);
+}
+
+// n steps in passes of at most kmax, what is left (n < 4) in n: plan(K, q)
+// gives the tiles, enq(q, par, second, m) launches.
+template <typename Pl, typename E>
+lbm_status tape_passes(int64_t &n, int kmax, int par, int slots, Pl &&plan, E &&enq)
+{
+    auto go = [&](int K, int64_t m) -> lbm_status {
+        PassPlan q;
+        if (!plan(K, q)) return fail(LBM_ERR_ARG, "no plan of a pass");
+        if (q.tiles <= slots) {
+            constexpr int64_t kMost = 1 << 16;
+            for (; m > 0; m -= std::min(m, kMost)) LBM_CUDA(enq(q, par, false, (int)std::min(m, kMost)));
+            return LBM_OK;
+        }
+        for (; m > 0; m -= 2) {
+            LBM_CUDA(enq(q, par, false, 1));
+            LBM_CUDA(enq(q, par ^ 1, true, 1));
+        }
+        return LBM_OK;
+    };
+    auto pair = [&](int Ka, int Kb) -> lbm_status {
+        PassPlan qa, qb;
+        if (!plan(Ka, qa) || !plan(Kb, qb)) return fail(LBM_ERR_ARG, "no plan of a pass");
+        LBM_CUDA(enq(qa, par, false, 1));
+        LBM_CUDA(enq(qb, par ^ 1, true, 1));
+        return LBM_OK;
+    };
+    return split_passes(n, kmax, go, pair);
 }
 
 // n recording steps of the handle from its current parity.
@@ -122,7 +202,17 @@ lbm_status record_steps(lbm_tape *t, int64_t n, int acc_loss)
     lbm_handle *h = t->h;
     const RecArgs r = rec_args(t, acc_loss);
     int par = h->parity;
-    lbm_status rc;
+    lbm_status rc = LBM_OK;
+    if (n > 0 && h->cp.mode != CRACK_NONE) h->pending = true;
+    if (h->pass_k && !h->own_bands && !h->bulk && t->ns <= kPassSensors) {
+        rc = tape_passes(
+            n, h->pass_k, par, t->rec_slots, [&](int K, PassPlan &q) { return pass_plan(h, K, h->pass_nw, h->pass_rpt, q); },
+            [&](const PassPlan &q, int p, bool second, int m) {
+                return h->esize == 8 ? enqueue_record<double>(t, q, p, second, m, acc_loss)
+                                     : enqueue_record<float>(t, q, p, second, m, acc_loss);
+            });
+        if (rc != LBM_OK) return rc;
+    }
     if (h->esize == 8) {
         rc = run_chunks(t->g_rec[acc_loss], h->gen, h->stream, t->cap, n, par, [&](int p, cudaStream_t s) {
             StepArgs<double, double> a;
@@ -139,25 +229,96 @@ lbm_status record_steps(lbm_tape *t, int64_t n, int acc_loss)
         });
     }
     h->parity = par;
-    if (n > 0 && h->cp.mode != CRACK_NONE) h->pending = true;
     return rc;
 }
 
-// n transposed steps from adjoint parity *apar.
+// Sum the load gradient of the steps whose edge values are kept.
+lbm_status sum_edges(lbm_tape *t)
+{
+    lbm_handle *h = t->h;
+    const int64_t lo = std::max<int64_t>(0, t->edge_hi - t->edge_count + 1), hi = std::min<int64_t>(t->edge_hi, t->T - 1);
+    int dir_mask = 0;
+    for (int e = 0; e < 4; ++e)
+        if (h->grid.edge[e] == LBM_EDGE_DIRICHLET) dir_mask |= 1 << e;
+    if (h->esize == 8)
+        LBM_CUDA(launch_grad_sum<double>(static_cast<const double *>(t->edge_m), t->edge_ring, t->edge_len, lo, hi - lo + 1, t->T,
+                                         h->grid.nx, h->grid.ny, dir_mask, h->g, t->grad, h->stream));
+    else
+        LBM_CUDA(launch_grad_sum<float>(static_cast<const float *>(t->edge_m), t->edge_ring, t->edge_len, lo, hi - lo + 1, t->T,
+                                        h->grid.nx, h->grid.ny, dir_mask, h->g, t->grad, h->stream));
+    t->edge_hi -= t->edge_count;
+    t->edge_count = 0;
+    return LBM_OK;
+}
+
+// n transposed steps from adjoint parity apar.
 lbm_status adjoint_steps(lbm_tape *t, int64_t n, int &apar)
 {
     lbm_handle *h = t->h;
-    if (h->esize == 8)
-        return run_chunks(t->g_adj, h->gen, h->stream, t->cap, n, apar, [&](int p, cudaStream_t s) {
-            AdjArgs<double> a;
-            make_adj_args(t, p, a);
-            return launch_adjoint<double>(a, h->n_bands, s);
-        });
-    return run_chunks(t->g_adj, h->gen, h->stream, t->cap, n, apar, [&](int p, cudaStream_t s) {
-        AdjArgs<float> a;
-        make_adj_args(t, p, a);
-        return launch_adjoint<float>(a, h->n_bands, s);
-    });
+    while (n > 0) {
+        int64_t c = std::min(n, t->edge_ring);
+        n -= c;
+        if (t->edge_count + c > t->edge_ring) {
+            const lbm_status rs = sum_edges(t);
+            if (rs != LBM_OK) return rs;
+        }
+        t->edge_count += c;
+        lbm_status rc = LBM_OK;
+        if (t->adj_k && !h->own_bands && !h->bulk) {
+            rc = tape_passes(
+                c, t->adj_k, apar, t->adj_slots,
+                [&](int K, PassPlan &q) { return pass_plan(h, K, t->adj_nw, t->adj_rpt, q, true); },
+                [&](const PassPlan &q, int p, bool second, int m) {
+                    return h->esize == 8 ? enqueue_sweep<double>(t, q, p, second, m) : enqueue_sweep<float>(t, q, p, second, m);
+                });
+            if (rc != LBM_OK) return rc;
+        }
+        if (h->esize == 8)
+            rc = run_chunks(t->g_adj, h->gen, h->stream, t->cap, c, apar, [&](int p, cudaStream_t s) {
+                AdjArgs<double> a;
+                make_adj_args(t, p, a);
+                return launch_adjoint<double>(a, h->n_bands, s);
+            });
+        else
+            rc = run_chunks(t->g_adj, h->gen, h->stream, t->cap, c, apar, [&](int p, cudaStream_t s) {
+                AdjArgs<float> a;
+                make_adj_args(t, p, a);
+                return launch_adjoint<float>(a, h->n_bands, s);
+            });
+        if (rc != LBM_OK) return rc;
+    }
+    return LBM_OK;
+}
+
+// The passes of the sweep: as the handle's, up to two rows shorter with the
+// transposed crack-face rule.
+void choose_sweep(lbm_tape *t)
+{
+    lbm_handle *h = t->h;
+    t->adj_k = 0;
+    t->rec_slots = t->adj_slots = 0;
+    if (!h->pass_k) return;
+    t->adj_nw = h->pass_nw;
+    auto slots = [&](const void *fn) {
+        int n = 0;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, 32 * h->pass_nw, 0) == cudaSuccess ? n * h->sms : 0;
+    };
+    t->rec_slots = slots(h->esize == 8 ? pass_kernel_ptr<double, double, kRecord>(h->pass_nw, h->pass_rpt, true)
+                                       : pass_kernel_ptr<float, float, kRecord>(h->pass_nw, h->pass_rpt, true));
+    if (t->ns > kPassSensors) return;
+    for (int K = h->pass_k; K >= 2; --K) {
+        PassPlan q;
+        t->adj_rpt = h->pass_nw == 4 ? 4 : 8;
+        if (!pass_plan(h, K, t->adj_nw, t->adj_rpt, q, true)) continue;
+        if (h->esize == 4 && q.tiles < 2 * h->sms) t->adj_rpt = 4;
+        bool shorter = true;
+        for (int k = K; k >= 2; --k) shorter = shorter && pass_plan(h, k, t->adj_nw, t->adj_rpt, q, true);
+        if (!shorter) continue;
+        t->adj_k = K;
+        break;
+    }
+    t->adj_slots = slots(h->esize == 8 ? pass_kernel_ptr<double, double, kAdjoint>(t->adj_nw, t->adj_rpt, true)
+                                       : pass_kernel_ptr<float, float, kAdjoint>(t->adj_nw, t->adj_rpt, true));
 }
 
 // Copy the handle's state (fields of the current parity with their pads,
@@ -273,6 +434,12 @@ lbm_status lbm_tape_create(lbm_handle *h, const int32_t *sensors, int32_t n_sens
     t->sens.assign(sensors, sensors + 2 * (size_t)n_sens);
     t->ck_pending.assign((size_t)t->n_ckpt, 0);
 
+    choose_sweep(t);
+    // about 500 steps of edge values between two sums, whole passes of them
+    t->edge_ring = std::min<int64_t>(n_steps + 1, t->adj_k ? 2 * t->adj_k * (512 / (2 * t->adj_k)) : 512);
+    t->edge_len = (std::max(nx, ny) + 3) / 4 * 4;
+    t->edge_hi = n_steps;
+    t->edge_count = 0;
     const size_t ns = (size_t)n_sens, T = (size_t)n_steps;
     const size_t dense = 2 * (size_t)nx * ny * h->esize;
     t->ck_w = 0;
@@ -289,7 +456,7 @@ lbm_status lbm_tape_create(lbm_handle *h, const int32_t *sensors, int32_t n_sens
     const size_t o_rs = off; off = align256(off + (size_t)t->ring * ns * 8);
     const size_t o_la = off; off = align256(off + ns * 8);
     const size_t o_lo = off; off = align256(off + 8);
-    const size_t o_pt = off; off = align256(off + T * 4 * (size_t)t->slots * 8);
+    const size_t o_ed = off; off = align256(off + (size_t)t->edge_ring * 4 * (size_t)t->edge_len * h->esize);
     const size_t o_gr = off; off = align256(off + 4 * T * 8);
     const size_t o_if = off; off = align256(off + T * 4);
     const size_t o_il = off; off = align256(off + T * 4);
@@ -316,7 +483,7 @@ lbm_status lbm_tape_create(lbm_handle *h, const int32_t *sensors, int32_t n_sens
     t->resid = reinterpret_cast<double *>(b + o_rs);
     t->loss_acc = reinterpret_cast<double *>(b + o_la);
     t->loss = reinterpret_cast<double *>(b + o_lo);
-    t->part = reinterpret_cast<double *>(b + o_pt);
+    t->edge_m = b + o_ed;
     t->grad = reinterpret_cast<double *>(b + o_gr);
     t->i_first = reinterpret_cast<int32_t *>(b + o_if);
     t->i_last = reinterpret_cast<int32_t *>(b + o_il);
@@ -415,7 +582,8 @@ lbm_status lbm_tape_backward(lbm_tape *t, double *dL_dload, int32_t load_on_devi
     if ((dL_dw0 || dL_dwdot0) && dtype != (h->esize == 8 ? LBM_F64 : LBM_F32))
         return fail(LBM_ERR_ARG, "dtype must be LBM_F64 for F64 storage, LBM_F32 for F32");
     cudaStream_t s = h->stream;
-    LBM_CUDA(cudaMemsetAsync(t->part, 0, (size_t)t->T * 4 * (size_t)t->slots * 8, s));
+    t->edge_hi = t->T;
+    t->edge_count = 0;
     LBM_CUDA(cudaMemsetAsync(t->mbase[0], 0, h->plane_bytes, s));
     LBM_CUDA(cudaMemsetAsync(t->mbase[1], 0, h->plane_bytes, s));
     LBM_CUDA(cudaMemsetAsync(t->abase, 0, h->plane_bytes, s));
@@ -436,10 +604,7 @@ lbm_status lbm_tape_backward(lbm_tape *t, double *dL_dload, int32_t load_on_devi
         if ((rc = adjoint_steps(t, 1, apar)) != LBM_OK) return rc;   // transposed step 0
         if ((rc = snapshot(t, nseg, false)) != LBM_OK) return rc;    // back to the end of the run
     }
-    int dir_mask = 0;
-    for (int e = 0; e < 4; ++e)
-        if (h->grid.edge[e] == LBM_EDGE_DIRICHLET) dir_mask |= 1 << e;
-    LBM_CUDA(launch_grad_sum(t->part, t->T, t->slots, dir_mask, h->g, t->grad, s));
+    if ((rc = sum_edges(t)) != LBM_OK) return rc;
     const int nx = h->grid.nx, ny = h->grid.ny;
     const size_t nf = (size_t)nx * ny;
     if (dL_dw0 || dL_dwdot0) {

@@ -106,3 +106,32 @@ def test_passes_equal_single_steps(gpu, name, p, storage, n):
         for k in a:
             np.testing.assert_array_equal(a[k], b[k], err_msg=k)
     assert st == st1
+
+
+TAPES = ["macro_growth", "bb_growth", "bb_periodic", "all_dirichlet", "scaled_units", "no_crack", "wide_macro", "wide_bb"]
+
+
+@pytest.mark.parametrize("storage", ["f32", "f64"])
+@pytest.mark.parametrize("every", [0, 13])
+@pytest.mark.parametrize("kind", TAPES)
+def test_tape_passes_equal_single_steps(gpu, kind, every, storage):
+    """The recording and the sweep in passes against single steps (a launch
+    shape of the user's own keeps a lattice to those): the same losses and
+    gradients, bit for bit (the load gradient's sum does not depend on the
+    route)."""
+    lbm = gpu
+    T = 59
+    p, loaded, w0, wd0, sens, tgt = W.adjoint_case(kind, T, seed=5, ns=23)
+    got = []
+    for rows in (0, 7):
+        lat = lbm.Lattice(p, storage)
+        lat.set_launch(rows)
+        lat.set_fields(w0, wd0)
+        tape = lbm.Tape(lat, sens, T, checkpoint_every=every)
+        loss = tape.forward(tgt)
+        mis = tape.misfits() if every == 0 else np.zeros(1)
+        got.append((loss, mis, *tape.backward(device=False), *lat.fields(), lat.history(T)["K"]))
+        tape.close()
+        lat.close()
+    for a, b in zip(*got):
+        np.testing.assert_array_equal(a, b)
