@@ -2039,6 +2039,14 @@ struct lbm_batch {
     cudaStream_t stream;
     cudaStream_t cap_stream;
     ChunkGraph graph;    // graphs of runs of batched steps
+    // passes of several steps (lbm_pass.cuh) of 8, 4 and 2 steps: descriptors
+    // (four per lattice: parity + 2 second) and tiles, in an allocation of their own
+    static constexpr int kPassKinds = 3;
+    void *pblock;        // null: single steps only
+    void *pdescs[kPassKinds];
+    BatchUnit *punits[kPassKinds];
+    int n_punits[kPassKinds];
+    bool own_shape;      // lbm_batch_set_shape or _lookahead chose the shape of the single steps: no passes
     bool owns;           // made by lbm_create_batch: the member handles are destroyed with the batch
 };
 
@@ -2495,6 +2503,85 @@ lbm_status batch_build(lbm_batch *b, int threads, int rows, int la)
     return LBM_OK;
 }
 
+constexpr int kBatchPassSteps[lbm_batch::kPassKinds] = {8, 4, 2};
+
+// The batch's passes, if every lattice takes them (FP32 arithmetic; their
+// scratch planes exist and the tiles can follow their cracks).  The tables do
+// not depend on the shape of the single steps.
+template <typename T, typename D>
+lbm_status batch_build_passes(lbm_batch *b)
+{
+    const size_t n = b->hs.size(), desc_bytes = align256(4 * n * sizeof(lbm::PassArgs<T, D>));
+    std::vector<std::vector<BatchUnit>> units(lbm_batch::kPassKinds);
+    std::vector<std::vector<lbm::PassPlan>> plans(lbm_batch::kPassKinds);
+    size_t need = 0;
+    for (int k = 0; k < lbm_batch::kPassKinds; ++k) {
+        for (const lbm_handle *h : b->hs) {
+            lbm::PassPlan q;
+            if (!h->alt[0] || !pass_plan(h, kBatchPassSteps[k], 8, 8, q)) return LBM_OK;
+            plans[k].push_back(q);
+        }
+        for (int strip = 1; strip >= 0; --strip)
+            for (size_t i = 0; i < n; ++i) {
+                const lbm::PassPlan &q = plans[k][i];
+                for (int u = strip ? 0 : q.ms; u < (strip ? q.ms : q.tiles); ++u) units[k].push_back(BatchUnit{(int32_t)i, u, 0, 0});
+            }
+        need += desc_bytes + align256(units[k].size() * sizeof(BatchUnit));
+    }
+    char *block = static_cast<char *>(batch_alloc(b, need));
+    if (!block) return LBM_OK;   // no room: single steps
+    std::vector<char> host(need);
+    size_t off = 0;
+    for (int k = 0; k < lbm_batch::kPassKinds; ++k) {
+        auto *d = reinterpret_cast<lbm::PassArgs<T, D> *>(host.data() + off);
+        for (size_t i = 0; i < n; ++i)
+            for (int which = 0; which < 4; ++which) {
+                std::memset((void *)&d[4 * i + which], 0, sizeof d[0]);
+                make_pass_args(b->hs[i], which & 1, which >= 2, plans[k][i], d[4 * i + which]);
+            }
+        b->pdescs[k] = block + off;
+        off += desc_bytes;
+        std::memcpy(host.data() + off, units[k].data(), units[k].size() * sizeof(BatchUnit));
+        b->punits[k] = reinterpret_cast<BatchUnit *>(block + off);
+        b->n_punits[k] = (int)units[k].size();
+        off += align256(units[k].size() * sizeof(BatchUnit));
+    }
+    b->pblock = block;
+    cudaError_t e = cudaMemcpyAsync(block, host.data(), need, cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);   // the host tables go out of scope
+    return e == cudaSuccess ? LBM_OK : cuda_fail(e, "uploading the batch's passes");
+}
+
+lbm_status batch_build_passes(lbm_batch *b)
+{
+    if (b->q != 5 || b->line) return LBM_OK;
+    switch (b->storage) {
+    case LBM_F32: return batch_build_passes<float, float>(b);
+    case LBM_F32_WD_BF16: return batch_build_passes<float, __nv_bfloat16>(b);
+    case LBM_F32_WD_F16: return batch_build_passes<float, __half>(b);
+    case LBM_F32_LEAPFROG: return batch_build_passes<float, Lf>(b);
+    default: return LBM_OK;
+    }
+}
+
+template <typename T, typename D>
+cudaError_t enqueue_batch_pass_t(const lbm_batch *b, int k, int which, cudaStream_t s)
+{
+    return launch_pass_batch(static_cast<const lbm::PassArgs<T, D> *>(b->pdescs[k]), b->punits[k], b->n_punits[k], which, s);
+}
+
+// One pass of kBatchPassSteps[k] steps of every lattice.
+cudaError_t enqueue_batch_pass(const lbm_batch *b, int k, int par, bool second, cudaStream_t s)
+{
+    const int which = par + (second ? 2 : 0);
+    switch (b->storage) {
+    case LBM_F32: return enqueue_batch_pass_t<float, float>(b, k, which, s);
+    case LBM_F32_WD_BF16: return enqueue_batch_pass_t<float, __nv_bfloat16>(b, k, which, s);
+    case LBM_F32_WD_F16: return enqueue_batch_pass_t<float, __half>(b, k, which, s);
+    default: return enqueue_batch_pass_t<float, Lf>(b, k, which, s);
+    }
+}
+
 // Shapes chosen by lbm_batch_tune in this process, keyed by the device's SM
 // count, the storage and the lattices' sizes and crack bands.
 std::mutex g_tune_mu;
@@ -2596,8 +2683,11 @@ lbm_status lbm_batch_create(lbm_handle *const *handles, int32_t n, int32_t band_
     b->custom_alloc = allocator && allocator->alloc && allocator->release;
     if (b->custom_alloc) b->alloc = *allocator;
     b->owns = false;
+    b->pblock = nullptr;
+    b->own_shape = false;
     auto bail = [&](lbm_status rc) {
         batch_release_block(b);
+        batch_free(b, b->pblock);
         batch_free(b, b->bar);
         if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
         delete b;
@@ -2618,6 +2708,8 @@ lbm_status lbm_batch_create(lbm_handle *const *handles, int32_t n, int32_t band_
     // many CTAs, no need to fit one wave; lbm_batch_tune picks a better shape
     lbm_status rc = batch_build(b, kThreads, band_rows != 0 ? band_rows : 16, 1);
     if (rc != LBM_OK) return bail(rc);
+    rc = batch_build_passes(b);
+    if (rc != LBM_OK) return bail(rc);
     cudaError_t e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) return bail(cuda_fail(e, "creating the capture stream"));
     *out = b;
@@ -2632,6 +2724,7 @@ lbm_status lbm_batch_set_shape(lbm_batch *b, int32_t threads, int32_t band_rows)
     if (rc != LBM_OK) return rc;
     for (lbm_handle *h : b->hs) LBM_CUDA(cudaStreamSynchronize(h->stream));
     rc = batch_build(b, threads, band_rows, b->lookahead);
+    if (rc == LBM_OK) b->own_shape = true;
     if (rc == LBM_OK) clear_error();
     return rc;
 }
@@ -2644,6 +2737,7 @@ lbm_status lbm_batch_set_lookahead(lbm_batch *b, int32_t rows)
     if (rc != LBM_OK) return rc;
     for (lbm_handle *h : b->hs) LBM_CUDA(cudaStreamSynchronize(h->stream));
     rc = batch_build(b, b->threads, b->band_rows, rows);
+    if (rc == LBM_OK) b->own_shape = true;
     if (rc == LBM_OK) clear_error();
     return rc;
 }
@@ -2691,6 +2785,7 @@ lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *threads, i
             for (lbm_handle *h : b->hs) LBM_CUDA(cudaStreamSynchronize(h->stream));
             rc = batch_build(b, it->second.threads, it->second.rows, it->second.la);
             if (rc != LBM_OK) return rc;
+            b->own_shape = false;
             if (threads) *threads = b->threads;
             if (band_rows) *band_rows = b->band_rows;
             if (us_per_step) *us_per_step = 0.0;
@@ -2782,6 +2877,7 @@ lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *threads, i
     // snapshot: partition again for the chosen shape
     rc = batch_build(b, best_t, best_r, best_la);
     if (rc != LBM_OK) return done(rc);
+    b->own_shape = false;
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         g_tune_cache[key] = BatchShape{best_t, best_r, best_la};
@@ -2811,6 +2907,14 @@ lbm_status lbm_batch_step(lbm_batch *b, int64_t n)
         par ^= (int)(n & 1);
         left = 0;
     }
+    if (left > 0 && b->pblock && !b->own_shape) {
+        // pairs of passes of 8, 4 and 2 steps, then single steps
+        for (int k = 0; k < lbm_batch::kPassKinds; ++k)
+            for (; left >= 2 * kBatchPassSteps[k]; left -= 2 * kBatchPassSteps[k]) {
+                LBM_CUDA(enqueue_batch_pass(b, k, par, false, b->stream));
+                LBM_CUDA(enqueue_batch_pass(b, k, par ^ 1, true, b->stream));
+            }
+    }
     if (left > 0) {
         // runs of steps replay graphs of 64, 32, ..., 2 batched steps
         const lbm_status rc = run_chunks(b->graph, 0, b->stream, b->cap_stream, left, par,
@@ -2839,6 +2943,7 @@ void lbm_batch_destroy(lbm_batch *b)
     b->graph.reset();
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
     batch_release_block(b);
+    batch_free(b, b->pblock);
     batch_free(b, b->bar);
     if (b->owns)
         for (lbm_handle *h : b->hs) lbm_destroy(h);

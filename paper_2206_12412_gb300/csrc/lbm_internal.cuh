@@ -369,6 +369,10 @@ cudaError_t launch_step(const StepArgs<T, D> &a, int bands, cudaStream_t s, bool
 template <typename T, typename D, int MODE = kForward>
 cudaError_t launch_pass(const PassArgs<T, D> &a, int n_pass, cudaStream_t s);
 template <typename T, typename D, int MODE = kForward> const void *pass_kernel_ptr(int nw, int rpt, bool run);
+// One pass of every lattice of a batch (FP32 arithmetic); which: parity + 2 if
+// the second pass of a pair.
+template <typename T, typename D>
+cudaError_t launch_pass_batch(const PassArgs<T, D> *descs, const BatchUnit *units, int n_units, int which, cudaStream_t s);
 template <typename T, typename D> cudaError_t launch_edge_rule(const StepArgs<T, D> &a, cudaStream_t s);
 template <typename T, typename D> int edge_rule_count(const StepArgs<T, D> &a);
 template <typename T, typename D>

@@ -43,6 +43,7 @@
 #include "lbm_internal.cuh"
 #include "lbm_rows.cuh"
 
+#include <cstddef>
 #include <type_traits>
 
 namespace lbm {
@@ -1606,6 +1607,34 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW)
         pass_cta<T, D, NW, RPT, true, MODE>(a, B, blockIdx.x, sh, sen);
         if (it + 1 < n_pass && !grid_barrier(a.bar, gridDim.x, a.budget, a.s.err)) return;
     }
+}
+
+// One pass of every lattice of a batch: CTA u takes tile units[u].cb of
+// lattice units[u].inst, with that lattice's arguments (descriptor par + 2
+// second of its four) copied to shared memory.  The crack strips' tiles come
+// first: a growing end's tile runs a chain of FP64 steps that the bulk tiles
+// of all lattices hide.
+template <typename T, typename D>
+__global__ void __launch_bounds__(256, 2) pass_batch_kernel(const PassArgs<T, D> *descs, const BatchUnit *units, int which)
+{
+    __shared__ PassShared<T, 8> sh;
+    __shared__ PassSensors<T, kForward> sen;
+    __shared__ __align__(16) PassArgs<T, D> sa;
+    const BatchUnit u = units[blockIdx.x];
+    const uint32_t *src = reinterpret_cast<const uint32_t *>(descs + 4 * u.inst + which);
+    uint32_t *dst = reinterpret_cast<uint32_t *>(&sa);
+    typedef PassArgs<T, D> Args;
+    for (int q = threadIdx.x; q < (int)(offsetof(Args, rec) / 4); q += 256) dst[q] = src[q];
+    __syncthreads();
+    const PassBuf<T, D> B = {sa.s.w_in, sa.wd_in, sa.s.w_out, sa.s.wd, sa.s.s_in, sa.s.s_out, nullptr, nullptr};
+    pass_cta<T, D, 8, 8, false, kForward>(sa, B, u.cb, sh, sen);
+}
+
+template <typename T, typename D>
+cudaError_t launch_pass_batch(const PassArgs<T, D> *descs, const BatchUnit *units, int n_units, int which, cudaStream_t s)
+{
+    pass_batch_kernel<T, D><<<(unsigned)n_units, 256, 0, s>>>(descs, units, which);
+    return cudaGetLastError();
 }
 
 template <typename T, typename D, int MODE> const void *pass_kernel_ptr(int nw, int rpt, bool run)

@@ -135,3 +135,35 @@ def test_tape_passes_equal_single_steps(gpu, kind, every, storage):
         lat.close()
     for a, b in zip(*got):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("storage", ["f32", "f32_bf16", "f32_f16", "f32_lf"])
+def test_batch_passes_equal_single_steps(gpu, storage):
+    """A batch of uneven lattices in passes (pairs of 8, 4 and 2 steps, then
+    single ones) against the same lattices stepped alone, one step a call."""
+    lbm = gpu
+    probs = [_strip(97, 41, v_rel=0.6), _strip(300, 150, mode="kcrit", K_C=KC), _strip(33, 25, mode=None),
+             _strip(500, 80, mode="kcrit", K_C=6e-5, start=200.0, tip=215.0, two_tips=True),
+             _strip(260, 120, mode="kcrit", bc="macroscopic_edges", K_C=KC),
+             _strip(240, 70, bc="bounceback", v_rel=0.5, edges=("periodic", "periodic", "dirichlet", "free"), start=150.0,
+                    tip=200.0)]
+    solo = [lbm.Lattice(p, storage) for p in probs]
+    lats = [lbm.Lattice(p, storage) for p in probs]
+    for k, (a, b) in enumerate(zip(solo, lats)):
+        w0, wd0 = W.random_state(a.nx, a.ny, 30 + k)
+        a.set_fields(w0, wd0)
+        b.set_fields(w0, wd0)
+    batch = lbm.Batch(lats)
+    for n in (3, 16 + 8 + 4 + 3, 21):
+        batch.step(n)
+        for a in solo:
+            for _ in range(n):
+                a.step(1)
+    for a, b in zip(solo, lats):
+        for x, y in zip(a.fields(), b.fields()):
+            np.testing.assert_array_equal(x, y)
+        assert a.crack_state() == b.crack_state()
+        ha, hb = a.history(60), b.history(60)
+        for key in ha:
+            np.testing.assert_array_equal(ha[key], hb[key])
+    batch.close()
