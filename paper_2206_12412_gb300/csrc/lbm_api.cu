@@ -393,6 +393,8 @@ cudaError_t enqueue_pass_t(const lbm_handle *h, const lbm::PassPlan &q, int par,
     lbm::NvtxRange r("K1 pass");
     lbm::PassArgs<T, D> a;
     make_pass_args(h, par, second, q, a);
+    if constexpr (std::is_same<T, D>::value)
+        if (h->q == 9) return launch_pass<T, D, lbm::kNine>(a, n_pass, s);
     return launch_pass(a, n_pass, s);
 }
 
@@ -987,7 +989,7 @@ lbm_status create_impl(const lbm_grid *grid, const lbm_lattice *lattice, const l
     const size_t alt_bytes = h->esize_d ? plane_d : plane;
     const size_t o_a0 = off; off = align256(off + alt_bytes);
     const size_t o_a1 = off; if (!h->esize_d) off = align256(off + alt_bytes);
-    bool scratch = !line && !d2q9 && !slab && grid->edge[LBM_BOTTOM] != LBM_EDGE_PERIODIC &&
+    bool scratch = !line && !slab && grid->edge[LBM_BOTTOM] != LBM_EDGE_PERIODIC &&
                    off - h->state_bytes <= kMaxPassScratch;
     h->block_bytes = scratch ? off : h->state_bytes;
     h->block = dev_alloc(h, h->block_bytes);

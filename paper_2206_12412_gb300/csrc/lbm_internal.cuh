@@ -224,7 +224,7 @@ struct PassPlan {
     int32_t jt, mt, pt;        // rows [jt, ny) above it (a lattice without a crack: all rows)
     int32_t ms, ps;            // column tiles of the strip and their nominal width
     int32_t zb, za;            // strip: no tile boundary less than zb behind or up to za ahead of a tip
-    int32_t grow;              // strip: most columns an end can cut in a pass
+    int32_t grow, back;        // strip: the columns ahead of and behind an end's next that a pass can cut
     int32_t tiles, edge_macro;
 };
 
@@ -252,9 +252,9 @@ struct RecArgs {
     int32_t ns, acc_loss;
 };
 
-// What a pass does besides stepping: nothing, the adjoint's recording, or the
-// transposed steps of its sweep (m and a in place of w and wdot).
-enum { kForward = 0, kRecord = 1, kAdjoint = 2 };
+// What a pass does: steps, steps recorded for the adjoint, the transposed steps
+// of its sweep (m and a in place of w and wdot), or D2Q9 steps.
+enum { kForward = 0, kRecord = 1, kAdjoint = 2, kNine = 3 };
 constexpr int kPassSensors = 64;   // most sensors of a recording or sweep in passes
 
 // The sweep's part of a pass's arguments (see AdjArgs); edge_m: the values of m

@@ -40,6 +40,7 @@
 
 #include "lbm_barrier.cuh"
 #include "lbm_crack.cuh"
+#include "lbm_d2q9.cuh"
 #include "lbm_internal.cuh"
 #include "lbm_rows.cuh"
 
@@ -165,6 +166,38 @@ __device__ __forceinline__ void row_sites(const Row<T, N> &cu, const Row<T, N> &
     }
 }
 
+// The same with eight neighbours: axis and diag hold the sums over the axis
+// and the diagonal neighbours.
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+template <typename T, int N>
+__device__ __forceinline__ void row_sites9(const Row<T, N> &cu, const Row<T, N> &axis, const Row<T, N> &diag, Row<T, N> &d, T ga,
+                                           T gd, T dt, Row<T, N> &out)
+{
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int k = 0; k < N; k += 2) {
+            const uint64_t c = pk2(cu.v[k], cu.v[k + 1]), m4 = pk2(-4.0f, -4.0f);
+            const uint64_t ax = fma2(m4, c, pk2(axis.v[k], axis.v[k + 1])), di = fma2(m4, c, pk2(diag.v[k], diag.v[k + 1]));
+            // d9_rate and d9_integrate
+            const uint64_t r = add2(pk2(d.v[k], d.v[k + 1]), fma2(pk2(ga, ga), ax, mul2(pk2(gd, gd), di)));
+            up2(r, d.v[k], d.v[k + 1]);
+            up2(fma2(pk2(dt, dt), r, c), out.v[k], out.v[k + 1]);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const T ax = axis.v[k] - (T)4 * cu.v[k], di = diag.v[k] - (T)4 * cu.v[k];
+            d.v[k] = d9_rate(d.v[k], ax, di, ga, gd);
+            out.v[k] = d9_integrate(cu.v[k], d.v[k], dt);
+        }
+    }
+}
+
 // The crack state in force during one update of a pass, and the records of
 // the crack step before it (lazy: its K and pairs are formed at the end).
 struct PassTip {
@@ -196,6 +229,7 @@ template <typename T, int MODE> struct PassSensors {
     T v[kPassSteps][2 * kPassSensors];
 };
 template <typename T> struct PassSensors<T, kForward> {};
+template <typename T> struct PassSensors<T, kNine> {};
 
 struct TileGeo {
     int xl, x0, x1, yl, y0, y1;   // first column held, own columns [x0, x1); first row held, own rows [y0, y1)
@@ -677,7 +711,8 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
     if (MODE != kAdjoint && KIND == 2 && face) stg_row(&sh.pair[s][below ? 0 : 1][lane * N], F.template cur<PH>(below ? RPT - 1 : 0));
 
     const bool dir_l = KIND != 0 && a.edge[LEFT] == EDGE_DIRICHLET, dir_r = KIND != 0 && a.edge[RIGHT] == EDGE_DIRICHLET;
-    const bool em = MODE == kForward && KIND != 0 && A.q.edge_macro != 0, em_side = em && c.side;
+    constexpr bool kNineQ = MODE == kNine;
+    const bool em = (MODE == kForward || kNineQ) && KIND != 0 && A.q.edge_macro != 0, em_side = em && c.side;
     const bool last_r = KIND != 0 && c.kr == N - 1;
     T tl = (T)0, tr = (T)0;
     R first, last;                                         // the first and last rows before the update
@@ -692,6 +727,7 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
             // columns, as neighbours: the row update itself knows no edge
 #pragma unroll
             for (int r = 0; r < RPT; ++r) {
+                if (kNineQ) break;   // (a D2Q9 diagonal sends back its own site's value, not its neighbour's)
                 if (r + 1 < RPT && jb + r == ny - 1)
                     F.template cur<PH>(r + 1 < RPT ? r + 1 : r) =
                         edge_image<T, N>(F.template cur<PH>(r), a.edge[TOP] == EDGE_DIRICHLET, sh.ws2[TOP][s]);
@@ -736,7 +772,7 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
     // on latency more than on issue, update them before the barrier (row 1's
     // new values take the slot of row 0, whose old values and neighbour are
     // kept); larger ones sweep all rows after it.
-    constexpr bool kEarly = RPT <= 4;
+    constexpr bool kEarly = RPT <= 4 && !kNineQ;
     R old0, old1, hs0, hsT;
     if (kEarly && PH == 0) {
         old0 = F.template cur<PH>(0);
@@ -758,7 +794,8 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
         if (warp == 0) {
             pass_crack_step<T, PassShared<T, NW>::W>(p, A.q, sh.top[b][kBelowWarp], sh.bot[b][kBelowWarp + 1], c.org_r,
                                                      c.org_l, sh.S, sh.log[s + 1], c.ev_r, c.ev_l, win);
-            if (lane == 0) sh.reach[b ^ 1] = crack_cut_in_reach(p, sh.S) ? 1 : 0;
+            // (D2Q9: any advance can pass a diagonal crossing)
+            if (lane == 0) sh.reach[b ^ 1] = kNineQ || crack_cut_in_reach(p, sh.S) ? 1 : 0;
         }
         // rows next to the crack wait for the decision only where it can cut a link
         if (reach) __syncthreads();
@@ -766,7 +803,7 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
     R dnx, upx;
     ld_row(&sh.top[b][warp > 0 ? warp - 1 : 0][lane * N], dnx);
     ld_row(&sh.bot[b][warp < NW - 1 ? warp + 1 : warp][lane * N], upx);
-    if (KIND != 0 && (c.has_t || c.has_b)) {
+    if (KIND != 0 && !kNineQ && (c.has_t || c.has_b)) {
         // the images beyond the bottom and top rows
         if (c.has_t) upx = edge_image<T, N>(last, a.edge[TOP] == EDGE_DIRICHLET, sh.ws2[TOP][s]);
         if (c.has_b) dnx = edge_image<T, N>(first, a.edge[BOTTOM] == EDGE_DIRICHLET, sh.ws2[BOTTOM][s]);
@@ -786,11 +823,101 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
             if (c.per) q = q < 0 ? q + nx : (q >= nx ? q - nx : q);
             cut[k] = q >= f && q <= l;
             cutp[k] = q >= fp && q <= lp;
-            upx.v[k] = cut[k] && below ? last.v[k] : upx.v[k];
-            dnx.v[k] = cut[k] && !below ? first.v[k] : dnx.v[k];
+            if (!kNineQ) {
+                upx.v[k] = cut[k] && below ? last.v[k] : upx.v[k];
+                dnx.v[k] = cut[k] && !below ? first.v[k] : dnx.v[k];
+            }
         }
     }
-    if (kEarly && PH == 0) {
+    if constexpr (kNineQ) {
+        const T ga = gg * (T)(2.0 / 3.0), gd = gg * (T)(1.0 / 6.0);
+        // the severed diagonals: crossings of the crack line between the tips
+        // in force, left and right of each column
+        bool dl[N], dr[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) dl[k] = dr[k] = false;
+        if (KIND == 2 && face) {
+            const int64_t rq = c.known ? sh.log[s + 1].tr : (c.ev_r ? sh.S.r.tip_q : sh.in.r.tip_q);
+            const int64_t lq = !p.two_tips ? p.start_q : (c.known ? sh.log[s + 1].tl : (c.ev_l ? sh.S.l.tip_q : sh.in.l.tip_q));
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                int q = x0 + k;
+                if (c.per) q = q < 0 ? q + nx : (q >= nx ? q - nx : q);
+                const int64_t ml = (int64_t)q << kQBits, mr = (int64_t)(q + 1) << kQBits;
+                dl[k] = q >= 1 && lq <= ml && ml <= rq;
+                dr[k] = q + 1 <= nx - 1 && lq <= mr && mr <= rq;
+            }
+        }
+        const TwoWs<T> two_ws{sh.ws2[LEFT][s], sh.ws2[RIGHT][s], sh.ws2[BOTTOM][s], sh.ws2[TOP][s]};
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+            const int r = PH == 0 ? q : RPT - 1 - q, j = jb + r;
+            const R cu = F.template cur<PH>(r);
+            const R up = r + 1 < RPT ? F.template cur<PH>(r + 1 < RPT ? r + 1 : r) : upx;
+            const R dn = r > 0 ? F.template cur<PH>(r > 0 ? r - 1 : r) : dnx;
+            const bool crow = KIND == 2 && face && r == (below ? RPT - 1 : 0);
+            const bool top = KIND != 0 && j == ny - 1, bot = KIND != 0 && j == 0;
+            R axis, diag;
+            if (KIND != 0 && (crow || top || bot || c.odd)) {
+                // a row with links that leave the body or cross the crack:
+                // each diagonal by itself
+                const T lc = __shfl_up_sync(kFull, cu.v[N - 1], 1), rc = __shfl_down_sync(kFull, cu.v[0], 1);
+                const T la = __shfl_up_sync(kFull, up.v[N - 1], 1), ra = __shfl_down_sync(kFull, up.v[0], 1);
+                const T lb = __shfl_up_sync(kFull, dn.v[N - 1], 1), rb = __shfl_down_sync(kFull, dn.v[0], 1);
+#pragma unroll
+                for (int k = 0; k < N; ++k) {
+                    const T w0 = cu.v[k];
+                    const bool lft = c.is_l && k == 0, rgt = k == c.kr;
+                    T wl = k == 0 ? lc : cu.v[k > 0 ? k - 1 : 0], wr = k == N - 1 ? rc : cu.v[k < N - 1 ? k + 1 : k];
+                    T al = k == 0 ? la : up.v[k > 0 ? k - 1 : 0], ar = k == N - 1 ? ra : up.v[k < N - 1 ? k + 1 : k];
+                    T bl = k == 0 ? lb : dn.v[k > 0 ? k - 1 : 0], br = k == N - 1 ? rb : dn.v[k < N - 1 ? k + 1 : k];
+                    T u = up.v[k], v = dn.v[k];
+                    if (lft) wl = leaving(a.edge, two_ws, true, false, -1, 0, w0);
+                    if (rgt) wr = leaving(a.edge, two_ws, true, false, 1, 0, w0);
+                    if (top) u = leaving(a.edge, two_ws, false, true, 0, 1, w0);
+                    else if (crow && below && cut[k]) u = w0;
+                    if (bot) v = leaving(a.edge, two_ws, false, true, 0, -1, w0);
+                    else if (crow && !below && cut[k]) v = w0;
+                    if (crow && below && dl[k]) al = w0;
+                    else if (lft || top) al = leaving(a.edge, two_ws, lft, top, -1, 1, w0);
+                    if (crow && below && dr[k]) ar = w0;
+                    else if (rgt || top) ar = leaving(a.edge, two_ws, rgt, top, 1, 1, w0);
+                    if (crow && !below && dl[k]) bl = w0;
+                    else if (lft || bot) bl = leaving(a.edge, two_ws, lft, bot, -1, -1, w0);
+                    if (crow && !below && dr[k]) br = w0;
+                    else if (rgt || bot) br = leaving(a.edge, two_ws, rgt, bot, 1, -1, w0);
+                    axis.v[k] = (u + v) + (wl + wr);
+                    diag.v[k] = (al + bl) + (ar + br);
+                }
+            } else {
+                // from the column sums of the rows above and below
+                R sc;
+#pragma unroll
+                for (int k = 0; k < N; ++k) sc.v[k] = up.v[k] + dn.v[k];
+                T sl = __shfl_up_sync(kFull, sc.v[N - 1], 1), sr = __shfl_down_sync(kFull, sc.v[0], 1);
+                if (KIND != 0) {
+                    T il = cu.v[0], ir = cu.v[N - 1];
+                    if (dir_l) il = tl - il;
+                    if (dir_r) ir = tr - ir;
+                    sl = c.is_l ? il + il : sl;
+                    sr = last_r ? ir + ir : sr;
+                }
+                const R hs = sides(cu);
+#pragma unroll
+                for (int k = 0; k < N; ++k) {
+                    axis.v[k] = sc.v[k] + hs.v[k];
+                    diag.v[k] = (k == 0 ? sl : sc.v[k > 0 ? k - 1 : 0]) + (k == N - 1 ? sr : sc.v[k < N - 1 ? k + 1 : k]);
+                }
+            }
+            R out;
+            row_sites9<T, N>(cu, axis, diag, F.b[r], ga, gd, dt, out);
+            F.template next<PH>(r) = out;
+        }
+#pragma unroll
+        for (int k = 0; k < N; ++k) cut[k] = cut[k] || dl[k] || dr[k];   // the crack-face points
+    }
+    if constexpr (kNineQ) {
+    } else if (kEarly && PH == 0) {
         R out;
         row_sites<T, D, N>(old0, old1, dnx, hs0, F.template rate<PH>(0), gg, dt, wd_scale, wd_inv, out);
         // the last row: its old values and its neighbour's are still in place
@@ -867,7 +994,15 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
             wB.v[k] = (T)1.5 * w2 - (T)0.5 * w3;
             w0.v[k] = below ? last.v[k] : first.v[k];
         }
-        const R rt = kLf ? wB : rate_of(wB, w0, dt);
+        R rt = wB;
+        if (kNineQ) {
+            // (the D2Q9 face rule multiplies by 1 / dt)
+            const T inv_dt = dt == (T)1 ? (T)1 : div_dt((T)1, dt);
+#pragma unroll
+            for (int k = 0; k < N; ++k) rt.v[k] = (wB.v[k] - w0.v[k]) * inv_dt;
+        } else if (!kLf) {
+            rt = rate_of(wB, w0, dt);
+        }
 #pragma unroll
         for (int k = 0; k < N; ++k) {
             if (!kLf) {
@@ -1174,7 +1309,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
             sh.log[tid].l = q >= 0 ? A.adj.i_last[qc] : 0;
         }
     }
-    if constexpr (MODE != kForward) pass_sensors<T, D, NW, RPT, MODE>(A, B, g, c.n, sen);
+    if constexpr (MODE == kRecord || MODE == kAdjoint) pass_sensors<T, D, NW, RPT, MODE>(A, B, g, c.n, sen);
     if (MODE != kAdjoint && KIND == 2) {
         c.known = p.mode != CRACK_KCRIT;
         c.f0 = sh.in.i_first;
@@ -1182,17 +1317,17 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
         hist0 = p.hist_cap > 0 ? sh.in.hist_n % p.hist_cap : 0;   // the ring slot of the first record
         rec0 = sh.in.r.decided ? 1 : 0;   // the first update whose crack step is still to run
         const int cr = tip_col_r(c.f0, c.l0, nx), cl = tip_col_l(c.f0, c.l0, nx);
-        const int hc = A.q.hc, grow = A.q.grow;
+        const int hc = A.q.hc, grow = A.q.grow, back = A.q.back;
         // (periodic sides: the column itself, then its images beyond either side)
         for (int q = 0; q < (per ? 3 : 1); ++q) {
             const int o = q == 0 ? 0 : (q == 1 ? -nx : nx);
             if (cr + o >= g.x0 && cr + o < g.x1) c.own_r = true;
             if (p.two_tips && cl + o >= g.x0 && cl + o < g.x1) c.own_l = true;
-            if (!c.ev_r && g.x0 - hc <= cr + o + grow && g.x1 + hc > cr + o) {
+            if (!c.ev_r && g.x0 - hc <= cr + o + grow && g.x1 + hc > cr + o - back) {
                 c.ev_r = true;
                 c.org_r = g.xl - o;
             }
-            if (p.two_tips && !c.ev_l && g.x0 - hc <= cl + o && g.x1 + hc > cl + o - grow) {
+            if (p.two_tips && !c.ev_l && g.x0 - hc <= cl + o + back && g.x1 + hc > cl + o - grow) {
                 c.ev_l = true;
                 c.org_l = g.xl - o;
             }
@@ -1208,7 +1343,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
         } else {
             if (tid == 0) {
                 sh.S = sh.in;
-                sh.reach[0] = crack_cut_in_reach(p, sh.S) ? 1 : 0;
+                sh.reach[0] = MODE == kNine || crack_cut_in_reach(p, sh.S) ? 1 : 0;
                 sh.log[0].tr = sh.S.r.tip_q;
                 sh.log[0].tl = sh.S.l.tip_q;
                 sh.log[0].f = c.f0;
@@ -1263,8 +1398,8 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
     c.has_b = KIND != 0 && jb == 0;
     c.odd = KIND != 0 && ((jb < 0 && jb + RPT > 0) || (jb < ny && jb + RPT > ny) ||
                           __any_sync(kFull, c.kr >= 0 && c.kr < N - 1));
-    if (KIND != 0 || MODE != kForward) __syncthreads();   // w*, the cuts of the pass, the sensors
-    if constexpr (MODE != kForward) {
+    if (KIND != 0 || MODE == kRecord || MODE == kAdjoint) __syncthreads();   // w*, the cuts of the pass, the sensors
+    if constexpr (MODE == kRecord || MODE == kAdjoint) {
         for (int e = 0; e < sen.n; ++e) {
             const int r0 = sen.j[e] - jb, k0 = sen.i[e] - x0;
             c.senses |= r0 >= 0 && r0 < RPT && k0 >= 0 && k0 < N;

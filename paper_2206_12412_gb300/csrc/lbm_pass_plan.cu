@@ -95,7 +95,11 @@ bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q, bool ad
     } else if (crack) {
         // columns an end can cut in a pass, and the reach of its K window
         const int64_t dq = p.mode == CRACK_KCRIT ? p.dq_max : p.mode == CRACK_PRESCRIBED ? p.dq_prescribed : 0;
-        q.grow = (int)((dq * K) >> kQBits) + 2;
+        // (D2Q9: a diagonal crossing lies up to half a spacing behind the next
+        // vertical link and belongs to the columns on both of its sides)
+        const int d9 = h->q == 9 ? 2 : 0;
+        q.grow = (int)((dq * K) >> kQBits) + 2 + d9;
+        q.back = d9;
         const double v = p.mode == CRACK_KCRIT ? p.v_max : p.mode == CRACK_PRESCRIBED ? p.v_rel : 0.0;
         const double r_min = p.r_min_fixed > 0.0 ? p.r_min_fixed : p.r0 / (1.0 - v);
         const double reach = (r_min + p.fit_width) / p.dh;
@@ -122,7 +126,7 @@ bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q, bool ad
             q.ps = nx;
         } else {
             if (!(reach < (double)W)) return false;
-            q.zb = std::max((int)std::ceil(reach) + 4 + K - q.hc, q.hc) + 1;
+            q.zb = std::max((int)std::ceil(reach) + 4 + K - q.hc, q.hc) + 1 + d9;
             q.za = q.grow + q.hc + 1;
             const int Z = q.zb + q.za + 1;
             const int moved = p.two_tips ? Z + 2 * N : Z / 2 + N;   // how much wider moved boundaries can make a tile
@@ -161,7 +165,9 @@ void choose_pass(lbm_handle *h)
         bool shorter = true;   // every shorter pass too: a call's last passes
         for (int k = K; k >= 2; --k) shorter = shorter && pass_plan(h, k, h->pass_nw, h->pass_rpt, q);
         if (!shorter) continue;
-        const void *fn = h->lat.storage == LBM_F64           ? pass_kernel_ptr<double, double>(h->pass_nw, h->pass_rpt, true)
+        const void *fn = h->q == 9 ? (h->esize == 8 ? pass_kernel_ptr<double, double, kNine>(h->pass_nw, h->pass_rpt, true)
+                                                    : pass_kernel_ptr<float, float, kNine>(h->pass_nw, h->pass_rpt, true))
+                         : h->lat.storage == LBM_F64           ? pass_kernel_ptr<double, double>(h->pass_nw, h->pass_rpt, true)
                          : h->lat.storage == LBM_F32_WD_BF16 ? pass_kernel_ptr<float, __nv_bfloat16>(h->pass_nw, h->pass_rpt, true)
                          : h->lat.storage == LBM_F32_WD_F16  ? pass_kernel_ptr<float, __half>(h->pass_nw, h->pass_rpt, true)
                          : h->lat.storage == LBM_F32_LEAPFROG ? pass_kernel_ptr<float, Lf>(h->pass_nw, h->pass_rpt, true)

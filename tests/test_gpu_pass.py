@@ -61,6 +61,16 @@ def cases():
         out.append((f"rest_two_{k}", _strip(300, 150, mode="kcrit", K_C=kc, start=140.2, tip=143.9, two_tips=True), "f32", 91))
         out.append((f"rest_wide_{k}", _strip(700, 300, mode="kcrit", K_C=kc, start=140.0, tip=181.0, two_tips=True,
                                              fit_width=3.5), "f64", 60))
+    nine = []
+    for nm, p, st, n in out:   # the same on nine velocities
+        if st in ("f32", "f64"):
+            nine.append((nm + "_q9", dict(p, lattice="D2Q9"), st, n))
+    out += nine
+    for k, kw in enumerate((dict(edges=("dirichlet",) * 4, bc="bounceback", v_rel=0.7, start=30.0),
+                            dict(mode="kcrit", jc=12, K_C=KC), dict(mode=None),
+                            dict(mode="prescribed", bc="macroscopic_edges", start=20.0, v_rel=0.5,
+                                 edges=("dirichlet", "free", "free", "dirichlet")))):
+        out.append((f"q9_{k}", dict(_strip(250, 110, **kw), lattice="D2Q9"), "f32", 50))
     out += [
         ("no_crack", _strip(300, 170, mode=None), "f32", 70),
         ("no_crack_edges", _strip(300, 170, mode=None, bc="macroscopic_edges"), "f32", 70),
