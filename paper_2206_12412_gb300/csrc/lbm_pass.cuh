@@ -74,6 +74,23 @@ template <typename D, typename T> __device__ __forceinline__ void wd_put(D *p, T
     else WdIO<D>::put(p, v, scale);
 }
 
+// Two neighbouring ones at once: the packed conversions run at the ALU's
+// rate, the scalar ones at an eighth of it (8192 x 8192 BF16: 68 us a step
+// with those, against 32 us for FP32 wdot).
+template <typename D> __device__ __forceinline__ void wd_round2(float &a, float &b, float scale, float inv)
+{
+    if constexpr (std::is_same<D, __nv_bfloat16>::value) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+        const uint32_t u = *reinterpret_cast<const uint32_t *>(&h);
+        a = __uint_as_float(u << 16);
+        b = __uint_as_float(u & 0xffff0000u);
+    } else if constexpr (std::is_same<D, __half>::value) {
+        const float2 f = __half22float2(__floats2half2_rn(a * scale, b * scale));
+        a = f.x * inv;
+        b = f.y * inv;
+    }
+}
+
 // Two FP32 operations in one instruction (each rounded as the scalar one).
 // They do not raise the FP32 rate, but halve the instructions a row issues,
 // and a tile is bound by instruction issue.
@@ -148,10 +165,8 @@ __device__ __forceinline__ void row_sites(const Row<T, N> &cu, const Row<T, N> &
             } else {
                 const uint64_t dn2 = fma2(pk2(g, g), lap, pk2(d.v[k], d.v[k + 1]));
                 up2(fma2(pk2(dt, dt), dn2, c), out.v[k], out.v[k + 1]);
-                float d0, d1;
-                up2(dn2, d0, d1);
-                d.v[k] = wd_round<D, T>(d0, wd_scale, wd_inv);
-                d.v[k + 1] = wd_round<D, T>(d1, wd_scale, wd_inv);
+                up2(dn2, d.v[k], d.v[k + 1]);
+                wd_round2<D>(d.v[k], d.v[k + 1], wd_scale, wd_inv);
             }
         }
     } else {
