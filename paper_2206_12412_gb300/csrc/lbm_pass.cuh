@@ -578,10 +578,10 @@ __device__ __forceinline__ void cg_row(const double *p, Row<double, 2> &r)
     const double2 q = __ldcg(reinterpret_cast<const double2 *>(p));
     r.v[0] = q.x; r.v[1] = q.y;
 }
-template <typename D, typename T, int N> __device__ __forceinline__ void cg_rate(const D *p, Row<T, N> &r, T inv)
+template <typename D, typename Raw> __device__ __forceinline__ void cg_raw(const D *p, Raw &r)
 {
     if constexpr (std::is_same<D, Lf>::value) cg_row(reinterpret_cast<const float *>(p), r);
-    else if constexpr (sizeof(D) == 2) WdIO<D>::unpack(__ldcg(reinterpret_cast<const uint2 *>(p)), r, inv);
+    else if constexpr (sizeof(D) == 2) r = __ldcg(reinterpret_cast<const uint2 *>(p));
     else cg_row(p, r);
 }
 template <typename T> __device__ __forceinline__ T cg_get(const T *p) { return __ldcg(p); }
@@ -1274,22 +1274,33 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
         const T *wp = B.w_in + (int64_t)jb * P + x0;
         const D *dp = B.wd_in + (int64_t)jb * P + x0;
         const bool whole = KIND == 0 ? x0 < nx : (x0 >= 0 && x0 + N <= nx);
+        // every load before any conversion, so that they are in flight together
+        typename WdIO<D>::Raw raw[RPT];
 #pragma unroll
         for (int r = 0; r < RPT; ++r) {
-            R &w = F.template cur<0>(r), &d = F.b[r];
+            R &w = F.template cur<0>(r);
 #pragma unroll
-            for (int k = 0; k < N; ++k) w.v[k] = d.v[k] = (T)0;
+            for (int k = 0; k < N; ++k) w.v[k] = (T)0;
+            raw[r] = typename WdIO<D>::Raw{};
             const int j = jb + r;
-            if (j < 0 || j >= ny) continue;
-            if (whole) {
+            if (whole && j >= 0 && j < ny) {
                 if (COOP) {
                     cg_row(wp + (int64_t)r * P, w);
-                    cg_rate(dp + (int64_t)r * P, d, wd_inv);
+                    cg_raw(dp + (int64_t)r * P, raw[r]);
                 } else {
                     ldg_row(wp + (int64_t)r * P, w);
-                    WdIO<D>::load(dp + (int64_t)r * P, d, wd_inv);
+                    WdIO<D>::fetch(dp + (int64_t)r * P, raw[r]);
                 }
-            } else if (KIND != 0) {
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) WdIO<D>::unpack(raw[r], F.b[r], wd_inv);
+        if (KIND != 0 && !whole) {
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) {
+                const int j = jb + r;
+                if (j < 0 || j >= ny) continue;
+                R &w = F.template cur<0>(r), &d = F.b[r];
 #pragma unroll
                 for (int k = 0; k < N; ++k) {
                     int q = x0 + k;
