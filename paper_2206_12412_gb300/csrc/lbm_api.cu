@@ -1264,6 +1264,20 @@ lbm_status lbm_step(lbm_handle *h, int64_t n)
     return LBM_OK;
 }
 
+// A plane of the handle to / from device memory of the caller's.
+static cudaError_t plane_out(const lbm_handle *h, const void *plane, void *dst, int64_t stride)
+{
+    const int nx = h->grid.nx, ny = h->grid.ny;
+    return h->esize == 8 ? launch_plane_out<double>(static_cast<const double *>(plane), h->pitch, nx, ny, static_cast<double *>(dst), stride, h->stream)
+                         : launch_plane_out<float>(static_cast<const float *>(plane), h->pitch, nx, ny, static_cast<float *>(dst), stride, h->stream);
+}
+static cudaError_t plane_in(const lbm_handle *h, void *plane, const void *src, int64_t stride)
+{
+    const int nx = h->grid.nx, ny = h->grid.ny;
+    return h->esize == 8 ? launch_plane_in<double>(static_cast<double *>(plane), h->pitch, nx, ny, static_cast<const double *>(src), stride, h->stream)
+                         : launch_plane_in<float>(static_cast<float *>(plane), h->pitch, nx, ny, static_cast<const float *>(src), stride, h->stream);
+}
+
 // The dtype a field is exchanged in: the arithmetic precision (FP64 for F64
 // storage, FP32 otherwise; 16-bit wdot planes are converted).
 static int32_t exchange_dtype(const lbm_handle *h) { return h->esize == 8 ? LBM_F64 : LBM_F32; }
@@ -1291,7 +1305,8 @@ lbm_status lbm_fields(lbm_handle *h, int32_t which, void *dst, int32_t dst_on_de
             LBM_CUDA(cudaMemcpyAsync(dst, conv, (size_t)h->grid.nx * h->grid.ny * 4, cudaMemcpyDeviceToHost, h->stream));
     } else {
         const void *src = which == LBM_FIELD_W ? h->w[h->parity] : h->wd;
-        LBM_CUDA(cudaMemcpy2DAsync(dst, row, src, (size_t)h->pitch * h->esize, row, (size_t)h->grid.ny, kind, h->stream));
+        if (dst_on_device) LBM_CUDA(plane_out(h, src, dst, h->grid.nx));
+        else LBM_CUDA(cudaMemcpy2DAsync(dst, row, src, (size_t)h->pitch * h->esize, row, (size_t)h->grid.ny, kind, h->stream));
     }
     if (!dst_on_device) return check_sticky(h);
     return LBM_OK;
@@ -1325,8 +1340,9 @@ lbm_status lbm_set_fields(lbm_handle *h, int32_t which, const void *src, int32_t
         LBM_CUDA(wd_from_f32(h, conv, h->wd_scale, h->stream));
     } else {
         void *dst = which == LBM_FIELD_W ? h->w[h->parity] : h->wd;
-        LBM_CUDA(cudaMemcpy2DAsync(dst, (size_t)h->pitch * h->esize, src, row, row, (size_t)h->grid.ny,
-                                   src_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream));
+        if (src_on_device) LBM_CUDA(plane_in(h, dst, src, h->grid.nx));
+        else LBM_CUDA(cudaMemcpy2DAsync(dst, (size_t)h->pitch * h->esize, src, row, row, (size_t)h->grid.ny,
+                                        cudaMemcpyHostToDevice, h->stream));
         if (which == LBM_FIELD_W) {
             cudaError_t e = h->esize == 4
                 ? launch_fill_pads<float>(static_cast<float *>(dst), h->pitch, h->grid.nx, h->grid.ny, h->grid.edge, h->stream)
