@@ -506,13 +506,10 @@ lbm_status finalize(lbm_handle *h)
     return LBM_OK;
 }
 
-lbm_status check_sticky(lbm_handle *h)
+// The state and the error word, after everything enqueued so far, in one
+// synchronisation.
+lbm_status read_state(lbm_handle *h, CrackState &hs, uint32_t &err)
 {
-    if (h->sticky != LBM_OK) return fail(h->sticky, "the handle is in an error state");
-    lbm_status rc = finalize(h);
-    if (rc != LBM_OK) return rc;
-    CrackState hs;
-    uint32_t err = 0;
     cudaError_t e = cudaMemcpyAsync(&hs, h->st + h->parity, sizeof hs, cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&err, h->err, sizeof err, cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -520,6 +517,12 @@ lbm_status check_sticky(lbm_handle *h)
         h->sticky = LBM_ERR_CUDA;
         return cuda_fail(e, "synchronising the lattice stream");
     }
+    return LBM_OK;
+}
+
+// The sticky device errors they tell of.
+lbm_status sticky_of(lbm_handle *h, const CrackState &hs, uint32_t err)
+{
     if (err & ERR_TIMEOUT) {
         h->sticky = LBM_ERR_TIMEOUT;
         return fail(LBM_ERR_TIMEOUT, "a bounded device wait gave up (grid barrier of a persistent batched step or of a launch of several passes)");
@@ -529,6 +532,17 @@ lbm_status check_sticky(lbm_handle *h)
         return fail(LBM_ERR_UNSTABLE, "non-finite value in the fields or in K");
     }
     return LBM_OK;
+}
+
+lbm_status check_sticky(lbm_handle *h)
+{
+    if (h->sticky != LBM_OK) return fail(h->sticky, "the handle is in an error state");
+    lbm_status rc = finalize(h);
+    if (rc != LBM_OK) return rc;
+    CrackState hs;
+    uint32_t err = 0;
+    rc = read_state(h, hs, err);
+    return rc == LBM_OK ? sticky_of(h, hs, err) : rc;
 }
 
 }  // namespace host
@@ -1533,8 +1547,9 @@ lbm_status crack_state_impl(lbm_handle *h, bool left, lbm_crack_state_t *now, do
     lbm_status rc = finalize(h);
     if (rc != LBM_OK) return rc;
     CrackState hs;
-    LBM_CUDA(cudaMemcpyAsync(&hs, h->st + h->parity, sizeof hs, cudaMemcpyDeviceToHost, h->stream));
-    LBM_CUDA(cudaStreamSynchronize(h->stream));
+    uint32_t err = 0;
+    rc = read_state(h, hs, err);
+    if (rc != LBM_OK) return rc;
     const TipState &E = left ? hs.l : hs.r;
     int64_t n_cut = hs.i_last >= hs.i_first ? (int64_t)(hs.i_last - hs.i_first + 1) : 0;
     if (h->line && now) {
@@ -1565,26 +1580,25 @@ lbm_status crack_state_impl(lbm_handle *h, bool left, lbm_crack_state_t *now, do
         n = hs.hist_n < hcap ? hs.hist_n : hcap;
         if (n > cap) n = cap;
         const int64_t first = hs.hist_n - n;
-        std::vector<double> K((size_t)hcap), v((size_t)hcap);
-        std::vector<int64_t> tip((size_t)hcap);
-        std::vector<int32_t> np((size_t)hcap);
-        LBM_CUDA(cudaMemcpyAsync(K.data(), left ? h->hist.Kl : h->hist.K, (size_t)hcap * 8, cudaMemcpyDeviceToHost, h->stream));
-        LBM_CUDA(cudaMemcpyAsync(v.data(), left ? h->hist.vl : h->hist.v, (size_t)hcap * 8, cudaMemcpyDeviceToHost, h->stream));
-        LBM_CUDA(cudaMemcpyAsync(tip.data(), left ? h->hist.tipl : h->hist.tip, (size_t)hcap * 8, cudaMemcpyDeviceToHost,
-                                 h->stream));
-        LBM_CUDA(cudaMemcpyAsync(np.data(), left ? h->hist.npl : h->hist.np, (size_t)hcap * 4, cudaMemcpyDeviceToHost,
-                                 h->stream));
+        // the records asked for, straight from the ring (one or two runs of it)
+        auto copy = [&](auto *dst, const auto *ring) {
+            for (int64_t q = 0; dst && q < n;) {
+                const int64_t at = (first + q) % hcap, m = std::min(n - q, hcap - at);
+                const cudaError_t e = cudaMemcpyAsync(dst + q, ring + at, (size_t)m * sizeof *dst, cudaMemcpyDeviceToHost, h->stream);
+                if (e != cudaSuccess) return e;
+                q += m;
+            }
+            return cudaSuccess;
+        };
+        LBM_CUDA(copy(K_hist, left ? h->hist.Kl : h->hist.K));
+        LBM_CUDA(copy(v_hist, left ? h->hist.vl : h->hist.v));
+        LBM_CUDA(copy(tip_hist, left ? h->hist.tipl : h->hist.tip));
+        LBM_CUDA(copy(npairs_hist, left ? h->hist.npl : h->hist.np));
         LBM_CUDA(cudaStreamSynchronize(h->stream));
-        for (int64_t q = 0; q < n; ++q) {
-            const size_t r = (size_t)((first + q) % hcap);
-            if (K_hist) K_hist[q] = K[r];
-            if (v_hist) v_hist[q] = v[r];
-            if (tip_hist) tip_hist[q] = tip[r];
-            if (npairs_hist) npairs_hist[q] = np[r];
-        }
     }
     if (n_written) *n_written = n;
-    return check_sticky(h);
+    if (h->sticky != LBM_OK) return fail(h->sticky, "the handle is in an error state");
+    return sticky_of(h, hs, err);
 }
 
 }  // namespace

@@ -87,6 +87,11 @@ def cases():
         ("two_wide_windows", _strip(400, 90, mode="kcrit", K_C=KC, start=150.0, tip=158.0, two_tips=True, fit_width=5.0,
                                     r0=1.0), "f32", 64),
         ("far_window", _strip(400, 90, mode="kcrit", K_C=KC, tip=150.0, r_min=30.0), "f32", 64),
+        ("many_tiles", _strip(3072, 1700, mode="kcrit", K_C=KC), "f32", 45),
+        ("many_tiles_periodic", _strip(3001, 1777, bc="bounceback", v_rel=0.5, start=1000.0, tip=1200.0,
+                                     edges=("periodic", "periodic", "dirichlet", "free")), "f32_f16", 41),
+        ("many_tiles_no_crack", _strip(2900, 2000, mode=None), "f32_lf", 37),
+        ("many_tiles_bf16", _strip(3500, 1500, v_rel=0.5), "f32_bf16", 26),
         ("tall", _strip(120, 1500, mode="kcrit", K_C=KC), "f32", 40),
         ("example", W.kcrit_centre_crack(), "f32", 200),
     ]
