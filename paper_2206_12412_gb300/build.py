@@ -18,7 +18,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD_DIR = os.path.join(PKG, "_build")
 LIB_PATH = os.path.join(PKG, "liblbm.so")
 SOURCES = ["lbm_kernels.cu", "lbm_adjoint.cu", "lbm_api.cu", "lbm_tape.cu", "lbm_decomp.cu", "lbm_d2q9.cu", "lbm_line.cu",
-           "lbm_pass.cu", "lbm_pass16.cu", "lbm_pass_tape.cu", "lbm_pass_batch.cu", "lbm_pass9.cu",
+           "lbm_pass.cu", "lbm_pass16.cu", "lbm_pass_tape.cu", "lbm_pass_batch.cu", "lbm_pass9.cu", "lbm_pass_f64.cu",
            "lbm_pass_plan.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["--split-compile=0", "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2", "-I" + INCLUDE, "-I" + CSRC]

@@ -405,7 +405,9 @@ cudaError_t enqueue_pass(const lbm_handle *h, const lbm::PassPlan &q, int par, b
     case LBM_F32_WD_BF16: return enqueue_pass_t<float, __nv_bfloat16>(h, q, par, second, n_pass, s);
     case LBM_F32_WD_F16: return enqueue_pass_t<float, __half>(h, q, par, second, n_pass, s);
     case LBM_F32_LEAPFROG: return enqueue_pass_t<float, Lf>(h, q, par, second, n_pass, s);
-    default: return enqueue_pass_t<double, double>(h, q, par, second, n_pass, s);
+    default:
+        return h->pass_narrow ? enqueue_pass_t<double, lbm::NarrowF64>(h, q, par, second, n_pass, s)
+                              : enqueue_pass_t<double, double>(h, q, par, second, n_pass, s);
     }
 }
 
@@ -1240,7 +1242,7 @@ lbm_status lbm_step(lbm_handle *h, int64_t n)
         if (h->pass_k && !h->own_bands && !h->bulk) {
             auto go = [&](int K, int64_t m) -> lbm_status {
                 lbm::PassPlan q;
-                if (!pass_plan(h, K, h->pass_nw, h->pass_rpt, q)) return fail(LBM_ERR_ARG, "no plan of a pass");
+                if (!pass_plan(h, K, h->pass_nw, h->pass_rpt, q, false, h->pass_narrow)) return fail(LBM_ERR_ARG, "no plan of a pass");
                 if (q.tiles <= h->pass_slots) {
                     // every tile resident: the passes in one launch
                     for (; m > 0; m -= std::min(m, kMaxPasses))
@@ -1255,7 +1257,8 @@ lbm_status lbm_step(lbm_handle *h, int64_t n)
             };
             auto pair = [&](int Ka, int Kb) -> lbm_status {
                 lbm::PassPlan qa, qb;
-                if (!pass_plan(h, Ka, h->pass_nw, h->pass_rpt, qa) || !pass_plan(h, Kb, h->pass_nw, h->pass_rpt, qb))
+                if (!pass_plan(h, Ka, h->pass_nw, h->pass_rpt, qa, false, h->pass_narrow) ||
+                    !pass_plan(h, Kb, h->pass_nw, h->pass_rpt, qb, false, h->pass_narrow))
                     return fail(LBM_ERR_ARG, "no plan of a pass");
                 LBM_CUDA(enqueue_pass(h, qa, par, false, 1, h->stream));
                 LBM_CUDA(enqueue_pass(h, qb, par ^ 1, true, 1, h->stream));

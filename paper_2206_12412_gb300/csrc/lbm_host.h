@@ -130,6 +130,7 @@ struct lbm_handle {
     // that the buffers end where an even number of single steps leaves them
     lbm::host::ChunkGraph passes;  // graphs of runs of passes of pass_k steps
     int32_t pass_k;      // steps of a pass (0: single steps only)
+    bool pass_narrow;    // FP64: one column a thread
     int32_t pass_slots;  // tiles resident at once
     int32_t pass_nw, pass_rpt;   // warps of its tiles, rows per thread of the bulk ones
     lbm::GridBarrier *pass_bar;  // of the cooperative launches of several passes, device
@@ -211,8 +212,10 @@ inline void make_step_args(const lbm_handle *h, int par, StepArgs<T, D> &a)
 // The tiles of a pass of K steps of this lattice (lbm_pass_plan.cu); false
 // where a pass of K steps cannot be split so that every tile that needs a
 // crack decision holds what decides it.
-// adjoint: the plan of the sweep's transposed steps.
-bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, lbm::PassPlan &q, bool adjoint = false);
+// adjoint: the plan of the sweep's transposed steps; narrow: one column a
+// thread (FP64).
+bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, lbm::PassPlan &q, bool adjoint = false,
+               bool narrow = false);
 // Choose the pass of this lattice: h->pass_k, h->pass_nw, h->pass_rpt.
 void choose_pass(lbm_handle *h);
 

@@ -219,10 +219,12 @@ struct PassPlan {
     int64_t w_q;               // the window's width
     double k_inv;              // 1 / K_C
     float k_unit, k_rest;      // mu / 4 sqrt(2 pi / dh) 2^16; just below K_C
-    int32_t mx, px;            // column tiles of the bulk and their width
-    int32_t jb, mb, pb;        // rows [0, jb) below the strip: mb row tiles of pb rows
-    int32_t jt, mt, pt;        // rows [jt, ny) above it (a lattice without a crack: all rows)
+    // column tiles of the bulk: of px vectors, the first ex of them of one more
+    int32_t mx, px, ex;
+    int32_t jb, mb, pb, eb;    // rows [0, jb) below the strip: mb row tiles of pb rows, the first eb of one more
+    int32_t jt, mt, pt, et;    // rows [jt, ny) above it (a lattice without a crack: all rows)
     int32_t ms, ps;            // column tiles of the strip and their nominal width
+    int32_t free;              // narrow tiles: the strip's columns as the bulk's (the cuts need no K, a window holds at most one pair)
     int32_t zb, za;            // strip: no tile boundary less than zb behind or up to za ahead of a tip
     int32_t grow, back;        // strip: the columns ahead of and behind an end's next that a pass can cut
     int32_t tiles, edge_macro;
@@ -366,6 +368,7 @@ cudaError_t launch_batch_pieces(const StepArgs<T, D> *descs, const BatchPiece *p
 template <typename T, typename D>
 cudaError_t launch_step(const StepArgs<T, D> &a, int bands, cudaStream_t s, bool bulk = false);
 // n_pass passes of several time steps (more than one: one cooperative launch).
+struct NarrowF64;
 template <typename T, typename D, int MODE = kForward>
 cudaError_t launch_pass(const PassArgs<T, D> &a, int n_pass, cudaStream_t s);
 template <typename T, typename D, int MODE = kForward> const void *pass_kernel_ptr(int nw, int rpt, bool run);

@@ -52,6 +52,28 @@ namespace lbm {
 constexpr int kPassSteps = 8;     // most steps of a pass (and no more than a tile has warps)
 constexpr int kStripRpt = 4;      // rows per thread of a strip tile
 
+// FP64 storage taken one column a thread (32-column tiles of four warps): FP64
+// runs at two results a cycle and SM, so a pass lasts as long as its busiest
+// SM's tile, and on small lattices the tiles have to be many and small (128^2
+// with a stationary crack: 4.4 -> 3.2 us per step, 256^2 prescribed 5.9 -> 4.8).
+// Where the decisions need no K, a strip tile lies anywhere (PassPlan::free):
+// 32 columns would not hold the zones around the tips.
+struct NarrowF64 {
+    double v;
+};
+template <> struct WdIO<NarrowF64> {
+    typedef Row<double, 1> Raw;
+    static __device__ __forceinline__ void fetch(const NarrowF64 *p, Raw &r) { r.v[0] = p->v; }
+    static __device__ __forceinline__ void unpack(const Raw &q, Row<double, 1> &r, double) { r = q; }
+    static __device__ __forceinline__ void store(NarrowF64 *p, const Row<double, 1> &r, double) { p->v = r.v[0]; }
+    static __device__ __forceinline__ void put(NarrowF64 *p, double v, double) { p->v = v; }
+};
+template <typename T, typename D> struct PassVec { static constexpr int N = Vec<T>::N; };
+template <> struct PassVec<double, NarrowF64> { static constexpr int N = 1; };
+__device__ __forceinline__ void ldg_row(const double *p, Row<double, 1> &r) { r.v[0] = __ldg(p); }
+__device__ __forceinline__ void ld_row(const double *p, Row<double, 1> &r) { r.v[0] = *p; }
+__device__ __forceinline__ void stg_row(double *p, const Row<double, 1> &r) { *p = r.v[0]; }
+
 // One site's wdot as the next step reads it back from storage.
 template <typename D, typename T> __device__ __forceinline__ T wd_round(T v, T, T) { return v; }
 template <> __device__ __forceinline__ float wd_round<__nv_bfloat16, float>(float v, float, float)
@@ -222,9 +244,9 @@ struct PassTip {
     int32_t arr_r, arr_l, lazy, pad;
 };
 
-template <typename T, int NW>
+template <typename T, int NW, int N = Vec<T>::N>
 struct PassShared {
-    static constexpr int W = 32 * Vec<T>::N;
+    static constexpr int W = 32 * N;
     alignas(16) T top[2][NW][W];    // each warp's last row, by step parity
     alignas(16) T bot[2][NW][W];    // each warp's first row
     alignas(16) T pair[kPassSteps][2][W];   // rows jc - 1 and jc of a strip tile at each step
@@ -306,16 +328,6 @@ __device__ __forceinline__ PassPair pass_pair(int dir, int64_t tip, int64_t lo_q
     r.in = r.d >= lo_q && r.d < hi_q && i >= f && i <= l;
     r.col = (int)i;
     return r;
-}
-// a / b for a divisor known in advance, y = 1 / b rounded: the residual of a y
-// is exact in one FMA, and adding its share rounds to the quotient (Markstein,
-// IBM J. Res. Dev. 34, 1990; equal to the division in 1.2e8 random quotients
-// over the divisors used here).  Three FP64 instructions instead of ten, at
-// 64 cycles each.
-__device__ __forceinline__ double div_known(double a, double b, double y)
-{
-    const double q = a * y;
-    return fma(fma(-q, b, a), y, q);
 }
 
 // sqrt(r / 2 pi) of a pair, and K from it (the sums of crack_eval_pairs over one pair).
@@ -573,6 +585,7 @@ __device__ __forceinline__ void cg_row(const float *p, Row<float, 4> &r)
     const float4 q = __ldcg(reinterpret_cast<const float4 *>(p));
     r.v[0] = q.x; r.v[1] = q.y; r.v[2] = q.z; r.v[3] = q.w;
 }
+__device__ __forceinline__ void cg_row(const double *p, Row<double, 1> &r) { r.v[0] = __ldcg(p); }
 __device__ __forceinline__ void cg_row(const double *p, Row<double, 2> &r)
 {
     const double2 q = __ldcg(reinterpret_cast<const double2 *>(p));
@@ -581,6 +594,7 @@ __device__ __forceinline__ void cg_row(const double *p, Row<double, 2> &r)
 template <typename D, typename Raw> __device__ __forceinline__ void cg_raw(const D *p, Raw &r)
 {
     if constexpr (std::is_same<D, Lf>::value) cg_row(reinterpret_cast<const float *>(p), r);
+    else if constexpr (std::is_same<D, NarrowF64>::value) cg_row(reinterpret_cast<const double *>(p), r);
     else if constexpr (sizeof(D) == 2) r = __ldcg(reinterpret_cast<const uint2 *>(p));
     else cg_row(p, r);
 }
@@ -588,6 +602,7 @@ template <typename T> __device__ __forceinline__ T cg_get(const T *p) { return _
 template <typename D, typename T> __device__ __forceinline__ T cg_rate_get(const D *p, T inv)
 {
     if constexpr (std::is_same<D, Lf>::value) return __ldcg(reinterpret_cast<const float *>(p));
+    else if constexpr (std::is_same<D, NarrowF64>::value) return __ldcg(reinterpret_cast<const double *>(p));
     else if constexpr (sizeof(D) == 2) {
         const unsigned short u = __ldcg(reinterpret_cast<const unsigned short *>(p));
         if constexpr (std::is_same<D, __half>::value) return __half2float(__ushort_as_half(u)) * inv;
@@ -641,7 +656,7 @@ struct PassCtx {
 // planes change places; the other forms shift the rows of w by one slot, up
 // in one step (PH = 0, rows swept upwards) and down in the next (PH = 1).
 template <typename T, typename D, int RPT> struct PassRows {
-    static constexpr int N = Vec<T>::N;
+    static constexpr int N = PassVec<T, D>::N;
     typedef Row<T, N> R;
     static constexpr bool kLf = std::is_same<D, Lf>::value;
     R a[RPT + (kLf ? 0 : 1)];
@@ -671,7 +686,7 @@ template <typename T, typename D, int RPT> struct PassRows {
 template <typename T, typename D, int RPT, typename F>
 __device__ __forceinline__ void pass_edge_rows(const PassArgs<T, D> &A, const PassCtx &c, int s, F &&row)
 {
-    constexpr int N = Vec<T>::N;
+    constexpr int N = PassVec<T, D>::N;
     const PassAdj<T> &d = A.adj;
     const int64_t n = c.n - s;
     if (n < 0 || n >= d.n_steps || !(c.on_edge || c.side)) return;
@@ -707,9 +722,9 @@ __device__ __forceinline__ void pass_edge_rows(const PassArgs<T, D> &A, const Pa
 // One time step of a tile.
 template <typename T, typename D, int NW, int RPT, int KIND, int PH, int MODE>
 __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx &c, int s, PassRows<T, D, RPT> &F,
-                                          PassShared<T, NW> &sh, PassSensors<T, MODE> &sen, PassWindow &win)
+                                          PassShared<T, NW, PassVec<T, D>::N> &sh, PassSensors<T, MODE> &sen, PassWindow &win)
 {
-    constexpr int N = Vec<T>::N;
+    constexpr int N = PassVec<T, D>::N;
     constexpr int kBelowWarp = NW / 2 - 1;   // strip: the warp whose last row is jc - 1; the next one's first is jc
     constexpr bool kLf = std::is_same<D, Lf>::value;
     typedef Row<T, N> R;
@@ -807,7 +822,7 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
     if (MODE != kAdjoint && KIND == 2 && c.follow) {
         const bool reach = sh.reach[b] != 0;
         if (warp == 0) {
-            pass_crack_step<T, PassShared<T, NW>::W>(p, A.q, sh.top[b][kBelowWarp], sh.bot[b][kBelowWarp + 1], c.org_r,
+            pass_crack_step<T, PassShared<T, NW, PassVec<T, D>::N>::W>(p, A.q, sh.top[b][kBelowWarp], sh.bot[b][kBelowWarp + 1], c.org_r,
                                                      c.org_l, sh.S, sh.log[s + 1], c.ev_r, c.ev_l, win);
             // (D2Q9: any advance can pass a diagonal crossing)
             if (lane == 0) sh.reach[b ^ 1] = kNineQ || crack_cut_in_reach(p, sh.S) ? 1 : 0;
@@ -1030,7 +1045,7 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
             oB = cut[k] && !below ? wB.v[k] : oB;
         }
     }
-    if (em) {
+    if constexpr (N > 1) if (em) {
         // the macroscopic rule on the outer edges (the two levels of
         // edge_rule_at): the edge columns, the crack-face points on
         // them, then the bottom and top rows and the corners
@@ -1247,10 +1262,10 @@ __device__ __forceinline__ void pass_misfits(const PassArgs<T, D> &A, const Pass
 // outer edges, 2 a crack-strip tile (with edges where it meets them).
 template <typename T, typename D, int NW, int RPT, int KIND, bool COOP, int MODE>
 __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf<T, D> &B, const TileGeo g,
-                                          PassShared<T, NW> &sh, PassSensors<T, MODE> &sen)
+                                          PassShared<T, NW, PassVec<T, D>::N> &sh, PassSensors<T, MODE> &sen)
 {
-    constexpr int N = Vec<T>::N;
-    constexpr int W = PassShared<T, NW>::W;
+    constexpr int N = PassVec<T, D>::N;
+    constexpr int W = PassShared<T, NW, PassVec<T, D>::N>::W;
     typedef Row<T, N> R;
     const unsigned kFull = 0xffffffffu;
     const StepArgs<T, D> &a = A.s;
@@ -1380,7 +1395,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
                 pass_window(A.q, sh.S, lane < 16 ? c.org_r : c.org_l, lane < 16 ? c.ev_r : c.ev_l, win);
             }
         }
-        if ((c.own_r || c.own_l) && A.q.one_pair && warp == 1 && lane < 2 * kPassSteps) {
+        if ((c.own_r || c.own_l || (N == 1 && A.q.free)) && A.q.one_pair && warp == 1 && lane < 2 * kPassSteps) {
             // the part of the K fits that needs no fields (an FP64 root and
             // division), while the loads are under way: lane st of the right
             // end, st + 8 of the left, for the tip before update st (K-
@@ -1501,7 +1516,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
     if (__any_sync(kFull, !isfinite(acc)) && lane == 0) atomicOr(a.err, (uint32_t)ERR_NONFINITE);
 
     if constexpr (MODE == kRecord) pass_misfits<T, D, NW>(A, B, sen);
-    if (MODE != kAdjoint && KIND == 2 && (c.own_r || c.own_l)) {
+    if (MODE != kAdjoint && KIND == 2 && (c.own_r || c.own_l || (N == 1 && A.q.free))) {
         __syncthreads();   // the last crack step
         // the records of the pass's crack steps, and the K fits their decisions
         // did not wait for.  A window of one spacing holds at most one pair, so
@@ -1549,22 +1564,45 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
         const double v_prev = p.mode == CRACK_PRESCRIBED ? p.v_rel : 0.0;
         if (A.q.one_pair) {
             const int st = lane & (kPassSteps - 1), dir = lane < kPassSteps ? +1 : -1;
-            if (warp == 1 && lane < 2 * kPassSteps && st >= rec0 && st < K && (dir > 0 ? c.own_r : c.own_l)) {
-                double Kf = 0.0;
-                int np = 0;
-                if (sh.log[st + 1].lazy) {
-                    const PassTip &q = sh.log[st];
-                    const int64_t tip = dir > 0 ? q.tr : q.tl;
-                    PassPair w = pass_pair(dir, tip, A.q.lo_q, A.q.hi_q, q.f, q.l);
-                    if (tip != fit_tip || w.in != fit_pair.in) fit_sf = w.in ? pass_sf(p, w.d) : 0.0;   // it has moved since
-                    const int e = w.col - (dir > 0 ? c.org_r : c.org_l);
-                    if (w.in && e >= 0 && e < W) {
-                        const CrackSums f = pass_sums<T>(fit_sf, sh.pair[st][1][e], sh.pair[st][0][e], 0.0);
-                        Kf = pass_K(p, f);
-                        np = 1;
+            if constexpr (N == 1) {
+                bool mine = dir > 0 ? c.own_r : c.own_l;
+                if (warp == 1 && lane < 2 * kPassSteps && st >= rec0 && st < K && (mine || (A.q.free && (dir > 0 || p.two_tips)))) {
+                    double Kf = 0.0;
+                    int np = 0;
+                    if (sh.log[st + 1].lazy) {
+                        const PassTip &q = sh.log[st];
+                        const int64_t tip = dir > 0 ? q.tr : q.tl;
+                        PassPair w = pass_pair(dir, tip, A.q.lo_q, A.q.hi_q, q.f, q.l);
+                        if (tip != fit_tip || w.in != fit_pair.in) fit_sf = w.in ? pass_sf(p, w.d) : 0.0;   // it has moved since
+                        // (free: the tile that owns the step's pair forms it, whichever tile owns the tip)
+                        if (A.q.free && w.in) mine = w.col >= g.x0 && w.col < g.x1;
+                        const int e = w.col - (A.q.free ? g.xl : (dir > 0 ? c.org_r : c.org_l));
+                        if (w.in && e >= 0 && e < W) {
+                            const CrackSums f = pass_sums<T>(fit_sf, sh.pair[st][1][e], sh.pair[st][0][e], 0.0);
+                            Kf = pass_K(p, f);
+                            np = 1;
+                        }
                     }
+                    if (mine) record(st, dir, Kf, np, A.q.r_min);
                 }
-                record(st, dir, Kf, np, A.q.r_min);
+            } else {
+                if (warp == 1 && lane < 2 * kPassSteps && st >= rec0 && st < K && (dir > 0 ? c.own_r : c.own_l)) {
+                    double Kf = 0.0;
+                    int np = 0;
+                    if (sh.log[st + 1].lazy) {
+                        const PassTip &q = sh.log[st];
+                        const int64_t tip = dir > 0 ? q.tr : q.tl;
+                        PassPair w = pass_pair(dir, tip, A.q.lo_q, A.q.hi_q, q.f, q.l);
+                        if (tip != fit_tip || w.in != fit_pair.in) fit_sf = w.in ? pass_sf(p, w.d) : 0.0;   // it has moved since
+                        const int e = w.col - (dir > 0 ? c.org_r : c.org_l);
+                        if (w.in && e >= 0 && e < W) {
+                            const CrackSums f = pass_sums<T>(fit_sf, sh.pair[st][1][e], sh.pair[st][0][e], 0.0);
+                            Kf = pass_K(p, f);
+                            np = 1;
+                        }
+                    }
+                    record(st, dir, Kf, np, A.q.r_min);
+                }
             }
         } else if (warp >= rec0 && warp < K) {
             for (int dir = 1; dir >= (c.own_l ? -1 : 1); dir -= 2) {
@@ -1640,12 +1678,15 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
     }
 }
 
+// Where the i-th of the tiles of `len` items begins, the first `more` of them of one more.
+__device__ __forceinline__ int pass_split(int i, int len, int more) { return i * len + min(i, more); }
+
 // Tile t of a pass.
 template <typename T, typename D, int NW, int RPT, bool COOP, int MODE>
-__device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<T, D> &B, int t, PassShared<T, NW> &sh,
+__device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<T, D> &B, int t, PassShared<T, NW, PassVec<T, D>::N> &sh,
                                          PassSensors<T, MODE> &sen)
 {
-    constexpr int N = Vec<T>::N;
+    constexpr int N = PassVec<T, D>::N;
     const StepArgs<T, D> &a = A.s;
     const PassPlan &q = A.q;
     const int nx = a.nx, ny = a.ny;
@@ -1679,8 +1720,8 @@ __device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<
     TileGeo g;
     if (MODE == kAdjoint && t < q.ms) {
         // the recorded cuts need no tips: columns as the bulk splits them
-        g.x0 = t * q.ps;
-        g.x1 = min(g.x0 + q.ps, nx);
+        g.x0 = N * pass_split(t, q.px, q.ex);
+        g.x1 = min(N * pass_split(t + 1, q.px, q.ex), nx);
         g.xl = g.x0 == 0 && !per ? 0 : g.x0 - q.hc;
         g.yl = a.p.jc - NW * kStripRpt / 2;
         g.y0 = q.jb;
@@ -1699,9 +1740,14 @@ __device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<
             hi0 = max(hi0, hi1);
             two = false;
         }
-        g.x0 = t == 0 && !per ? 0 : pass_boundary<N>(t * q.ps, nx, per, lo0, hi0, lo1, hi1, two);
-        if (t + 1 < q.ms) g.x1 = pass_boundary<N>((t + 1) * q.ps, nx, per, lo0, hi0, lo1, hi1, two);
-        else g.x1 = per ? nx + pass_boundary<N>(0, nx, per, lo0, hi0, lo1, hi1, two) : nx;
+        if (N == 1 && q.free) {
+            g.x0 = N * pass_split(t, q.px, q.ex);
+            g.x1 = min(N * pass_split(t + 1, q.px, q.ex), nx);
+        } else {
+            g.x0 = t == 0 && !per ? 0 : pass_boundary<N>(t * q.ps, nx, per, lo0, hi0, lo1, hi1, two);
+            if (t + 1 < q.ms) g.x1 = pass_boundary<N>((t + 1) * q.ps, nx, per, lo0, hi0, lo1, hi1, two);
+            else g.x1 = per ? nx + pass_boundary<N>(0, nx, per, lo0, hi0, lo1, hi1, two) : nx;
+        }
         if (q.ms == 1) {
             g.x0 = 0;
             g.x1 = nx;
@@ -1716,14 +1762,14 @@ __device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<
     }
     t -= q.ms;
     const int cx = t % q.mx, ry = t / q.mx;
-    g.x0 = cx * q.px;
-    g.x1 = min(g.x0 + q.px, nx);
+    g.x0 = N * pass_split(cx, q.px, q.ex);
+    g.x1 = min(N * pass_split(cx + 1, q.px, q.ex), nx);
     if (ry < q.mb) {
-        g.y0 = ry * q.pb;
-        g.y1 = min(g.y0 + q.pb, q.jb);
+        g.y0 = pass_split(ry, q.pb, q.eb);
+        g.y1 = pass_split(ry + 1, q.pb, q.eb);
     } else {
-        g.y0 = q.jt + (ry - q.mb) * q.pt;
-        g.y1 = min(g.y0 + q.pt, ny);
+        g.y0 = q.jt + pass_split(ry - q.mb, q.pt, q.et);
+        g.y1 = q.jt + pass_split(ry - q.mb + 1, q.pt, q.et);
     }
     g.xl = g.x0 == 0 && !per ? 0 : g.x0 - q.hc;
     g.yl = g.y0 == 0 ? 0 : (g.y1 == ny ? ny - NW * RPT : g.y0 - q.K);
@@ -1736,7 +1782,7 @@ __device__ __forceinline__ void pass_cta(const PassArgs<T, D> &A, const PassBuf<
 template <typename T, typename D, int NW, int RPT, int MODE>
 __global__ void __launch_bounds__(32 * NW, 16 / NW) pass_kernel(const __grid_constant__ PassArgs<T, D> a)
 {
-    __shared__ PassShared<T, NW> sh;
+    __shared__ PassShared<T, NW, PassVec<T, D>::N> sh;
     __shared__ PassSensors<T, MODE> sen;
     pdl_wait();
     pdl_trigger();
@@ -1752,7 +1798,7 @@ template <typename T, typename D, int NW, int RPT, int MODE>
 __global__ void __launch_bounds__(32 * NW, 16 / NW)
     pass_run_kernel(const __grid_constant__ PassArgs<T, D> a, int n_pass)
 {
-    __shared__ PassShared<T, NW> sh;
+    __shared__ PassShared<T, NW, PassVec<T, D>::N> sh;
     __shared__ PassSensors<T, MODE> sen;
     for (int it = 0; it < n_pass; ++it) {
         const bool odd = (it & 1) != 0;
@@ -1800,7 +1846,10 @@ cudaError_t launch_pass_batch(const PassArgs<T, D> *descs, const BatchUnit *unit
 
 template <typename T, typename D, int MODE> const void *pass_kernel_ptr(int nw, int rpt, bool run)
 {
-    if constexpr (sizeof(T) == 8)
+    if constexpr (PassVec<T, D>::N == 1)
+        return run ? reinterpret_cast<const void *>(&pass_run_kernel<T, D, 4, 4, MODE>)
+                   : reinterpret_cast<const void *>(&pass_kernel<T, D, 4, 4, MODE>);
+    else if constexpr (sizeof(T) == 8)
         if (nw == 4)
             return run ? reinterpret_cast<const void *>(&pass_run_kernel<T, D, 4, 4, MODE>)
                        : reinterpret_cast<const void *>(&pass_kernel<T, D, 4, 4, MODE>);
@@ -1808,8 +1857,9 @@ template <typename T, typename D, int MODE> const void *pass_kernel_ptr(int nw, 
         if (rpt == 4)
             return run ? reinterpret_cast<const void *>(&pass_run_kernel<T, D, 8, 4, MODE>)
                        : reinterpret_cast<const void *>(&pass_kernel<T, D, 8, 4, MODE>);
-    return run ? reinterpret_cast<const void *>(&pass_run_kernel<T, D, 8, 8, MODE>)
-               : reinterpret_cast<const void *>(&pass_kernel<T, D, 8, 8, MODE>);
+    if constexpr (PassVec<T, D>::N > 1)
+        return run ? reinterpret_cast<const void *>(&pass_run_kernel<T, D, 8, 8, MODE>)
+                   : reinterpret_cast<const void *>(&pass_kernel<T, D, 8, 8, MODE>);
 }
 
 template <typename T, typename D, int MODE> cudaError_t launch_pass(const PassArgs<T, D> &a, int n_pass, cudaStream_t s)

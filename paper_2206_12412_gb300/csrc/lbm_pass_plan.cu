@@ -14,34 +14,46 @@ namespace {
 int ceil_div(int a, int b) { return (a + b - 1) / b; }
 int round_up(int a, int n) { return ceil_div(a, n) * n; }
 
-// FP64 lattices up to kPass64Sites sites are stepped in passes, those up to
-// kPass64Small in tiles of four warps.
-constexpr int64_t kPass64Sites = (int64_t)1 << 19, kPass64Small = (int64_t)1 << 17;
+// FP64 runs at two results a cycle and SM, so recomputed halos cost more than
+// saved launches and traffic give once every SM has its tile.
+// Time per step in passes and (in parentheses) in single steps, K-criterion:
+// 128^2 6.8 (9.3), 362^2 10.4 (11.1), 512^2 10.1 (13.3), 724^2 18.4 (14.2),
+// 1024 x 512 18.4 us (14.3 us): passes while there are no more tiles of eight
+// warps than SMs.  The edge rule: 512 x 256 11.7 (15.2), 512^2 19.9 us (16.1 us):
+// up to kPass64Small sites, which take tiles of four warps.  Up to
+// kPass64Narrow they are one column a thread (a stationary crack on 128^2:
+// 3.2 us, two columns a thread 4.5 us, single steps 10.9 us).
+constexpr int64_t kPass64Small = (int64_t)1 << 17, kPass64Narrow = (int64_t)1 << 16;
+
+// n items in m tiles: of p, the first e of one more.
+void even(int n, int m, int &p, int &e)
+{
+    p = m > 0 ? n / m : 0;
+    e = m > 0 ? n % m : 0;
+}
 
 // Row tiles of H held rows, K of them halo on each side that is no lattice
-// edge, over a region of `len` rows; at least `least` tiles.
-void split_rows(int len, int H, int K, bool edge0, bool edge1, int least, int &m, int &p)
+// edge, over a region of `len` rows; at least `least` tiles.  Even: the rules
+// next to an edge span three rows of a tile.
+void split_rows(int len, int H, int K, bool edge0, bool edge1, int least, int &m, int &p, int &e)
 {
     m = 0;
-    p = 1;
-    if (len <= 0) return;
-    const int one = H - (edge0 ? 0 : K) - (edge1 ? 0 : K);
-    if (len <= one) m = 1;
-    else if (edge0 && edge1 && len <= 2 * (H - K)) m = 2;
-    else m = ceil_div(len, H - 2 * K);
-    m = std::max(m, std::min(least, len));
-    p = ceil_div(len, m);
-    // no last tile thinner than the three rows the rules next to an edge span
-    while (m > 1 && p > 3 && len - (ceil_div(len, p) - 1) * p < 3) --p;
-    m = ceil_div(len, p);
+    if (len > 0) {
+        const int one = H - (edge0 ? 0 : K) - (edge1 ? 0 : K);
+        if (len <= one) m = 1;
+        else if (edge0 && edge1 && len <= 2 * (H - K)) m = 2;
+        else m = ceil_div(len, H - 2 * K);
+        m = std::max(m, std::min(least, len));
+    }
+    even(len, m, p, e);
 }
 
 }  // namespace
 
-bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q, bool adjoint)
+bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q, bool adjoint, bool narrow)
 {
     const int nx = h->grid.nx, ny = h->grid.ny;
-    const int N = (int)(16 / h->esize), W = 32 * N, H = nw * rpt;
+    const int N = narrow ? 1 : (int)(16 / h->esize), W = 32 * N, H = nw * rpt;
     const int strip_half = nw * 4 / 2;   // kStripRpt rows a warp
     const bool per = h->grid.edge[LBM_LEFT] == LBM_EDGE_PERIODIC;
     const bool crack = h->cp.mode != CRACK_NONE;
@@ -58,15 +70,15 @@ bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q, bool ad
 
     // bulk columns
     const int ow = W - 2 * q.hc;
-    if (nx + (per ? 2 * q.hc : 0) <= W) {
-        q.mx = 1;
-        q.px = nx;
+    if (nx + (per ? 2 * q.hc : 0) <= W) q.mx = 1;
+    else q.mx = !per && nx <= 2 * (W - q.hc) ? 2 : ceil_div(nx, ow);
+    if (N == 1) {
+        even(nx, q.mx, q.px, q.ex);
     } else {
-        q.mx = !per && nx <= 2 * (W - q.hc) ? 2 : ceil_div(nx, ow);
-        q.px = round_up(ceil_div(nx, q.mx), N);
+        q.px = ceil_div(ceil_div(nx, q.mx), N);
         // no last tile narrower than the columns the rules next to an edge span
-        while (nx - (ceil_div(nx, q.px) - 1) * q.px < 4 && q.px > N) q.px -= N;
-        q.mx = ceil_div(nx, q.px);
+        while (nx - (ceil_div(nx, q.px * N) - 1) * q.px * N < 4 && q.px > 1) --q.px;
+        q.mx = ceil_div(nx, q.px * N);
     }
 
     // rows: the crack strip, and the bulk below and above it (all of it without a crack)
@@ -79,10 +91,10 @@ bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q, bool ad
         region1 = std::min(ny, p.jc + so);
         q.jb = region0;
         q.jt = region1;
-        split_rows(q.jb, H, K, true, false, 1, q.mb, q.pb);
-        split_rows(ny - q.jt, H, K, false, true, 1, q.mt, q.pt);
+        split_rows(q.jb, H, K, true, false, 1, q.mb, q.pb, q.eb);
+        split_rows(ny - q.jt, H, K, false, true, 1, q.mt, q.pt, q.et);
     } else {
-        split_rows(ny, H, K, true, true, h->edge_macro ? 2 : 1, q.mt, q.pt);
+        split_rows(ny, H, K, true, true, h->edge_macro ? 2 : 1, q.mt, q.pt, q.et);
     }
     // the edge rule is applied by tiles whose rows 0 .. 2 (or ny-1 .. ny-3) lie
     // in one thread: tiles held from row 0 or up to row ny - 1, not the strip
@@ -91,7 +103,6 @@ bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q, bool ad
 
     if (crack && adjoint) {
         q.ms = q.mx;
-        q.ps = q.px;
     } else if (crack) {
         // columns an end can cut in a pass, and the reach of its K window
         const int64_t dq = p.mode == CRACK_KCRIT ? p.dq_max : p.mode == CRACK_PRESCRIBED ? p.dq_prescribed : 0;
@@ -121,7 +132,10 @@ bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q, bool ad
         q.k_rest = (float)(p.K_C * 0.999);
         // both ends are fitted at once by half a warp each: at most 16 columns
         if (!(p.fit_width / p.dh <= 12.0)) return false;
-        if (nx + (per ? 2 * q.hc : 0) <= W) {
+        q.free = narrow && p.mode != CRACK_KCRIT && q.one_pair;
+        if (q.free) {
+            q.ms = q.mx;
+        } else if (nx + (per ? 2 * q.hc : 0) <= W) {
             q.ms = 1;
             q.ps = nx;
         } else {
@@ -149,36 +163,45 @@ bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q, bool ad
 void choose_pass(lbm_handle *h)
 {
     h->pass_k = 0;
+    h->pass_narrow = false;
     if (!h->alt[0]) return;
     const int64_t sites = (int64_t)h->grid.nx * h->grid.ny;
-    // FP64: two results per cycle and SM, so recomputed halos cost more than
-    // launches save on large lattices, and on small ones the tiles have to be
-    // many and small (see kPass64*)
-    if (h->esize == 8 && sites > kPass64Sites) return;
-    h->pass_nw = h->esize == 8 && sites <= kPass64Small ? 4 : 8;
-    const int kmax = h->esize == 8 ? 4 : 8;
-    for (int K = kmax; K >= 2; --K) {
+    const bool f64 = h->esize == 8;
+    if (f64 && sites > kPass64Small && (h->edge_macro || (h->q == 5 && h->cp.mode != CRACK_KCRIT))) return;
+    auto feasible = [&](int K, bool narrow) {
         PassPlan q;
+        h->pass_nw = f64 && (narrow || sites <= kPass64Small) ? 4 : 8;
         h->pass_rpt = h->pass_nw == 4 ? 4 : 8;
-        if (!pass_plan(h, K, h->pass_nw, h->pass_rpt, q)) continue;
-        if (h->esize == 4 && q.tiles < 2 * h->sms) h->pass_rpt = 4;
-        bool shorter = true;   // every shorter pass too: a call's last passes
-        for (int k = K; k >= 2; --k) shorter = shorter && pass_plan(h, k, h->pass_nw, h->pass_rpt, q);
-        if (!shorter) continue;
-        const void *fn = h->q == 9 ? (h->esize == 8 ? pass_kernel_ptr<double, double, kNine>(h->pass_nw, h->pass_rpt, true)
-                                                    : pass_kernel_ptr<float, float, kNine>(h->pass_nw, h->pass_rpt, true))
-                         : h->lat.storage == LBM_F64           ? pass_kernel_ptr<double, double>(h->pass_nw, h->pass_rpt, true)
-                         : h->lat.storage == LBM_F32_WD_BF16 ? pass_kernel_ptr<float, __nv_bfloat16>(h->pass_nw, h->pass_rpt, true)
-                         : h->lat.storage == LBM_F32_WD_F16  ? pass_kernel_ptr<float, __half>(h->pass_nw, h->pass_rpt, true)
-                         : h->lat.storage == LBM_F32_LEAPFROG ? pass_kernel_ptr<float, Lf>(h->pass_nw, h->pass_rpt, true)
-                                                              : pass_kernel_ptr<float, float>(h->pass_nw, h->pass_rpt, true);
-        int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * h->pass_nw, 0) != cudaSuccess || per_sm < 1)
-            return;
-        h->pass_slots = per_sm * h->sms;
-        h->pass_k = K;
+        if (!pass_plan(h, K, h->pass_nw, h->pass_rpt, q, false, narrow)) return false;
+        if (f64 && sites > kPass64Small && (K < 4 || q.tiles > h->sms)) return false;
+        if (!f64 && q.tiles < 2 * h->sms) h->pass_rpt = 4;
+        bool all = true;   // every shorter pass too: a call's last passes
+        for (int k = K; k >= 2; --k) all = all && pass_plan(h, k, h->pass_nw, h->pass_rpt, q, false, narrow);
+        return all;
+    };
+    // (the edge rule, nine velocities and a tape's passes take two columns a thread)
+    if (f64 && sites <= kPass64Narrow && !h->edge_macro && h->q == 5 && feasible(4, true) && feasible(4, false)) {
+        h->pass_k = 4;
+        h->pass_narrow = true;
+    }
+    for (int K = f64 ? 4 : 8; K >= 2 && !h->pass_k; --K)
+        if (feasible(K, false)) h->pass_k = K;
+    if (!h->pass_k) return;
+    const int nw = h->pass_nw, rpt = h->pass_rpt;
+    const void *fn = h->q == 9 ? (f64 ? pass_kernel_ptr<double, double, kNine>(nw, rpt, true)
+                                      : pass_kernel_ptr<float, float, kNine>(nw, rpt, true))
+                     : h->pass_narrow                     ? pass_kernel_ptr<double, NarrowF64>(nw, rpt, true)
+                     : h->lat.storage == LBM_F64          ? pass_kernel_ptr<double, double>(nw, rpt, true)
+                     : h->lat.storage == LBM_F32_WD_BF16  ? pass_kernel_ptr<float, __nv_bfloat16>(nw, rpt, true)
+                     : h->lat.storage == LBM_F32_WD_F16   ? pass_kernel_ptr<float, __half>(nw, rpt, true)
+                     : h->lat.storage == LBM_F32_LEAPFROG ? pass_kernel_ptr<float, Lf>(nw, rpt, true)
+                                                          : pass_kernel_ptr<float, float>(nw, rpt, true);
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * nw, 0) != cudaSuccess || per_sm < 1) {
+        h->pass_k = 0;
         return;
     }
+    h->pass_slots = per_sm * h->sms;
 }
 
 }  // namespace host

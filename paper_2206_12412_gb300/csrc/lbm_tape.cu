@@ -204,7 +204,7 @@ lbm_status record_steps(lbm_tape *t, int64_t n, int acc_loss)
     int par = h->parity;
     lbm_status rc = LBM_OK;
     if (n > 0 && h->cp.mode != CRACK_NONE) h->pending = true;
-    if (h->pass_k && !h->own_bands && !h->bulk && t->ns <= kPassSensors) {
+    if (t->rec_slots && !h->own_bands && !h->bulk && t->ns <= kPassSensors) {
         rc = tape_passes(
             n, h->pass_k, par, t->rec_slots, [&](int K, PassPlan &q) { return pass_plan(h, K, h->pass_nw, h->pass_rpt, q); },
             [&](const PassPlan &q, int p, bool second, int m) {
@@ -297,7 +297,9 @@ void choose_sweep(lbm_tape *t)
     lbm_handle *h = t->h;
     t->adj_k = 0;
     t->rec_slots = t->adj_slots = 0;
-    if (!h->pass_k) return;
+    // (FP64 in tiles of eight warps: 512^2 25.2 us a step, recorded and swept, in
+    // single steps 21.2; of four warps, 362^2: 16.8 and 19.9 us)
+    if (!h->pass_k || (h->esize == 8 && h->pass_nw == 8)) return;
     t->adj_nw = h->pass_nw;
     auto slots = [&](const void *fn) {
         int n = 0;

@@ -95,6 +95,17 @@ def cases():
         ("tall", _strip(120, 1500, mode="kcrit", K_C=KC), "f32", 40),
         ("example", W.kcrit_centre_crack(), "f32", 200),
     ]
+    for k, (nx, ny) in enumerate([(16, 20), (32, 25), (33, 31), (47, 60), (129, 128), (255, 257), (256, 256)]):   # FP64, one column a thread
+        out.append((f"narrow_{nx}x{ny}", _strip(nx, ny, v_rel=0.7), "f64", 41 + k))
+        out.append((f"narrow_rest_{nx}x{ny}", _strip(nx, ny, mode="stationary", bc="bounceback", start=nx * 0.3,
+                                                     tip=nx * 0.6, two_tips=True), "f64", 40))
+        out.append((f"narrow_bulk_{nx}x{ny}", _strip(nx, ny, mode=None), "f64", 43))
+        out.append((f"narrow_periodic_{nx}x{ny}", _strip(nx, ny, bc="bounceback", v_rel=0.5, start=nx * 0.5, tip=nx * 0.8,
+                                                         edges=("periodic", "periodic", "dirichlet", "free")), "f64", 45))
+        out.append((f"narrow_kcrit_{nx}x{ny}", _strip(nx, ny, mode="kcrit", K_C=KC), "f64", 60))
+    for tip in (110.2, 117.9, 119.5, 223.4):   # ends that a step moves over a tile boundary, towards either side
+        out.append((f"over_{tip}", _strip(400, 80, v_rel=0.9, start=236.6 - tip / 2, tip=tip + 130, two_tips=True), "f32", 48))
+        out.append((f"over_f64_{tip}", _strip(250, 80, v_rel=0.9, start=tip - 90, tip=tip, two_tips=True), "f64", 60))
     return out
 
 
