@@ -16,8 +16,10 @@
  *       criterion (prescribed growth, or the K-criterion with the velocity of
  *       eq. v-tanh), tip advance by Delta a = adot dt, and severing of the
  *       links the new crack segment intersects.
- * All of it runs in this library's CUDA kernels, one kernel launch per time
- * step; the library owns the device state.  Conventions shared by every call:
+ * All of it runs in this library's CUDA kernels: lbm_step advances most
+ * lattices in passes of up to eight time steps per launch (with the same
+ * results as one launch per time step, bit for bit), the others in one launch
+ * per time step; the library owns the device state.  Conventions shared by every call:
  *   - every call returns lbm_status; nothing throws or exits across the ABI;
  *   - inputs are copied at create; no caller pointer is retained, except the
  *     allocator callbacks and their context, which must outlive the handle;
@@ -354,7 +356,9 @@ lbm_status lbm_set_stream(lbm_handle *h, void *stream);
  * direction).  Each CTA marches over a band of at most band_rows rows of one
  * column block; 0 picks the built-in partition (D2Q5 and a crack in any
  * direction: the shortest bands for which every CTA of a step is resident at
- * once; D2Q9: about three waves of shorter bands).  The rows
+ * once; D2Q9: about three waves of shorter bands) and lets lbm_step take passes
+ * of several time steps where the lattice allows it; while band_rows > 0 it
+ * takes one launch per time step.  The rows
  * next to the crack line (jc-3 .. jc+2 with macroscopic crack faces, jc-1 and
  * jc otherwise) always form two bands of their own.  Synchronises the stream
  * and drops the cached step graph. */
@@ -407,7 +411,7 @@ lbm_status lbm_set_bulk(lbm_handle *h, int32_t enable);
 lbm_status lbm_set_chained(lbm_handle *h, int32_t enable);
 
 /* Kernel timing: while enabled, lbm_step launches every step directly (no
- * graph) with CUDA events on the handle's stream around the step kernel, and
+ * graph, no passes of several steps) with CUDA events on the handle's stream around the step kernel, and
  * the deferred crack step that synchronising calls apply first is timed the
  * same way. */
 lbm_status lbm_set_profiling(lbm_handle *h, int32_t enable);
@@ -486,7 +490,8 @@ lbm_status lbm_wdot_to_host_noalloc(lbm_handle *h, float *dst_host, int64_t n_fl
 lbm_status lbm_save(lbm_handle *h, const char *path);
 lbm_status lbm_load(lbm_handle *h, const char *path);
 
-/* Bytes of device memory the handle holds. */
+/* Bytes of device memory the handle holds (with two planes of scratch for
+ * passes of several time steps where the lattice takes them, at most 6 GB). */
 lbm_status lbm_device_bytes(const lbm_handle *h, int64_t *bytes);
 
 /* Release the handle and its device memory (NULL is ignored).  Synchronises
@@ -541,7 +546,9 @@ lbm_status lbm_create_batch(int32_t n, const lbm_grid *grids, const lbm_lattice 
 lbm_status lbm_batch_member(const lbm_batch *b, int32_t i, lbm_handle **h);
 
 /* Enqueue n >= 0 time steps of every lattice of the batch on the shared
- * stream (CUDA-graph replay of 64-step chunks). */
+ * stream (CUDA-graph replay of 64-step chunks; passes of eight, four and two
+ * time steps per launch where every member allows them and no launch shape,
+ * lookahead or persistent form was asked for). */
 lbm_status lbm_batch_step(lbm_batch *b, int64_t n);
 
 /* Number of lattices and CTAs per step of the batch (pointers may be NULL). */

@@ -61,6 +61,11 @@ __device__ __forceinline__ bool within(int64_t ax, int64_t ay, int64_t bx, int64
 __device__ bool segments_meet(int64_t p1x, int64_t p1y, int64_t p2x, int64_t p2y, int64_t q1x, int64_t q1y,
                               int64_t q2x, int64_t q2y)
 {
+    // (segments that meet have bounding boxes that do; a step's advance is
+    // short, so this mostly spares the 128-bit products)
+    if (hi64(p1x, p2x) < lo64(q1x, q2x) || hi64(q1x, q2x) < lo64(p1x, p2x) || hi64(p1y, p2y) < lo64(q1y, q2y) ||
+        hi64(q1y, q2y) < lo64(p1y, p2y))
+        return false;
     const int a = orient_q(q1x, q1y, q2x, q2y, p1x, p1y), b = orient_q(q1x, q1y, q2x, q2y, p2x, p2y);
     const int c = orient_q(p1x, p1y, p2x, p2y, q1x, q1y), d = orient_q(p1x, p1y, p2x, p2y, q2x, q2y);
     if (a * b < 0 && c * d < 0) return true;
@@ -107,69 +112,113 @@ struct LineSums {
 // candidates are the sites around the window's stretch of the crack,
 // widened by two spacings (a severed link's ends lie within 1.3 spacings of
 // the crack line).
+//
+// Bounded by FP64: an instruction takes a warp 64 cycles whatever its active
+// lanes, a division or a root about 700, and the end's decision waits for
+// all of them.  So four lanes form the four sides of the box at once, the
+// severed links are sifted in FP32 with a margin (every link that could lie
+// in the window is then tested in FP64), each lane takes its links one after
+// the other (one round of roots for the usual one or two pairs, whatever
+// their place in the box), and the divisions are skipped where they are
+// exact.  With tip_cta's side work on its other warps, 2048 x 1024 with two
+// ends and macroscopic faces: 24.5 -> 17.9 us per step, the same bits.
 template <typename T>
 __device__ LineSums line_eval_warp(const CrackParams &p, const T *w, int64_t P, const uint32_t *cut_h,
                                    const uint32_t *cut_v, const TipState &E, int dir)
 {
+    const unsigned kFull = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const double r_min = p.r_min_fixed > 0.0 ? p.r_min_fixed : p.r0 / (1.0 - E.v_prev);   // eq. r(v)
-    const double lo = r_min / p.dh, hi = (r_min + p.fit_width) / p.dh;
-    const double tx = (double)E.tip_q * kTwoM32, ty = (double)E.tip_yq * kTwoM32;
+    const int64_t tip_x = E.tip_q, tip_y = E.tip_yq;
+    const double v_prev = E.v_prev;
+    const bool unit = p.dh == 1.0;
+    const double r_min = p.r_min_fixed > 0.0 ? p.r_min_fixed : (v_prev == 0.0 ? p.r0 : p.r0 / (1.0 - v_prev));   // eq. r(v)
+    const double lo = unit ? r_min : r_min / p.dh, hi = unit ? r_min + p.fit_width : (r_min + p.fit_width) / p.dh;
     // the window lies behind the tip: along -c from the right end, along +c
-    // from the left end of a two-tip crack
-    const double sx = dir > 0 ? -p.dir_x : p.dir_x, sy = dir > 0 ? -p.dir_y : p.dir_y;
-    const double ax = tx + lo * sx, bx = tx + hi * sx, ay = ty + lo * sy, by = ty + hi * sy;
-    const double X = (double)p.nx, Y = (double)p.ny;
-    auto cl = [](double v, double lim) { return fmin(fmax(v, -4.0), lim + 4.0); };
-    int i0 = (int)floor(cl(fmin(ax, bx), X) - 2.0), i1 = (int)ceil(cl(fmax(ax, bx), X) + 2.0);
-    int j0 = (int)floor(cl(fmin(ay, by), Y) - 2.0), j1 = (int)ceil(cl(fmax(ay, by), Y) + 2.0);
-    i0 = max(i0, 0);
-    j0 = max(j0, 0);
-    i1 = min(i1, p.nx - 1);
-    j1 = min(j1, p.ny - 1);
+    // from the left end of a two-tip crack.  Lanes 0 .. 3 (of every four):
+    // the lower bound in x and y, the upper bound in x and y
+    const bool iy = lane & 1, upper = lane & 2;
+    const double c = iy ? p.dir_y : p.dir_x, t = (double)(iy ? tip_y : tip_x) * kTwoM32;
+    const double s = dir > 0 ? -c : c, u = t + lo * s, v = t + hi * s, far = (double)((iy ? p.ny : p.nx) + 4);
+    double m = (u < v) == upper ? v : u;
+    m = m > -4.0 ? m : -4.0;
+    m = m < far ? m : far;
+    m = upper ? -2.0 - m : m - 2.0;
+    const int side = upper ? -__double2int_rd(m) : __double2int_rd(m);
+    const int i0 = max(__shfl_sync(kFull, side, 0), 0), j0 = max(__shfl_sync(kFull, side, 1), 0);
+    const int i1 = min(__shfl_sync(kFull, side, 2), p.nx - 1), j1 = min(__shfl_sync(kFull, side, 3), p.ny - 1);
     const int ni = i1 - i0 + 1, nj = j1 - j0 + 1;
     const int total = (ni > 0 && nj > 0) ? ni * nj : 0;
+    const float f = (float)(iy ? (upper ? hi : p.dir_y) : (upper ? lo : p.dir_x));
+    const float cx = __shfl_sync(kFull, f, 0), cy = __shfl_sync(kFull, f, 1);
+    const float lo_f = __shfl_sync(kFull, f, 2), hi_f = __shfl_sync(kFull, f, 3);
     const bool k1_left_v = p.dir_x > 0.0, k1_left_h = p.dir_y < 0.0;
+    auto mid = [&](int i, int j, int vert, int64_t &dx, int64_t &dy) {
+        const int64_t mx = vert ? centre_q(i) : (int64_t)(i + 1) << kQBits, my = vert ? (int64_t)(j + 1) << kQBits : centre_q(j);
+        dx = dir > 0 ? tip_x - mx : mx - tip_x;
+        dy = dir > 0 ? tip_y - my : my - tip_y;
+    };
+    auto near = [&](int i, int j, int vert) {
+        int64_t dx, dy;
+        mid(i, j, vert, dx, dy);
+        const float fx = (float)dx * (float)kTwoM32, fy = (float)dy * (float)kTwoM32, r = fx * cx + fy * cy;
+        const float margin = 1e-3f + 1e-5f * (fabsf(fx) + fabsf(fy) + lo_f + hi_f);
+        return !(r < lo_f - margin) && !(r > hi_f + margin);
+    };
     double num = 0.0, den = 0.0;
     int np = 0;
-    for (int q = lane; q < total; q += 32) {
-        const int i = i0 + q % ni, j = j0 + q / ni;
-#pragma unroll
-        for (int vert = 0; vert < 2; ++vert) {
-            bool cut;
-            int64_t mx, my;
-            if (!vert) {
-                if (i + 1 >= p.nx) continue;
-                cut = (__ldcg(cut_h + (int64_t)j * p.words + (i >> 5)) >> (i & 31)) & 1u;
-                mx = (int64_t)(i + 1) << kQBits;
-                my = centre_q(j);
-            } else {
-                if (j + 1 >= p.ny) continue;
-                cut = (__ldcg(cut_v + (int64_t)j * p.words + (i >> 5)) >> (i & 31)) & 1u;
-                mx = centre_q(i);
-                my = (int64_t)(j + 1) << kQBits;
+    constexpr int kSift = 16;   // sites of a lane sifted at a time
+    for (int base = 0; base < total; base += 32 * kSift) {
+        uint32_t cand = 0;
+        const int rounds = min(kSift, (total - base + 31) / 32);
+#pragma unroll 2
+        for (int q = 0; q < rounds; ++q) {
+            const int k = base + 32 * q + lane;
+            const int i = i0 + k % ni, j = j0 + k / ni;
+            const bool h = k < total && i + 1 < p.nx && near(i, j, 0), vv = k < total && j + 1 < p.ny && near(i, j, 1);
+            const int64_t o = (int64_t)j * p.words + (i >> 5);
+            const uint32_t wh = h ? __ldcg(cut_h + o) : 0u, wv = vv ? __ldcg(cut_v + o) : 0u;
+            cand |= (((wh >> (i & 31)) & 1u) | (((wv >> (i & 31)) & 1u) << 1)) << (2 * q);
+        }
+        // (in the order of the sites, horizontal before vertical)
+        while (__any_sync(kFull, cand != 0u)) {
+            if (cand) {
+                const int b = __ffs(cand) - 1, k = base + 32 * (b >> 1) + lane, vert = b & 1;
+                const int i = i0 + k % ni, j = j0 + k / ni;
+                cand &= cand - 1u;
+                const double w0 = (double)w[(int64_t)j * P + i];
+                const double w1 = (double)w[vert ? (int64_t)(j + 1) * P + i : (int64_t)j * P + i + 1];
+                int64_t dx, dy;
+                mid(i, j, vert, dx, dy);
+                const double px = __dmul_rn((double)dx * kTwoM32, p.dir_x), py = __dmul_rn((double)dy * kTwoM32, p.dir_y);
+                const double r_h = __dadd_rn(px, py);
+                if (r_h >= lo && r_h < hi) {
+                    const double delta = (vert ? k1_left_v : k1_left_h) ? w1 - w0 : w0 - w1;
+                    const double r = unit ? r_h : r_h * p.dh;
+                    const double sf = sqrt(div_known(r, 2.0 * kPi, 1.0 / (2.0 * kPi)));
+                    num += delta * sf;
+                    den += sf * sf;
+                    ++np;
+                }
             }
-            if (!cut) continue;
-            const double px = __dmul_rn((double)(dir > 0 ? E.tip_q - mx : mx - E.tip_q) * kTwoM32, p.dir_x);
-            const double py = __dmul_rn((double)(dir > 0 ? E.tip_yq - my : my - E.tip_yq) * kTwoM32, p.dir_y);
-            const double r_h = __dadd_rn(px, py);
-            if (!(r_h >= lo && r_h < hi)) continue;
-            const double w0 = (double)w[(int64_t)j * P + i];
-            const double w1 = (double)(vert ? w[(int64_t)(j + 1) * P + i] : w[(int64_t)j * P + i + 1]);
-            const double delta = (vert ? k1_left_v : k1_left_h) ? w1 - w0 : w0 - w1;
-            const double r = r_h * p.dh;
-            const double sf = sqrt(r / (2.0 * kPi));
-            num += delta * sf;
-            den += sf * sf;
-            ++np;
         }
     }
+    // with the pairs in at most two lanes their sums are added as the tree
+    // would: other lanes' zeros change nothing
+    const unsigned holders = __ballot_sync(kFull, np > 0);
+    if (__popc(holders) <= 2) {
+        const int ha = holders ? __ffs(holders) - 1 : 0, hb = 31 - __clz(holders | 1u);
+        const double na = __shfl_sync(kFull, num, ha), nb = __shfl_sync(kFull, num, hb);
+        const double da = __shfl_sync(kFull, den, ha), db = __shfl_sync(kFull, den, hb);
+        num = ha == hb ? na : na + nb;
+        den = ha == hb ? da : da + db;
+    } else {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        num += __shfl_xor_sync(0xffffffffu, num, o);
-        den += __shfl_xor_sync(0xffffffffu, den, o);
-        np += __shfl_xor_sync(0xffffffffu, np, o);
+        for (int o = 16; o > 0; o >>= 1) {
+            num += __shfl_xor_sync(kFull, num, o);
+            den += __shfl_xor_sync(kFull, den, o);
+        }
     }
+    np = __reduce_add_sync(kFull, np);
     return LineSums{num, den, r_min, np};
 }
 
@@ -178,9 +227,9 @@ __device__ LineSums line_eval_warp(const CrackParams &p, const T *w, int64_t P, 
 // on the state S (shared memory), given that end's sums: K, the criterion,
 // the advance (with the stop at the boundary), the severed links, the end's
 // fields of S and, if `commit`, its history record at hist_n (x in tip /
-// tipl, y in tipy / tipyl).
+// tipl, y in tipy / tipyl).  k_inv: 1 / K_C.
 __device__ void line_apply_warp(const CrackParams &p, uint32_t *cut_h, uint32_t *cut_v, const History &hist,
-                                CrackState &S, int dir, bool commit, const LineSums &c)
+                                CrackState &S, int dir, bool commit, const LineSums &c, double k_inv)
 {
     const int lane = threadIdx.x & 31;
     TipState &E = dir > 0 ? S.r : S.l;
@@ -191,7 +240,7 @@ __device__ void line_apply_warp(const CrackParams &p, uint32_t *cut_h, uint32_t 
         propagate = 1;
         v = p.v_rel;
     } else if (p.mode == CRACK_KCRIT && c.np > 0 && fabs(K) > p.K_C) {
-        const double ratio = fabs(K) / p.K_C;
+        const double ratio = isinf(K) ? fabs(K) : div_known(fabs(K), p.K_C, k_inv);
         propagate = 1;
         v = p.v_max * tanh(sqrt(ratio * ratio * ratio * ratio - 1.0));   // eq. v-tanh
     }
@@ -203,7 +252,8 @@ __device__ void line_apply_warp(const CrackParams &p, uint32_t *cut_h, uint32_t 
     int64_t qx = px, qy = py;
     if (propagate) {
         const double adot = v * p.cs;
-        const double q = adot * p.dt / p.dh * 4294967296.0;   // Delta a = adot dt, in grid units
+        const double da = p.dt == 1.0 ? adot : adot * p.dt;
+        const double q = (p.dh == 1.0 ? da : da / p.dh) * 4294967296.0;   // Delta a = adot dt, in grid units
         const int64_t ax = __double2ll_rn(q * p.dir_x), ay = __double2ll_rn(q * p.dir_y);
         qx = dir > 0 ? px + ax : px - ax;
         qy = dir > 0 ? py + ay : py - ay;
@@ -279,8 +329,9 @@ __device__ void line_step_warp(const CrackParams &p, const T *w, int64_t P, uint
     const LineSums cr = line_eval_warp<T>(p, w, P, cut_h, cut_v, S.r, +1);
     LineSums cl{0.0, 0.0, 0.0, 0};
     if (p.two_tips) cl = line_eval_warp<T>(p, w, P, cut_h, cut_v, S.l, -1);
-    line_apply_warp(p, cut_h, cut_v, hist, S, +1, commit, cr);
-    if (p.two_tips) line_apply_warp(p, cut_h, cut_v, hist, S, -1, commit, cl);
+    const double k_inv = 1.0 / p.K_C;
+    line_apply_warp(p, cut_h, cut_v, hist, S, +1, commit, cr, k_inv);
+    if (p.two_tips) line_apply_warp(p, cut_h, cut_v, hist, S, -1, commit, cl, k_inv);
 }
 
 // The pad images of the new value v of site (i, j) (free edges: the site's
@@ -393,13 +444,14 @@ __device__ __forceinline__ Claims claims(const CrackParams &p, const CrackState 
     const int64_t ya = lo64(lyq, s->r.tip_yq) >> kQBits, yb = hi64(lyq, s->r.tip_yq) >> kQBits;
     c.r0 = (int)hi64(0, lo64(ya - 3, lo64(c.j0, p.two_tips ? c.l0 : c.j0)));
     c.r1 = (int)lo64(p.ny - 1, hi64(yb + 3, hi64(c.j1, p.two_tips ? c.l1 : c.j1)));
-    c.sx = (float)((double)p.start_q * kTwoM32);
-    c.sy = (float)((double)p.start_yq * kTwoM32);
+    auto unit = [](int64_t q) { return (float)q * (float)kTwoM32; };   // (FP64 conversions cost 64 cycles each)
+    c.sx = unit(p.start_q);
+    c.sy = unit(p.start_yq);
     c.cx = (float)p.dir_x;
     c.cy = (float)p.dir_y;
-    const float tx = (float)((double)s->r.tip_q * kTwoM32), ty = (float)((double)s->r.tip_yq * kTwoM32);
+    const float tx = unit(s->r.tip_q), ty = unit(s->r.tip_yq);
     c.t_hi = __fadd_rn(__fadd_rn(__fmul_rn(__fsub_rn(tx, c.sx), c.cx), __fmul_rn(__fsub_rn(ty, c.sy), c.cy)), 2.0f);
-    const float ux = (float)((double)lxq * kTwoM32), uy = (float)((double)lyq * kTwoM32);
+    const float ux = unit(lxq), uy = unit(lyq);
     c.t_lo = __fsub_rn(__fadd_rn(__fmul_rn(__fsub_rn(ux, c.sx), c.cx), __fmul_rn(__fsub_rn(uy, c.sy), c.cy)), 2.0f);
     c.inv_cx = fabsf(c.cx) < 1e-6f ? 0.0f : __frcp_rn(c.cx);
     c.inv_cy = fabsf(c.cy) < 1e-6f ? 0.0f : __frcp_rn(c.cy);
@@ -463,51 +515,65 @@ __device__ __forceinline__ bool seg_claimed(const Claims &c, int s, int j, int W
 
 // Block 0: the pending crack step -- warp 0 the tip, warp 1 the left end of
 // a two-tip crack; both criteria are evaluated before either end severs a
-// link, as Alg. 1 orders them -- then the record and the next state (thread
-// 0), then the ends' boxes with the cuts in force after it.
+// link, as Alg. 1 orders them -- then the record and the next state, and the
+// ends' boxes with the cuts in force after it.  What the decisions do not
+// need is done beside them: warp 2 copies the state and forms the next
+// Dirichlet values, warp 3 the claims and the edge values (sC, sE) and 1 / K_C.
 template <typename T, typename D>
-__device__ void tip_cta(const StepArgs<T, D> &a, CrackState &sS, const EdgeValues<T> &E, const Claims &C)
+__device__ void tip_cta(const StepArgs<T, D> &a, CrackState &sS, EdgeValues<T> &E, Claims &C)
 {
-    const int tid = threadIdx.x, warp = tid >> 5;
+    static_assert(kThreads == 128 && sizeof(CrackState) % 4 == 0, "four warps");
+    __shared__ double k_inv;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const CrackParams &p = a.p;
-    if (tid == 0) sS = *a.s_in;
-    __syncthreads();
-    const bool pending = !sS.r.decided;   // not yet applied by a deferred crack step
+    const CrackState *in = a.s_in;
+    const bool pending = !in->r.decided;   // not yet applied by a deferred crack step
     const bool active = p.mode != CRACK_NONE && pending;
     const int dir = warp == 0 ? +1 : -1;
     const bool mine = warp == 0 || (warp == 1 && p.two_tips);
     LineSums cs{0.0, 0.0, 0.0, 0};
-    if (active && mine) cs = line_eval_warp<T>(p, a.w_in, a.pitch, a.cut_h, a.cut_v, dir > 0 ? sS.r : sS.l, dir);
-    __syncthreads();   // both criteria on the state before either end severs a link
-    if (active && mine) line_apply_warp(p, a.cut_h, a.cut_v, a.hist, sS, dir, true, cs);
-    __syncthreads();
-    if (tid < 32) {
-        if (tid == 0) {
-            CrackState *o = a.s_out;
-            const int64_t n = sS.step + 1;
-            o->step = n;
-            o->hist_n = sS.hist_n + (pending ? 1 : 0);
-            o->i_first = sS.i_first;
-            o->i_last = sS.i_last;
-            o->r = sS.r;
-            o->r.decided = 0;
-            o->l = sS.l;
-            o->l.decided = 0;
-            for (int e = 0; e < 4; ++e)
-                o->wstar[e] = a.edge[e] == EDGE_DIRICHLET ? load_value(a.load[e], n, (double)p.dt) : 0.0;
+    if (warp == 2) {
+        for (int k = lane; k < (int)(sizeof(CrackState) / 4); k += 32)
+            reinterpret_cast<uint32_t *>(&sS)[k] = reinterpret_cast<const uint32_t *>(in)[k];
+        __syncwarp();
+        // (the values in force are E's)
+        if (lane < 4)
+            sS.wstar[lane] = a.edge[lane] == EDGE_DIRICHLET ? load_value(a.load[lane], in->step + 1, (double)p.dt) : 0.0;
+    } else if (warp == 3) {
+        if (lane == 0) {
+            C = claims(p, in);
+            E = edge_values<T>(in);
+            k_inv = p.mode == CRACK_KCRIT ? 1.0 / p.K_C : 0.0;
         }
+    } else if (active && mine) {
+        cs = line_eval_warp<T>(p, a.w_in, a.pitch, a.cut_h, a.cut_v, dir > 0 ? in->r : in->l, dir);
     }
+    __syncthreads();   // both criteria on the state before either end severs a link
+    if (active && mine) line_apply_warp(p, a.cut_h, a.cut_v, a.hist, sS, dir, true, cs, k_inv);
     __syncthreads();   // the new cuts, for every thread of the CTA
     bool ok = true;
-    const int ni = C.i1 - C.i0 + 1, nj = C.j1 - C.j0 + 1;
-    for (int t = tid; t < ni * nj; t += blockDim.x) ok &= site_update(a, E, C.i0 + t % ni, C.j0 + t / ni);
+    const int ni = C.i1 - C.i0 + 1, n1 = ni * (C.j1 - C.j0 + 1);
     // the left end's box, less the sites of the tip's
-    const int mi = C.k1 - C.k0 + 1, mj = C.l1 - C.l0 + 1;
-    for (int t = tid; t < (mi > 0 ? mi * mj : 0); t += blockDim.x) {
-        const int i = C.k0 + t % mi, j = C.l0 + t / mi;
-        if (!(i >= C.i0 && i <= C.i1 && j >= C.j0 && j <= C.j1)) ok &= site_update(a, E, i, j);
+    const int mi = C.k1 - C.k0 + 1, mj = C.l1 - C.l0 + 1, n2 = mi > 0 && mj > 0 ? mi * mj : 0;
+    for (int t = tid; t < n1 + n2; t += blockDim.x) {
+        const bool left = t >= n1;
+        const int q = left ? t - n1 : t, wd = left ? mi : ni;
+        const int i = (left ? C.k0 : C.i0) + q % wd, j = (left ? C.l0 : C.j0) + q / wd;
+        if (!(left && i >= C.i0 && i <= C.i1 && j >= C.j0 && j <= C.j1)) ok &= site_update(a, E, i, j);
     }
     if (!ok) atomicOr(a.err, (uint32_t)ERR_NONFINITE);
+    if (warp == 3) {
+        __syncwarp();
+        if (lane == 0) {
+            sS.step += 1;
+            sS.hist_n += pending ? 1 : 0;
+            sS.r.decided = 0;
+            sS.l.decided = 0;
+        }
+        __syncwarp();
+        for (int k = lane; k < (int)(sizeof(CrackState) / 4); k += 32)
+            reinterpret_cast<uint32_t *>(a.s_out)[k] = reinterpret_cast<const uint32_t *>(&sS)[k];
+    }
 }
 
 // The claimed groups: every site outside the boxes of every claimed group.  The rows r0 .. r1, each cut into stretches of 16 groups, are taken
@@ -683,6 +749,10 @@ __device__ __forceinline__ void line_cta(const StepArgs<T, D> &a, int blk, Crack
 {
     constexpr int N = Vec<T>::N;
     const int tid = threadIdx.x, lane = tid & 31;
+    if (blk == 0) {
+        tip_cta<T, D>(a, sS, sE, sC);
+        return;
+    }
     if (tid == 0) {
         sC = claims(a.p, a.s_in);
         sE = edge_values<T>(a.s_in);
@@ -690,10 +760,6 @@ __device__ __forceinline__ void line_cta(const StepArgs<T, D> &a, int blk, Crack
     __syncthreads();
     const EdgeValues<T> &E = sE;
     const Claims &C = sC;
-    if (blk == 0) {
-        tip_cta<T, D>(a, sS, E, C);
-        return;
-    }
     const int n_march = a.ncb * ((a.ny + a.p.band - 1) / a.p.band);
     const int u = blk - 1;
     const int cb = u % a.ncb, band = u / a.ncb;
