@@ -534,7 +534,8 @@ lbm_status lbm_batch_create(lbm_handle *const *handles, int32_t n, int32_t band_
  * lbm_batch_destroy destroys them too (lbm_batch_member gives each handle,
  * for reading fields, masks and crack states; do not destroy those handles).
  * The paper has no batches: many independent runs of the method (Sec. 3,
- * Alg. 1), each exactly as one lattice, advance in one launch per step.
+ * Alg. 1), each exactly as one lattice, advance together, one launch per step or per
+ * pass of several (lbm_batch_step).
  * loads and n_loads are both NULL or both given.  On error nothing is left
  * allocated and the message names the member that failed. */
 lbm_status lbm_create_batch(int32_t n, const lbm_grid *grids, const lbm_lattice *lattices, const lbm_material *materials,

@@ -1000,12 +1000,14 @@ lbm_status create_impl(const lbm_grid *grid, const lbm_lattice *lattice, const l
     size_t o_ser[4];
     for (int q = 0; q < 4; ++q) { o_ser[q] = off; off = align256(off + (size_t)h->load[q].n * 8); }
     h->state_bytes = off;
-    // scratch planes of the passes, for lattices that can take them and whose
-    // scratch is a small part of the device's memory
+    // scratch planes of the passes, for lattices that can take them (FP64 ones
+    // of more than 2^19 sites have more tiles than SMs) and whose scratch is a
+    // small part of the device's memory
     const size_t alt_bytes = h->esize_d ? plane_d : plane;
     const size_t o_a0 = off; off = align256(off + alt_bytes);
     const size_t o_a1 = off; if (!h->esize_d) off = align256(off + alt_bytes);
     bool scratch = !line && !slab && grid->edge[LBM_BOTTOM] != LBM_EDGE_PERIODIC &&
+                   !(h->esize == 8 && (int64_t)grid->nx * grid->ny > (int64_t)1 << 19) &&
                    off - h->state_bytes <= kMaxPassScratch;
     h->block_bytes = scratch ? off : h->state_bytes;
     h->block = dev_alloc(h, h->block_bytes);

@@ -73,7 +73,7 @@ struct CrackSums {
 // gets the sums.  tip, v_prev: the end's tip and previous speed; i_first,
 // i_last: the severed columns; fetch(i, above, below) reads the pair of
 // column i and tells whether its link is severed.  All 32 lanes of the warp
-// must call it, but for G = 1, where each calling lane fits on its own.
+// must call it.
 template <typename T, int G, typename F>
 __device__ __forceinline__ CrackSums crack_eval_pairs(const CrackParams &p, int64_t tip, double v_prev, int i_first,
                                                       int i_last, int dir, F &&fetch)
@@ -114,7 +114,6 @@ __device__ __forceinline__ CrackSums crack_eval_pairs(const CrackParams &p, int6
         den += sf * sf;
         ++np;
     }
-    if constexpr (G == 1) return CrackSums{num, den, r_min, np};   // a lane on its own
     // with the pairs in one lane of the group (the one-pair window W = dh
     // always), that lane's sums are the group's: adding the other lanes'
     // zeros cannot change them, so one shuffle replaces the reduction tree

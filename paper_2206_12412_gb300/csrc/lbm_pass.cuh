@@ -20,13 +20,19 @@
 // step, for an eighth of its memory traffic and launches.
 //
 // Measured, one GB300, time per step of a run against one launch per step:
-// 4096 x 2048 FP32, K-criterion 20.0 -> 8.6 us; 8192 x 8192 BF16 wdot 161 ->
-// 69 us; 16384 x 16384 leapfrog 575 -> 187 us; 1001 x 777 FP16 wdot, periodic
-// sides 6.0 -> 3.4 us; 512 x 192 with the edge rule and two tips 10.7 -> 5.3 us.
-// What bounds a bulk tile is instruction issue: with scalar FP32 and the rows
-// moved back after each step the leapfrog kernel issued 85.7 M instructions
-// per 4096^2 pass (120 us), without the moves 69.8 M (110 us), packed 50.7 M
-// (98 us; FP32 pipes 44 % busy, DRAM 27 %).
+// 4096 x 2048 FP32, K-criterion 20.0 -> 6.9 us; the same on nine velocities
+// 25.8 -> 9.3 us; 8192 x 8192 BF16 wdot 149 -> 36 us; 16384 x 16384 leapfrog 575
+// -> 166 us; 1001 x 777 FP16 wdot, periodic sides 6.0 -> 2.3 us; 512 x 192 with
+// the edge rule and two tips 11.6 -> 3.1 us; 128 x 128 FP64 10.9 -> 3.2 us.
+// What bounds a bulk tile is instruction issue: half the issue slots and 45 %
+// of the FMA pipes are busy, DRAM half of its copy rate.  With scalar FP32 and
+// the rows moved back after each step the leapfrog kernel issued 85.7 M
+// instructions per 4096^2 pass (120 us), without the moves 69.8 M (110 us),
+// packed 50.7 M (98 us).  Loading the next tile's rows during a tile's steps
+// (asynchronous copies, persistent CTAs) was slower (8192^2 FP32 32.8 -> 36.3
+// us per step): the second resident CTA hides the loads already.  A strip
+// tile's step takes 1250 cycles, an edge tile's 700 (chains of a few shuffles,
+// one barrier and the rules); small lattices are bound by these.
 //
 // The crack strip.  The rows within 16 - K of the crack line form tiles of
 // their own (32 rows, the line between warps 3 and 4), which apply the cuts
@@ -446,12 +452,13 @@ __device__ __forceinline__ void pass_crack_step(const CrackParams &p, const Pass
                 d.K = pass_K(p, c);
                 d.flags = E.flags;
                 const double Ka = fabs(d.K);
+                const bool bad = (__double_as_longlong(d.K) & 0x7ff0000000000000ll) == 0x7ff0000000000000ll;
                 if (c.np > 0 && Ka > p.K_C) {
-                    const double ratio = div_known(Ka, p.K_C, q.k_inv);
+                    const double ratio = bad ? Ka : div_known(Ka, p.K_C, q.k_inv);
                     d.propagate = 1;
                     d.v = p.v_max * tanh(sqrt(ratio * ratio * ratio * ratio - 1.0));   // eq. v-tanh
                 }
-                if ((__double_as_longlong(d.K) & 0x7ff0000000000000ll) == 0x7ff0000000000000ll) d.flags |= FLAG_NONFINITE;
+                if (bad) d.flags |= FLAG_NONFINITE;
                 if (E.arrested) {
                     d.propagate = 0;
                     d.v = 0.0;
@@ -1523,10 +1530,10 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
         // one warp forms the fits of all steps, a lane each (an FP64
         // instruction takes a warp 64 cycles whatever its active lanes); a
         // wider one takes a warp per step.
-        auto fit = [&](int st, int dir, double v_prev, double &Kf, int &np, double &r_min, auto group) {
+        auto fit = [&](int st, int dir, double v_prev, double &Kf, int &np, double &r_min) {
             const PassTip &q = sh.log[st];
             const int org = dir > 0 ? c.org_r : c.org_l;
-            const CrackSums f = crack_eval_pairs<T, decltype(group)::value>(
+            const CrackSums f = crack_eval_pairs<T, 32>(
                 p, dir > 0 ? q.tr : q.tl, v_prev, q.f, q.l, dir, [&](int i, T &ab, T &be) {
                     const int e = i - org;
                     if (e < 0 || e >= W) return false;
@@ -1609,7 +1616,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs<T, D> &A, const PassBuf
                 if (dir > 0 && !c.own_r) continue;
                 double Kf = 0.0, r_min = 0.0;
                 int np = 0;
-                if (sh.log[warp + 1].lazy) fit(warp, dir, v_prev, Kf, np, r_min, std::integral_constant<int, 32>());
+                if (sh.log[warp + 1].lazy) fit(warp, dir, v_prev, Kf, np, r_min);
                 if (lane == 0) record(warp, dir, Kf, np, r_min);
             }
         }

@@ -15,14 +15,17 @@ int ceil_div(int a, int b) { return (a + b - 1) / b; }
 int round_up(int a, int n) { return ceil_div(a, n) * n; }
 
 // FP64 runs at two results a cycle and SM, so recomputed halos cost more than
-// saved launches and traffic give once every SM has its tile.
-// Time per step in passes and (in parentheses) in single steps, K-criterion:
-// 128^2 6.8 (9.3), 362^2 10.4 (11.1), 512^2 10.1 (13.3), 724^2 18.4 (14.2),
-// 1024 x 512 18.4 us (14.3 us): passes while there are no more tiles of eight
-// warps than SMs.  The edge rule: 512 x 256 11.7 (15.2), 512^2 19.9 us (16.1 us):
-// up to kPass64Small sites, which take tiles of four warps.  Up to
-// kPass64Narrow they are one column a thread (a stationary crack on 128^2:
-// 3.2 us, two columns a thread 4.5 us, single steps 10.9 us).
+// saved launches and traffic give once every SM has its tile.  Time per step
+// in passes and (in parentheses) in single steps.  Above kPass64Small sites:
+// the K-criterion 512^2 10.1 (13.3), 640^2 11.6 (12.6), 724^2 18.4 us (14.2 us)
+// and nine velocities 512^2 16.4 (24.8), 640^2 18.6 (26.8), 724^2 30.5 us (29.7
+// us): passes of four steps while there are no more tiles of eight warps than
+// SMs.  Prescribed growth 600^2 10.0 (10.1), 1500 x 90 10.0 (8.7), periodic sides
+// 1500 x 90 9.3 us (5.8 us) and the edge rule 512^2 19.9 us (16.1 us): single
+// steps.  Up to kPass64Small sites, in tiles of four warps: 362^2 7.3 (9.0), K-
+// criterion 10.4 (11.1), nine velocities 13.0 (18.4), the edge rule 9.7 us (13.7
+// us) on 1000 x 120.  Up to kPass64Narrow they are one column a thread (128^2,
+// stationary crack: 3.2 us, two columns a thread 4.4 us, single steps 10.9 us).
 constexpr int64_t kPass64Small = (int64_t)1 << 17, kPass64Narrow = (int64_t)1 << 16;
 
 // n items in m tiles: of p, the first e of one more.
@@ -174,7 +177,12 @@ void choose_pass(lbm_handle *h)
         h->pass_rpt = h->pass_nw == 4 ? 4 : 8;
         if (!pass_plan(h, K, h->pass_nw, h->pass_rpt, q, false, narrow)) return false;
         if (f64 && sites > kPass64Small && (K < 4 || q.tiles > h->sms)) return false;
-        if (!f64 && q.tiles < 2 * h->sms) h->pass_rpt = 4;
+        // shorter tiles while the taller ones would leave a good part of the SMs
+        // with one: four and (in parentheses) eight rows a thread, prescribed
+        // growth, 512 x 192 1.32 (1.38), 1024^2 1.74 (1.76), 1400 x 1024 2.09
+        // (1.89), 1600 x 1400 2.83 us (2.26 us); FP16 rates, periodic sides 1001 x
+        // 777 2.29 (2.90), 1400 x 1024 2.99 us (2.82 us)
+        if (!f64 && q.tiles < 7 * h->sms / 4) h->pass_rpt = 4;
         bool all = true;   // every shorter pass too: a call's last passes
         for (int k = K; k >= 2; --k) all = all && pass_plan(h, k, h->pass_nw, h->pass_rpt, q, false, narrow);
         return all;

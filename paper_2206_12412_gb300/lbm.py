@@ -596,7 +596,7 @@ def lbm_batch_member(b: int, i: int) -> int:
 
 
 class Batch:
-    """Several Lattice objects advanced together, one kernel launch per step."""
+    """Several Lattice objects advanced together, one kernel launch per step or per pass of several."""
 
     def __init__(self, lattices, band_rows: int = 0, torch_allocator: bool = True):
         self.lattices = list(lattices)
