@@ -21,7 +21,7 @@ SOURCES = ["lbm_kernels.cu", "lbm_adjoint.cu", "lbm_api.cu", "lbm_tape.cu", "lbm
            "lbm_pass.cu", "lbm_pass16.cu", "lbm_pass_tape.cu", "lbm_pass_batch.cu", "lbm_pass9.cu", "lbm_pass_f64.cu",
            "lbm_pass_plan.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["--split-compile=0", "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2", "-I" + INCLUDE, "-I" + CSRC]
+FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2", "-I" + INCLUDE, "-I" + CSRC]
 
 _lock = threading.Lock()
 
