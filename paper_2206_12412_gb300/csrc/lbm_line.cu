@@ -364,7 +364,7 @@ __device__ __forceinline__ void site_pads(const StepArgs<T, D> &a, int i, int j,
 // The update of one site with its severed links (the update of the march,
 // site by site); returns whether the new w is finite.
 template <typename T, typename D>
-__device__ __forceinline__ bool site_update(const StepArgs<T, D> &a, const EdgeValues<T> &E, int i, int j)
+__device__ __forceinline__ bool update_site(const StepArgs<T, D> &a, const EdgeValues<T> &E, int i, int j)
 {
     const int nx = a.nx, ny = a.ny, words = a.words;
     const int64_t P = a.pitch;
@@ -390,8 +390,8 @@ __device__ __forceinline__ bool site_update(const StepArgs<T, D> &a, const EdgeV
     if (i == nx - 1 && a.edge[RIGHT] == EDGE_DIRICHLET) wr = E.two_ws[RIGHT] - w0;
     else if ((hr_w >> (i & 31)) & 1u) wr = w0;
     const T lap = ((u + d) + (wl + wr)) - (T)4 * w0;
-    const T wdn = wdo + a.g * lap;
-    const T wn = w0 + a.dt * wdn;
+    T wn, wdn;
+    site_update<T, D>(w0, wdo, lap, a.g, a.dt, wn, wdn);
     a.w_out[o] = wn;
     WdIO<D>::put(a.wd + o, wdn, a.wd_scale);
     site_pads(a, i, j, wn);
@@ -559,7 +559,7 @@ __device__ void tip_cta(const StepArgs<T, D> &a, CrackState &sS, EdgeValues<T> &
         const bool left = t >= n1;
         const int q = left ? t - n1 : t, wd = left ? mi : ni;
         const int i = (left ? C.k0 : C.i0) + q % wd, j = (left ? C.l0 : C.j0) + q / wd;
-        if (!(left && i >= C.i0 && i <= C.i1 && j >= C.j0 && j <= C.j1)) ok &= site_update(a, E, i, j);
+        if (!(left && i >= C.i0 && i <= C.i1 && j >= C.j0 && j <= C.j1)) ok &= update_site(a, E, i, j);
     }
     if (!ok) atomicOr(a.err, (uint32_t)ERR_NONFINITE);
     if (warp == 3) {
@@ -598,7 +598,7 @@ __device__ void claimed_groups(const StepArgs<T, D> &a, const EdgeValues<T> &E, 
             const int g = g0 + t;
             if (!((g >= sa && g <= sb) || box_group(C, g, j, kGroup))) continue;
             const int i = g * kGroup + lane;
-            if (i < a.nx && !in_box(C, i, j)) ok &= site_update(a, E, i, j);
+            if (i < a.nx && !in_box(C, i, j)) ok &= update_site(a, E, i, j);
         }
     }
     if (!ok) atomicOr(a.err, (uint32_t)ERR_NONFINITE);
@@ -647,8 +647,7 @@ __device__ __forceinline__ T line_march_bare(const StepArgs<T, D> &a, int x0, in
         for (int k = 0; k < N; ++k) {
             const T wl = k == 0 ? lc : c.v[k - 1], wr = k == N - 1 ? rc : c.v[k + 1];
             const T lap = ((up.v[k] + dn.v[k]) + (wl + wr)) - (T)4 * c.v[k];
-            wdnew.v[k] = wdv.v[k] + g * lap;
-            wn.v[k] = c.v[k] + dt * wdnew.v[k];
+            site_update<T, D>(c.v[k], wdv.v[k], lap, g, dt, wn.v[k], wdnew.v[k]);
         }
         stg_row(wout + (int64_t)j * P, wn);
         WdIO<D>::store(wdp + (int64_t)j * P, wdnew, wd_scale);
@@ -719,8 +718,7 @@ __device__ __forceinline__ T line_march_edge(const StepArgs<T, D> &a, const Edge
                 for (int k = 0; k < N; ++k) {
                     const T wl = k == 0 ? lc : c.v[k - 1], wr = k == N - 1 ? rc : c.v[k + 1];
                     const T lap = ((up.v[k] + dn.v[k]) + (wl + wr)) - (T)4 * c.v[k];
-                    wdnew.v[k] = wdv.v[k] + a.g * lap;
-                    wn.v[k] = c.v[k] + a.dt * wdnew.v[k];
+                    site_update<T, D>(c.v[k], wdv.v[k], lap, a.g, a.dt, wn.v[k], wdnew.v[k]);
                 }
                 stg_row(a.w_out + x0 + (int64_t)j * P, wn);
                 WdIO<D>::store(a.wd + x0 + (int64_t)j * P, wdnew, a.wd_scale);

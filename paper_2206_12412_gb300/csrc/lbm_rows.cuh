@@ -161,18 +161,30 @@ template <> struct WdIO<Lf> {
     static __device__ __forceinline__ void put(Lf *, float, float) {}
 };
 
+// Operations with one fixed rounding, which the compiler neither contracts nor
+// splits.  Every kernel that advances a site (single steps, passes, batches,
+// slabs, the adjoint) forms it from these, so that all give the same bits
+// whatever else they hold.
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 // One site's update: wdot' = wdot + g lap, w' = w + dt wdot' (moment form),
 // or, with leapfrog storage (the second argument is then w_{n-1}),
-// w' = w + ((w - w_{n-1}) + g dt lap).
+// w' = w + ((w - w_{n-1}) + g dt lap).  Each sum takes its product unrounded:
+// left to the compiler, the FP16 form took the (exact) product of the stored
+// rate and its scale that way instead of g lap, in single steps but not in
+// passes, and differed wherever g is no power of two.
 template <typename T, typename D>
 __device__ __forceinline__ void site_update(T w0, T wdv, T lap, T g, T dt, T &wnew, T &wdnew)
 {
     if constexpr (std::is_same<D, Lf>::value) {
-        wnew = w0 + ((w0 - wdv) + (g * dt) * lap);
+        wnew = w0 + fma_rn(mul_rn(g, dt), lap, w0 - wdv);
         wdnew = wnew;
     } else {
-        wdnew = wdv + g * lap;
-        wnew = w0 + dt * wdnew;
+        wdnew = fma_rn(g, lap, wdv);
+        wnew = fma_rn(dt, wdnew, w0);
     }
 }
 
