@@ -22,12 +22,6 @@ SOURCES = ["lbm_kernels.cu", "lbm_adjoint.cu", "lbm_api.cu", "lbm_tape.cu", "lbm
            "lbm_pass_plan.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2", "-I" + INCLUDE, "-I" + CSRC]
-# Units whose kernels are compiled in parallel parts: the transposed step's
-# multiply-adds are then contracted alike in its single steps and its passes
-# (compiled whole they differ in the last bit where dt is not 1).  The other
-# units lose 2-8 % of their speed that way and are compiled whole.
-PARTS = ("lbm_adjoint.cu", "lbm_pass_tape.cu")
-
 _lock = threading.Lock()
 
 
@@ -64,8 +58,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         for src in SOURCES:
             obj = os.path.join(BUILD_DIR, os.path.splitext(src)[0] + ".o")
             objs.append(obj)
-            parts = ["--split-compile=0"] if src in PARTS else []
-            cmd = [nvcc, *ARCH, *parts, *FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
+            cmd = [nvcc, *ARCH, *FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
             if verbose:
                 print(" ".join(cmd))
             procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))

@@ -76,7 +76,7 @@ __device__ __forceinline__ void add_sources(const AdjArgs<T> &a, const SrcTab<T>
         for (int kk = 0; kk < N; ++kk)
             if (kk == di) {
                 anew.v[kk] += v;
-                mnew.v[kk] += a.dt * v;
+                mnew.v[kk] = fma_rn(a.dt, v, mnew.v[kk]);
             }
     }
     const int64_t srow = S.srow;
@@ -90,7 +90,7 @@ __device__ __forceinline__ void add_sources(const AdjArgs<T> &a, const SrcTab<T>
         for (int kk = 0; kk < N; ++kk)
             if (kk == di) {
                 anew.v[kk] += v;
-                mnew.v[kk] += a.dt * v;
+                mnew.v[kk] = fma_rn(a.dt, v, mnew.v[kk]);
             }
     }
 }
@@ -171,8 +171,7 @@ __device__ __forceinline__ void adj_march(const AdjArgs<T> &a, int cb, int j0, i
                 const T ml = k == 0 ? left0 : mc.v[k - 1];
                 const T mr = k == N - 1 ? rightN : mc.v[k + 1];
                 const T lap = ((ma.v[k] + mb.v[k]) + (ml + mr)) - (T)4 * mc.v[k];
-                anew.v[k] = av.v[k] + g * lap;
-                mnew.v[k] = mc.v[k] + dt * anew.v[k];
+                site_update<T, T>(mc.v[k], av.v[k], lap, g, dt, mnew.v[k], anew.v[k]);
             }
             if (SRC) add_sources<T, N>(a, S, x0, j, anew, mnew);
             stg_row(mout + (int64_t)j * P, mnew);
@@ -253,15 +252,8 @@ __device__ __noinline__ T adj_crack_rows(const AdjArgs<T> *sa, int cb, int j0, i
         const T inv_dt = (T)1 / a.dt;
 #pragma unroll
         for (int k = 0; k < N; ++k)
-            if ((cut_p >> k) & 1u) {
-                const T mB = o[qb].v[k];
-                od[qb].v[k] -= mB * inv_dt;
-                o[qb].v[k] = (T)0;
-                od[qi].v[k] += (T)1.5 * mB * inv_dt;
-                o[qi].v[k] += (T)1.5 * mB;
-                od[qii].v[k] -= (T)0.5 * mB * inv_dt;
-                o[qii].v[k] -= (T)0.5 * mB;
-            }
+            if ((cut_p >> k) & 1u)
+                face_transposed(inv_dt, o[qb].v[k], od[qb].v[k], o[qi].v[k], od[qi].v[k], o[qii].v[k], od[qii].v[k]);
     }
     if (x0 < a.nx) {
 #pragma unroll

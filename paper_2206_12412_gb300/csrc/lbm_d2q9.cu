@@ -415,8 +415,8 @@ __device__ __forceinline__ void d2q9_face_at(const StepArgs<T, T> &a, int i)
     const int64_t P = a.pitch;
     const T *wn = a.w_out;
     const T inv_dt = (T)1 / a.dt;
-    const T up = (T)1.5 * wn[(int64_t)(jc + 1) * P + i] - (T)0.5 * wn[(int64_t)(jc + 2) * P + i];
-    const T dn = (T)1.5 * wn[(int64_t)(jc - 2) * P + i] - (T)0.5 * wn[(int64_t)(jc - 3) * P + i];
+    const T up = face_value(wn[(int64_t)(jc + 1) * P + i], wn[(int64_t)(jc + 2) * P + i]);
+    const T dn = face_value(wn[(int64_t)(jc - 2) * P + i], wn[(int64_t)(jc - 3) * P + i]);
     const int64_t ou = (int64_t)jc * P + i, od = (int64_t)(jc - 1) * P + i;
     const T wdu = (up - a.w_in[ou]) * inv_dt, wdd = (dn - a.w_in[od]) * inv_dt;
     a.w_out[ou] = up;

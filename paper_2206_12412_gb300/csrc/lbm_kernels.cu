@@ -155,7 +155,7 @@ __device__ __noinline__ T crack_rows(const T *w_in_, T *w_out_, D *wd_, T wd_sca
 #pragma unroll
         for (int k = 0; k < N; ++k)
             if ((cut >> k) & 1u) {
-                const T wB = (T)1.5 * o[qi].v[k] - (T)0.5 * o[qii].v[k];
+                const T wB = face_value(o[qi].v[k], o[qii].v[k]);
                 od[qb].v[k] = (wB - w[qb + 1].v[k]) / a.dt;
                 o[qb].v[k] = wB;
             }
@@ -1316,7 +1316,7 @@ __device__ __forceinline__ void edge_rule_at(const StepArgs<T, D> &a, int t)
         // a crack-face point on an edge column (eh >= 0): its x_I, x_II are
         // the edge points one and two rows further from the crack
         const int s = j == jc ? 1 : -1;
-        v = (T)1.5 * R.point(eh, i, j + s) - (T)0.5 * R.point(eh, i, j + 2 * s);
+        v = face_value(R.point(eh, i, j + s), R.point(eh, i, j + 2 * s));
     } else if (eh >= 0 && ev >= 0) {
         const int e = (a.edge[eh] == EDGE_DIRICHLET && a.edge[ev] != EDGE_DIRICHLET) ? eh : ev;
         const int o = e == eh ? ev : eh;

@@ -989,7 +989,7 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
                     for (int k = 0; k < N; ++k)
                         if (r == r0 && k == k0) {
                             F.template rate<PH>(r).v[k] += v;
-                            F.template next<PH>(r).v[k] += dt * v;
+                            F.template next<PH>(r).v[k] = fma_rn(dt, v, F.template next<PH>(r).v[k]);
                         }
             }
         if (KIND == 2 && p.macro && face) {
@@ -997,27 +997,12 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
             const T inv_dt = dt == (T)1 ? (T)1 : div_dt((T)1, dt);
 #pragma unroll
             for (int k = 0; k < N; ++k) {
-                const T mB = below ? F.template next<PH>(RPT - 1).v[k] : F.template next<PH>(0).v[k];
                 T &oT = F.template next<PH>(RPT - 1).v[k], &oT1 = F.template next<PH>(RPT - 2).v[k], &oT2 = F.template next<PH>(RPT - 3).v[k];
                 T &oB = F.template next<PH>(0).v[k], &oB1 = F.template next<PH>(1).v[k], &oB2 = F.template next<PH>(2).v[k];
                 T &aT = F.b[RPT - 1].v[k], &aT1 = F.b[RPT - 2].v[k], &aT2 = F.b[RPT - 3].v[k];
                 T &aB = F.b[0].v[k], &aB1 = F.b[1].v[k], &aB2 = F.b[2].v[k];
-                if (cutp[k] && below) {
-                    aT -= mB * inv_dt;
-                    oT = (T)0;
-                    aT1 += (T)1.5 * mB * inv_dt;
-                    oT1 += (T)1.5 * mB;
-                    aT2 -= (T)0.5 * mB * inv_dt;
-                    oT2 -= (T)0.5 * mB;
-                }
-                if (cutp[k] && !below) {
-                    aB -= mB * inv_dt;
-                    oB = (T)0;
-                    aB1 += (T)1.5 * mB * inv_dt;
-                    oB1 += (T)1.5 * mB;
-                    aB2 -= (T)0.5 * mB * inv_dt;
-                    oB2 -= (T)0.5 * mB;
-                }
+                if (cutp[k] && below) face_transposed(inv_dt, oT, aT, oT1, aT1, oT2, aT2);
+                if (cutp[k] && !below) face_transposed(inv_dt, oB, aB, oB1, aB1, oB2, aB2);
             }
         }
     }
@@ -1028,7 +1013,7 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
         for (int k = 0; k < N; ++k) {
             const T w2 = below ? F.template next<PH>(RPT - 2).v[k] : F.template next<PH>(1).v[k];
             const T w3 = below ? F.template next<PH>(RPT - 3).v[k] : F.template next<PH>(2).v[k];
-            wB.v[k] = (T)1.5 * w2 - (T)0.5 * w3;
+            wB.v[k] = face_value(w2, w3);
             w0.v[k] = below ? last.v[k] : first.v[k];
         }
         R rt = wB;
@@ -1111,7 +1096,7 @@ __device__ __forceinline__ void pass_step(const PassArgs<T, D> &A, const PassCtx
                     if (!(cut[k] && ((on_l && k == 0) || (on_r && k == c.kr)))) continue;
                     const T v1 = below ? F.template next<PH>(RPT - 2).v[k] : F.template next<PH>(1).v[k];
                     const T v2 = below ? F.template next<PH>(RPT - 3).v[k] : F.template next<PH>(2).v[k];
-                    const T v = (T)1.5 * v1 - (T)0.5 * v2;
+                    const T v = face_value(v1, v2);
                     Row<T, 1> wn, wo;
                     wn.v[0] = v;
                     wo.v[0] = below ? last.v[k] : first.v[k];

@@ -188,6 +188,23 @@ __device__ __forceinline__ void site_update(T w0, T wdv, T lap, T g, T dt, T &wn
     }
 }
 
+// The macroscopic rule's value at a boundary point from its two sites along the
+// inward normal (free edges and crack faces): w_B = 1.5 w_I - 0.5 w_II.
+template <typename T> __device__ __forceinline__ T face_value(T wI, T wII) { return fma_rn((T)1.5, wI, (T)-0.5 * wII); }
+
+// Its transpose: m and a of the boundary point (mB, aB) go to the two sites.
+template <typename T>
+__device__ __forceinline__ void face_transposed(T inv_dt, T &mB, T &aB, T &mI, T &aI, T &mII, T &aII)
+{
+    const T m = mB, nI = mul_rn((T)1.5, m), nII = mul_rn((T)0.5, m);
+    aB = fma_rn(-m, inv_dt, aB);
+    mB = (T)0;
+    aI = fma_rn(nI, inv_dt, aI);
+    mI += nI;
+    aII = fma_rn(-nII, inv_dt, aII);
+    mII -= nII;
+}
+
 // Pad images of the new values of row j, for the next step's neighbours.
 template <typename A, typename T, int N>
 __device__ __forceinline__ void write_pads(const A &a, int x0, int j, const Row<T, N> &wnew)
@@ -298,8 +315,8 @@ struct EdgeRule {
     __device__ __forceinline__ T rule(int e, T wI, T wII) const
     {
         if (dir[e])
-            return (T)(8.0 / 15.0) * ws[e] + (T)(2.0 / 3.0) * wI - (T)0.2 * wII;
-        return (T)1.5 * wI - (T)0.5 * wII;
+            return fma_rn((T)-0.2, wII, fma_rn((T)(2.0 / 3.0), wI, mul_rn((T)(8.0 / 15.0), ws[e])));
+        return face_value(wI, wII);
     }
     // a non-corner point of edge e from its two sites along the inward normal
     __device__ __forceinline__ T point(int e, int i, int j) const
