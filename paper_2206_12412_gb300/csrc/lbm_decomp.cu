@@ -204,9 +204,9 @@ lbm_status lbm_decomp_create(const lbm_grid *grid, const lbm_lattice *lattice, c
     d->esize = d->slabs[0]->esize;
     d->row_bytes = d->slabs[0]->pitch * (int64_t)d->esize;
     if (lattice->storage == LBM_F32_WD_F16) {
-        // the scale the undivided lattice takes: the smallest over the slabs
-        double scale = 0.0;
-        for (lbm_handle *h : d->slabs) scale = scale == 0.0 ? h->wd_scale : std::min(scale, h->wd_scale);
+        // the scale of the undivided lattice (a slab without a loaded edge would
+        // take another, which rounds small rates otherwise)
+        const double scale = fp16_wd_scale(grid, loads, n_loads);
         for (lbm_handle *h : d->slabs) {
             lbm_status rc = lbm_set_wd_scale(h, scale);
             if (rc != LBM_OK) {

@@ -111,6 +111,21 @@ def test_batch_equals_lattices_alone(gpu, storage):
     batch.close()
 
 
+@pytest.mark.parametrize("storage", STORAGES)
+def test_slabs_equal_lattice(gpu, storage):
+    lbm = gpu
+    p = _strip(300, 150, **FORMS["kcrit"])
+    w0, wd0 = W.random_state(300, 150, 11)
+    lat, dec = lbm.Lattice(p, storage), lbm.Decomp(p, 3, storage)
+    for x in (lat, dec):
+        x.set_fields(w0, wd0)
+        x.step(30)
+    for a, b in zip(lat.fields(), dec.fields()):
+        np.testing.assert_array_equal(a, b)
+    lat.close()
+    dec.close()
+
+
 @pytest.mark.parametrize("storage", ["f32", "f64"])
 @pytest.mark.parametrize("kind", ["macro_growth", "bb_growth", "bb_periodic", "all_dirichlet", "no_crack", "wide_macro"])
 def test_tape_passes_equal_single_steps(gpu, kind, storage):
