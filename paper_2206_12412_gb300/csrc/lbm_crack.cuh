@@ -32,16 +32,21 @@ __device__ __forceinline__ double load_value(const LoadDesc L, int64_t n, double
     }
 }
 
-// a / b for a divisor known in advance, y = 1 / b rounded: the residual of a y
-// is exact in one FMA, and adding its share rounds to the quotient (Markstein,
-// IBM J. Res. Dev. 34, 1990; equal to the division in 1.2e8 random quotients
-// over the divisors used here).  Three FP64 instructions instead of ten, at
-// 64 cycles each.
+// a / b for a divisor known in advance, y = 1 / b: the residual of a y is exact in
+// one FMA, and adding its share rounds to the quotient (Markstein, IBM J. Res.
+// Dev. 34, 1990; equal to the division in 3e8 random quotients).  Three FP64
+// instructions instead of ten, at 64 cycles each.  For operands whose products
+// and residual are normal numbers: distances over 2 pi, and K over K_C where K_C is
+// a known_divisor and K is not huge.
 __device__ __forceinline__ double div_known(double a, double b, double y)
 {
     const double q = a * y;
     return fma(fma(-q, b, a), y, q);
 }
+// K from 2^500 on, infinities and NaN (by its bits: FP64 comparisons cost 64 cycles).
+__device__ __forceinline__ bool huge_K(double Ka) { return __double2hiint(Ka) >= 1523 << 20; }
+// The division as a call, so that it is not computed beside the other form.
+static __device__ __noinline__ double div_call(double a, double b) { return a / b; }
 
 // ------------------------------------------------------------ crack step
 //

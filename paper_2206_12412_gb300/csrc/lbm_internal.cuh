@@ -33,6 +33,9 @@ namespace lbm {
 constexpr int kQBits = 32;                          // tip fixed point: 1 dh = 2^32 units
 constexpr double kTwoM32 = 2.3283064365386963e-10;  // 2^-32
 constexpr double kPi = 3.14159265358979323846;
+// Critical values whose quotients are formed by their inverse (div_known); others take the division.
+__host__ __device__ __forceinline__ bool known_divisor(double b) { return b > 0x1p-500 && b < 0x1p500; }
+__host__ __device__ __forceinline__ double known_inverse(double b) { return known_divisor(b) ? 1.0 / b : 0.0; }
 constexpr int kThreads = 128;                       // threads per CTA of the step kernel
 constexpr int kMinBlocks = 8;                       // resident CTAs per SM the kernel is built for
 constexpr int64_t kChainedSites = int64_t(1) << 18;  // lattices up to this size launch their steps chained
@@ -214,10 +217,10 @@ struct PassPlan {
     int64_t lo_q, hi_q;
     double r_min;
     int32_t one_pair;
-    int32_t unit;              // dh = dt = 1
+    int32_t unit;              // dh = dt = 1, and K_C a known_divisor
     float lo_f;                // r_min at rest
     int64_t w_q;               // the window's width
-    double k_inv;              // 1 / K_C
+    double k_inv;              // 1 / K_C (unit only)
     float k_unit, k_rest;      // mu / 4 sqrt(2 pi / dh) 2^16; just below K_C
     // column tiles of the bulk: of px vectors, the first ex of them of one more
     int32_t mx, px, ex;

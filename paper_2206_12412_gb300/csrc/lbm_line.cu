@@ -227,7 +227,7 @@ __device__ LineSums line_eval_warp(const CrackParams &p, const T *w, int64_t P, 
 // on the state S (shared memory), given that end's sums: K, the criterion,
 // the advance (with the stop at the boundary), the severed links, the end's
 // fields of S and, if `commit`, its history record at hist_n (x in tip /
-// tipl, y in tipy / tipyl).  k_inv: 1 / K_C.
+// tipl, y in tipy / tipyl).  k_inv: known_inverse(K_C).
 __device__ void line_apply_warp(const CrackParams &p, uint32_t *cut_h, uint32_t *cut_v, const History &hist,
                                 CrackState &S, int dir, bool commit, const LineSums &c, double k_inv)
 {
@@ -240,7 +240,8 @@ __device__ void line_apply_warp(const CrackParams &p, uint32_t *cut_h, uint32_t 
         propagate = 1;
         v = p.v_rel;
     } else if (p.mode == CRACK_KCRIT && c.np > 0 && fabs(K) > p.K_C) {
-        const double ratio = isinf(K) ? fabs(K) : div_known(fabs(K), p.K_C, k_inv);
+        const double Ka = fabs(K);
+        const double ratio = __double_as_longlong(k_inv) == 0 || huge_K(Ka) ? div_call(Ka, p.K_C) : div_known(Ka, p.K_C, k_inv);
         propagate = 1;
         v = p.v_max * tanh(sqrt(ratio * ratio * ratio * ratio - 1.0));   // eq. v-tanh
     }
@@ -329,7 +330,7 @@ __device__ void line_step_warp(const CrackParams &p, const T *w, int64_t P, uint
     const LineSums cr = line_eval_warp<T>(p, w, P, cut_h, cut_v, S.r, +1);
     LineSums cl{0.0, 0.0, 0.0, 0};
     if (p.two_tips) cl = line_eval_warp<T>(p, w, P, cut_h, cut_v, S.l, -1);
-    const double k_inv = 1.0 / p.K_C;
+    const double k_inv = known_inverse(p.K_C);
     line_apply_warp(p, cut_h, cut_v, hist, S, +1, commit, cr, k_inv);
     if (p.two_tips) line_apply_warp(p, cut_h, cut_v, hist, S, -1, commit, cl, k_inv);
 }
@@ -518,7 +519,7 @@ __device__ __forceinline__ bool seg_claimed(const Claims &c, int s, int j, int W
 // link, as Alg. 1 orders them -- then the record and the next state, and the
 // ends' boxes with the cuts in force after it.  What the decisions do not
 // need is done beside them: warp 2 copies the state and forms the next
-// Dirichlet values, warp 3 the claims and the edge values (sC, sE) and 1 / K_C.
+// Dirichlet values, warp 3 the claims and the edge values (sC, sE) and the inverse of K_C.
 template <typename T, typename D>
 __device__ void tip_cta(const StepArgs<T, D> &a, CrackState &sS, EdgeValues<T> &E, Claims &C)
 {
@@ -543,7 +544,7 @@ __device__ void tip_cta(const StepArgs<T, D> &a, CrackState &sS, EdgeValues<T> &
         if (lane == 0) {
             C = claims(p, in);
             E = edge_values<T>(in);
-            k_inv = p.mode == CRACK_KCRIT ? 1.0 / p.K_C : 0.0;
+            k_inv = p.mode == CRACK_KCRIT ? known_inverse(p.K_C) : 0.0;
         }
     } else if (active && mine) {
         cs = line_eval_warp<T>(p, a.w_in, a.pitch, a.cut_h, a.cut_v, dir > 0 ? in->r : in->l, dir);

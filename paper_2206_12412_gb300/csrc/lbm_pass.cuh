@@ -452,13 +452,12 @@ __device__ __forceinline__ void pass_crack_step(const CrackParams &p, const Pass
                 d.K = pass_K(p, c);
                 d.flags = E.flags;
                 const double Ka = fabs(d.K);
-                const bool bad = (__double_as_longlong(d.K) & 0x7ff0000000000000ll) == 0x7ff0000000000000ll;
                 if (c.np > 0 && Ka > p.K_C) {
-                    const double ratio = bad ? Ka : div_known(Ka, p.K_C, q.k_inv);
+                    const double ratio = div_known(Ka, p.K_C, q.k_inv);
                     d.propagate = 1;
                     d.v = p.v_max * tanh(sqrt(ratio * ratio * ratio * ratio - 1.0));   // eq. v-tanh
                 }
-                if (bad) d.flags |= FLAG_NONFINITE;
+                full = huge_K(Ka);
                 if (E.arrested) {
                     d.propagate = 0;
                     d.v = 0.0;

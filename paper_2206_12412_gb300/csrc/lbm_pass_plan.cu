@@ -127,10 +127,10 @@ bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q, bool ad
         q.hi_q = (int64_t)std::ceil(std::min(hi, 1e6) * 4294967296.0);
         q.one_pair = p.fit_width <= p.dh && q.hi_q - q.lo_q <= ((int64_t)1 << kQBits);
         // (a fixed r_min does not follow the speed: the general step)
-        q.unit = p.dh == 1.0 && p.dt == 1.0 && !(p.r_min_fixed > 0.0);
+        q.unit = p.dh == 1.0 && p.dt == 1.0 && !(p.r_min_fixed > 0.0) && known_divisor(p.K_C);
         q.lo_f = (float)p.r0;
         q.w_q = (int64_t)std::llrint(std::min(p.fit_width / p.dh, 1e6) * 4294967296.0);
-        q.k_inv = p.K_C > 0.0 ? 1.0 / p.K_C : 0.0;
+        q.k_inv = known_inverse(p.K_C);
         q.k_unit = (float)(p.mu / 4.0 * std::sqrt(2.0 * kPi / p.dh) * 65536.0);
         q.k_rest = (float)(p.K_C * 0.999);
         // both ends are fitted at once by half a warp each: at most 16 columns
