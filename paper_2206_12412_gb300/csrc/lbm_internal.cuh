@@ -218,7 +218,8 @@ struct PassPlan {
     double r_min;
     int32_t one_pair;
     int32_t unit;              // dh = dt = 1, and K_C a known_divisor
-    float lo_f;                // r_min at rest
+    float lo_f, lo_max;        // r_min at rest; no more than this in the crack step's FP32 form,
+    uint32_t slack;            // where it is off by less than this (units of 2^-32, modulo 1)
     int64_t w_q;               // the window's width
     double k_inv;              // 1 / K_C (unit only)
     float k_unit, k_rest;      // mu / 4 sqrt(2 pi / dh) 2^16; just below K_C

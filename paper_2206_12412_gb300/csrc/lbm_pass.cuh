@@ -49,6 +49,7 @@
 #include "lbm_d2q9.cuh"
 #include "lbm_internal.cuh"
 #include "lbm_rows.cuh"
+#include "lbm_window.h"
 
 #include <cstddef>
 #include <type_traits>
@@ -438,13 +439,13 @@ __device__ __forceinline__ void pass_crack_step(const CrackParams &p, const Pass
         bool full = !q.one_pair || !q.unit;
         if (!full && head) {
             // dh = dt = 1 and a window of at most one pair: its column from
-            // r_min in FP32 (exact unless a column lies within 2^-17 of the
+            // r_min in FP32 (exact unless a column lies within the slack of the
             // window's ends), and no FP64 operation that does not decide
-            const float lo = rest ? q.lo_f : q.lo_f / (1.0f - (float)E.v_prev);
-            const int64_t lo_q = (int64_t)(lo * 4294967296.0f), slack = (int64_t)1 << 15;
+            const float lo = rest ? q.lo_f : window_start(q.lo_f, E.v_prev);
+            const int64_t lo_q = (int64_t)(lo * 4294967296.0f);
             const PassPair w = pass_pair(dir, E.tip_q, lo_q, lo_q + ((int64_t)1 << kQBits), S.i_first, S.i_last);
             const int64_t past = w.d - lo_q;   // in [0, 2^32)
-            full = !(lo < 24.0f) || past < slack || past > ((int64_t)1 << kQBits) - slack || llabs(past - q.w_q) < slack;
+            full = !(lo < q.lo_max) || (uint32_t)past + q.slack < 2u * q.slack || (uint32_t)(past - q.w_q) + q.slack < 2u * q.slack;
             const int k = w.col - org;
             if (w.in && past < q.w_q && k >= 0 && k < W) c = pass_sums<T>(pass_sf(p, w.d), above[k], below[k], 0.0);
             if (!full) {

@@ -1,6 +1,7 @@
 // lbm_pass_plan.cu -- host side of the passes (lbm_pass.cuh): how the
 // lattice is split into tiles for a pass of K steps.
 #include "lbm_host.h"
+#include "lbm_window.h"
 
 #include <algorithm>
 #include <cmath>
@@ -127,8 +128,10 @@ bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q, bool ad
         q.hi_q = (int64_t)std::ceil(std::min(hi, 1e6) * 4294967296.0);
         q.one_pair = p.fit_width <= p.dh && q.hi_q - q.lo_q <= ((int64_t)1 << kQBits);
         // (a fixed r_min does not follow the speed: the general step)
-        q.unit = p.dh == 1.0 && p.dt == 1.0 && !(p.r_min_fixed > 0.0) && known_divisor(p.K_C);
+        q.unit = p.dh == 1.0 && p.dt == 1.0 && !(p.r_min_fixed > 0.0) && known_divisor(p.K_C) && p.r0 >= kWindowR0;
         q.lo_f = (float)p.r0;
+        q.lo_max = (float)std::min((double)kWindowLo, 1.001 * p.r0 / (1.0 - p.v_max));
+        q.slack = q.unit ? (uint32_t)window_slack(q.lo_f, q.lo_max) : 0u;
         q.w_q = (int64_t)std::llrint(std::min(p.fit_width / p.dh, 1e6) * 4294967296.0);
         q.k_inv = known_inverse(p.K_C);
         q.k_unit = (float)(p.mu / 4.0 * std::sqrt(2.0 * kPi / p.dh) * 65536.0);

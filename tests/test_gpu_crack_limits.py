@@ -1,5 +1,5 @@
 """The crack step at the ends of its parameters' ranges: critical values that
-1 / K_C or K / K_C does not fit a double for."""
+1 / K_C or K / K_C does not fit a double for, and speeds near that of shear waves."""
 import numpy as np
 import pytest
 
@@ -71,3 +71,10 @@ def test_smallest_critical_values_any_direction(gpu, K_C, two):
         got.append(_run(gpu, p, "f32", [50]))
     assert got[1][1]["v"] == 0.85
     _same(*got)
+
+
+@pytest.mark.parametrize("r0", [0.6, 1.0, 2.0])
+@pytest.mark.parametrize("v_max", [0.92, 0.95, 0.99])
+def test_fast_ends(gpu, r0, v_max):
+    p = _problem(900, 90, K_C=2e-7, v_max=v_max, r0=r0, x_start=430.2, x_tip=460.7, two_tips=True)
+    _same(_run(gpu, p, "f32", [230]), _run(gpu, p, "f32", [1] * 230))
