@@ -222,7 +222,7 @@ struct PassPlan {
     uint32_t slack;            // where it is off by less than this (units of 2^-32, modulo 1)
     int64_t w_q;               // the window's width
     double k_inv;              // 1 / K_C (unit only)
-    float k_unit, k_rest;      // mu / 4 sqrt(2 pi / dh) 2^16; just below K_C
+    float k_unit, k_rest;      // mu / 4 sqrt(2 pi / dh) 2^16; just below K_C (0: no such test)
     // column tiles of the bulk: of px vectors, the first ex of them of one more
     int32_t mx, px, ex;
     int32_t jb, mb, pb, eb;    // rows [0, jb) below the strip: mb row tiles of pb rows, the first eb of one more

@@ -134,8 +134,13 @@ bool pass_plan(const lbm_handle *h, int K, int nw, int rpt, PassPlan &q, bool ad
         q.slack = q.unit ? (uint32_t)window_slack(q.lo_f, q.lo_max) : 0u;
         q.w_q = (int64_t)std::llrint(std::min(p.fit_width / p.dh, 1e6) * 4294967296.0);
         q.k_inv = known_inverse(p.K_C);
-        q.k_unit = (float)(p.mu / 4.0 * std::sqrt(2.0 * kPi / p.dh) * 65536.0);
-        q.k_rest = (float)(p.K_C * 0.999);
+        // the FP32 test that an end at rest stays there has a margin of 1e-3: taken
+        // where neither its factors nor an FP64 jump too small for FP32 (off by
+        // 2^-150 at most, times up to 16 units) round by as much; else an end is
+        // never seen to rest by it
+        const double unit = p.mu / 4.0 * std::sqrt(2.0 * kPi / p.dh) * 65536.0;
+        q.k_unit = (float)unit;
+        q.k_rest = unit >= 0x1p-60 && unit <= 0x1p90 && p.K_C >= 0x1p-100 && p.K_C >= unit * 0x1p-135 ? (float)(p.K_C * 0.999) : 0.0f;
         // both ends are fitted at once by half a warp each: at most 16 columns
         if (!(p.fit_width / p.dh <= 12.0)) return false;
         q.free = narrow && p.mode != CRACK_KCRIT && q.one_pair;

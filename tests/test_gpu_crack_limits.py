@@ -1,5 +1,6 @@
 """The crack step at the ends of its parameters' ranges: critical values that
-1 / K_C or K / K_C does not fit a double for, and speeds near that of shear waves."""
+1 / K_C or K / K_C does not fit a double for, speeds near that of shear waves,
+and fields far below FP32's range."""
 import numpy as np
 import pytest
 
@@ -78,3 +79,17 @@ def test_smallest_critical_values_any_direction(gpu, K_C, two):
 def test_fast_ends(gpu, r0, v_max):
     p = _problem(900, 90, K_C=2e-7, v_max=v_max, r0=r0, x_start=430.2, x_tip=460.7, two_tips=True)
     _same(_run(gpu, p, "f32", [230]), _run(gpu, p, "f32", [1] * 230))
+
+
+@pytest.mark.parametrize("K_C", [3e-5, 1.2e-4])
+def test_fields_below_fp32(gpu, K_C):
+    """A problem scaled by powers of two gives the scaled results, also where its
+    jumps are no FP32 numbers: ends rest and grow in the same steps."""
+    su, sm = 2.0 ** -150, 2.0 ** 100
+    a = _run(gpu, _problem(150, 90, K_C=K_C), "f64", [120])
+    b = _run(gpu, _problem(150, 90, scale_mu=sm, scale_u=su, K_C=K_C * sm * su), "f64", [120], su)
+    assert a[1]["tip_q"] > int(150 / 4 * 2.0 ** 32)   # it grows
+    assert a[1]["tip_q"] == b[1]["tip_q"]
+    for x, y in zip(a[0][:2], b[0][:2]):
+        np.testing.assert_array_equal(x * su, y)
+    np.testing.assert_array_equal(a[0][2], b[0][2])
