@@ -1284,17 +1284,17 @@ lbm_status lbm_step(lbm_handle *h, int64_t n)
 }
 
 // A plane of the handle to / from device memory of the caller's.
-static cudaError_t plane_out(const lbm_handle *h, const void *plane, void *dst, int64_t stride)
+static cudaError_t plane_out(const lbm_handle *h, const void *plane, void *dst)
 {
     const int nx = h->grid.nx, ny = h->grid.ny;
-    return h->esize == 8 ? launch_plane_out<double>(static_cast<const double *>(plane), h->pitch, nx, ny, static_cast<double *>(dst), stride, h->stream)
-                         : launch_plane_out<float>(static_cast<const float *>(plane), h->pitch, nx, ny, static_cast<float *>(dst), stride, h->stream);
+    return h->esize == 8 ? launch_plane_out<double>(static_cast<const double *>(plane), h->pitch, nx, ny, static_cast<double *>(dst), h->stream)
+                         : launch_plane_out<float>(static_cast<const float *>(plane), h->pitch, nx, ny, static_cast<float *>(dst), h->stream);
 }
-static cudaError_t plane_in(const lbm_handle *h, void *plane, const void *src, int64_t stride)
+static cudaError_t plane_in(const lbm_handle *h, void *plane, const void *src)
 {
     const int nx = h->grid.nx, ny = h->grid.ny;
-    return h->esize == 8 ? launch_plane_in<double>(static_cast<double *>(plane), h->pitch, nx, ny, static_cast<const double *>(src), stride, h->stream)
-                         : launch_plane_in<float>(static_cast<float *>(plane), h->pitch, nx, ny, static_cast<const float *>(src), stride, h->stream);
+    return h->esize == 8 ? launch_plane_in<double>(static_cast<double *>(plane), h->pitch, nx, ny, static_cast<const double *>(src), h->stream)
+                         : launch_plane_in<float>(static_cast<float *>(plane), h->pitch, nx, ny, static_cast<const float *>(src), h->stream);
 }
 
 // The dtype a field is exchanged in: the arithmetic precision (FP64 for F64
@@ -1324,7 +1324,7 @@ lbm_status lbm_fields(lbm_handle *h, int32_t which, void *dst, int32_t dst_on_de
             LBM_CUDA(cudaMemcpyAsync(dst, conv, (size_t)h->grid.nx * h->grid.ny * 4, cudaMemcpyDeviceToHost, h->stream));
     } else {
         const void *src = which == LBM_FIELD_W ? h->w[h->parity] : h->wd;
-        if (dst_on_device) LBM_CUDA(plane_out(h, src, dst, h->grid.nx));
+        if (dst_on_device) LBM_CUDA(plane_out(h, src, dst));
         else LBM_CUDA(cudaMemcpy2DAsync(dst, row, src, (size_t)h->pitch * h->esize, row, (size_t)h->grid.ny, kind, h->stream));
     }
     if (!dst_on_device) return check_sticky(h);
@@ -1359,7 +1359,7 @@ lbm_status lbm_set_fields(lbm_handle *h, int32_t which, const void *src, int32_t
         LBM_CUDA(wd_from_f32(h, conv, h->wd_scale, h->stream));
     } else {
         void *dst = which == LBM_FIELD_W ? h->w[h->parity] : h->wd;
-        if (src_on_device) LBM_CUDA(plane_in(h, dst, src, h->grid.nx));
+        if (src_on_device) LBM_CUDA(plane_in(h, dst, src));
         else LBM_CUDA(cudaMemcpy2DAsync(dst, (size_t)h->pitch * h->esize, src, row, row, (size_t)h->grid.ny,
                                         cudaMemcpyHostToDevice, h->stream));
         if (which == LBM_FIELD_W) {

@@ -407,12 +407,9 @@ cudaError_t launch_grad_sum(const T *edge, int64_t edge_ring, int64_t edge_len, 
                             int nx, int ny, int dir_mask, double g, double *grad, cudaStream_t s);
 template <typename T>
 cudaError_t launch_adjoint_out(const T *a, const T *m, int64_t pitch, int nx, int ny, T dt, T *dw, T *dwd, cudaStream_t s);
-// A plane (element (0, 0) of padded rows) to / from an array of the caller's
-// whose rows lie `stride` elements apart.
-template <typename T>
-cudaError_t launch_plane_out(const T *w, int64_t pitch, int nx, int ny, T *dst, int64_t stride, cudaStream_t s);
-template <typename T>
-cudaError_t launch_plane_in(T *w, int64_t pitch, int nx, int ny, const T *src, int64_t stride, cudaStream_t s);
+// A plane (element (0, 0) of padded rows) to / from a dense array of the caller's.
+template <typename T> cudaError_t launch_plane_out(const T *w, int64_t pitch, int nx, int ny, T *dst, cudaStream_t s);
+template <typename T> cudaError_t launch_plane_in(T *w, int64_t pitch, int nx, int ny, const T *src, cudaStream_t s);
 template <typename D>
 cudaError_t launch_wd_to_f32(const D *wd, int64_t pitch, int nx, int ny, float scale, float *dst, cudaStream_t s);
 // Leapfrog storage: wdot_n = (w_n - w_{n-1}) / dt into a dense array, and

@@ -29,6 +29,7 @@
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+#include <algorithm>
 #include <type_traits>
 
 namespace lbm {
@@ -994,35 +995,41 @@ cudaError_t launch_batch_pieces(const StepArgs<T, D> *descs, const BatchPiece *p
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
-// --------------------------------- planes to and from dense or strided arrays
+// ------------------------------------------- planes to and from dense arrays
 //
 // Exchange of the padded planes with the caller's arrays.  A thread takes
 // four neighbouring columns of one row (two in FP64), as one 16-byte access
-// on each side where the caller's rows allow it (base and stride whole
-// vectors, no ragged end), column by column elsewhere; a CTA marches down its
+// on each side where the caller's rows allow it (base and width whole
+// vectors), column by column elsewhere; a CTA marches down its
 // rows, so that no element costs a division.  Bound by HBM: 8192 x 8192 FP32,
 // one plane in 0.13 ms, against 0.3 ms through cudaMemcpy2DAsync and 0.25 ms
 // for the 16-bit and leapfrog conversions with a thread per element.
 
-constexpr int kCopyThreads = 128, kCopyRows = 16;
+// A grid is at most kCopyBlocks CTAs high (a grid may be 65535): the CTAs of a
+// taller lattice take several blocks of rows each.
+
+constexpr int kCopyThreads = 128, kCopyRows = 16, kCopyBlocks = 32768;
 
 // f(padded offset, dense offset, number of columns) for this thread's pieces.
 template <int N, typename F>
-__device__ __forceinline__ void for_pieces(int64_t P, int64_t stride, int nx, int ny, F &&f)
+__device__ __forceinline__ void for_pieces(int64_t P, int nx, int ny, F &&f)
 {
-    const int i = (blockIdx.x * kCopyThreads + threadIdx.x) * N;
+    const int64_t i = ((int64_t)blockIdx.x * kCopyThreads + threadIdx.x) * N;
     if (i >= nx) return;
-    const int j1 = min(ny, (int)(blockIdx.y + 1) * kCopyRows);
+    const int m = (int)min((int64_t)N, nx - i);
+    for (int64_t j0 = (int64_t)blockIdx.y * kCopyRows; j0 < ny; j0 += (int64_t)kCopyBlocks * kCopyRows) {
+        const int64_t j1 = min((int64_t)ny, j0 + kCopyRows);
 #pragma unroll 4
-    for (int j = blockIdx.y * kCopyRows; j < j1; ++j) f((int64_t)j * P + i, (int64_t)j * stride + i, min(N, nx - i));
+        for (int64_t j = j0; j < j1; ++j) f(j * P + i, j * nx + i, m);
+    }
 }
 
 // get(plane offset, k): the value of column k of a piece.
 template <typename T, bool VEC, typename G>
-__device__ __forceinline__ void copy_out(int64_t P, int64_t stride, int nx, int ny, T *dst, G &&get)
+__device__ __forceinline__ void copy_out(int64_t P, int nx, int ny, T *dst, G &&get)
 {
     constexpr int N = Vec<T>::N;
-    for_pieces<N>(P, stride, nx, ny, [&](int64_t o, int64_t q, int m) {
+    for_pieces<N>(P, nx, ny, [&](int64_t o, int64_t q, int m) {
         Row<T, N> r;
         get(o, r);
         if (VEC) stg_row(dst + q, r);
@@ -1033,10 +1040,10 @@ __device__ __forceinline__ void copy_out(int64_t P, int64_t stride, int nx, int 
     });
 }
 template <typename T, bool VEC, typename S>
-__device__ __forceinline__ void copy_in(int64_t P, int64_t stride, int nx, int ny, const T *src, S &&set)
+__device__ __forceinline__ void copy_in(int64_t P, int nx, int ny, const T *src, S &&set)
 {
     constexpr int N = Vec<T>::N;
-    for_pieces<N>(P, stride, nx, ny, [&](int64_t o, int64_t q, int m) {
+    for_pieces<N>(P, nx, ny, [&](int64_t o, int64_t q, int m) {
         Row<T, N> r;
         if (VEC) ldg_row(src + q, r);
         else
@@ -1047,28 +1054,28 @@ __device__ __forceinline__ void copy_in(int64_t P, int64_t stride, int nx, int n
 }
 
 // Whole vectors on the caller's side.
-template <typename T> bool whole_vectors(const void *p, int64_t stride, int nx)
+template <typename T> bool whole_vectors(const void *p, int nx)
 {
     constexpr int N = Vec<T>::N;
-    return reinterpret_cast<uintptr_t>(p) % 16 == 0 && stride % N == 0 && nx % N == 0;
+    return reinterpret_cast<uintptr_t>(p) % 16 == 0 && nx % N == 0;
 }
 template <typename T> dim3 copy_grid(int nx, int ny)
 {
-    const int cols = kCopyThreads * Vec<T>::N;
-    return dim3((unsigned)((nx + cols - 1) / cols), (unsigned)((ny + kCopyRows - 1) / kCopyRows));
+    const int64_t cols = kCopyThreads * Vec<T>::N, rows = ((int64_t)ny + kCopyRows - 1) / kCopyRows;
+    return dim3((unsigned)((nx + cols - 1) / cols), (unsigned)std::min<int64_t>(rows, kCopyBlocks));
 }
 
 // (The padded rows hold whole vectors beyond column nx - 1: reading them is
 // harmless, writing them is not, since a pad next to it may hold an image.)
 template <typename T, bool VEC>
-__global__ void __launch_bounds__(kCopyThreads) plane_out_kernel(const T *w, int64_t P, int nx, int ny, T *dst, int64_t stride)
+__global__ void __launch_bounds__(kCopyThreads) plane_out_kernel(const T *w, int64_t P, int nx, int ny, T *dst)
 {
-    copy_out<T, VEC>(P, stride, nx, ny, dst, [&](int64_t o, Row<T, Vec<T>::N> &r) { ldg_row(w + o, r); });
+    copy_out<T, VEC>(P, nx, ny, dst, [&](int64_t o, Row<T, Vec<T>::N> &r) { ldg_row(w + o, r); });
 }
 template <typename T, bool VEC>
-__global__ void __launch_bounds__(kCopyThreads) plane_in_kernel(T *w, int64_t P, int nx, int ny, const T *src, int64_t stride)
+__global__ void __launch_bounds__(kCopyThreads) plane_in_kernel(T *w, int64_t P, int nx, int ny, const T *src)
 {
-    copy_in<T, VEC>(P, stride, nx, ny, src, [&](int64_t o, int m, const Row<T, Vec<T>::N> &r) {
+    copy_in<T, VEC>(P, nx, ny, src, [&](int64_t o, int m, const Row<T, Vec<T>::N> &r) {
         if (VEC) stg_row(w + o, r);
         else
 #pragma unroll
@@ -1079,12 +1086,12 @@ __global__ void __launch_bounds__(kCopyThreads) plane_in_kernel(T *w, int64_t P,
 template <typename D, bool VEC>
 __global__ void __launch_bounds__(kCopyThreads) wd_out_kernel(const D *wd, int64_t P, int nx, int ny, float inv, float *dst)
 {
-    copy_out<float, VEC>(P, nx, nx, ny, dst, [&](int64_t o, Row<float, 4> &r) { WdIO<D>::load(wd + o, r, inv); });
+    copy_out<float, VEC>(P, nx, ny, dst, [&](int64_t o, Row<float, 4> &r) { WdIO<D>::load(wd + o, r, inv); });
 }
 template <typename D, bool VEC>
 __global__ void __launch_bounds__(kCopyThreads) wd_in_kernel(D *wd, int64_t P, int nx, int ny, float scale, const float *src)
 {
-    copy_in<float, VEC>(P, nx, nx, ny, src, [&](int64_t o, int m, const Row<float, 4> &r) {
+    copy_in<float, VEC>(P, nx, ny, src, [&](int64_t o, int m, const Row<float, 4> &r) {
         if (VEC) WdIO<D>::store(wd + o, r, scale);
         else
 #pragma unroll
@@ -1094,29 +1101,29 @@ __global__ void __launch_bounds__(kCopyThreads) wd_in_kernel(D *wd, int64_t P, i
 }
 
 template <typename T>
-cudaError_t launch_plane_out(const T *w, int64_t pitch, int nx, int ny, T *dst, int64_t stride, cudaStream_t s)
+cudaError_t launch_plane_out(const T *w, int64_t pitch, int nx, int ny, T *dst, cudaStream_t s)
 {
-    if (whole_vectors<T>(dst, stride, nx)) plane_out_kernel<T, true><<<copy_grid<T>(nx, ny), kCopyThreads, 0, s>>>(w, pitch, nx, ny, dst, stride);
-    else plane_out_kernel<T, false><<<copy_grid<T>(nx, ny), kCopyThreads, 0, s>>>(w, pitch, nx, ny, dst, stride);
+    if (whole_vectors<T>(dst, nx)) plane_out_kernel<T, true><<<copy_grid<T>(nx, ny), kCopyThreads, 0, s>>>(w, pitch, nx, ny, dst);
+    else plane_out_kernel<T, false><<<copy_grid<T>(nx, ny), kCopyThreads, 0, s>>>(w, pitch, nx, ny, dst);
     return cudaGetLastError();
 }
 template <typename T>
-cudaError_t launch_plane_in(T *w, int64_t pitch, int nx, int ny, const T *src, int64_t stride, cudaStream_t s)
+cudaError_t launch_plane_in(T *w, int64_t pitch, int nx, int ny, const T *src, cudaStream_t s)
 {
-    if (whole_vectors<T>(src, stride, nx)) plane_in_kernel<T, true><<<copy_grid<T>(nx, ny), kCopyThreads, 0, s>>>(w, pitch, nx, ny, src, stride);
-    else plane_in_kernel<T, false><<<copy_grid<T>(nx, ny), kCopyThreads, 0, s>>>(w, pitch, nx, ny, src, stride);
+    if (whole_vectors<T>(src, nx)) plane_in_kernel<T, true><<<copy_grid<T>(nx, ny), kCopyThreads, 0, s>>>(w, pitch, nx, ny, src);
+    else plane_in_kernel<T, false><<<copy_grid<T>(nx, ny), kCopyThreads, 0, s>>>(w, pitch, nx, ny, src);
     return cudaGetLastError();
 }
-template cudaError_t launch_plane_out<float>(const float *, int64_t, int, int, float *, int64_t, cudaStream_t);
-template cudaError_t launch_plane_out<double>(const double *, int64_t, int, int, double *, int64_t, cudaStream_t);
-template cudaError_t launch_plane_in<float>(float *, int64_t, int, int, const float *, int64_t, cudaStream_t);
-template cudaError_t launch_plane_in<double>(double *, int64_t, int, int, const double *, int64_t, cudaStream_t);
+template cudaError_t launch_plane_out<float>(const float *, int64_t, int, int, float *, cudaStream_t);
+template cudaError_t launch_plane_out<double>(const double *, int64_t, int, int, double *, cudaStream_t);
+template cudaError_t launch_plane_in<float>(float *, int64_t, int, int, const float *, cudaStream_t);
+template cudaError_t launch_plane_in<double>(double *, int64_t, int, int, const double *, cudaStream_t);
 
 template <typename D>
 cudaError_t launch_wd_to_f32(const D *wd, int64_t pitch, int nx, int ny, float scale, float *dst, cudaStream_t s)
 {
     const float inv = 1.0f / scale;
-    if (whole_vectors<float>(dst, nx, nx)) wd_out_kernel<D, true><<<copy_grid<float>(nx, ny), kCopyThreads, 0, s>>>(wd, pitch, nx, ny, inv, dst);
+    if (whole_vectors<float>(dst, nx)) wd_out_kernel<D, true><<<copy_grid<float>(nx, ny), kCopyThreads, 0, s>>>(wd, pitch, nx, ny, inv, dst);
     else wd_out_kernel<D, false><<<copy_grid<float>(nx, ny), kCopyThreads, 0, s>>>(wd, pitch, nx, ny, inv, dst);
     return cudaGetLastError();
 }
@@ -1124,7 +1131,7 @@ cudaError_t launch_wd_to_f32(const D *wd, int64_t pitch, int nx, int ny, float s
 template <typename D>
 cudaError_t launch_wd_from_f32(D *wd, int64_t pitch, int nx, int ny, float scale, const float *src, cudaStream_t s)
 {
-    if (whole_vectors<float>(src, nx, nx)) wd_in_kernel<D, true><<<copy_grid<float>(nx, ny), kCopyThreads, 0, s>>>(wd, pitch, nx, ny, scale, src);
+    if (whole_vectors<float>(src, nx)) wd_in_kernel<D, true><<<copy_grid<float>(nx, ny), kCopyThreads, 0, s>>>(wd, pitch, nx, ny, scale, src);
     else wd_in_kernel<D, false><<<copy_grid<float>(nx, ny), kCopyThreads, 0, s>>>(wd, pitch, nx, ny, scale, src);
     return cudaGetLastError();
 }
@@ -1134,7 +1141,7 @@ cudaError_t launch_wd_from_f32(D *wd, int64_t pitch, int nx, int ny, float scale
 template <bool VEC>
 __global__ void __launch_bounds__(kCopyThreads) lf_wdot_kernel(const float *w, const float *wprev, int64_t P, int nx, int ny, float dt, float *dst)
 {
-    copy_out<float, VEC>(P, nx, nx, ny, dst, [&](int64_t o, Row<float, 4> &r) {
+    copy_out<float, VEC>(P, nx, ny, dst, [&](int64_t o, Row<float, 4> &r) {
         Row<float, 4> p;
         ldg_row(w + o, r);
         ldg_row(wprev + o, p);
@@ -1146,7 +1153,7 @@ __global__ void __launch_bounds__(kCopyThreads) lf_wdot_kernel(const float *w, c
 template <bool VEC>
 __global__ void __launch_bounds__(kCopyThreads) lf_set_wdot_kernel(const float *w, float *wprev, int64_t P, int nx, int ny, float dt, const float *src)
 {
-    copy_in<float, VEC>(P, nx, nx, ny, src, [&](int64_t o, int m, const Row<float, 4> &r) {
+    copy_in<float, VEC>(P, nx, ny, src, [&](int64_t o, int m, const Row<float, 4> &r) {
         Row<float, 4> q;
         ldg_row(w + o, q);
 #pragma unroll
@@ -1162,7 +1169,7 @@ __global__ void __launch_bounds__(kCopyThreads) lf_set_wdot_kernel(const float *
 cudaError_t launch_lf_wdot(const float *w, const float *wprev, int64_t pitch, int nx, int ny, float dt, float *dst,
                            cudaStream_t s)
 {
-    if (whole_vectors<float>(dst, nx, nx)) lf_wdot_kernel<true><<<copy_grid<float>(nx, ny), kCopyThreads, 0, s>>>(w, wprev, pitch, nx, ny, dt, dst);
+    if (whole_vectors<float>(dst, nx)) lf_wdot_kernel<true><<<copy_grid<float>(nx, ny), kCopyThreads, 0, s>>>(w, wprev, pitch, nx, ny, dt, dst);
     else lf_wdot_kernel<false><<<copy_grid<float>(nx, ny), kCopyThreads, 0, s>>>(w, wprev, pitch, nx, ny, dt, dst);
     return cudaGetLastError();
 }
@@ -1170,7 +1177,7 @@ cudaError_t launch_lf_wdot(const float *w, const float *wprev, int64_t pitch, in
 cudaError_t launch_lf_set_wdot(const float *w, float *wprev, int64_t pitch, int nx, int ny, float dt, const float *src,
                                cudaStream_t s)
 {
-    if (whole_vectors<float>(src, nx, nx)) lf_set_wdot_kernel<true><<<copy_grid<float>(nx, ny), kCopyThreads, 0, s>>>(w, wprev, pitch, nx, ny, dt, src);
+    if (whole_vectors<float>(src, nx)) lf_set_wdot_kernel<true><<<copy_grid<float>(nx, ny), kCopyThreads, 0, s>>>(w, wprev, pitch, nx, ny, dt, src);
     else lf_set_wdot_kernel<false><<<copy_grid<float>(nx, ny), kCopyThreads, 0, s>>>(w, wprev, pitch, nx, ny, dt, src);
     return cudaGetLastError();
 }
