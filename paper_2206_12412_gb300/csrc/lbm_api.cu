@@ -1283,16 +1283,38 @@ lbm_status lbm_step(lbm_handle *h, int64_t n)
     return LBM_OK;
 }
 
+// Whether the copy kernels may access device memory of the caller's: whole
+// elements, allocated on the handle's device.  Other memory (of another GPU, which
+// kernels reach with peer access only; managed; off the elements' alignment) goes
+// through the copy engine, as dense rows.
+static bool direct(const lbm_handle *h, const void *p)
+{
+    int dev = -1;
+    cudaPointerAttributes at;
+    if (reinterpret_cast<uintptr_t>(p) % h->esize != 0) return false;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == dev;
+}
+
 // A plane of the handle to / from device memory of the caller's.
 static cudaError_t plane_out(const lbm_handle *h, const void *plane, void *dst)
 {
     const int nx = h->grid.nx, ny = h->grid.ny;
+    const size_t row = (size_t)nx * h->esize;
+    if (!direct(h, dst))
+        return cudaMemcpy2DAsync(dst, row, plane, (size_t)h->pitch * h->esize, row, (size_t)ny, cudaMemcpyDeviceToDevice, h->stream);
     return h->esize == 8 ? launch_plane_out<double>(static_cast<const double *>(plane), h->pitch, nx, ny, static_cast<double *>(dst), h->stream)
                          : launch_plane_out<float>(static_cast<const float *>(plane), h->pitch, nx, ny, static_cast<float *>(dst), h->stream);
 }
 static cudaError_t plane_in(const lbm_handle *h, void *plane, const void *src)
 {
     const int nx = h->grid.nx, ny = h->grid.ny;
+    const size_t row = (size_t)nx * h->esize;
+    if (!direct(h, src))
+        return cudaMemcpy2DAsync(plane, (size_t)h->pitch * h->esize, src, row, row, (size_t)ny, cudaMemcpyDeviceToDevice, h->stream);
     return h->esize == 8 ? launch_plane_in<double>(static_cast<double *>(plane), h->pitch, nx, ny, static_cast<const double *>(src), h->stream)
                          : launch_plane_in<float>(static_cast<float *>(plane), h->pitch, nx, ny, static_cast<const float *>(src), h->stream);
 }
@@ -1312,16 +1334,14 @@ lbm_status lbm_fields(lbm_handle *h, int32_t which, void *dst, int32_t dst_on_de
     const cudaMemcpyKind kind = dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     if (which == LBM_FIELD_WDOT && h->esize_d == 0) {
         // leapfrog storage: wdot_n = (w_n - w_{n-1}) / dt
-        float *conv = dst_on_device ? static_cast<float *>(dst) : h->staging;
+        float *conv = dst_on_device && direct(h, dst) ? static_cast<float *>(dst) : h->staging;
         LBM_CUDA(launch_lf_wdot(static_cast<const float *>(h->w[h->parity]), static_cast<const float *>(h->w[h->parity ^ 1]),
                                 h->pitch, h->grid.nx, h->grid.ny, (float)h->grid.dt, conv, h->stream));
-        if (!dst_on_device)
-            LBM_CUDA(cudaMemcpyAsync(dst, conv, (size_t)h->grid.nx * h->grid.ny * 4, cudaMemcpyDeviceToHost, h->stream));
+        if (conv != dst) LBM_CUDA(cudaMemcpyAsync(dst, conv, (size_t)h->grid.nx * h->grid.ny * 4, kind, h->stream));
     } else if (which == LBM_FIELD_WDOT && wd16(h)) {
-        float *conv = dst_on_device ? static_cast<float *>(dst) : h->staging;
+        float *conv = dst_on_device && direct(h, dst) ? static_cast<float *>(dst) : h->staging;
         LBM_CUDA(wd_to_f32(h, conv, h->wd_scale, h->stream));
-        if (!dst_on_device)
-            LBM_CUDA(cudaMemcpyAsync(dst, conv, (size_t)h->grid.nx * h->grid.ny * 4, cudaMemcpyDeviceToHost, h->stream));
+        if (conv != dst) LBM_CUDA(cudaMemcpyAsync(dst, conv, (size_t)h->grid.nx * h->grid.ny * 4, kind, h->stream));
     } else {
         const void *src = which == LBM_FIELD_W ? h->w[h->parity] : h->wd;
         if (dst_on_device) LBM_CUDA(plane_out(h, src, dst));
@@ -1341,19 +1361,20 @@ lbm_status lbm_set_fields(lbm_handle *h, int32_t which, const void *src, int32_t
     lbm_status rc = finalize(h);   // the pending crack step reads the fields being replaced
     if (rc != LBM_OK) return rc;
     const size_t row = (size_t)h->grid.nx * h->esize;
+    const cudaMemcpyKind kind = src_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     if (which == LBM_FIELD_WDOT && h->esize_d == 0) {
         // leapfrog storage: w_{n-1} = w_n - dt wdot_n, against the current w
         const float *conv = static_cast<const float *>(src);
-        if (!src_on_device) {
-            LBM_CUDA(cudaMemcpyAsync(h->staging, src, (size_t)h->grid.nx * h->grid.ny * 4, cudaMemcpyHostToDevice, h->stream));
+        if (!src_on_device || !direct(h, src)) {
+            LBM_CUDA(cudaMemcpyAsync(h->staging, src, (size_t)h->grid.nx * h->grid.ny * 4, kind, h->stream));
             conv = h->staging;
         }
         LBM_CUDA(launch_lf_set_wdot(static_cast<const float *>(h->w[h->parity]), static_cast<float *>(h->w[h->parity ^ 1]),
                                     h->pitch, h->grid.nx, h->grid.ny, (float)h->grid.dt, conv, h->stream));
     } else if (which == LBM_FIELD_WDOT && wd16(h)) {
         const float *conv = static_cast<const float *>(src);
-        if (!src_on_device) {
-            LBM_CUDA(cudaMemcpyAsync(h->staging, src, (size_t)h->grid.nx * h->grid.ny * 4, cudaMemcpyHostToDevice, h->stream));
+        if (!src_on_device || !direct(h, src)) {
+            LBM_CUDA(cudaMemcpyAsync(h->staging, src, (size_t)h->grid.nx * h->grid.ny * 4, kind, h->stream));
             conv = h->staging;
         }
         LBM_CUDA(wd_from_f32(h, conv, h->wd_scale, h->stream));

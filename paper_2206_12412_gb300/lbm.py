@@ -327,6 +327,7 @@ class Lattice:
         self.nx, self.ny = int(problem["nx"]), int(problem["ny"])
         self.np_dtype = np.float64 if storage == "f64" else np.float32
         self.torch_dtype = torch.float64 if storage == "f64" else torch.float32
+        self.device = torch.device("cuda", torch.cuda.current_device())   # the handle's
         if stream is None:
             stream = torch.cuda.current_stream()
         self.stream_obj = stream
@@ -394,7 +395,7 @@ class Lattice:
             if arr is None:
                 continue
             if isinstance(arr, self.torch.Tensor) and arr.is_cuda:
-                t = arr.to(self.torch_dtype).contiguous()
+                t = arr.to(self.device, self.torch_dtype).contiguous()
                 assert t.numel() == self.nx * self.ny
                 lbm_set_fields(self.h, A.FIELD[which], t.data_ptr(), True, self.dtype_code)
                 self.torch.cuda.current_stream().synchronize()
@@ -415,7 +416,7 @@ class Lattice:
         """(w, wdot) as CUDA tensors (copies, enqueued on the handle's stream)."""
         out = []
         for which in ("w", "wdot"):
-            t = self.torch.empty((self.ny, self.nx), dtype=self.torch_dtype, device="cuda")
+            t = self.torch.empty((self.ny, self.nx), dtype=self.torch_dtype, device=self.device)
             lbm_fields(self.h, A.FIELD[which], t.data_ptr(), True, self.dtype_code)
             out.append(t)
         return tuple(out)
@@ -853,6 +854,7 @@ class Slab(Lattice):
         self.global_ny = int(problem["ny"])
         self.np_dtype = np.float64 if storage == "f64" else np.float32
         self.torch_dtype = torch.float64 if storage == "f64" else torch.float32
+        self.device = torch.device("cuda", torch.cuda.current_device())   # the handle's
         if stream is None:
             stream = torch.cuda.current_stream()
         self.stream_obj = stream

@@ -45,3 +45,37 @@ def test_tall_lattice_round_trip(gpu, storage):
         for got, want in zip(out, (w, wd)):
             np.testing.assert_array_equal(got.cpu().numpy(), want)
     lat.close()
+
+
+@pytest.mark.parametrize("offset", [1, 2, 4, 8, 16])
+@pytest.mark.parametrize("nx", [64, 61])
+@pytest.mark.parametrize("storage", STORAGES)
+def test_device_memory_at_any_address(gpu, storage, nx, offset):
+    """Device arrays that start `offset` bytes into an allocation, off the elements'
+    alignment among them."""
+    import torch
+    ny = 33
+    lat = gpu.Lattice(W.base_problem(nx, ny), storage)
+    if storage == "f32_f16":
+        gpu.lbm_set_wd_scale(lat.h, 1.0)
+    want = [_values(ny, nx, storage, s) for s in (5, 6)]
+    raw = torch.zeros(2, ny * nx * want[0].itemsize + 32, dtype=torch.uint8, device="cuda")
+    size = want[0].nbytes
+    for k, a in enumerate(want):
+        raw[k, offset:offset + size] = torch.from_numpy(a.view(np.uint8).reshape(-1)).cuda()
+    torch.cuda.synchronize()
+    for k, which in enumerate(("w", "wdot")):
+        gpu.lbm_set_fields(lat.h, A.FIELD[which], raw[k].data_ptr() + offset, True, lat.dtype_code)
+    lat.sync()
+    for got, a in zip(lat.fields(), want):
+        np.testing.assert_array_equal(got, a)
+    raw.zero_()
+    torch.cuda.synchronize()
+    for k, which in enumerate(("w", "wdot")):
+        gpu.lbm_fields(lat.h, A.FIELD[which], raw[k].data_ptr() + offset, True, lat.dtype_code)
+    lat.sync()
+    back = raw.cpu().numpy()
+    for k, a in enumerate(want):
+        np.testing.assert_array_equal(back[k, offset:offset + size], a.view(np.uint8).reshape(-1))
+        assert not back[k, :offset].any() and not back[k, offset + size:].any()
+    lat.close()
