@@ -123,10 +123,12 @@ __device__ __forceinline__ CrackSums crack_eval_pairs(const CrackParams &p, int6
     // always), that lane's sums are the group's: adding the other lanes'
     // zeros cannot change them, so one shuffle replaces the reduction tree
     // (only where that holds for every group of the warp: the shuffles of
-    // both branches name all 32 lanes, so the warp takes one of them whole)
+    // both branches name all 32 lanes, so the warp takes one of them whole;
+    // the one ballot tells it to every lane)
     const unsigned gmask = G == 32 ? 0xffffffffu : (0xffffu << (threadIdx.x & 16));
-    const unsigned holders = __ballot_sync(0xffffffffu, np > 0) & gmask;
-    if (__all_sync(0xffffffffu, __popc(holders) <= 1)) {
+    const unsigned all = __ballot_sync(0xffffffffu, np > 0), holders = all & gmask;
+    const unsigned g0 = G == 32 ? all : all & 0xffffu, g1 = G == 32 ? 0u : all & 0xffff0000u;
+    if ((g0 & (g0 - 1u)) == 0u && (g1 & (g1 - 1u)) == 0u) {
         const int src = holders ? __ffs(holders) - 1 : (threadIdx.x & 31 & ~(G - 1));
         num = __shfl_sync(0xffffffffu, num, src);
         den = __shfl_sync(0xffffffffu, den, src);
