@@ -548,8 +548,9 @@ lbm_status lbm_batch_member(const lbm_batch *b, int32_t i, lbm_handle **h);
 
 /* Enqueue n >= 0 time steps of every lattice of the batch on the shared
  * stream (CUDA-graph replay of 64-step chunks; passes of eight, four and two
- * time steps per launch where every member allows them and no launch shape,
- * lookahead or persistent form was asked for). */
+ * time steps per launch where every member allows them, the shape and lookahead
+ * are the default ones or lbm_batch_tune's, and no persistent form was asked
+ * for). */
 lbm_status lbm_batch_step(lbm_batch *b, int64_t n);
 
 /* Number of lattices and CTAs per step of the batch (pointers may be NULL). */
@@ -604,7 +605,9 @@ lbm_status lbm_batch_get_lookahead(const lbm_batch *b, int32_t *rows);
  * applies any pending crack step, copies every member's device state to a
  * scratch allocation of the same total size (from the batch's allocator;
  * LBM_ERR_OOM if it fails) and copies it back afterwards: the lattices end as
- * they were.  Synchronises the stream.  Outputs may be NULL. */
+ * they were.  A batch that takes passes takes the shape for the few steps they
+ * leave over: *us_per_step is the time of a single step, not the batch's.
+ * Synchronises the stream.  Outputs may be NULL. */
 lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *threads, int32_t *band_rows,
                           double *us_per_step, int32_t *from_cache);
 

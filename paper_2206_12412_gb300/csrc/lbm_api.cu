@@ -2067,6 +2067,10 @@ void lbm_destroy(lbm_handle *h)
 
 }  // extern "C"
 
+struct BatchShape {
+    int threads, rows, la;
+};
+
 struct lbm_batch {
     std::vector<lbm_handle *> hs;
     int storage;
@@ -2104,7 +2108,9 @@ struct lbm_batch {
     void *pdescs[kPassKinds];
     BatchUnit *punits[kPassKinds];
     int n_punits[kPassKinds];
-    bool own_shape;      // lbm_batch_set_shape or _lookahead chose the shape of the single steps: no passes
+    // the shape of the single steps that the library chose (the default, or
+    // lbm_batch_tune's): in another one, the caller's, the batch takes no passes
+    BatchShape base;
     bool owns;           // made by lbm_create_batch: the member handles are destroyed with the batch
 };
 
@@ -2643,9 +2649,6 @@ cudaError_t enqueue_batch_pass(const lbm_batch *b, int k, int par, bool second, 
 // Shapes chosen by lbm_batch_tune in this process, keyed by the device's SM
 // count, the storage and the lattices' sizes and crack bands.
 std::mutex g_tune_mu;
-struct BatchShape {
-    int threads, rows, la;
-};
 std::map<std::string, BatchShape> g_tune_cache;
 
 std::string batch_key(const lbm_batch *b)
@@ -2742,7 +2745,7 @@ lbm_status lbm_batch_create(lbm_handle *const *handles, int32_t n, int32_t band_
     if (b->custom_alloc) b->alloc = *allocator;
     b->owns = false;
     b->pblock = nullptr;
-    b->own_shape = false;
+    b->base = BatchShape{kThreads, 16, 1};
     auto bail = [&](lbm_status rc) {
         batch_release_block(b);
         batch_free(b, b->pblock);
@@ -2782,7 +2785,6 @@ lbm_status lbm_batch_set_shape(lbm_batch *b, int32_t threads, int32_t band_rows)
     if (rc != LBM_OK) return rc;
     for (lbm_handle *h : b->hs) LBM_CUDA(cudaStreamSynchronize(h->stream));
     rc = batch_build(b, threads, band_rows, b->lookahead);
-    if (rc == LBM_OK) b->own_shape = true;
     if (rc == LBM_OK) clear_error();
     return rc;
 }
@@ -2795,7 +2797,6 @@ lbm_status lbm_batch_set_lookahead(lbm_batch *b, int32_t rows)
     if (rc != LBM_OK) return rc;
     for (lbm_handle *h : b->hs) LBM_CUDA(cudaStreamSynchronize(h->stream));
     rc = batch_build(b, b->threads, b->band_rows, rows);
-    if (rc == LBM_OK) b->own_shape = true;
     if (rc == LBM_OK) clear_error();
     return rc;
 }
@@ -2843,7 +2844,7 @@ lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *threads, i
             for (lbm_handle *h : b->hs) LBM_CUDA(cudaStreamSynchronize(h->stream));
             rc = batch_build(b, it->second.threads, it->second.rows, it->second.la);
             if (rc != LBM_OK) return rc;
-            b->own_shape = false;
+            b->base = it->second;
             if (threads) *threads = b->threads;
             if (band_rows) *band_rows = b->band_rows;
             if (us_per_step) *us_per_step = 0.0;
@@ -2935,10 +2936,10 @@ lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *threads, i
     // snapshot: partition again for the chosen shape
     rc = batch_build(b, best_t, best_r, best_la);
     if (rc != LBM_OK) return done(rc);
-    b->own_shape = false;
+    b->base = BatchShape{best_t, best_r, best_la};
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
-        g_tune_cache[key] = BatchShape{best_t, best_r, best_la};
+        g_tune_cache[key] = b->base;
     }
     if (threads) *threads = best_t;
     if (band_rows) *band_rows = best_r;
@@ -2965,7 +2966,8 @@ lbm_status lbm_batch_step(lbm_batch *b, int64_t n)
         par ^= (int)(n & 1);
         left = 0;
     }
-    if (left > 0 && b->pblock && !b->own_shape) {
+    const bool own_shape = b->threads != b->base.threads || b->band_rows != b->base.rows || b->lookahead != b->base.la;
+    if (left > 0 && b->pblock && !own_shape) {
         // pairs of passes of 8, 4 and 2 steps, then single steps
         for (int k = 0; k < lbm_batch::kPassKinds; ++k)
             for (; left >= 2 * kBatchPassSteps[k]; left -= 2 * kBatchPassSteps[k]) {
