@@ -3,8 +3,8 @@
 // snapshots every k steps, and the reverse sweep of the adjoint kernel, in
 // passes of several steps (lbm_pass.cuh) where the lattice and its sensors
 // allow, all replayed as CUDA graphs of 64-launch chunks on the handle's stream.
-// 1024^2 FP32, 2000 steps, 64 sensors: 25.8 -> 12.9 ms, with square-root
-// checkpoints 42.8 -> 20.7 ms.
+// 1024^2 FP32, 2000 steps, 64 sensors: 25.8 -> 11.7 ms, with square-root
+// checkpoints 42.8 -> 19.1 ms.
 #include "lbm_adjoint.h"
 #include "lbm_host.h"
 
