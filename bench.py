@@ -16,8 +16,9 @@ eight of them in one launch.
 Timing: the lattice first runs --prelude steps, then --warmup untimed steps
 and the call to be timed once; the --steps timed steps are one call between
 two CUDA events on the lattice's stream.  The state is 16x the L2, so no flush
-is needed.  The single-step kernel is also timed by the library's own event
-hooks (the roofline figure).  The rest of the JSON line: the former 4096 x 2048
+is needed.  `roofline` is of the kernel that the timed call launches, a pass of
+several steps: the two planes read and written once a pass.  The single-step kernel
+is also timed, by the library's own event hooks (`single_step`).  The rest of the JSON line: the former 4096 x 2048
 K-criterion headline (L2 flushed between steps), the 128 x 128 FP64
 configuration as graph replay, the 16-bit storage forms, the extensions
 (D2Q9, cracks in other directions, the Sec. 5.2 example), and last the
@@ -51,11 +52,15 @@ sys.path.insert(0, ROOT)
 METRIC = "GLUPS and HBM GB/s vs GB300 roofline; batched and adjoint vs plain FP32 forward"
 UNIT = "GLUPS"
 HEADLINE_STORAGE = "f32_lf"    # FP32 leapfrog storage: the state as w_n, w_{n-1}
-BYTES_PER_SITE = 12            # read w_n and w_{n-1}, write w_{n+1} (FP32)
+BYTES_PER_SITE = 12            # a single step: read w_n and w_{n-1}, write w_{n+1} (FP32)
+PASS_BYTES_PER_SITE = 16       # a pass of any number of steps: read both planes, write both
 WORKLOAD = "prescribed_v05_16384x16384_f32"
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "step_kernel_leapfrog_f32_8192x8192.md")
+PASS_SUMMARY = os.path.join(ROOT, "profiles", "pass_kernel_leapfrog_f32_8192x8192.md")
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_2206_12412_gb300", "csrc", f)
                   for f in ("lbm_kernels.cu", "lbm_rows.cuh", "lbm_internal.cuh", "lbm_crack.cuh")]
+PASS_SOURCES = [os.path.join(ROOT, "paper_2206_12412_gb300", "csrc", f)
+                for f in ("lbm_pass.cuh", "lbm_rows.cuh", "lbm_internal.cuh", "lbm_crack.cuh", "lbm_pass_plan.cu")]
 
 
 def r4(x):
@@ -110,23 +115,24 @@ def pass_launches(n: int, most: int = 8) -> int:
     return launches + 2 * m
 
 
-def kernel_source_sha256() -> str:
-    """Hash of the files that define the step kernel (concatenated)."""
+def kernel_source_sha256(sources=None) -> str:
+    """Hash of the files that define a kernel, the step kernel by default (concatenated)."""
     h = hashlib.sha256()
-    for path in KERNEL_SOURCES:
+    for path in sources or KERNEL_SOURCES:
         with open(path, "rb") as f:
             h.update(f.read())
     return h.hexdigest()
 
 
-def traffic_from_profile(sites: int):
-    """DRAM bytes of one step-kernel launch on `sites` sites, scaled from the
-    committed ncu summary of the 8192 x 8192 lattice (1 GB of state, so the
-    writes cannot stay in L2) by the sites per launch; None if there is no
-    summary or the kernel source changed since it was taken."""
+def traffic_from_profile(sites: int, summary=None, sources=None):
+    """DRAM bytes of one launch (of the step kernel by default) on `sites`
+    sites, scaled from the committed ncu summary of the 8192 x 8192 lattice
+    (0.5 GB of state, so most writes cannot stay in L2) by the sites of the
+    lattice; None if there is no summary or the kernel source changed since it
+    was taken."""
     try:
-        text = open(PROFILE_SUMMARY).read()
-        src = kernel_source_sha256()
+        text = open(summary or PROFILE_SUMMARY).read()
+        src = kernel_source_sha256(sources)
     except OSError:
         return None
     m = re.search(r"kernel_source_sha256:\s*([0-9a-f]{64})", text)
@@ -324,35 +330,35 @@ def profile_batched(lbm, W, torch, stream, steps, shape, count=256):
 
 
 def measure_batched(lbm, W, torch, stream, steps, peak, count=256, full_steps=None):
-    """Batched form: 256 independent lattices of uneven sizes, one launch per
-    step (graph replay), against the same lattices stepped one after another
-    with the single-lattice path.  The 840 MB of state exceed L2.  With
-    full_steps, the tuned batch then runs the configuration's whole length
-    (20 000 steps) as one timed run."""
+    """Batched form: 256 independent lattices of uneven sizes in passes of
+    several steps, against the same lattices stepped one after another with the
+    single-lattice path and against the batch's own single steps (one launch a
+    step, graph replay; the tuned shape with the other row lookahead, which is a
+    shape of the caller's own).  The 840 MB of state exceed L2.  With full_steps,
+    the batch then runs the configuration's whole length (20 000 steps) as one
+    timed run."""
     problems = W.batch_problems(count, seed=3)
     sites = sum(p["nx"] * p["ny"] for p in problems)
     lats = [lbm.Lattice(p, "f32", stream=stream) for p in problems]
     batch = lbm.Batch(lats)
-    batch.step(128)
-    t_d = timed(torch, stream, lambda: batch.step(steps))      # the default shape: 128 threads, 16-row bands
     batch.tune(trial_steps=8)
     batch.step(64)
     t_b = timed(torch, stream, lambda: batch.step(steps))
     info = batch.info()
-    # the tuned shape with the other row lookahead of the march
+    # single steps
     la = info["lookahead"]
     batch.set_lookahead(3 - la)
+    ctas = batch.info()["ctas"]
     batch.step(16)
     t_o = timed(torch, stream, lambda: batch.step(steps))
     batch.set_lookahead(la)
-    lookahead_ab = {str(la): r4(sites * steps / t_b / 1e9), str(3 - la): r4(sites * steps / t_o / 1e9)}
     full = None
     if full_steps:
         for l in lats:
             l.reset()
         t_f = timed(torch, stream, lambda: batch.step(full_steps))
         full = {"steps": full_steps, "s": r4(t_f), "glups": r4(sites * full_steps / t_f / 1e9)}
-    # the same shape as one persistent cooperative launch (grid barrier between steps)
+    # single steps as one persistent cooperative launch (grid barrier between steps)
     batch.set_persistent(True)
     batch.step(8)
     t_p = timed(torch, stream, lambda: batch.step(steps))
@@ -368,19 +374,15 @@ def measure_batched(lbm, W, torch, stream, steps, peak, count=256, full_steps=No
     blf.tune(trial_steps=8)
     blf.step(64)
     t_lf = timed(torch, stream, lambda: blf.step(steps))
-    lf_shape = blf.info()
     blf.close()
     for l in lf:
         l.close()
-    return {"n": len(problems), "sites": sites, "steps": steps, "ctas": info["ctas"],
-            "shape": [info["threads"], info["band_rows"], info["lookahead"]],
-            "glups_default_shape": r4(sites * steps / t_d / 1e9), "glups_by_lookahead": lookahead_ab,
-            "glups_persistent": r4(sites * steps / t_p / 1e9),
-            "glups_sequential": r4(sites * steps / t_s / 1e9), "speedup": r4(t_s / t_b),
-            "glups": r4(sites * steps / t_b / 1e9), "frac": r4(16 * sites * steps / t_b / 1e9 / peak),
-            "full_run": full,
-            "leapfrog": {"glups": r4(sites * steps / t_lf / 1e9), "frac": r4(12 * sites * steps / t_lf / 1e9 / peak),
-                         "shape": [lf_shape["threads"], lf_shape["band_rows"], lf_shape["lookahead"]]}}
+    return {"n": len(problems), "sites": sites, "steps": steps, "glups": r4(sites * steps / t_b / 1e9),
+            "glups_sequential": r4(sites * steps / t_s / 1e9), "speedup": r4(t_s / t_b), "full_run": full,
+            "single_steps": {"shape": [info["threads"], info["band_rows"], 3 - la], "ctas": ctas,
+                             "glups": r4(sites * steps / t_o / 1e9), "frac": r4(16 * sites * steps / t_o / 1e9 / peak),
+                             "glups_persistent": r4(sites * steps / t_p / 1e9)},
+            "leapfrog": {"glups": r4(sites * steps / t_lf / 1e9)}}
 
 
 def measure_adjoint(lbm, W, torch, stream, n_steps=None):
@@ -652,6 +654,11 @@ def run_profile(args, W, lbm, torch, rank):
         lat.set_bulk(True)
     lat.step(args.prelude)
     lat.sync()
+    if args.passes:   # one call of --steps steps, in passes
+        lat.step(args.steps)
+        lat.sync()
+        lat.close()
+        return 0
     big = p["nx"] * p["ny"] * 16 > (1 << 30)
     flush = None if big else torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
     lat.set_profiling(True)
@@ -735,8 +742,14 @@ def run_ours(args, rank, world, local):
     kern_bulk_s = kernel_seconds(lat)
     lat.set_bulk(False)
     lat.set_profiling(False)
-    achieved = BYTES_PER_SITE * sites / kern_s / 1e9
-    traffic = traffic_from_profile(sites)
+    single = {"kernel": "step_kernel<float, Lf>", "us": r4(kern_s * 1e6), "bytes_per_site": BYTES_PER_SITE,
+              "frac": r4(BYTES_PER_SITE * sites / kern_s / 1e9 / peak), "traffic": traffic_from_profile(sites),
+              "bulk_march_us": r4(kern_bulk_s * 1e6), "launch": lat.launch()}
+    # the passes of the timed call: the planes read and written once each
+    n_pass = pass_launches(args.steps)
+    pass_s = step_ms * 1e-3 / n_pass
+    achieved = PASS_BYTES_PER_SITE * sites / pass_s / 1e9
+    traffic = traffic_from_profile(sites, PASS_SUMMARY, PASS_SOURCES)
 
     # end to end through the public API with host buffers: upload the state
     # from pinned memory, run the steps, read back the fields and the
@@ -762,7 +775,6 @@ def run_ours(args, rank, world, local):
     plane = sites * 4
     h2d = 2 * plane / args.steps
     d2h = (2 * plane + len(hist["K"]) * (8 + 8 + 8 + 4)) / args.steps
-    launch = lat.launch()
     lat.close()
     del w_h, wd_h
     torch.cuda.empty_cache()
@@ -801,15 +813,15 @@ def run_ours(args, rank, world, local):
                    "crack": "prescribed v=0.5", "bc_mode": problem["bc_mode"], "prelude_steps": args.prelude + args.steps,
                    "l2": "inputs larger than L2 (2.1 GB state), no flush",
                    "parallelism": f"{world} independent replicas" if world > 1 else "single GPU",
-                   "launch": launch},
+                   "steps_per_launch": args.steps / n_pass},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
-                     "kernel": "step_kernel<float, Lf>", "kernel_ms": kern_s * 1e3, "bytes_per_site": BYTES_PER_SITE},
+                     "kernel": "pass_kernel<float, Lf>", "kernel_ms": pass_s * 1e3, "bytes_per_site": PASS_BYTES_PER_SITE,
+                     "limit": "instruction issue"},
         "e2e": {"value": world * sites * args.steps / e2e_s / 1e9, "unit": UNIT,
                 "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
         "gpu_launches": pass_launches(args.steps),
-        "bulk_march": {"us": r4(kern_bulk_s * 1e6), "frac": r4(BYTES_PER_SITE * sites / kern_bulk_s / 1e9 / peak),
-                       "register_us": r4(kern_s * 1e6)},
+        "single_step": single,
         "clocks": clk,
         "wall_s": r4(wall),
     }
@@ -857,6 +869,8 @@ def main():
     ap.add_argument("--storage", default="f32", choices=["f32", "f32_lf", "f32_bf16", "f32_f16", "f64"],
                     help="with --profile-only: the storage form")
     ap.add_argument("--bulk", action="store_true", help="with --profile-only: the bulk-copy march (lbm_set_bulk)")
+    ap.add_argument("--passes", action="store_true",
+                    help="with --profile-only: the steps as one call, in passes, instead of one by one")
     args = ap.parse_args()
     args.warmup = max(args.warmup, 3)
     rank, world, local = dist_env()
